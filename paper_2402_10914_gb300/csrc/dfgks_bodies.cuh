@@ -182,9 +182,6 @@ DFK_HD int lines_body(const Mesh& m, const SchemeConsts& S, const double* __rest
             al[s] = alpha[c];
         }
         CharBasis B = make_basis(Wc[2], Wc[3], S);
-        double Q[6][4];
-#pragma unroll
-        for (int s = 0; s < 6; ++s) project(B, Wc[s], Q[s]);
         const bool dfL = nn_less(nn_max(nn_max(al[1], al[2]), al[3]), S.alpha_thres);   // Eq. 34, cell f-1
         const bool dfR = nn_less(nn_max(nn_max(al[2], al[3]), al[4]), S.alpha_thres);   // Eq. 34, cell f
         ndf = (int)dfL + (int)dfR;
@@ -193,70 +190,103 @@ DFK_HD int lines_body(const Mesh& m, const SchemeConsts& S, const double* __rest
         // the cell-average reading of the DF states, stored before the reconstructions so that
         // the two cell states need not stay live through them
         if (S.df_states) lines[LR_DFC * ls + li] = df_alpha(Wc[2], Wc[3], S);
-        double qL[4], qLn[4], qR[4], qRn[4];
         // the limiter weight so far as tn / td (1 until a reconstruction gives less); fractions are
-        // compared by cross-multiplication (denominators >= 2), one division at the end
+        // compared by cross-multiplication, one division at the end
         double tn = 1.0, td = 1.0;
         int tlk = -1;                                     // the reconstruction that set it
+        double out[16];
+        if constexpr (!TAPE) {
+            const DiffBasis D = diff_basis(B);
+            double F[5][4];                               // first differences of the characteristic variables
 #pragma unroll
-        for (int k = 0; k < 4; ++k) {
-            double sL[5] = {Q[0][k], Q[1][k], Q[2][k], Q[3][k], Q[4][k]};
-            double sR[5] = {Q[5][k], Q[4][k], Q[3][k], Q[2][k], Q[1][k]};   // mirrored about cell f
-            double v, sl;
-            if (!TAPE) {
-                // both reconstructions at once: the mirrored stencils share two of their three
-                // quadratic second differences, and the weights' normalisers one division
+            for (int s = 0; s < 5; ++s) {
+                const double dW[4] = {Wc[s + 1][0] - Wc[s][0], Wc[s + 1][1] - Wc[s][1], Wc[s + 1][2] - Wc[s][2],
+                                      Wc[s + 1][3] - Wc[s][3]};
+                project_diff(D, dW, F[s]);
+            }
+            double qL[4], qLn[4], qR[4], qRn[4];          // face value minus cell value, slope
+            double xhi = 1.0, xlo = 1.0;                  // limiter: (1 + rmax^2) / (1 + rmin^2), the largest so far
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                const double s1 = F[1][k] - F[0][k], s2 = F[2][k] - F[1][k], s3 = F[3][k] - F[2][k], s4 = F[4][k] - F[3][k];
+                const double f3 = F[2][k], hf = 0.5 * f3;
+                // both sides' central quadratics at the face: cell f-1 at xi = +1/2, cell f mirrored
+                const double baseL = fma(-1.0 / 6.0, s2, hf), baseR = fma(-1.0 / 6.0, s3, -hf);
                 if (!dfL || !dfR || S.time_limiter) {
-                    const double h = 0.5 * kS13;
-                    const double d01 = h * (Q[0][k] - 2.0 * Q[1][k] + Q[2][k]);
-                    const double d12 = h * (Q[1][k] - 2.0 * Q[2][k] + Q[3][k]);
-                    const double d23 = h * (Q[2][k] - 2.0 * Q[3][k] + Q[4][k]);
-                    const double d34 = h * (Q[3][k] - 2.0 * Q[4][k] + Q[5][k]);
-                    const double aL[3] = {d01, d12, d23}, aR[3] = {d34, d23, d12};
-                    AO oL, oR;
-                    ao_finish_pair(ao_core(sL, aL, S), ao_core(sR, aR, S), S, oL, oR);
+                    const double eps = (k == 0 || k == 3) ? 4.0 * S.eps : S.eps;
+                    const double t1 = s2 - s1, t2 = s3 - s2, t3 = s4 - s3;
+                    const double w1 = second_difference_energy(s1, eps), w2 = second_difference_energy(s2, eps);
+                    const double w3 = second_difference_energy(s3, eps), w4 = second_difference_energy(s4, eps);
+                    const AOWeights L = ao_weights<+1>(F[1][k], f3, s1, s2, s3, w1, w2, w3, fma(0.5, s2, F[1][k]), t1 + t2,
+                                                       t2 - t1, eps, S);
+                    const AOWeights R = ao_weights<-1>(F[3][k], f3, s4, s3, s2, w4, w3, w2, fma(-0.5, s3, F[3][k]), t2 + t3,
+                                                       t3 - t2, eps, S);
+                    if (S.time_limiter) {
+                        if (nn_less(xhi * L.xmin, L.xmax * xlo)) { xhi = L.xmax; xlo = L.xmin; tlk = 2 * k; }
+                        if (nn_less(xhi * R.xmin, R.xmax * xlo)) { xhi = R.xmax; xlo = R.xmin; tlk = 2 * k + 1; }
+                    }
+                    const double h2 = 0.5 * t2, h12 = (1.0 / 12.0) * t2, h20 = (1.0 / 20.0) * t2, d03 = (1.0 / 3.0) * S.d[0];
+                    if (!dfL) {
+                        const double iv = ao_inverse_sum(L), p = L.y0 * t1;
+                        const double v = fma(d03, fma(h2, L.y2, p), L.x3 * fma(1.0 / 30.0, t1, h20));
+                        qL[k] = fma(-iv, v, baseL);
+                        qLn[k] = idn * fma(-iv, fma(S.d[0], p, L.x3 * h12), f3);
+                    }
+                    if (!dfR) {
+                        const double iv = ao_inverse_sum(R), p = R.y0 * t3;
+                        const double v = fma(d03, fma(h2, R.y2, p), R.x3 * fma(1.0 / 30.0, t3, h20));
+                        qR[k] = fma(iv, v, baseR);
+                        qRn[k] = idn * fma(-iv, fma(S.d[0], p, R.x3 * h12), f3);
+                    }
+                }
+                if (dfL) { qL[k] = al[2] * baseL; qLn[k] = idn * (al[2] * f3); }
+                if (dfR) { qR[k] = al[3] * baseR; qRn[k] = idn * (al[3] * f3); }
+            }
+            tn = 2.0 * xlo;
+            td = xhi + xlo;
+            back_project_diff(D, qL, out + LR_WL);
+            back_project_diff(D, qLn, out + LR_WLN);
+            back_project_diff(D, qR, out + LR_WR);
+            back_project_diff(D, qRn, out + LR_WRN);
+#pragma unroll
+            for (int k = 0; k < 4; ++k) { out[LR_WL + k] += Wc[2][k]; out[LR_WR + k] += Wc[3][k]; }
+        } else {
+            double Q[6][4], qL[4], qLn[4], qR[4], qRn[4];
+#pragma unroll
+            for (int s = 0; s < 6; ++s) project(B, Wc[s], Q[s]);
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                double sL[5] = {Q[0][k], Q[1][k], Q[2][k], Q[3][k], Q[4][k]};
+                double sR[5] = {Q[5][k], Q[4][k], Q[3][k], Q[2][k], Q[1][k]};   // mirrored about cell f
+                double v, sl;
+                if (!dfL || S.time_limiter) {
+                    AO o = weno_ao_t(sL, S, PlaneTape{ltape + li, ls}, 2 * k * AT_COUNT);
                     if (S.time_limiter) {
                         double n, d;
-                        limiter_fraction(oL, n, d);
+                        limiter_fraction(o, n, d);
                         if (nn_less(n * td, tn * d)) { tn = n; td = d; tlk = 2 * k; }
-                        limiter_fraction(oR, n, d);
+                    }
+                    if (!dfL) ao_at_right_edge(o, sL[2], v, sl);
+                }
+                if (dfL) df_at_right_edge(sL, al[2], v, sl);
+                qL[k] = v; qLn[k] = sl * idn;
+                if (!dfR || S.time_limiter) {
+                    AO o = weno_ao_t(sR, S, PlaneTape{ltape + li, ls}, (2 * k + 1) * AT_COUNT);
+                    if (S.time_limiter) {
+                        double n, d;
+                        limiter_fraction(o, n, d);
                         if (nn_less(n * td, tn * d)) { tn = n; td = d; tlk = 2 * k + 1; }
                     }
-                    if (!dfL) { ao_at_right_edge(oL, sL[2], v, sl); qL[k] = v; qLn[k] = sl * idn; }
-                    if (!dfR) { ao_at_right_edge(oR, sR[2], v, sl); qR[k] = v; qRn[k] = -sl * idn; }
+                    if (!dfR) ao_at_right_edge(o, sR[2], v, sl);
                 }
-                if (dfL) { df_at_right_edge(sL, al[2], v, sl); qL[k] = v; qLn[k] = sl * idn; }
-                if (dfR) { df_at_right_edge(sR, al[3], v, sl); qR[k] = v; qRn[k] = -sl * idn; }
-                continue;
+                if (dfR) df_at_right_edge(sR, al[3], v, sl);
+                qR[k] = v; qRn[k] = -sl * idn;
             }
-            if (!dfL || S.time_limiter) {
-                AO o = TAPE ? weno_ao_t(sL, S, PlaneTape{ltape + li, ls}, 2 * k * AT_COUNT) : weno_ao(sL, S);
-                if (S.time_limiter) {
-                    double n, d;
-                    limiter_fraction(o, n, d);
-                    if (nn_less(n * td, tn * d)) { tn = n; td = d; tlk = 2 * k; }
-                }
-                if (!dfL) ao_at_right_edge(o, sL[2], v, sl);
-            }
-            if (dfL) df_at_right_edge(sL, al[2], v, sl);
-            qL[k] = v; qLn[k] = sl * idn;
-            if (!dfR || S.time_limiter) {
-                AO o = TAPE ? weno_ao_t(sR, S, PlaneTape{ltape + li, ls}, (2 * k + 1) * AT_COUNT) : weno_ao(sR, S);
-                if (S.time_limiter) {
-                    double n, d;
-                    limiter_fraction(o, n, d);
-                    if (nn_less(n * td, tn * d)) { tn = n; td = d; tlk = 2 * k + 1; }
-                }
-                if (!dfR) ao_at_right_edge(o, sR[2], v, sl);
-            }
-            if (dfR) df_at_right_edge(sR, al[3], v, sl);
-            qR[k] = v; qRn[k] = -sl * idn;
+            back_project(B, qL, out + LR_WL);
+            back_project(B, qLn, out + LR_WLN);
+            back_project(B, qR, out + LR_WR);
+            back_project(B, qRn, out + LR_WRN);
         }
-        double out[16];
-        back_project(B, qL, out + LR_WL);
-        back_project(B, qLn, out + LR_WLN);
-        back_project(B, qR, out + LR_WR);
-        back_project(B, qRn, out + LR_WRN);
 #pragma unroll
         for (int q = 0; q < 16; ++q) lines[q * ls + li] = out[q];
         lines[LR_TL * ls + li] = tn / td;
@@ -295,66 +325,81 @@ DFK_HD int faces_body(const Mesh& m, const SchemeConsts& S, const double* __rest
         B.ic = lines[LR_IC * ls + l0]; B.H = lines[LR_H * ls + l0]; B.b1 = lines[LR_B1 * ls + l0];
         B.b2 = lines[LR_B2 * ls + l0]; B.q2 = lines[LR_Q2 * ls + l0];
         const int wbase = side == 0 ? LR_WL : LR_WR;
-        double Q[5][4];
-#pragma unroll
-        for (int b = 0; b < 5; ++b) {
-            long long lb = g.line(f, t + Geo<DIR>::sigma * (b - 2));
-            double Wl[4];
-#pragma unroll
-            for (int k = 0; k < 4; ++k) Wl[k] = lines[(wbase + k) * ls + lb];
-            project(B, Wl, Q[b]);
-        }
         const int ncell = f - 1 + side;
         double al[3];
 #pragma unroll
         for (int b = 0; b < 3; ++b) al[b] = alpha[g.cell(m, ncell, t + Geo<DIR>::sigma * (b - 1))];
         const bool df = nn_less(nn_max(nn_max(al[0], al[1]), al[2]), S.alpha_thres);    // Eq. 34, tangential
         ndf = (int)df;
-        double qv[2][4], qt[2][4];
+        double Wv[2][4], Wd[2][4];               // values and tangential slopes at the two Gauss points
         const double idt = g.idtan;
         const long long e = (long long)side * g.nfaces() + g.face(f, t);
-        if (!TAPE && !df) {
-            // the four components' reconstructions in two pairs, one division per pair
+        double Wl[5][4];
 #pragma unroll
-            for (int k = 0; k < 4; k += 2) {
-                const double sa[5] = {Q[0][k], Q[1][k], Q[2][k], Q[3][k], Q[4][k]};
-                const double sb[5] = {Q[0][k + 1], Q[1][k + 1], Q[2][k + 1], Q[3][k + 1], Q[4][k + 1]};
-                double da[3], db[3];
-                ao_second_differences(sa, da);
-                ao_second_differences(sb, db);
-                AO oa, ob;
-                ao_finish_pair(ao_core(sa, da, S), ao_core(sb, db, S), S, oa, ob);
+        for (int b = 0; b < 5; ++b) {
+            const long long lb = g.line(f, t + Geo<DIR>::sigma * (b - 2));
+#pragma unroll
+            for (int k = 0; k < 4; ++k) Wl[b][k] = lines[(wbase + k) * ls + lb];
+        }
+        if constexpr (!TAPE) {
+            const DiffBasis D = diff_basis(B);
+            double F[4][4], qv[2][4], qt[2][4];
+#pragma unroll
+            for (int b = 0; b < 4; ++b) {
+                const double dW[4] = {Wl[b + 1][0] - Wl[b][0], Wl[b + 1][1] - Wl[b][1], Wl[b + 1][2] - Wl[b][2],
+                                      Wl[b + 1][3] - Wl[b][3]};
+                project_diff(D, dW, F[b]);
+            }
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                const double s0 = F[1][k] - F[0][k], s1 = F[2][k] - F[1][k], s2 = F[3][k] - F[2][k];
+                const double a11 = fma(0.5, s1, F[1][k]);
                 double v[2], s[2];
-                ao_at_gauss(oa, sa[2], v, s);
+                if (df) df_diff_at_gauss(a11, s1, al[1], v, s);
+                else {
+                    const double eps = (k == 0 || k == 3) ? 4.0 * S.eps : S.eps;
+                    const double t1 = s1 - s0, t2 = s2 - s1, T = t1 + t2, U = t2 - t1;
+                    const AOWeights o = ao_weights<+1>(F[1][k], F[2][k], s0, s1, s2, second_difference_energy(s0, eps),
+                                                       second_difference_energy(s1, eps), second_difference_energy(s2, eps),
+                                                       a11, T, U, eps, S);
+                    ao_diff_at_gauss(o, a11, s1, t1, t2, T, U, S, v, s);
+                }
                 qv[0][k] = v[0]; qv[1][k] = v[1];
                 qt[0][k] = s[0] * idt; qt[1][k] = s[1] * idt;
-                ao_at_gauss(ob, sb[2], v, s);
-                qv[0][k + 1] = v[0]; qv[1][k + 1] = v[1];
-                qt[0][k + 1] = s[0] * idt; qt[1][k + 1] = s[1] * idt;
+            }
+#pragma unroll
+            for (int mm = 0; mm < 2; ++mm) {
+                back_project_diff(D, qv[mm], Wv[mm]);
+                back_project_diff(D, qt[mm], Wd[mm]);
+#pragma unroll
+                for (int k = 0; k < 4; ++k) Wv[mm][k] += Wl[2][k];
             }
         } else {
+            double Q[5][4], qv[2][4], qt[2][4];
+#pragma unroll
+            for (int b = 0; b < 5; ++b) project(B, Wl[b], Q[b]);
 #pragma unroll
             for (int k = 0; k < 4; ++k) {
                 double sq[5] = {Q[0][k], Q[1][k], Q[2][k], Q[3][k], Q[4][k]};
                 double v[2], s[2];
                 if (df) df_at_gauss(sq, al[1], v, s);
                 else {
-                    AO o = TAPE ? weno_ao_t(sq, S, PlaneTape{ftape + e, gs}, k * AT_COUNT) : weno_ao(sq, S);
+                    AO o = weno_ao_t(sq, S, PlaneTape{ftape + e, gs}, k * AT_COUNT);
                     ao_at_gauss(o, sq[2], v, s);
                 }
                 qv[0][k] = v[0]; qv[1][k] = v[1];
                 qt[0][k] = s[0] * idt; qt[1][k] = s[1] * idt;
             }
+#pragma unroll
+            for (int mm = 0; mm < 2; ++mm) { back_project(B, qv[mm], Wv[mm]); back_project(B, qt[mm], Wd[mm]); }
         }
         const int nbase = side == 0 ? LR_WLN : LR_WRN;
         int fbits = 0;
 #pragma unroll
         for (int mm = 0; mm < 2; ++mm) {
             double Wg[4], Wt[4], Wn[4];
-            back_project(B, qv[mm], Wg);
-            back_project(B, qt[mm], Wt);
 #pragma unroll
-            for (int k = 0; k < 4; ++k) Wn[k] = lines[(nbase + k) * ls + l0];
+            for (int k = 0; k < 4; ++k) { Wg[k] = Wv[mm][k]; Wt[k] = Wd[mm][k]; Wn[k] = lines[(nbase + k) * ls + l0]; }
             if (S.gp_fallback && !physical_state(Wg, S.gm1)) {
                 long long c = g.cell(m, ncell, t);
 #pragma unroll
