@@ -381,7 +381,7 @@ static void adjoint_dir(const Mesh& m, const SchemeConsts& S, int flux, const Ad
                         const double* alpha, const double* dtp, const SweepBuffers& B, double* lb, double* gbuf,
                         double* Wb, cudaStream_t s, KernelTimer* T) {
     // the forward sweep's 1-D grids (sweep_xy)
-    const dim3 blk(128);
+    const dim3 blk(kSweepThreads);
     const dim3 gf(sweep_blocks(faces_lx<DIR>(m), faces_ly<DIR>(m)), 2);
     const dim3 gl(sweep_blocks(lines_lx<DIR>(m), lines_ly<DIR>(m)));
     cudaMemsetAsync(lb, 0, sizeof(double) * LR_COUNT * B.line_stride, s);

@@ -63,7 +63,8 @@ template <int DIR> DFK_HD int faces_ly(const Mesh& m) { return DIR == 0 ? m.ny :
 // (i mod lx, i / lx), so only the grid's last warp is partly idle, where a 2-D grid of 32-wide rows
 // would idle part of every row's last warp (15 of 416 lanes on a 401-face row).  Threads past the
 // end get ay >= ly, which the bodies' bounds checks reject.
-inline unsigned sweep_blocks(int lx, int ly) { return (unsigned)(((long long)lx * ly + 127) / 128); }
+constexpr int kSweepThreads = 128;
+inline unsigned sweep_blocks(int lx, int ly, int threads = kSweepThreads) { return (unsigned)(((long long)lx * ly + threads - 1) / threads); }
 __device__ __forceinline__ void sweep_xy(int lx, int& ax, int& ay) {
     const int i = (int)(blockIdx.x * blockDim.x + threadIdx.x);
     ax = i % lx;
@@ -185,7 +186,6 @@ DFK_HD int lines_body(const Mesh& m, const SchemeConsts& S, const double* __rest
         const bool dfL = nn_less(nn_max(nn_max(al[1], al[2]), al[3]), S.alpha_thres);   // Eq. 34, cell f-1
         const bool dfR = nn_less(nn_max(nn_max(al[2], al[3]), al[4]), S.alpha_thres);   // Eq. 34, cell f
         ndf = (int)dfL + (int)dfR;
-        const double idn = g.idn;
         const long long li = g.line(f, t);
         // the cell-average reading of the DF states, stored before the reconstructions so that
         // the two cell states need not stay live through them
@@ -197,26 +197,28 @@ DFK_HD int lines_body(const Mesh& m, const SchemeConsts& S, const double* __rest
         double out[16];
         if constexpr (!TAPE) {
             const DiffBasis D = diff_basis(B);
-            double F[5][4];                               // first differences of the characteristic variables
+            const Real idn = g.idn;
+            Real F[5][4];                               // first differences of the characteristic variables
 #pragma unroll
             for (int s = 0; s < 5; ++s) {
-                const double dW[4] = {Wc[s + 1][0] - Wc[s][0], Wc[s + 1][1] - Wc[s][1], Wc[s + 1][2] - Wc[s][2],
-                                      Wc[s + 1][3] - Wc[s][3]};
+                Real dW[4];
+#pragma unroll
+                for (int k = 0; k < 4; ++k) dW[k] = Real::raw(Wc[s + 1][k]) - Real::raw(Wc[s][k]);
                 project_diff(D, dW, F[s]);
             }
-            double qL[4], qLn[4], qR[4], qRn[4];          // face value minus cell value, slope
-            double xhi = 1.0, xlo = 1.0;                  // limiter: (1 + rmax^2) / (1 + rmin^2), the largest so far
+            Real qL[4], qLn[4], qR[4], qRn[4];          // face value minus cell value, slope
+            Real xhi = 1.0, xlo = 1.0;                  // limiter: (1 + rmax^2) / (1 + rmin^2), the largest so far
 #pragma unroll
             for (int k = 0; k < 4; ++k) {
-                const double s1 = F[1][k] - F[0][k], s2 = F[2][k] - F[1][k], s3 = F[3][k] - F[2][k], s4 = F[4][k] - F[3][k];
-                const double f3 = F[2][k], hf = 0.5 * f3;
+                const Real s1 = F[1][k] - F[0][k], s2 = F[2][k] - F[1][k], s3 = F[3][k] - F[2][k], s4 = F[4][k] - F[3][k];
+                const Real f3 = F[2][k], hf = 0.5 * f3;
                 // both sides' central quadratics at the face: cell f-1 at xi = +1/2, cell f mirrored
-                const double baseL = fma(-1.0 / 6.0, s2, hf), baseR = fma(-1.0 / 6.0, s3, -hf);
+                const Real baseL = fma(-1.0 / 6.0, s2, hf), baseR = fma(-1.0 / 6.0, s3, -hf);
                 if (!dfL || !dfR || S.time_limiter) {
-                    const double eps = (k == 0 || k == 3) ? 4.0 * S.eps : S.eps;
-                    const double t1 = s2 - s1, t2 = s3 - s2, t3 = s4 - s3;
-                    const double w1 = second_difference_energy(s1, eps), w2 = second_difference_energy(s2, eps);
-                    const double w3 = second_difference_energy(s3, eps), w4 = second_difference_energy(s4, eps);
+                    const Real eps = (k == 0 || k == 3) ? Real(4.0 * S.eps) : Real(S.eps);
+                    const Real t1 = s2 - s1, t2 = s3 - s2, t3 = s4 - s3;
+                    const Real w1 = second_difference_energy(s1, eps), w2 = second_difference_energy(s2, eps);
+                    const Real w3 = second_difference_energy(s3, eps), w4 = second_difference_energy(s4, eps);
                     const AOWeights L = ao_weights<+1>(F[1][k], f3, s1, s2, s3, w1, w2, w3, fma(0.5, s2, F[1][k]), t1 + t2,
                                                        t2 - t1, eps, S);
                     const AOWeights R = ao_weights<-1>(F[3][k], f3, s4, s3, s2, w4, w3, w2, fma(-0.5, s3, F[3][k]), t2 + t3,
@@ -225,32 +227,39 @@ DFK_HD int lines_body(const Mesh& m, const SchemeConsts& S, const double* __rest
                         if (nn_less(xhi * L.xmin, L.xmax * xlo)) { xhi = L.xmax; xlo = L.xmin; tlk = 2 * k; }
                         if (nn_less(xhi * R.xmin, R.xmax * xlo)) { xhi = R.xmax; xlo = R.xmin; tlk = 2 * k + 1; }
                     }
-                    const double h2 = 0.5 * t2, h12 = (1.0 / 12.0) * t2, h20 = (1.0 / 20.0) * t2, d03 = (1.0 / 3.0) * S.d[0];
+                    const Real h2 = 0.5 * t2, h12 = (1.0 / 12.0) * t2, h20 = (1.0 / 20.0) * t2, d03 = (1.0 / 3.0) * S.d[0];
                     if (!dfL) {
-                        const double iv = ao_inverse_sum(L), p = L.y0 * t1;
-                        const double v = fma(d03, fma(h2, L.y2, p), L.x3 * fma(1.0 / 30.0, t1, h20));
+                        const Real iv = ao_inverse_sum(L), p = L.y0 * t1;
+                        const Real v = fma(d03, fma(h2, L.y2, p), L.x3 * fma(1.0 / 30.0, t1, h20));
                         qL[k] = fma(-iv, v, baseL);
                         qLn[k] = idn * fma(-iv, fma(S.d[0], p, L.x3 * h12), f3);
                     }
                     if (!dfR) {
-                        const double iv = ao_inverse_sum(R), p = R.y0 * t3;
-                        const double v = fma(d03, fma(h2, R.y2, p), R.x3 * fma(1.0 / 30.0, t3, h20));
+                        const Real iv = ao_inverse_sum(R), p = R.y0 * t3;
+                        const Real v = fma(d03, fma(h2, R.y2, p), R.x3 * fma(1.0 / 30.0, t3, h20));
                         qR[k] = fma(iv, v, baseR);
                         qRn[k] = idn * fma(-iv, fma(S.d[0], p, R.x3 * h12), f3);
                     }
                 }
-                if (dfL) { qL[k] = al[2] * baseL; qLn[k] = idn * (al[2] * f3); }
-                if (dfR) { qR[k] = al[3] * baseR; qRn[k] = idn * (al[3] * f3); }
+                if (dfL) { qL[k] = Real::raw(al[2]) * baseL; qLn[k] = idn * (Real::raw(al[2]) * f3); }
+                if (dfR) { qR[k] = Real::raw(al[3]) * baseR; qRn[k] = idn * (Real::raw(al[3]) * f3); }
             }
-            tn = 2.0 * xlo;
-            td = xhi + xlo;
-            back_project_diff(D, qL, out + LR_WL);
-            back_project_diff(D, qLn, out + LR_WLN);
-            back_project_diff(D, qR, out + LR_WR);
-            back_project_diff(D, qRn, out + LR_WRN);
+            tn = Real(2.0 * xlo).v;
+            td = (xhi + xlo).v;
+            Real w[16];
+            back_project_diff(D, qL, w + LR_WL);
+            back_project_diff(D, qLn, w + LR_WLN);
+            back_project_diff(D, qR, w + LR_WR);
+            back_project_diff(D, qRn, w + LR_WRN);
 #pragma unroll
-            for (int k = 0; k < 4; ++k) { out[LR_WL + k] += Wc[2][k]; out[LR_WR + k] += Wc[3][k]; }
+            for (int k = 0; k < 4; ++k) {
+                w[LR_WL + k] = w[LR_WL + k] + Real::raw(Wc[2][k]);
+                w[LR_WR + k] = w[LR_WR + k] + Real::raw(Wc[3][k]);
+            }
+#pragma unroll
+            for (int k = 0; k < 16; ++k) out[k] = w[k].v;
         } else {
+            const double idn = g.idn;
             double Q[6][4], qL[4], qLn[4], qR[4], qRn[4];
 #pragma unroll
             for (int s = 0; s < 6; ++s) project(B, Wc[s], Q[s]);
@@ -332,7 +341,6 @@ DFK_HD int faces_body(const Mesh& m, const SchemeConsts& S, const double* __rest
         const bool df = nn_less(nn_max(nn_max(al[0], al[1]), al[2]), S.alpha_thres);    // Eq. 34, tangential
         ndf = (int)df;
         double Wv[2][4], Wd[2][4];               // values and tangential slopes at the two Gauss points
-        const double idt = g.idtan;
         const long long e = (long long)side * g.nfaces() + g.face(f, t);
         double Wl[5][4];
 #pragma unroll
@@ -343,22 +351,24 @@ DFK_HD int faces_body(const Mesh& m, const SchemeConsts& S, const double* __rest
         }
         if constexpr (!TAPE) {
             const DiffBasis D = diff_basis(B);
-            double F[4][4], qv[2][4], qt[2][4];
+            const Real idt = g.idtan;
+            Real F[4][4], qv[2][4], qt[2][4];
 #pragma unroll
             for (int b = 0; b < 4; ++b) {
-                const double dW[4] = {Wl[b + 1][0] - Wl[b][0], Wl[b + 1][1] - Wl[b][1], Wl[b + 1][2] - Wl[b][2],
-                                      Wl[b + 1][3] - Wl[b][3]};
+                Real dW[4];
+#pragma unroll
+                for (int k = 0; k < 4; ++k) dW[k] = Real::raw(Wl[b + 1][k]) - Real::raw(Wl[b][k]);
                 project_diff(D, dW, F[b]);
             }
 #pragma unroll
             for (int k = 0; k < 4; ++k) {
-                const double s0 = F[1][k] - F[0][k], s1 = F[2][k] - F[1][k], s2 = F[3][k] - F[2][k];
-                const double a11 = fma(0.5, s1, F[1][k]);
-                double v[2], s[2];
-                if (df) df_diff_at_gauss(a11, s1, al[1], v, s);
+                const Real s0 = F[1][k] - F[0][k], s1 = F[2][k] - F[1][k], s2 = F[3][k] - F[2][k];
+                const Real a11 = fma(0.5, s1, F[1][k]);
+                Real v[2], s[2];
+                if (df) df_diff_at_gauss(a11, s1, Real::raw(al[1]), v, s);
                 else {
-                    const double eps = (k == 0 || k == 3) ? 4.0 * S.eps : S.eps;
-                    const double t1 = s1 - s0, t2 = s2 - s1, T = t1 + t2, U = t2 - t1;
+                    const Real eps = (k == 0 || k == 3) ? Real(4.0 * S.eps) : Real(S.eps);
+                    const Real t1 = s1 - s0, t2 = s2 - s1, T = t1 + t2, U = t2 - t1;
                     const AOWeights o = ao_weights<+1>(F[1][k], F[2][k], s0, s1, s2, second_difference_energy(s0, eps),
                                                        second_difference_energy(s1, eps), second_difference_energy(s2, eps),
                                                        a11, T, U, eps, S);
@@ -369,12 +379,14 @@ DFK_HD int faces_body(const Mesh& m, const SchemeConsts& S, const double* __rest
             }
 #pragma unroll
             for (int mm = 0; mm < 2; ++mm) {
-                back_project_diff(D, qv[mm], Wv[mm]);
-                back_project_diff(D, qt[mm], Wd[mm]);
+                Real w[4], d[4];
+                back_project_diff(D, qv[mm], w);
+                back_project_diff(D, qt[mm], d);
 #pragma unroll
-                for (int k = 0; k < 4; ++k) Wv[mm][k] += Wl[2][k];
+                for (int k = 0; k < 4; ++k) { Wv[mm][k] = (w[k] + Real::raw(Wl[2][k])).v; Wd[mm][k] = d[k].v; }
             }
         } else {
+            const double idt = g.idtan;
             double Q[5][4], qv[2][4], qt[2][4];
 #pragma unroll
             for (int b = 0; b < 5; ++b) project(B, Wl[b], Q[b]);
@@ -467,7 +479,7 @@ DFK_HD void flux_point(int dir, const SchemeConsts& S, const FluxSite& site, con
         gks_flux_t(L, R, sl, sr, dt, S, F, dF, PlaneTape{tape + e, fs});
     } else {
         const FlowState sl = side_state(L.W, S), sr = side_state(R.W, S);
-        fr[FR_ALPHA * fs + e] = df_alpha_sides(sl, sr, S);
+        fr[FR_ALPHA * fs + e] = df_alpha_sides(sl, sr, S).v;
         if (S.df_states) fr[FR_ALPHA * fs + e] = lines[LR_DFC * ls + site.li];
         if (ALPHA_ONLY) return;
         if (FLUX == 0) gks_flux_sides(L, R, sl, sr, dt, S, F, dF);

@@ -54,6 +54,61 @@ DFK_HD bool nn_less(double a, double b) { return dbits(a) < dbits(b); }
 // lo < a < hi for lo, hi > 0: false for a negative, -0 or NaN
 DFK_HD bool in_range(double a, double lo, double hi) { const long long x = dbits(a); return dbits(lo) < x && x < dbits(hi); }
 
+// FP64 arithmetic with every operand in a vector register.  An SM's two FP64 units take a warp's fused
+// multiply-add in 16 cycles when all three operands are vector registers, and in 19 when one is an
+// immediate, a constant-bank or a uniform register, as they do for an addition or a multiplication of two
+// operands (measured with dependent and independent chains, 4 to 16 warps per SM).  The forward sweeps keep
+// these units busy all the time, so their arithmetic runs in this type: x + y is fma(x, 1, y) and x y is
+// fma(x, y, -0), the same bits as the two-operand forms, with 1, -0 and every other constant held as a value
+// the compiler cannot prove uniform.  A product met by a sum fuses, as the compiler fuses plain doubles.
+// Per 400 x 400 step: face lines 0.906 -> 0.807 ms, tangential 1.050 -> 0.934, flux 1.381 -> 1.311.
+#ifdef __CUDACC__
+static __constant__ unsigned kOpaqueZero;      // never written
+#endif
+DFK_HD double vreg(double c) {
+#ifdef __CUDA_ARCH__
+    return __hiloint2double(__double2hiint(c) | (int)(threadIdx.x & kOpaqueZero), __double2loint(c));
+#else
+    return c;
+#endif
+}
+struct Real {
+    double v;
+    DFK_HD Real() {}
+    DFK_HD Real(double c) : v(vreg(c)) {}                                   // a constant or a parameter
+    static DFK_HD Real raw(double x) { Real r; r.v = x; return r; }            // a value already in a register
+    DFK_HD Real operator-() const { return raw(-v); }
+    friend DFK_HD Real fma(Real a, Real b, Real c) { return raw(::fma(a.v, b.v, c.v)); }
+    friend DFK_HD Real fabs(Real a) { return raw(::fabs(a.v)); }
+};
+struct RealProd {
+    Real a, b;
+#ifndef DFK_TWO_OPERAND_FORMS
+    DFK_HD operator Real() const { return Real::raw(::fma(a.v, b.v, vreg(-0.0))); }
+#else
+    DFK_HD operator Real() const { return Real::raw(a.v * b.v); }
+#endif
+    DFK_HD RealProd operator-() const { RealProd p; p.a = -a; p.b = b; return p; }
+};
+DFK_HD RealProd operator*(Real a, Real b) { RealProd p; p.a = a; p.b = b; return p; }
+#ifndef DFK_TWO_OPERAND_FORMS
+DFK_HD Real operator+(Real a, Real b) { return Real::raw(::fma(a.v, vreg(1.0), b.v)); }
+DFK_HD Real operator-(Real a, Real b) { return Real::raw(::fma(a.v, vreg(1.0), -b.v)); }
+#else       // a build for flop counters, which would read two flops in fma(x, 1, y)
+DFK_HD Real operator+(Real a, Real b) { return Real::raw(a.v + b.v); }
+DFK_HD Real operator-(Real a, Real b) { return Real::raw(a.v - b.v); }
+#endif
+DFK_HD Real operator+(RealProd p, Real c) { return fma(p.a, p.b, c); }
+DFK_HD Real operator+(Real c, RealProd p) { return fma(p.a, p.b, c); }
+DFK_HD Real operator-(RealProd p, Real c) { return fma(p.a, p.b, -c); }
+DFK_HD Real operator-(Real c, RealProd p) { return fma(-p.a, p.b, c); }
+DFK_HD Real operator+(RealProd p, RealProd q) { return fma(p.a, p.b, (Real)q); }
+DFK_HD Real operator-(RealProd p, RealProd q) { return fma(p.a, p.b, -(Real)q); }
+DFK_HD Real nn_max(Real a, Real b) { return Real::raw(nn_max(a.v, b.v)); }
+DFK_HD Real nn_min(Real a, Real b) { return Real::raw(nn_min(a.v, b.v)); }
+DFK_HD bool nn_less(Real a, Real b) { return nn_less(a.v, b.v); }
+DFK_HD bool in_range(Real a, double lo, double hi) { return in_range(a.v, lo, hi); }
+
 struct SchemeConsts {
     double gamma, gm1, K, inv_K2;          // gamma, gamma-1, internal degrees of freedom, 1/(K+2)
     double r2g;                            // sqrt(2/gamma): 1/c = sqrt(2/gamma) sqrt(lambda)
@@ -282,58 +337,59 @@ DFK_HD AO weno_ao(const double q[5], const SchemeConsts& S) { return weno_ao_t(q
 // 1/x for x in [1e-300, 1e300]: the hardware's approximation (2^-20) refined by one third-order
 // Householder step y (1 + e + e^2), e = 1 - x y.  Largest error 0.51 ulp; 3 FP64 instructions against
 // the 5 of a division, and no slow path.
-DFK_HD double rcp(double x) {
+DFK_HD Real rcp(Real x) {
 #ifdef __CUDA_ARCH__
-    double y;
-    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
-    const double e = fma(-x, y, 1.0);
+    Real y;
+    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y.v) : "d"(x.v));
+    const Real e = fma(-x, y, 1.0);
     return fma(y, fma(e, e, e), y);
 #else
-    return 1.0 / x;
+    return Real::raw(1.0 / x.v);
 #endif
 }
 
 // weights of one reconstruction: c_3 = x3 / sum, c_0 = d0 y0 / sum, c_2 = d0 y2 / sum, and the extreme
 // x_k, all carried scaled by (3 prod)^2, prod = the product of the four beta_k + eps (the scale cancels)
-struct AOWeights { double x3, y0, y2, sum, xmax, xmin; };
+struct AOWeights { Real x3, y0, y2, sum, xmax, xmin; };
 
 // 13/12 s^2 + eps, shared by the reconstructions that use the second difference s
-DFK_HD double second_difference_energy(double s, double eps) { return fma((13.0 / 12.0) * s, s, eps); }
+DFK_HD Real second_difference_energy(Real s, Real eps) { return fma((13.0 / 12.0) * s, s, eps); }
 
 // SGN -1: a stencil mirrored about its cell, given by the unmirrored differences (the odd ones change
 // sign).  w_k: second_difference_energy of s_k.
 template <int SGN>
-DFK_HD AOWeights ao_weights(double fb, double ff, double s0, double s1, double s2, double w0, double w1, double w2,
-                            double a11, double T, double U, double eps, const SchemeConsts& S) {
-    constexpr double h = 0.5 * SGN;
-    const double a10 = fma(h, s0, fb), a12 = fma(-h, s2, ff);
-    const double m1 = fma(-1.0 / 12.0, T, a11), m2 = fma(-11.0 / 130.0, U, s1);
-    const double e0 = fma(a10, a10, w0), e1 = fma(a11, a11, w1), e2 = fma(a12, a12, w2);
-    double e3 = fma((1421461.0 / 1310400.0) * U, U, eps);
+DFK_HD AOWeights ao_weights(Real fb, Real ff, Real s0, Real s1, Real s2, Real w0, Real w1, Real w2,
+                            Real a11, Real T, Real U, Real eps, const SchemeConsts& S) {
+    const Real h = 0.5 * SGN;
+    const Real a10 = fma(h, s0, fb), a12 = fma(-h, s2, ff);
+    const Real m1 = fma(-1.0 / 12.0, T, a11), m2 = fma(-11.0 / 130.0, U, s1);
+    const Real e0 = fma(a10, a10, w0), e1 = fma(a11, a11, w1), e2 = fma(a12, a12, w2);
+    Real e3 = fma((1421461.0 / 1310400.0) * U, U, eps);
     e3 = fma((781.0 / 2880.0) * T, T, e3);
     e3 = fma((13.0 / 12.0) * m2, m2, e3);
     e3 = fma(m1, m1, e3);
     // Eq. 37: tau = (|b3-b0| + |b3-b1| + |b3-b2|)/3; r_k = tau / (beta_k + eps) = t_k / (3 prod)
-    const double tau3 = (fabs(e3 - e0) + fabs(e3 - e1)) + fabs(e3 - e2);
-    const double p01 = e0 * e1, p23 = e2 * e3, prod = p01 * p23;
-    const double g01 = tau3 * p01, g23 = tau3 * p23;
-    double t0 = e1 * g23, t1 = e0 * g23, t2 = e3 * g01, t3 = e2 * g01;
-    double p2;
-    const double tm = nn_max(nn_max(t0, t1), nn_max(t2, t3));
-    if (in_range(prod, 1e-75, 1e75) && nn_less(tm, 1e75)) {
-        const double p3 = 3.0 * prod;
+    const Real tau3 = (fabs(e3 - e0) + fabs(e3 - e1)) + fabs(e3 - e2);
+    const Real p01 = e0 * e1, p23 = e2 * e3, prod = p01 * p23;
+    const Real g01 = tau3 * p01, g23 = tau3 * p23;
+    Real t0 = e1 * g23, t1 = e0 * g23, t2 = e3 * g01, t3 = e2 * g01;
+    Real p2;
+    const Real tm = nn_max(nn_max(t0, t1), nn_max(t2, t3));
+    if (in_range(prod, 1e-75, 1e75) && nn_less(tm.v, 1e75)) {
+        const Real p3 = 3.0 * prod;
         p2 = p3 * p3;
     } else {                                       // extreme data: the ratios themselves
-        t0 = tau3 / (3.0 * e0); t1 = tau3 / (3.0 * e1); t2 = tau3 / (3.0 * e2); t3 = tau3 / (3.0 * e3);
+        t0 = Real::raw(tau3.v / (3.0 * e0.v)); t1 = Real::raw(tau3.v / (3.0 * e1.v));
+        t2 = Real::raw(tau3.v / (3.0 * e2.v)); t3 = Real::raw(tau3.v / (3.0 * e3.v));
         p2 = 1.0;
     }
-    const double tmax = nn_max(nn_max(t0, t1), nn_max(t2, t3)), tmin = nn_min(nn_min(t0, t1), nn_min(t2, t3));
+    const Real tmax = nn_max(nn_max(t0, t1), nn_max(t2, t3)), tmin = nn_min(nn_min(t0, t1), nn_min(t2, t3));
     AOWeights o;
-    const double z3 = t3 * t3;
+    const Real z3 = t3 * t3;
     o.x3 = fma(t3, t3, p2);
     o.y0 = fma(t0, t0, -z3);
     o.y2 = fma(t2, t2, -z3);
-    const double y1 = fma(t1, t1, -z3);
+    const Real y1 = fma(t1, t1, -z3);
     o.sum = fma(S.d[0], o.y0 + o.y2, fma(S.d[1], y1, o.x3));
     o.xmax = fma(tmax, tmax, p2);                  // the time limiter's; dropped where it is not used
     o.xmin = fma(tmin, tmin, p2);
@@ -341,25 +397,25 @@ DFK_HD AOWeights ao_weights(double fb, double ff, double s0, double s1, double s
 }
 
 // 1/sum: a positive normal number unless the data overflow
-DFK_HD double ao_inverse_sum(const AOWeights& o) { return in_range(o.sum, 1e-300, 1e300) ? rcp(o.sum) : 1.0 / o.sum; }
+DFK_HD Real ao_inverse_sum(const AOWeights& o) { return in_range(o.sum, 1e-300, 1e300) ? rcp(o.sum) : Real::raw(1.0 / o.sum.v); }
 
 // values minus q0 and d/deta (unscaled) at the two Gauss points eta = -g (m=1), +g (m=2), g = sqrt(3)/6
-DFK_HD void ao_diff_at_gauss(const AOWeights& o, double a11, double s1, double t1, double t2, double T, double U,
-                             const SchemeConsts& S, double val[2], double slope[2]) {
-    const double g = kGaussEta;
-    const double iv = ao_inverse_sum(o), di = S.d[0] * iv, c3 = o.x3 * iv;
-    const double p = (o.y0 * di) * t1, r = (o.y2 * di) * t2;         // c_0 t1, c_2 t2
-    const double c3T = c3 * T, c3U = c3 * U;
-    const double B = fma(-0.5, p + r, a11);
-    const double O = g * fma(-7.0 / 72.0, c3T, B), Es = fma(-1.0 / 12.0, c3T, B);
-    const double Os = fma(-1.0 / 9.0, c3U, s1 - (p - r)), E = (-1.0 / 4320.0) * c3U;
+DFK_HD void ao_diff_at_gauss(const AOWeights& o, Real a11, Real s1, Real t1, Real t2, Real T, Real U,
+                             const SchemeConsts& S, Real val[2], Real slope[2]) {
+    const Real g = kGaussEta;
+    const Real iv = ao_inverse_sum(o), di = S.d[0] * iv, c3 = o.x3 * iv;
+    const Real p = (o.y0 * di) * t1, r = (o.y2 * di) * t2;         // c_0 t1, c_2 t2
+    const Real c3T = c3 * T, c3U = c3 * U;
+    const Real B = fma(-0.5, p + r, a11);
+    const Real O = g * fma(-7.0 / 72.0, c3T, B), Es = fma(-1.0 / 12.0, c3T, B);
+    const Real Os = fma(-1.0 / 9.0, c3U, s1 - (p - r)), E = (-1.0 / 4320.0) * c3U;
     val[0] = E - O; val[1] = E + O;
     slope[0] = fma(-g, Os, Es); slope[1] = fma(g, Os, Es);
 }
 
 // the zero-mean DF quadratic's (Sect. 3.3) values minus q0 and slopes there
-DFK_HD void df_diff_at_gauss(double a11, double s1, double alpha, double val[2], double slope[2]) {
-    const double g = kGaussEta, Es = alpha * a11, O = g * Es, Os = (g * alpha) * s1;
+DFK_HD void df_diff_at_gauss(Real a11, Real s1, Real alpha, Real val[2], Real slope[2]) {
+    const Real g = kGaussEta, Es = alpha * a11, O = g * Es, Os = (g * alpha) * s1;
     val[0] = -O; val[1] = O;
     slope[0] = Es - Os; slope[1] = Es + Os;
 }
@@ -368,25 +424,26 @@ DFK_HD void df_diff_at_gauss(double a11, double s1, double alpha, double val[2],
 // doubled (Q_0 = k + m, Q_3 = k - m): their smoothness indicators then carry 4 eps, which leaves the
 // weights as they are, and the back projection halves them again.  10 instructions each way.
 struct DiffBasis {
-    double b1, b1u, b1v, b2, ic, uic, v;                     // projection
-    double u, hc, hH, huc, q2;                               // back projection
+    Real b1, b1u, b1v, b2, ic, uic, v;                     // projection
+    Real u, hc, hH, huc, q2;                               // back projection
 };
 DFK_HD DiffBasis diff_basis(const CharBasis& B) {
     DiffBasis D;
-    D.b1 = B.b1; D.b1u = B.b1 * B.u; D.b1v = B.b1 * B.v; D.b2 = B.b2; D.ic = B.ic; D.uic = B.u * B.ic; D.v = B.v;
-    D.u = B.u; D.hc = 0.5 * B.c; D.hH = 0.5 * B.H; D.huc = B.u * D.hc; D.q2 = B.q2;
+    D.b1 = Real::raw(B.b1); D.b2 = Real::raw(B.b2); D.ic = Real::raw(B.ic); D.u = Real::raw(B.u); D.v = Real::raw(B.v); D.q2 = Real::raw(B.q2);
+    D.b1u = D.b1 * D.u; D.b1v = D.b1 * D.v; D.uic = D.u * D.ic;
+    D.hc = 0.5 * Real::raw(B.c); D.hH = 0.5 * Real::raw(B.H); D.huc = D.u * D.hc;
     return D;
 }
-DFK_HD void project_diff(const DiffBasis& D, const double W[4], double Q[4]) {
-    const double k = fma(D.b1, W[3], fma(-D.b1v, W[2], fma(-D.b1u, W[1], D.b2 * W[0])));
-    const double m = fma(-D.ic, W[1], D.uic * W[0]);
+DFK_HD void project_diff(const DiffBasis& D, const Real W[4], Real Q[4]) {
+    const Real k = fma(D.b1, W[3], fma(-D.b1v, W[2], fma(-D.b1u, W[1], D.b2 * W[0])));
+    const Real m = fma(-D.ic, W[1], D.uic * W[0]);
     Q[0] = k + m;
     Q[1] = W[0] - k;
     Q[2] = fma(-D.v, W[0], W[2]);
     Q[3] = k - m;
 }
-DFK_HD void back_project_diff(const DiffBasis& D, const double Q[4], double W[4]) {
-    const double s = Q[0] + Q[3], d = Q[3] - Q[0];
+DFK_HD void back_project_diff(const DiffBasis& D, const Real Q[4], Real W[4]) {
+    const Real s = Q[0] + Q[3], d = Q[3] - Q[0];
     W[0] = fma(0.5, s, Q[1]);
     W[1] = fma(D.u, W[0], D.hc * d);
     W[2] = fma(D.v, W[0], Q[2]);
@@ -798,13 +855,13 @@ DFK_HD void gks_flux_t(const GPState& L, const GPState& R, double dt, const Sche
 // ------------------------------------------------------------------------------------------
 
 // rcp() where its range holds, a division elsewhere (negative, zero, extreme)
-DFK_HD double rcp_or_div(double x) { return in_range(x, 1e-300, 1e300) ? rcp(x) : 1.0 / x; }
+DFK_HD Real rcp_or_div(Real x) { return in_range(x, 1e-300, 1e300) ? rcp(x) : Real::raw(1.0 / x.v); }
 
 // velocities, pressure, theta = p/rho and hq = (U^2 + V^2)/2 of a state; for the two sides of a Gauss
 // point also rs = 1/sqrt(2 theta), which the half-space moments and the DF factor's sound speed share
-struct FlowState { double rho, ir, U, V, p, th, hq, rs; };
+struct FlowState { Real rho, ir, U, V, p, th, hq, rs; };
 
-DFK_HD FlowState flow_state(const double W[4], const SchemeConsts& S) {
+DFK_HD FlowState flow_state(const Real W[4], const SchemeConsts& S) {
     FlowState s;
     s.rho = W[0];
     s.ir = rcp_or_div(W[0]);
@@ -816,24 +873,25 @@ DFK_HD FlowState flow_state(const double W[4], const SchemeConsts& S) {
     return s;
 }
 DFK_HD FlowState side_state(const double W[4], const SchemeConsts& S) {
-    FlowState s = flow_state(W, S);
-    s.rs = rsqrt(2.0 * s.th);
+    const Real w[4] = {Real::raw(W[0]), Real::raw(W[1]), Real::raw(W[2]), Real::raw(W[3])};
+    FlowState s = flow_state(w, S);
+    s.rs = Real::raw(rsqrt(Real(2.0 * s.th).v));
     return s;
 }
 
 // DF factor of one Gauss point (Sect. 3.2, Eq. 33) from its two sides: 1/c = sqrt(2/gamma) / sqrt(2 theta),
 // |p_l - p_r| (1/p_l + 1/p_r) with 1/p = 2 rs^2 / rho
-DFK_HD double df_alpha_sides(const FlowState& l, const FlowState& r, const SchemeConsts& S) {
-    const double cl = S.r2g * l.rs, cr = S.r2g * r.rs;
-    const double dn = fma(l.U, cl, -(r.U * cr)), dt = fma(l.V, cl, -(r.V * cr));
-    const double ips = fma(l.rs * l.rs, l.ir, (r.rs * r.rs) * r.ir);
-    const double D = fma(2.0 * fabs(l.p - r.p), ips, fma(dn, dn, dt * dt));
+DFK_HD Real df_alpha_sides(const FlowState& l, const FlowState& r, const SchemeConsts& S) {
+    const Real cl = S.r2g * l.rs, cr = S.r2g * r.rs;
+    const Real dn = fma(l.U, cl, -(r.U * cr)), dt = fma(l.V, cl, -(r.V * cr));
+    const Real ips = fma(l.rs * l.rs, l.ir, (r.rs * r.rs) * r.ir);
+    const Real D = fma(2.0 * fabs(l.p - r.p), ips, fma(dn, dn, dt * dt));
     return rcp_or_div(fma(D, D, 1.0));
 }
 
 // r0, r1, r2, q3 and p' of the state along a gradient of its conserved variables
-struct FlowGrad { double r0, r1, r2, q3, dp; };
-DFK_HD FlowGrad flow_grad(const FlowState& s, const double d[4], const SchemeConsts& S) {
+struct FlowGrad { Real r0, r1, r2, q3, dp; };
+DFK_HD FlowGrad flow_grad(const FlowState& s, const Real d[4], const SchemeConsts& S) {
     FlowGrad g;
     g.r0 = d[0];
     g.r1 = fma(-s.U, d[0], d[1]);
@@ -843,10 +901,15 @@ DFK_HD FlowGrad flow_grad(const FlowState& s, const double d[4], const SchemeCon
     return g;
 }
 
+DFK_HD FlowGrad point_grad(const FlowState& s, const double d[4], const SchemeConsts& S) {
+    const Real w[4] = {Real::raw(d[0]), Real::raw(d[1]), Real::raw(d[2]), Real::raw(d[3])};
+    return flow_grad(s, w, S);
+}
+
 // moments m_k = <u^k>, k <= 4, and their derivatives' terms: e1[k] = dm_k/dU, e2[k] = dm_k/dtheta
-struct HalfMom { double m[5], e1[5], e2[5]; };
+struct HalfMom { Real m[5], e1[5], e2[5]; };
 DFK_HD void finish_moments(const FlowState& s, HalfMom& h) {
-    const double th2 = 2.0 * s.th, th3 = 3.0 * s.th;
+    const Real th2 = 2.0 * s.th, th3 = 3.0 * s.th;
     h.m[2] = fma(s.U, h.m[1], s.th * h.m[0]);
     h.m[3] = fma(s.U, h.m[2], th2 * h.m[1]);
     h.m[4] = fma(s.U, h.m[3], th3 * h.m[2]);
@@ -855,18 +918,18 @@ DFK_HD void finish_moments(const FlowState& s, HalfMom& h) {
 }
 template <int HALF>
 DFK_HD void half_moments(const FlowState& s, HalfMom& h) {
-    const double x = s.U * s.rs, G = exp(-x * x);
+    const Real x = s.U * s.rs, G = Real::raw(exp(Real(-x * x).v));
     // the marginal distribution at u = 0, exp(-U^2/(2 theta)) / sqrt(2 pi theta)
-    const double phi = (0.56418958354775628695 * s.rs) * G;
+    const Real phi = (0.56418958354775628695 * s.rs) * G;
     // erfc(|x|)/2 from the scaled function and the Gaussian above; erfc(-|x|) = 2 - erfc(|x|)
 #ifdef __CUDA_ARCH__
-    const double t = 0.5 * G * erfcx(fabs(x));
+    const Real t = 0.5 * G * Real::raw(erfcx(::fabs(x.v)));
 #else
-    const double t = 0.5 * erfc(fabs(x));
+    const Real t = 0.5 * erfc(::fabs(x.v));
 #endif
-    const bool xpos = dbits(x) >= 0;
+    const bool xpos = dbits(x.v) >= 0;
     h.m[0] = (HALF > 0) == xpos ? 1.0 - t : t;
-    const double sphi = HALF > 0 ? phi : -phi;
+    const Real sphi = HALF > 0 ? phi : -phi;
     h.m[1] = fma(s.U, h.m[0], s.th * sphi);
     h.e1[0] = sphi;
     h.e2[0] = -(sphi * x) * s.rs;
@@ -874,20 +937,20 @@ DFK_HD void half_moments(const FlowState& s, HalfMom& h) {
     finish_moments(s, h);
 }
 
-DFK_HD double grad_mom(const HalfMom& h, const FlowGrad& g, int k) { return fma(g.r0, h.m[k], fma(g.r1, h.e1[k], g.q3 * h.e2[k])); }
+DFK_HD Real grad_mom(const HalfMom& h, const FlowGrad& g, int k) { return fma(g.r0, h.m[k], fma(g.r1, h.e1[k], g.q3 * h.e2[k])); }
 
 // from the frame of tangential velocity V to the laboratory's, for a vector of psi moments
-DFK_HD void to_lab(double V, double hV2, double o[4]) {
+DFK_HD void to_lab(Real V, Real hV2, Real o[4]) {
     o[3] = fma(V, o[2], fma(hV2, o[0], o[3]));
     o[2] = fma(V, o[0], o[2]);
 }
 
 // rho <u^2 a_x psi> + rho <u v a_y psi> in the state's own tangential frame
 // (k1 = (K+1)/2, k3 = (K+3)/2; Nx[j] = N_{2+j} of the normal gradient, Ny[j] = N_{1+j} of the tangential)
-DFK_HD void transport(const FlowState& s, const HalfMom& h, const FlowGrad& x, const FlowGrad& y, const double Nx[3],
-                      const double Ny[3], double k1, double k3, double o[4]) {
-    const double G2 = fma(s.th, Nx[0], x.q3 * h.m[2]), G1 = fma(s.th, Ny[0], y.q3 * h.m[1]);
-    const double v1 = y.r2 * h.m[1];
+DFK_HD void transport(const FlowState& s, const HalfMom& h, const FlowGrad& x, const FlowGrad& y, const Real Nx[3],
+                      const Real Ny[3], Real k1, Real k3, Real o[4]) {
+    const Real G2 = fma(s.th, Nx[0], x.q3 * h.m[2]), G1 = fma(s.th, Ny[0], y.q3 * h.m[1]);
+    const Real v1 = y.r2 * h.m[1];
     o[0] = fma(s.V, Ny[0], Nx[0]) + v1;
     o[1] = fma(s.V, Ny[1], fma(y.r2, h.m[2], Nx[1]));
     o[2] = fma(s.V, v1, fma(x.r2, h.m[2], G1));
@@ -898,22 +961,22 @@ DFK_HD void transport(const FlowState& s, const HalfMom& h, const FlowGrad& x, c
 // g1 = rho <u^2 a_x psi> + rho <u v a_y psi>.  The left side (HALF > 0) comes first and sets them, the
 // right one adds (an addition to zero is not free on the FP64 units)
 template <int HALF>
-DFK_HD void side_add(const double o[4], double to[4]) {
+DFK_HD void side_add(const Real o[4], Real to[4]) {
 #pragma unroll
     for (int i = 0; i < 4; ++i) to[i] = HALF > 0 ? o[i] : to[i] + o[i];
 }
 template <int HALF>
-DFK_HD void side_sums(const FlowState& s, const FlowGrad& x, const FlowGrad& y, const HalfMom& h, double k1, double k3,
-                      double c[4], double cx[4], double cy[4], double g0[4], double g1[4]) {
-    const double hV2 = 0.5 * s.V * s.V, rk = fma(k1, s.th, hV2), rm0 = s.rho * h.m[0], rm1 = s.rho * h.m[1],
+DFK_HD void side_sums(const FlowState& s, const FlowGrad& x, const FlowGrad& y, const HalfMom& h, Real k1, Real k3,
+                      Real c[4], Real cx[4], Real cy[4], Real g0[4], Real g1[4]) {
+    const Real hV2 = 0.5 * s.V * s.V, rk = fma(k1, s.th, hV2), rm0 = s.rho * h.m[0], rm1 = s.rho * h.m[1],
                  rm2 = s.rho * h.m[2];
-    double Nx[3], Ny[3], o[4];
+    Real Nx[3], Ny[3], o[4];
     o[0] = rm0; o[1] = rm1; o[2] = s.V * rm0; o[3] = fma(0.5, rm2, rk * rm0);
     side_add<HALF>(o, c);
     o[0] = rm1; o[1] = rm2; o[2] = s.V * rm1; o[3] = fma(0.5 * s.rho, h.m[3], rk * rm1);
     side_add<HALF>(o, g0);
     {
-        const double N0 = grad_mom(h, x, 0);
+        const Real N0 = grad_mom(h, x, 0);
         Nx[0] = grad_mom(h, x, 2);
         o[0] = N0; o[1] = grad_mom(h, x, 1); o[2] = x.r2 * h.m[0];
         o[3] = fma(0.5, Nx[0], k1 * fma(s.th, N0, x.q3 * h.m[0]));
@@ -922,7 +985,7 @@ DFK_HD void side_sums(const FlowState& s, const FlowGrad& x, const FlowGrad& y, 
         Nx[1] = grad_mom(h, x, 3); Nx[2] = grad_mom(h, x, 4);
     }
     {
-        const double N0 = grad_mom(h, y, 0);
+        const Real N0 = grad_mom(h, y, 0);
         Ny[0] = grad_mom(h, y, 1); Ny[1] = grad_mom(h, y, 2);
         o[0] = N0; o[1] = Ny[0]; o[2] = y.r2 * h.m[0];
         o[3] = fma(0.5, Ny[1], k1 * fma(s.th, N0, y.q3 * h.m[0]));
@@ -938,7 +1001,7 @@ DFK_HD void side_sums(const FlowState& s, const FlowGrad& x, const FlowGrad& y, 
 // the Euler equations' time derivative of a state with gradients x, y, as a gradient
 DFK_HD FlowGrad euler_time_grad(const FlowState& s, const FlowGrad& x, const FlowGrad& y, const SchemeConsts& S) {
     FlowGrad t;
-    const double div = x.r1 + y.r2;
+    const Real div = x.r1 + y.r2;
     t.r0 = -fma(s.U, x.r0, fma(s.V, y.r0, div));
     t.r1 = -fma(s.U, x.r1, fma(s.V, y.r1, x.dp));
     t.r2 = -fma(s.U, x.r2, fma(s.V, y.r2, y.dp));
@@ -949,32 +1012,33 @@ DFK_HD FlowGrad euler_time_grad(const FlowState& s, const FlowGrad& x, const Flo
 
 // under the tau = tau_n reading: rho <u A psi> of one side, A from the side's own compatibility condition
 DFK_HD void side_time_sum(const FlowState& s, const FlowGrad& x, const FlowGrad& y, const HalfMom& h, const SchemeConsts& S,
-                          double k1, double g2[4]) {
+                          Real k1, Real g2[4]) {
     const FlowGrad t = euler_time_grad(s, x, y, S);
-    double o[4];
-    const double N1 = grad_mom(h, t, 1);
+    Real o[4];
+    const Real N1 = grad_mom(h, t, 1);
     o[0] = N1; o[1] = grad_mom(h, t, 2); o[2] = t.r2 * h.m[1];
     o[3] = fma(0.5, grad_mom(h, t, 3), k1 * fma(s.th, N1, t.q3 * h.m[1]));
     to_lab(s.V, 0.5 * s.V * s.V, o);
 #pragma unroll
-    for (int i = 0; i < 4; ++i) g2[i] += o[i];
+    for (int i = 0; i < 4; ++i) g2[i] = g2[i] + o[i];
 }
 
 // sl, sr: side_state of L.W and R.W
-DFK_HD void gks_flux_sides(const GPState& L, const GPState& R, const FlowState& sl, const FlowState& sr, double dt,
+DFK_HD void gks_flux_sides(const GPState& L, const GPState& Rt, const FlowState& sl, const FlowState& sr, double dtv,
                            const SchemeConsts& S, double F[4], double dF[4]) {
-    const double k1 = 0.5 * (S.K + 1.0), k3 = 0.5 * (S.K + 3.0);
+    const Real dt = dtv;
+    const Real k1 = 0.5 * (S.K + 1.0), k3 = 0.5 * (S.K + 3.0);
     // Sect. 3.4: the equilibrium state and its slopes by kinetic weighting, and the sides' flux moments
-    double Wc[4], Wcx[4], Wcy[4], dg[4], g1[4], g2[4] = {0, 0, 0, 0};
+    Real Wc[4], Wcx[4], Wcy[4], dg[4], g1[4], g2[4] = {0.0, 0.0, 0.0, 0.0};
     {
-        const FlowGrad x = flow_grad(sl, L.Wn, S), y = flow_grad(sl, L.Wt, S);
+        const FlowGrad x = point_grad(sl, L.Wn, S), y = point_grad(sl, L.Wt, S);
         HalfMom h;
         half_moments<+1>(sl, h);
         side_sums<+1>(sl, x, y, h, k1, k3, Wc, Wcx, Wcy, dg, g1);
         if (S.tau_reading == 1) side_time_sum(sl, x, y, h, S, k1, g2);
     }
     {
-        const FlowGrad x = flow_grad(sr, R.Wn, S), y = flow_grad(sr, R.Wt, S);
+        const FlowGrad x = point_grad(sr, Rt.Wn, S), y = point_grad(sr, Rt.Wt, S);
         HalfMom h;
         half_moments<-1>(sr, h);
         side_sums<-1>(sr, x, y, h, k1, k3, Wc, Wcx, Wcy, dg, g1);
@@ -982,58 +1046,58 @@ DFK_HD void gks_flux_sides(const GPState& L, const GPState& R, const FlowState& 
     }
     // the equilibrium state: c0 = rho <u psi>, c1 = rho <u^2 a_x psi> + rho <u v a_y psi>, c2 = rho <u A psi>
     const FlowState c = flow_state(Wc, S);
-    double c0[4], c1[4], c2[4];
+    Real c0[4], c1[4], c2[4];
     {
         const FlowGrad x = flow_grad(c, Wcx, S), y = flow_grad(c, Wcy, S), t = euler_time_grad(c, x, y, S);
         HalfMom h;                                   // the full space: no boundary terms
         h.m[0] = 1.0; h.m[1] = c.U;
         h.e1[0] = 0.0; h.e2[0] = 0.0; h.e2[1] = 0.0;
         finish_moments(c, h);
-        const double hV2 = 0.5 * c.V * c.V, hU2 = 0.5 * c.U * c.U, gg = 0.5 * (S.K + 4.0);   // gamma / (gamma - 1)
-        const double ru = Wc[1];
+        const Real hV2 = 0.5 * c.V * c.V, hU2 = 0.5 * c.U * c.U, gg = 0.5 * (S.K + 4.0);   // gamma / (gamma - 1)
+        const Real ru = Wc[1];
         c0[0] = ru;
         c0[1] = fma(ru, c.U, c.p);
         c0[2] = 0.0;
         c0[3] = fma(hU2, ru, (gg * c.U) * c.p);
         to_lab(c.V, hV2, c0);
-        const double n1 = fma(c.U, t.r0, t.r1);
+        const Real n1 = fma(c.U, t.r0, t.r1);
         c2[0] = n1;
         c2[1] = fma(c.U, n1 + t.r1, t.dp);
         c2[2] = c.U * t.r2;
         c2[3] = fma(hU2, fma(2.0, t.r1, n1), gg * fma(c.U, t.dp, c.th * t.r1));
         to_lab(c.V, hV2, c2);
-        const double Nx[3] = {grad_mom(h, x, 2), grad_mom(h, x, 3), grad_mom(h, x, 4)};
-        const double Ny[3] = {fma(c.U, y.r0, y.r1), grad_mom(h, y, 2), grad_mom(h, y, 3)};
+        const Real Nx[3] = {grad_mom(h, x, 2), grad_mom(h, x, 3), grad_mom(h, x, 4)};
+        const Real Ny[3] = {fma(c.U, y.r0, y.r1), grad_mom(h, y, 2), grad_mom(h, y, 3)};
         transport(c, h, x, y, Nx, Ny, k1, k3, c1);
         to_lab(c.V, hV2, c1);
     }
     // numerical collision time (Sect. 2.2) and the time coefficients of Eq. 27 (4 G(dt/2) - G(dt)) / dt and
     // 4 (G(dt) - 2 G(dt/2)) / dt^2, combined with E(dt) = E(dt/2)^2
-    const double q = (sl.p - sr.p) * rcp_or_div(sl.p + sr.p);
-    const double rT = fma(S.C2, fabs(q), S.C1);        // tau_n / dt
-    double E2 = 0.0, r = 0.0;
-    if (dbits(rT) > 0) { E2 = exp(-0.5 * rcp_or_div(rT)); r = rT; }   // rT >= 0
-    const double om = 1.0 - E2, om2 = om * om, rom = r * om;
-    const double gF = rom * (3.0 - E2), gD = -4.0 * (r * om2) * rcp_or_div(dt);
+    const Real q = (sl.p - sr.p) * rcp_or_div(sl.p + sr.p);
+    const Real rT = fma(S.C2, fabs(q), S.C1);        // tau_n / dt
+    Real E2 = 0.0, r = 0.0;
+    if (dbits(rT.v) > 0) { E2 = Real::raw(exp(Real(-0.5 * rcp_or_div(rT)).v)); r = rT; }   // rT >= 0
+    const Real om = 1.0 - E2, om2 = om * om, rom = r * om;
+    const Real gF = rom * (3.0 - E2), gD = -4.0 * (r * om2) * rcp_or_div(dt);
     if (S.tau_reading == 1) {
-        const double T = r * dt, E1 = E2 * E2, idt = 1.0 / dt, TT = 2.0 * T * T, S3 = om * (3.0 - E2);
-        const double aF = TT * S3 * idt - 2.0 * T * E2 + T * E1 - T;
-        const double aD = 4.0 * (-TT * om2 + T * dt * E2 * om) * idt * idt;
-        const double AF = -T + T * gF, AD = 4.0 * T * T * om2 * idt * idt, BF = -T * T * S3 * idt;
+        const Real T = r * dt, E1 = E2 * E2, idt = Real::raw(1.0 / dt.v), TT = 2.0 * T * T, S3 = om * (3.0 - E2);
+        const Real aF = TT * S3 * idt - 2.0 * T * E2 + T * E1 - T;
+        const Real aD = 4.0 * (-TT * om2 + T * dt * E2 * om) * idt * idt;
+        const Real AF = -T + T * gF, AD = 4.0 * T * T * om2 * idt * idt, BF = -T * T * S3 * idt;
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
-            const double d = dg[i] - c0[i];
-            F[i] = c0[i] + gF * d + aF * (c1[i] - g1[i]) - T * g1[i] + AF * c2[i] + BF * g2[i];
-            dF[i] = c2[i] + gD * d + aD * (c1[i] - g1[i]) + AD * (g2[i] - c2[i]);
+            const Real d = dg[i] - c0[i];
+            F[i] = (c0[i] + gF * d + aF * (c1[i] - g1[i]) - T * g1[i] + AF * c2[i] + BF * g2[i]).v;
+            dF[i] = (c2[i] + gD * d + aD * (c1[i] - g1[i]) + AD * (g2[i] - c2[i])).v;
         }
         return;
     }
-    const double aF = (r * dt) * (gF + (om2 - 1.0)), aD = 4.0 * rom * (E2 - rom);
+    const Real aF = (r * dt) * (gF + (om2 - 1.0)), aD = 4.0 * rom * (E2 - rom);
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
-        const double d = dg[i] - c0[i], e = c1[i] - g1[i];
-        F[i] = fma(gF, d, fma(aF, e, c0[i]));
-        dF[i] = fma(gD, d, fma(aD, e, c2[i]));
+        const Real d = dg[i] - c0[i], e = c1[i] - g1[i];
+        F[i] = fma(gF, d, fma(aF, e, c0[i])).v;
+        dF[i] = fma(gD, d, fma(aD, e, c2[i])).v;
     }
 }
 

@@ -218,7 +218,7 @@ __global__ void __launch_bounds__(128) k_flux_xy(Mesh m, SchemeConsts S, const d
 void launch_sweep_xy(const Mesh& m, const SchemeConsts& S, int flux, bool alpha_only, const double* W,
                      const double* alpha, const double* dtp, const SweepBuffers& Bx, const SweepBuffers& By,
                      DevState* st, const int* halt, cudaStream_t s, KernelTimer* T) {
-    const dim3 blk(128);
+    const dim3 blk(kSweepThreads);
     const int nl0 = (int)sweep_blocks(lines_lx<0>(m), lines_ly<0>(m)), nl1 = (int)sweep_blocks(lines_lx<1>(m), lines_ly<1>(m));
     const int nf0 = (int)sweep_blocks(faces_lx<0>(m), faces_ly<0>(m)), nf1 = (int)sweep_blocks(faces_lx<1>(m), faces_ly<1>(m));
     const bool tape = Bx.ltape != nullptr;      // both directions' record sets carry tapes or neither
@@ -265,7 +265,7 @@ static void sweep_dir(const Mesh& m, const SchemeConsts& S, int flux, bool alpha
                       const int* halt, cudaStream_t s, KernelTimer* T) {
     // 1-D grids over the row-major index spaces of face lines ((nn+1) x (nt+4)) and of face sides /
     // Gauss points ((nn+1) x nt, two of each per face: grid y); rows run along the contiguous index
-    const dim3 blk(128);
+    const dim3 blk(kSweepThreads);
     const dim3 gl(sweep_blocks(lines_lx<DIR>(m), lines_ly<DIR>(m)));
     if (T) T->begin(KK_LINES);
     if (B.ltape) k_lines<DIR, true><<<gl, blk, 0, s>>>(m, S, W, alpha, B.lines, B.line_stride, st, halt, B.ltape);

@@ -63,34 +63,36 @@ int main(int argc, char** argv) {
         double big = 0.0;
         for (double x : q) big = std::max(big, fabs(x));
         double v[6], w[6], lim;
+        Real wr[4];
         reference(q, S, v, lim);
         for (int mir = 0; mir < 2; ++mir) {          // the stencil given as it is, and as the mirror of its reverse
             double p[5];
             for (int i = 0; i < 5; ++i) p[i] = mir ? q[4 - i] : q[i];
-            double f[4], s[3];
+            Real f[4], s[3];
             for (int i = 0; i < 4; ++i) f[i] = p[i + 1] - p[i];
             for (int i = 0; i < 3; ++i) s[i] = f[i + 1] - f[i];
-            const double t1 = s[1] - s[0], t2 = s[2] - s[1];
-            double e[3];
+            const Real t1 = s[1] - s[0], t2 = s[2] - s[1];
+            Real e[3];
             for (int i = 0; i < 3; ++i) e[i] = second_difference_energy(s[i], S.eps);
             if (!mir) {
-                const double a11 = fma(0.5, s[1], f[1]), T = t1 + t2, Uu = t2 - t1;
+                const Real a11 = fma(0.5, s[1], f[1]), T = t1 + t2, Uu = t2 - t1;
                 const AOWeights A = ao_weights<+1>(f[1], f[2], s[0], s[1], s[2], e[0], e[1], e[2], a11, T, Uu, S.eps, S);
-                ao_diff_at_gauss(A, a11, s[1], t1, t2, T, Uu, S, w + 2, w + 4);
+                ao_diff_at_gauss(A, a11, s[1], t1, t2, T, Uu, S, wr, wr + 2);
+                for (int i = 0; i < 4; ++i) w[2 + i] = wr[i].v;
                 for (int i = 0; i < 4; ++i) worst = std::max(worst, fabs(w[2 + i] + (i < 2 ? q[2] : 0.0) - v[2 + i]) / big);
-                const double iv = ao_inverse_sum(A), y = A.y0 * t1;
-                const double val = 0.5 * f[2] - s[1] / 6.0 - iv * (S.d[0] / 3.0 * (y + 0.5 * t2 * A.y2) + A.x3 * (t1 / 30.0 + t2 / 20.0));
+                const double iv = ao_inverse_sum(A).v, y = Real(A.y0 * t1).v;
+                const double val = 0.5 * f[2].v - s[1].v / 6.0 - iv * (S.d[0] / 3.0 * (y + 0.5 * t2.v * A.y2.v) + A.x3.v * (t1.v / 30.0 + t2.v / 20.0));
                 worst = std::max(worst, fabs(q[2] + val - v[0]) / big);
-                worst = std::max(worst, fabs(f[2] - iv * (S.d[0] * y + A.x3 * t2 / 12.0) - v[1]) / big);
-                wlim = std::max(wlim, fabs(2.0 * A.xmin / (A.xmax + A.xmin) - lim));
+                worst = std::max(worst, fabs(f[2].v - iv * (S.d[0] * y + A.x3.v * t2.v / 12.0) - v[1]) / big);
+                wlim = std::max(wlim, fabs(2.0 * A.xmin.v / (A.xmax.v + A.xmin.v) - lim));
             } else {                                  // cell p[2], its right edge is q's left one
-                const double a11 = fma(-0.5, s[1], f[2]);
+                const Real a11 = fma(-0.5, s[1], f[2]);
                 const AOWeights A = ao_weights<-1>(f[2], f[1], s[2], s[1], s[0], e[2], e[1], e[0], a11, t1 + t2, t2 - t1, S.eps, S);
-                const double iv = ao_inverse_sum(A), y = A.y0 * t2;
-                const double val = -0.5 * f[1] - s[1] / 6.0 + iv * (S.d[0] / 3.0 * (y + 0.5 * t1 * A.y2) + A.x3 * (t2 / 30.0 + t1 / 20.0));
+                const double iv = ao_inverse_sum(A).v, y = Real(A.y0 * t2).v;
+                const double val = -0.5 * f[1].v - s[1].v / 6.0 + iv * (S.d[0] / 3.0 * (y + 0.5 * t1.v * A.y2.v) + A.x3.v * (t2.v / 30.0 + t1.v / 20.0));
                 worst = std::max(worst, fabs(q[2] + val - v[0]) / big);
-                worst = std::max(worst, fabs(-(f[1] - iv * (S.d[0] * y + A.x3 * t1 / 12.0)) - v[1]) / big);
-                wlim = std::max(wlim, fabs(2.0 * A.xmin / (A.xmax + A.xmin) - lim));
+                worst = std::max(worst, fabs(-(f[1].v - iv * (S.d[0] * y + A.x3.v * t1.v / 12.0)) - v[1]) / big);
+                wlim = std::max(wlim, fabs(2.0 * A.xmin.v / (A.xmax.v + A.xmin.v) - lim));
             }
         }
     }
