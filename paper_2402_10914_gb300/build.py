@@ -22,7 +22,8 @@ ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 
 
 # the sources that define the single-problem forward kernels (the profiled ones)
-FORWARD_KERNEL_SOURCES = ["dfgks_device.cuh", "dfgks_bodies.cuh", "dfgks_kernels.cu", "dfgks_internal.h"]
+FORWARD_KERNEL_SOURCES = ["dfgks_device.cuh", "dfgks_bodies.cuh", "dfgks_kernels.cu", "dfgks_internal.h",
+                          "dfgks_erfcx_table.inc", "dfgks_exp2_table.inc"]
 
 
 def kernel_source_hash() -> str:

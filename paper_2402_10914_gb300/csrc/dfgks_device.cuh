@@ -851,7 +851,7 @@ DFK_HD void gks_flux_t(const GPState& L, const GPState& R, double dt, const Sche
 // The equilibrium state's time derivative is the Euler equations' (its compatibility condition in closed
 // form).  Moments end at u^4 instead of u^6.  590 FP64 instructions per Gauss point against 1028 with
 // slope coefficients and general products of moments, on a kernel bound by the FP64 units: 2.38 -> 1.38 ms
-// per 400 x 400 step, 158 instead of 250 registers.
+// per 400 x 400 step (1.09 with vector-register operands and the tables below), 158 instead of 250 registers.
 // ------------------------------------------------------------------------------------------
 
 // rcp() where its range holds, a division elsewhere (negative, zero, extreme)
@@ -916,18 +916,91 @@ DFK_HD void finish_moments(const FlowState& s, HalfMom& h) {
     h.e1[1] = h.m[0]; h.e1[2] = 2.0 * h.m[1]; h.e1[3] = 3.0 * h.m[2]; h.e1[4] = 4.0 * h.m[3];
     h.e2[2] = h.m[0]; h.e2[3] = 3.0 * h.m[1]; h.e2[4] = 6.0 * h.m[2];
 }
+// Gaussians and complementary error functions of the half-space moments from tables.  CUDA's exp and erfcx
+// are 16 and 40 FP64 instructions (19 cycles each: their constants are immediates), 112 of the flux's 600
+// for the two sides; the reductions below take 11 and 10, and table entries arrive in vector registers.
+// exp(-y): Tang's table-driven method, y = -n ln2/64 - r, a degree-5 polynomial in |r| <= ln2/128 and 2^(n/64)
+// from a table; relative error below 1.2 ulp.  erfcx: see the table.  The tables (0.5 and 12 KB) stay in L1:
+// neighbouring threads read neighbouring rows.  601 -> 514 FP64 instructions per Gauss point; flux kernel
+// 1.311 -> 1.090 ms per 400 x 400 step.
+#ifdef __CUDACC__
+static __device__ const double kExp2Dev[64] = {
+#include "dfgks_exp2_table.inc"
+};
+static __device__ __align__(16) const double kErfcxDev[193 * 8] = {
+#include "dfgks_erfcx_table.inc"
+};
+#endif
+static const double kExp2Host[64] = {
+#include "dfgks_exp2_table.inc"
+};
+static const double kErfcxHost[193 * 8] = {
+#include "dfgks_erfcx_table.inc"
+};
+constexpr double kRoundToInt = 6755399441055744.0;      // 1.5 2^52: x + this - this rounds x to an integer
+
+// exp(-y) for 0 <= y < 700
+DFK_HD Real exp_neg_table(Real y) {
+    const Real nf = fma(y, -92.33248261689366, kRoundToInt);                      // 64/ln2
+    const int n = (int)dbits(nf.v);
+    const Real m = nf - kRoundToInt;
+    // ln2/64 in 32 bits, exact times m, and the rest
+    const Real r = fma(m, -2.9815858269852933e-12, fma(m, -0.01083042469326756, -y));
+    Real p = fma(r, 1.0 / 120.0, 1.0 / 24.0);
+    p = fma(p, r, 1.0 / 6.0);
+    p = fma(p, r, 0.5);
+    p = fma(r * r, p, r);
+#ifdef __CUDA_ARCH__
+    const Real T = Real::raw(__ldg(kExp2Dev + (n & 63)));
+#else
+    const Real T = Real::raw(kExp2Host[n & 63]);
+#endif
+    const Real e = fma(T, p, T);
+    return Real::raw(dval(dbits(e.v) + ((long long)(n >> 6) << 52)));
+}
+// exp(-y), y >= 0
+DFK_HD Real exp_neg(Real y) {
+    if (nn_less(y.v, 700.0)) return exp_neg_table(y);
+    return Real::raw(exp(-y.v));
+}
+
+// G = exp(-x^2) and t = erfc(|x|)/2 = G erfcx(|x|)/2
+DFK_HD void gauss_erfc(Real x, Real& G, Real& t) {
+    const Real y = x * x, a = fabs(x);
+    if (nn_less(a.v, 6.0)) {
+        G = exp_neg_table(y);
+        const Real jf = fma(a, 32.0, kRoundToInt);
+        const int j = (int)dbits(jf.v);
+        const Real d = fma(jf - kRoundToInt, -1.0 / 32.0, a);
+#ifdef __CUDA_ARCH__
+        const double2* row = reinterpret_cast<const double2*>(kErfcxDev + 8 * j);
+        const double2 c01 = __ldg(row), c23 = __ldg(row + 1), c45 = __ldg(row + 2), c67 = __ldg(row + 3);
+        const double c[8] = {c01.x, c01.y, c23.x, c23.y, c45.x, c45.y, c67.x, c67.y};
+#else
+        const double* c = kErfcxHost + 8 * j;
+#endif
+        Real e = Real::raw(c[7]);
+#pragma unroll
+        for (int k = 6; k >= 0; --k) e = fma(e, d, Real::raw(c[k]));
+        t = G * e;
+    } else {                                   // t < 1e-17: beyond Mach 7, or not a number
+        G = Real::raw(exp(-y.v));
+#ifdef __CUDA_ARCH__
+        t = 0.5 * G * Real::raw(erfcx(a.v));
+#else
+        t = 0.5 * erfc(a.v);
+#endif
+    }
+}
+
 template <int HALF>
 DFK_HD void half_moments(const FlowState& s, HalfMom& h) {
-    const Real x = s.U * s.rs, G = Real::raw(exp(Real(-x * x).v));
+    const Real x = s.U * s.rs;
+    Real G, t;
+    gauss_erfc(x, G, t);
     // the marginal distribution at u = 0, exp(-U^2/(2 theta)) / sqrt(2 pi theta)
     const Real phi = (0.56418958354775628695 * s.rs) * G;
-    // erfc(|x|)/2 from the scaled function and the Gaussian above; erfc(-|x|) = 2 - erfc(|x|)
-#ifdef __CUDA_ARCH__
-    const Real t = 0.5 * G * Real::raw(erfcx(::fabs(x.v)));
-#else
-    const Real t = 0.5 * erfc(::fabs(x.v));
-#endif
-    const bool xpos = dbits(x.v) >= 0;
+    const bool xpos = dbits(x.v) >= 0;                    // erfc(-|x|) = 2 - erfc(|x|)
     h.m[0] = (HALF > 0) == xpos ? 1.0 - t : t;
     const Real sphi = HALF > 0 ? phi : -phi;
     h.m[1] = fma(s.U, h.m[0], s.th * sphi);
@@ -961,41 +1034,47 @@ DFK_HD void transport(const FlowState& s, const HalfMom& h, const FlowGrad& x, c
 // g1 = rho <u^2 a_x psi> + rho <u v a_y psi>.  The left side (HALF > 0) comes first and sets them, the
 // right one adds (an addition to zero is not free on the FP64 units)
 template <int HALF>
-DFK_HD void side_add(const Real o[4], Real to[4]) {
-#pragma unroll
-    for (int i = 0; i < 4; ++i) to[i] = HALF > 0 ? o[i] : to[i] + o[i];
-}
+DFK_HD Real acc(Real x, Real to) { return HALF > 0 ? x : x + to; }
+template <int HALF>
+DFK_HD Real acc(RealProd x, Real to) { return HALF > 0 ? (Real)x : x + to; }
 template <int HALF>
 DFK_HD void side_sums(const FlowState& s, const FlowGrad& x, const FlowGrad& y, const HalfMom& h, Real k1, Real k3,
                       Real c[4], Real cx[4], Real cy[4], Real g0[4], Real g1[4]) {
     const Real hV2 = 0.5 * s.V * s.V, rk = fma(k1, s.th, hV2), rm0 = s.rho * h.m[0], rm1 = s.rho * h.m[1],
-                 rm2 = s.rho * h.m[2];
+               rm2 = s.rho * h.m[2];
+    c[0] = acc<HALF>(rm0, c[0]);
+    c[1] = acc<HALF>(rm1, c[1]);
+    c[2] = acc<HALF>(s.V * rm0, c[2]);
+    c[3] = fma(0.5, rm2, acc<HALF>(rk * rm0, c[3]));
+    g0[0] = acc<HALF>(rm1, g0[0]);
+    g0[1] = acc<HALF>(rm2, g0[1]);
+    g0[2] = acc<HALF>(s.V * rm1, g0[2]);
+    g0[3] = fma(0.5 * s.rho, h.m[3], acc<HALF>(rk * rm1, g0[3]));
     Real Nx[3], Ny[3], o[4];
-    o[0] = rm0; o[1] = rm1; o[2] = s.V * rm0; o[3] = fma(0.5, rm2, rk * rm0);
-    side_add<HALF>(o, c);
-    o[0] = rm1; o[1] = rm2; o[2] = s.V * rm1; o[3] = fma(0.5 * s.rho, h.m[3], rk * rm1);
-    side_add<HALF>(o, g0);
     {
-        const Real N0 = grad_mom(h, x, 0);
+        const Real N0 = grad_mom(h, x, 0), p = x.r2 * h.m[0];
         Nx[0] = grad_mom(h, x, 2);
-        o[0] = N0; o[1] = grad_mom(h, x, 1); o[2] = x.r2 * h.m[0];
-        o[3] = fma(0.5, Nx[0], k1 * fma(s.th, N0, x.q3 * h.m[0]));
-        to_lab(s.V, hV2, o);
-        side_add<HALF>(o, cx);
-        Nx[1] = grad_mom(h, x, 3); Nx[2] = grad_mom(h, x, 4);
+        cx[0] = acc<HALF>(N0, cx[0]);
+        cx[1] = fma(x.r0, h.m[1], fma(x.r1, h.e1[1], acc<HALF>(x.q3 * h.e2[1], cx[1])));
+        cx[2] = fma(s.V, N0, acc<HALF>(p, cx[2]));
+        cx[3] = fma(s.V, p, fma(hV2, N0, fma(0.5, Nx[0], acc<HALF>(k1 * fma(s.th, N0, x.q3 * h.m[0]), cx[3]))));
+        Nx[1] = fma(x.r0, h.m[3], fma(x.r1, h.e1[3], acc<HALF>(x.q3 * h.e2[3], g1[1])));
+        Nx[2] = grad_mom(h, x, 4);
     }
     {
-        const Real N0 = grad_mom(h, y, 0);
+        const Real N0 = grad_mom(h, y, 0), p = y.r2 * h.m[0];
         Ny[0] = grad_mom(h, y, 1); Ny[1] = grad_mom(h, y, 2);
-        o[0] = N0; o[1] = Ny[0]; o[2] = y.r2 * h.m[0];
-        o[3] = fma(0.5, Ny[1], k1 * fma(s.th, N0, y.q3 * h.m[0]));
-        to_lab(s.V, hV2, o);
-        side_add<HALF>(o, cy);
+        cy[0] = acc<HALF>(N0, cy[0]);
+        cy[1] = acc<HALF>(Ny[0], cy[1]);
+        cy[2] = fma(s.V, N0, acc<HALF>(p, cy[2]));
+        cy[3] = fma(s.V, p, fma(hV2, N0, fma(0.5, Ny[1], acc<HALF>(k1 * fma(s.th, N0, y.q3 * h.m[0]), cy[3]))));
         Ny[2] = grad_mom(h, y, 3);
     }
-    transport(s, h, x, y, Nx, Ny, k1, k3, o);
-    to_lab(s.V, hV2, o);
-    side_add<HALF>(o, g1);
+    transport(s, h, x, y, Nx, Ny, k1, k3, o);       // o[1] has the sum so far through Nx[1]
+    g1[3] = acc<HALF>(Real(fma(s.V, o[2], fma(hV2, o[0], o[3]))), g1[3]);
+    g1[2] = fma(s.V, o[0], acc<HALF>(o[2], g1[2]));
+    g1[1] = o[1];
+    g1[0] = acc<HALF>(o[0], g1[0]);
 }
 
 // the Euler equations' time derivative of a state with gradients x, y, as a gradient
@@ -1076,7 +1155,7 @@ DFK_HD void gks_flux_sides(const GPState& L, const GPState& Rt, const FlowState&
     const Real q = (sl.p - sr.p) * rcp_or_div(sl.p + sr.p);
     const Real rT = fma(S.C2, fabs(q), S.C1);        // tau_n / dt
     Real E2 = 0.0, r = 0.0;
-    if (dbits(rT.v) > 0) { E2 = Real::raw(exp(Real(-0.5 * rcp_or_div(rT)).v)); r = rT; }   // rT >= 0
+    if (dbits(rT.v) > 0) { E2 = exp_neg(0.5 * rcp_or_div(rT)); r = rT; }   // rT >= 0
     const Real om = 1.0 - E2, om2 = om * om, rom = r * om;
     const Real gF = rom * (3.0 - E2), gD = -4.0 * (r * om2) * rcp_or_div(dt);
     if (S.tau_reading == 1) {
