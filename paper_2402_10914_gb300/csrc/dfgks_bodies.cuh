@@ -59,11 +59,15 @@ template <int DIR> DFK_HD int lines_ly(const Mesh& m) { return DIR == 0 ? m.ny +
 template <int DIR> DFK_HD int faces_lx(const Mesh& m) { return DIR == 0 ? m.nx + 1 : m.nx; }
 template <int DIR> DFK_HD int faces_ly(const Mesh& m) { return DIR == 0 ? m.ny : m.ny + 1; }
 
-// The sweep kernels run on 1-D grids of 128-thread blocks over such a space: thread i takes
+// The sweep kernels run on 1-D grids of one-warp blocks over such a space: thread i takes
 // (i mod lx, i / lx), so only the grid's last warp is partly idle, where a 2-D grid of 32-wide rows
 // would idle part of every row's last warp (15 of 416 lanes on a 401-face row).  Threads past the
 // end get ay >= ly, which the bodies' bounds checks reject.
-constexpr int kSweepThreads = 128;
+// One warp per block, because nothing is shared in a block and a launch's time is that of the SM with the most
+// warps: with 128 threads a mesh of about 100 x 100 gives some SMs twice the work of others.  128 -> 32
+// threads: 3 x 2 blocks of 100 x 100 cells 13.2 -> 11.6 ms per 4 steps, the reverse of a 67 x 83 stage
+// 0.84 -> 0.77 ms, a 97 x 61 stage 0.177 -> 0.172 ms, a 400 x 400 step the same.
+constexpr int kSweepThreads = 32;
 inline unsigned sweep_blocks(int lx, int ly, int threads = kSweepThreads) { return (unsigned)(((long long)lx * ly + threads - 1) / threads); }
 __device__ __forceinline__ void sweep_xy(int lx, int& ax, int& ay) {
     const int i = (int)(blockIdx.x * blockDim.x + threadIdx.x);
