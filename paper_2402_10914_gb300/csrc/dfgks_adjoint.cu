@@ -84,7 +84,7 @@ DFK_HD void ka_flux_body(const Mesh& m, const SchemeConsts& S, const AdjointArgs
     }
     GPStateBar Lbar, Rbar;
     for (int k = 0; k < 4; ++k) { Lbar.W[k] = Lbar.Wn[k] = Lbar.Wt[k] = Rbar.W[k] = Rbar.Wn[k] = Rbar.Wt[k] = 0.0; }
-    if (FLUX == 0 && TAPED) gks_flux_reverse(PlaneTape{tape + (long long)mm * nf + fid, fs}, L, R, dt, S, Fb, dFb, Lbar, Rbar);
+    if (FLUX == 0 && TAPED) gks_flux_reverse(PlaneTape{tape + (long long)mm * nf + fid, fs}, L, R, S, Fb, dFb, Lbar, Rbar);
     else if (FLUX == 0) gks_flux_vjp(L, R, dt, S, Fb, dFb, Lbar, Rbar);
     else lf_flux_vjp(L, R, S, Fb, dFb, Lbar, Rbar);
     for (int k = 0; k < 4; ++k) {

@@ -231,557 +231,359 @@ DFK_HD void df_at_gauss_vjp(double alpha, const double valb[2], const double slo
 }
 
 // ------------------------------------------------------------------------------------------
-// GKS flux
+// GKS flux: reverse of the gradient form
+//
+// The moments' own derivatives are e1 and e2, and the marginal distribution g = phi at u = 0, a Gaussian in U of
+// variance theta, obeys the heat equation dg/dtheta = g''/2, as every moment does.  So the adjoints of a side's
+// m_0 .. m_4, phi and e2_0 go straight to U and theta,
+//   U^ = sum m_k^ e1_k + 2 phi^ e2_0 + e2_0^ psi,  theta^ = sum m_k^ e2_k + phi^ psi + e2_0^ e2_0 (U^2/theta - 3)/(2 theta),
+//   e2_0 = -phi U/(2 theta),  psi = dphi/dtheta = phi (U^2/theta - 1)/(2 theta),
+// without going back through the recurrences, the Gaussian and the error function.  Bound by the FP64 units
+// like the forward; the reverse of the flux written with slope coefficients took 2343 FP64 instructions per
+// Gauss point, a tape of 172 values and that form's forward (1028 instructions).  10-step gradient on 256 x 256
+// 72.9 -> 53.1 ms, reverse of a 67 x 83 stage 0.775 -> 0.620 ms (that one also reads a tape now).
 // ------------------------------------------------------------------------------------------
-struct MaxwBar { double rho, ir, U, V, p, tl, il2, f4, qK; };
-struct MomBar { double mu[7], mv[6], mx[3]; };
-
-DFK_HD void zero(MaxwBar& b) { b.rho = b.ir = b.U = b.V = b.p = b.tl = b.il2 = b.f4 = b.qK = 0.0; }
-DFK_HD void zero(MomBar& b) {
-    for (int i = 0; i < 7; ++i) b.mu[i] = 0.0;
-    for (int i = 0; i < 6; ++i) b.mv[i] = 0.0;
-    for (int i = 0; i < 3; ++i) b.mx[i] = 0.0;
-}
-
-DFK_HD void maxw_of_vjp(const double W[4], const SchemeConsts& S, const Maxw& s, const MaxwBar& sb, double Wb[4]) {
-    double tlb = sb.tl + sb.f4 * 2.0 * s.tl * S.inv_K2;
-    double Ub = sb.U + sb.qK * 2.0 * s.U, Vb = sb.V + sb.qK * 2.0 * s.V;
-    double il2b = sb.il2 + sb.qK * (S.K + 2.0);
-    double pb = sb.p + il2b * s.ir;
-    double irb = sb.ir + il2b * s.p;
-    Wb[0] += tlb / s.p;
-    pb += -tlb * s.tl / s.p;
-    Wb[3] += pb * S.gm1;
-    Wb[0] += -pb * S.gm1 * 0.5 * (s.U * s.U + s.V * s.V);
-    Ub += -pb * S.gm1 * W[0] * s.U;
-    Vb += -pb * S.gm1 * W[0] * s.V;
-    Wb[1] += Ub * s.ir;
-    Wb[2] += Vb * s.ir;
-    irb += Ub * W[1] + Vb * W[2];
-    Wb[0] += -irb * s.ir * s.ir + sb.rho;
-}
-
-// adjoint of fill_moments; accumulates into the state's U, V, il2 and tl adjoints
-template <int HALF>
-DFK_HD void fill_moments_vjp(const Maxw& s, double K, const Mom& m, MomBar& mb, MaxwBar& sb) {
-    sb.il2 += mb.mx[1] * K + mb.mx[2] * K * (K + 2.0) * 2.0 * s.il2;
-    for (int n = 5; n >= 2; --n) {
-        double g = mb.mv[n];
-        sb.V += g * m.mv[n - 1];
-        mb.mv[n - 1] += g * s.V;
-        sb.il2 += g * (double)(n - 1) * m.mv[n - 2];
-        mb.mv[n - 2] += g * (double)(n - 1) * s.il2;
-    }
-    sb.V += mb.mv[1];
-    for (int n = 6; n >= 2; --n) {
-        double g = mb.mu[n];
-        sb.U += g * m.mu[n - 1];
-        mb.mu[n - 1] += g * s.U;
-        sb.il2 += g * (double)(n - 1) * m.mu[n - 2];
-        mb.mu[n - 2] += g * (double)(n - 1) * s.il2;
-    }
-    if (HALF == 0) {
-        sb.U += mb.mu[1];
-    } else {
-        double lam = 0.5 * s.tl;
-        double isl = rsqrt(lam);
-        double x = lam * isl * s.U;
-        double ex = exp(-x * x);
-        double e = ex * (0.28209479177387814347 * isl);
-        // mu1 = U mu0 +/- e
-        sb.U += mb.mu[1] * m.mu[0];
-        double mu0b = mb.mu[0] + mb.mu[1] * s.U;
-        double eb = HALF > 0 ? mb.mu[1] : -mb.mu[1];
-        // mu0 = erfc(-/+ x)/2: d/dx = +/- exp(-x^2)/sqrt(pi)
-        double xb = mu0b * (HALF > 0 ? 1.0 : -1.0) * ex * 0.56418958354775628695;
-        xb += eb * e * (-2.0 * x);
-        double islb = eb * ex * 0.28209479177387814347;
-        double lamb = xb * isl * s.U;
-        islb += xb * lam * s.U;
-        sb.U += xb * lam * isl;
-        lamb += -0.5 * islb * isl * isl * isl;
-        sb.tl += 0.5 * lamb;
-    }
-}
-
-template <int k, int l, int c>
-DFK_HD void M_vjp(const Mom& m, double g, MomBar& mb) {
-    mb.mu[k] += g * m.mv[l] * m.mx[c];
-    mb.mv[l] += g * m.mu[k] * m.mx[c];
-    mb.mx[c] += g * m.mu[k] * m.mv[l];
-}
-
-template <int k, int l, int c>
-DFK_HD void psi_mom_vjp(const Mom& m, const double ob[4], MomBar& mb) {
-    M_vjp<k, l, c>(m, ob[0], mb);
-    M_vjp<k + 1, l, c>(m, ob[1], mb);
-    M_vjp<k, l + 1, c>(m, ob[2], mb);
-    M_vjp<k + 2, l, c>(m, 0.5 * ob[3], mb);
-    M_vjp<k, l + 2, c>(m, 0.5 * ob[3], mb);
-    M_vjp<k, l, c + 1>(m, 0.5 * ob[3], mb);
-}
-
-// adjoint of the factorised a_mom (see its comment): ab += d out/d a ^T ob, moment adjoints accumulated
-template <int k, int l>
-DFK_HD void a_mom_vjp(const Mom& m, const double a[4], const double ob[4], MomBar& mb, double ab[4]) {
-    const double* mu = m.mu;
-    const double* mv = m.mv;
-    const double h = 0.5 * a[3], x1 = m.mx[1], x2 = m.mx[2], hx1 = h * x1;
-    double P[3], Qp[3];
-    for (int j = 0; j < 3; ++j) {
-        P[j] = a[0] * mu[k + j] + a[1] * mu[k + j + 1] + h * mu[k + j + 2];
-        Qp[j] = a[2] * mv[l + j + 1] + h * mv[l + j + 2] + hx1 * mv[l + j];
-    }
-    const double Ql = a[2] * mv[l + 1] + h * mv[l + 2];
-    const double g0 = ob[0], g1 = ob[1], g2 = ob[2], g3 = 0.5 * ob[3];
-    double Pb[3] = {0.0, 0.0, 0.0}, Qpb[3] = {0.0, 0.0, 0.0}, Qlb = 0.0, hb = 0.0;
-    // out0 = mv_l P0 + mu_k Qp0, out1 = mv_l P1 + mu_{k+1} Qp0, out2 = mv_{l+1} P0 + mu_k Qp1
-    mb.mv[l] += g0 * P[0] + g1 * P[1] + g3 * P[2];
-    mb.mu[k] += g0 * Qp[0] + g2 * Qp[1] + g3 * Qp[2];
-    mb.mu[k + 1] += g1 * Qp[0];
-    mb.mv[l + 1] += g2 * P[0];
-    Pb[0] += g0 * mv[l] + g2 * mv[l + 1] + g3 * mv[l + 2];
-    Pb[1] += g1 * mv[l];
-    Pb[2] += g3 * mv[l];
-    Qpb[0] += g0 * mu[k] + g1 * mu[k + 1] + g3 * mu[k + 2];
-    Qpb[1] += g2 * mu[k];
-    Qpb[2] += g3 * mu[k];
-    // out3 / 2 = G(k+2,l,0) + G(k,l+2,0) + G(k,l,1): the first two above, then
-    // G(k,l,1) = x1 (mv_l P0 + mu_k Ql) + h mu_k mv_l x2
-    mb.mu[k + 2] += g3 * Qp[0];
-    mb.mv[l + 2] += g3 * P[0];
-    {
-        const double gi = g3 * x1, t = g3 * h * x2;
-        mb.mx[1] += g3 * (mv[l] * P[0] + mu[k] * Ql);
-        mb.mv[l] += gi * P[0] + t * mu[k];
-        mb.mu[k] += gi * Ql + t * mv[l];
-        mb.mx[2] += g3 * h * mu[k] * mv[l];
-        Pb[0] += gi * mv[l];
-        Qlb += gi * mu[k];
-        hb += g3 * mu[k] * mv[l] * x2;
-    }
-    // Qp_j = a2 mv_{l+j+1} + h mv_{l+j+2} + h x1 mv_{l+j},  Ql = a2 mv_{l+1} + h mv_{l+2}
-    for (int j = 0; j < 3; ++j) {
-        ab[2] += Qpb[j] * mv[l + j + 1];
-        hb += Qpb[j] * (mv[l + j + 2] + x1 * mv[l + j]);
-        mb.mv[l + j + 1] += Qpb[j] * a[2];
-        mb.mv[l + j + 2] += Qpb[j] * h;
-        mb.mv[l + j] += Qpb[j] * hx1;
-        mb.mx[1] += Qpb[j] * h * mv[l + j];
-    }
-    ab[2] += Qlb * mv[l + 1];
-    hb += Qlb * mv[l + 2];
-    mb.mv[l + 1] += Qlb * a[2];
-    mb.mv[l + 2] += Qlb * h;
-    // P_j = a0 mu_{k+j} + a1 mu_{k+j+1} + h mu_{k+j+2}
-    for (int j = 0; j < 3; ++j) {
-        ab[0] += Pb[j] * mu[k + j];
-        ab[1] += Pb[j] * mu[k + j + 1];
-        hb += Pb[j] * mu[k + j + 2];
-        mb.mu[k + j] += Pb[j] * a[0];
-        mb.mu[k + j + 1] += Pb[j] * a[1];
-        mb.mu[k + j + 2] += Pb[j] * h;
-    }
-    ab[3] += 0.5 * hb;
-}
-
-// The reverse of several a_mom of one (m, a) at once (the factorised form of a_mom): the output
-// adjoints of each out<k, l> are accumulated into the adjoints of the shared P_k, Q_l, Qp_l terms
-// (out_vjp), whose own reverse runs once (finish).  Needs KLO <= k, k + 2 <= KHI, LLO <= l,
-// l + 2 <= LHI for every output.
-template <int KLO, int KHI, int LLO, int LHI>
-struct AMomRev {
-    double P[KHI - KLO + 1], Q[LHI - LLO + 1], Qp[LHI - LLO + 1], h, x1, x2;
-    double Pb[KHI - KLO + 1], Qb[LHI - LLO + 1], Qpb[LHI - LLO + 1], hb;
-    DFK_HD AMomRev(const Mom& m, const double a[4]) {
-        h = 0.5 * a[3];
-        x1 = m.mx[1];
-        x2 = m.mx[2];
-        const double hx1 = h * x1;
-        for (int j = KLO; j <= KHI; ++j) {
-            P[j - KLO] = a[0] * m.mu[j] + a[1] * m.mu[j + 1] + h * m.mu[j + 2];
-            Pb[j - KLO] = 0.0;
-        }
-        for (int j = LLO; j <= LHI; ++j) {
-            Q[j - LLO] = a[2] * m.mv[j + 1] + h * m.mv[j + 2];
-            Qp[j - LLO] = Q[j - LLO] + hx1 * m.mv[j];
-            Qb[j - LLO] = 0.0;
-            Qpb[j - LLO] = 0.0;
-        }
-        hb = 0.0;
-    }
-    template <int k, int l>
-    DFK_HD void out_vjp(const Mom& m, const double ob[4], MomBar& mb) {
-        const double* mu = m.mu;
-        const double* mv = m.mv;
-        const double g0 = ob[0], g1 = ob[1], g2 = ob[2], g3 = 0.5 * ob[3];
-        const int pk = k - KLO, ql = l - LLO;
-        // out0 = mv_l P_k + mu_k Qp_l, out1 = mv_l P_{k+1} + mu_{k+1} Qp_l, out2 = mv_{l+1} P_k + mu_k Qp_{l+1},
-        // out3 / 2 = G(k+2,l,0) + G(k,l+2,0) + G(k,l,1)
-        mb.mv[l] += g0 * P[pk] + g1 * P[pk + 1] + g3 * P[pk + 2];
-        mb.mu[k] += g0 * Qp[ql] + g2 * Qp[ql + 1] + g3 * Qp[ql + 2];
-        mb.mu[k + 1] += g1 * Qp[ql];
-        mb.mv[l + 1] += g2 * P[pk];
-        mb.mu[k + 2] += g3 * Qp[ql];
-        mb.mv[l + 2] += g3 * P[pk];
-        Pb[pk] += g0 * mv[l] + g2 * mv[l + 1] + g3 * mv[l + 2];
-        Pb[pk + 1] += g1 * mv[l];
-        Pb[pk + 2] += g3 * mv[l];
-        Qpb[ql] += g0 * mu[k] + g1 * mu[k + 1] + g3 * mu[k + 2];
-        Qpb[ql + 1] += g2 * mu[k];
-        Qpb[ql + 2] += g3 * mu[k];
-        // G(k,l,1) = x1 (mv_l P_k + mu_k Q_l) + h mu_k mv_l x2
-        const double gi = g3 * x1, t = g3 * h * x2;
-        mb.mx[1] += g3 * (mv[l] * P[pk] + mu[k] * Q[ql]);
-        mb.mv[l] += gi * P[pk] + t * mu[k];
-        mb.mu[k] += gi * Q[ql] + t * mv[l];
-        mb.mx[2] += g3 * h * mu[k] * mv[l];
-        Pb[pk] += gi * mv[l];
-        Qb[ql] += gi * mu[k];
-        hb += g3 * mu[k] * mv[l] * x2;
-    }
-    DFK_HD void finish(const Mom& m, const double a[4], MomBar& mb, double ab[4]) {
-        const double* mu = m.mu;
-        const double* mv = m.mv;
-        const double hx1 = h * x1;
-        for (int j = LLO; j <= LHI; ++j) {
-            const int q = j - LLO;
-            // Qp_j = Q_j + h x1 mv_j, Q_j = a2 mv_{j+1} + h mv_{j+2}
-            const double qb = Qb[q] + Qpb[q];
-            hb += Qpb[q] * x1 * mv[j] + qb * mv[j + 2];
-            mb.mx[1] += Qpb[q] * h * mv[j];
-            mb.mv[j] += Qpb[q] * hx1;
-            ab[2] += qb * mv[j + 1];
-            mb.mv[j + 1] += qb * a[2];
-            mb.mv[j + 2] += qb * h;
-        }
-        for (int j = KLO; j <= KHI; ++j) {
-            const double pb = Pb[j - KLO];
-            ab[0] += pb * mu[j];
-            ab[1] += pb * mu[j + 1];
-            hb += pb * mu[j + 2];
-            mb.mu[j] += pb * a[0];
-            mb.mu[j + 1] += pb * a[1];
-            mb.mu[j + 2] += pb * h;
-        }
-        ab[3] += 0.5 * hb;
-    }
-};
-
-// adjoint of slope_solve: bb += S^T ab, state adjoints accumulated
-DFK_HD void slope_solve_vjp(const Maxw& s, const double b[4], const double abin[4], double bb[4], MaxwBar& sb) {
-    double R2 = b[1] - s.U * b[0], R3 = b[2] - s.V * b[0], R4 = 2.0 * b[3] - s.qK * b[0];
-    double X = R4 - 2.0 * s.U * R2 - 2.0 * s.V * R3;
-    double a3 = s.f4 * X;
-    double a2 = s.tl * R3 - s.V * a3;
-    double a1 = s.tl * R2 - s.U * a3;
-    double ab0 = abin[0], ab1 = abin[1], ab2 = abin[2], ab3 = abin[3];
-    // a0 = b0 - U a1 - V a2 - a3 qK / 2
-    bb[0] += ab0;
-    sb.U += -ab0 * a1;
-    ab1 += -ab0 * s.U;
-    sb.V += -ab0 * a2;
-    ab2 += -ab0 * s.V;
-    ab3 += -ab0 * 0.5 * s.qK;
-    sb.qK += -ab0 * 0.5 * a3;
-    // a1 = tl R2 - U a3
-    sb.tl += ab1 * R2;
-    double R2b = ab1 * s.tl;
-    sb.U += -ab1 * a3;
-    ab3 += -ab1 * s.U;
-    // a2 = tl R3 - V a3
-    sb.tl += ab2 * R3;
-    double R3b = ab2 * s.tl;
-    sb.V += -ab2 * a3;
-    ab3 += -ab2 * s.V;
-    // a3 = f4 X
-    sb.f4 += ab3 * X;
-    double Xb = ab3 * s.f4;
-    double R4b = Xb;
-    sb.U += -Xb * 2.0 * R2;
-    R2b += -Xb * 2.0 * s.U;
-    sb.V += -Xb * 2.0 * R3;
-    R3b += -Xb * 2.0 * s.V;
-    bb[3] += 2.0 * R4b;
-    sb.qK += -R4b * b[0];
-    bb[0] += -R4b * s.qK;
-    bb[2] += R3b;
-    sb.V += -R3b * b[0];
-    bb[0] += -R3b * s.V;
-    bb[1] += R2b;
-    sb.U += -R2b * b[0];
-    bb[0] += -R2b * s.U;
-}
-
-// value and derivative with respect to tau_n/dt of the combined time coefficients of Eq. 27
-struct Dual { double v, d; };
-DFK_HD Dual dmul(Dual a, Dual b) { return Dual{a.v * b.v, a.d * b.v + a.v * b.d}; }
-DFK_HD Dual dadd(Dual a, Dual b) { return Dual{a.v + b.v, a.d + b.d}; }
-DFK_HD Dual dsub(Dual a, Dual b) { return Dual{a.v - b.v, a.d - b.d}; }
-DFK_HD Dual dscale(double c, Dual a) { return Dual{c * a.v, c * a.d}; }
-
-struct TimeCoeffs { Dual gcF, gcD, acF, acD, AcF, AcD, glrF, glrD, alrF, alrD, AlrF, AlrD; };
-
-DFK_HD TimeCoeffs time_coeffs(double rT, double dt, int tau_reading) {
-    Dual r = {rT, 1.0};
-    Dual T = dscale(dt, r);
-    Dual tau = tau_reading == 1 ? T : Dual{0.0, 0.0};
-    Dual E2 = {0.0, 0.0}, rr = {0.0, 0.0};
-    if (dbits(rT) > 0) { double e = exp(-0.5 / rT); E2 = Dual{e, e * 0.5 / (rT * rT)}; rr = r; }
-    Dual E1 = dmul(E2, E2);
-    Dual om = dsub(Dual{1.0, 0.0}, E2);
-    Dual S3 = dmul(om, dsub(Dual{3.0, 0.0}, E2));
-    double idt = 1.0 / dt;
-    TimeCoeffs c;
-    c.glrF = dmul(rr, S3);
-    c.glrD = dscale(-4.0 * idt, dmul(rr, dmul(om, om)));
-    c.gcF = dsub(Dual{1.0, 0.0}, c.glrF);
-    c.gcD = dscale(-1.0, c.glrD);
-    Dual TT = dadd(dmul(T, T), dmul(T, tau));
-    c.acF = dsub(dadd(dsub(dscale(idt, dmul(TT, S3)), dscale(2.0, dmul(T, E2))), dmul(T, E1)), tau);
-    c.acD = dscale(4.0 * idt * idt, dadd(dscale(-1.0, dmul(TT, dmul(om, om))), dscale(dt, dmul(T, dmul(E2, om)))));
-    c.AcF = dadd(dscale(-1.0, tau), dmul(tau, dmul(rr, S3)));
-    c.AcD = dsub(Dual{1.0, 0.0}, dscale(4.0 * idt * idt, dmul(dmul(T, tau), dmul(om, om))));
-    c.alrF = dsub(dscale(-1.0, c.acF), tau);
-    c.alrD = dscale(-1.0, c.acD);
-    c.AlrF = dscale(-idt, dmul(dmul(T, tau), S3));
-    c.AlrD = dscale(4.0 * idt * idt, dmul(dmul(T, tau), dmul(om, om)));
-    return c;
-}
-
 struct GPStateBar { double W[4], Wn[4], Wt[4]; };
+struct FlowBar { Real rho, U, V, p, th, hq; };
+struct GradBar { Real r0, r1, r2, q3, dp; };
+
+DFK_HD void zero(FlowBar& b) { b.rho = b.U = b.V = b.p = b.th = b.hq = 0.0; }
+DFK_HD void zero(GradBar& b) { b.r0 = b.r1 = b.r2 = b.q3 = b.dp = 0.0; }
 
 template <class Tape>
-DFK_HD Maxw tape_get_maxw(const Tape& tp, int b) {
-    Maxw s;
-    s.rho = tp.get(b); s.ir = tp.get(b + 1); s.U = tp.get(b + 2); s.V = tp.get(b + 3); s.p = tp.get(b + 4);
-    s.il2 = tp.get(b + 5); s.tl = tp.get(b + 6); s.f4 = tp.get(b + 7); s.qK = tp.get(b + 8);
+DFK_HD Real tape_real(const Tape& tp, int i) { return Real::raw(tp.get(i)); }
+
+// a state of which 1/rho is known
+DFK_HD FlowState flow_state_again(const Real W[4], Real ir, const SchemeConsts& S) {
+    FlowState s;
+    s.rho = W[0];
+    s.ir = ir;
+    s.U = W[1] * ir;
+    s.V = W[2] * ir;
+    s.hq = 0.5 * fma(s.U, s.U, s.V * s.V);
+    s.p = S.gm1 * fma(-W[0], s.hq, W[3]);
+    s.th = s.p * ir;
     return s;
 }
-template <class Tape>
-DFK_HD void tape_get_mom(const Tape& tp, int b, Mom& m) {
-    for (int n = 0; n < 7; ++n) m.mu[n] = tp.get(b + n);
-    for (int n = 0; n < 6; ++n) m.mv[n] = tp.get(b + 7 + n);
-    for (int n = 0; n < 3; ++n) m.mx[n] = tp.get(b + 13 + n);
-}
-template <class Tape>
-DFK_HD void tape_get_vec(const Tape& tp, int b, double v[4]) {
-    for (int i = 0; i < 4; ++i) v[i] = tp.get(b + i);
+
+// flow_state's reverse: the state adjoint to that of the conserved variables
+DFK_HD void flow_state_rev(const FlowState& s, const FlowBar& b, const SchemeConsts& S, Real Wb[4]) {
+    const Real pb = fma(b.th, s.ir, b.p), z = S.gm1 * pb, hqb = fma(-z, s.rho, b.hq);
+    const Real Ub = fma(hqb, s.U, b.U), Vb = fma(hqb, s.V, b.V);
+    Wb[0] = fma(-z, s.hq, fma(-s.ir, fma(b.th, s.th, fma(Ub, s.U, Vb * s.V)), b.rho));
+    Wb[1] = Ub * s.ir;
+    Wb[2] = Vb * s.ir;
+    Wb[3] = z;
 }
 
-// under the tau = tau_n reading, one side's slope coefficients A of the time derivative of its
-// Maxwellian (from the compatibility condition over the full velocity space) and <u A psi> over the
-// side's half space, recomputed from the tape.  SIGN +1: left side, -1: right side.
+// flow_grad's reverse: a gradient's adjoint to that of the conserved gradient and of the state
+DFK_HD void flow_grad_rev(const FlowState& s, const Real d0, const FlowGrad& g, const GradBar& b, const SchemeConsts& S,
+                          Real db[4], FlowBar& sb) {
+    const Real z = S.gm1 * (b.dp + b.q3);
+    const Real r1b = fma(-s.U, z, b.r1), r2b = fma(-s.V, z, b.r2);
+    sb.th = fma(-d0, b.q3, sb.th);
+    sb.hq = fma(-d0, z, sb.hq);
+    sb.U = fma(-g.r1, z, fma(-d0, r1b, sb.U));
+    sb.V = fma(-g.r2, z, fma(-d0, r2b, sb.V));
+    db[0] = fma(-s.th, b.q3, fma(-s.hq, z, fma(-s.U, r1b, fma(-s.V, r2b, b.r0))));
+    db[1] = r1b;
+    db[2] = r2b;
+    db[3] = z;
+}
+
+// to_lab's reverse: the laboratory frame's adjoint b to the own frame's (a); w0, w2 are the own frame's values
+DFK_HD void to_lab_rev(Real V, Real hV2, const Real b[4], Real w0, Real w2, Real a[4], Real& Vb) {
+    Vb = fma(b[2], w0, fma(b[3], fma(V, w0, w2), Vb));
+    a[0] = fma(hV2, b[3], fma(V, b[2], b[0]));
+    a[1] = b[1];
+    a[2] = fma(V, b[3], b[2]);
+    a[3] = b[3];
+}
+
+// adjoints of m_0 .. m_4, phi and e2_0
+struct MomAdj { Real m[5], phi, e; };
+
+// reverse of N_k = r0 m_k + r1 e1_k + q3 e2_k for k = LO .. HI, the adjoints being Nb[k - LO]
+template <int LO, int HI>
+DFK_HD void grad_mom_rev(const HalfMom& h, const FlowGrad& g, const Real* Nb, GradBar& b, MomAdj& mb) {
+#pragma unroll
+    for (int k = LO; k <= HI; ++k) {
+        const Real n = Nb[k - LO];
+        b.r0 = fma(n, h.m[k], b.r0);
+        b.r1 = fma(n, h.e1[k], b.r1);
+        b.q3 = fma(n, h.e2[k], b.q3);
+        mb.m[k] = fma(n, g.r0, mb.m[k]);
+        const Real n1 = n * g.r1, n3 = n * g.q3;
+        if (k == 0) { mb.phi = mb.phi + n1; mb.e = mb.e + n3; }
+        if (k >= 1) mb.m[k - 1] = fma((double)k, n1, mb.m[k - 1]);
+        if (k == 1) mb.phi = fma(0.5, n3, mb.phi);
+        if (k >= 2) mb.m[k - 2] = fma(0.5 * k * (k - 1), n3, mb.m[k - 2]);
+    }
+}
+
+// reverse of transport (own-frame adjoints a): the adjoints of N_2 .. N_4 of x are set, those of N_1 .. N_3 of y
+// set, the rest accumulated.  Nx[0] = N_2 of x, Ny[j] = N_{1+j} of y
+DFK_HD void transport_rev(const FlowState& s, const HalfMom& h, const FlowGrad& x, const FlowGrad& y, Real Nx0,
+                          const Real Ny[3], Real k1, Real k3, const Real a[4], Real Nxb[3], Real Nyb[3], GradBar& xb,
+                          GradBar& yb, MomAdj& mb, FlowBar& sb) {
+    const Real ka = k1 * a[3], ha = 0.5 * a[3], kt = k3 * s.th;
+    const Real v1 = y.r2 * h.m[1], G1 = fma(s.th, Ny[0], y.q3 * h.m[1]);
+    const Real v1b = fma(kt, a[3], fma(s.V, a[2], a[0])), G1b = fma(s.V, ka, a[2]);
+    Nxb[0] = fma(s.th, ka, a[0]);
+    Nxb[1] = a[1];
+    Nxb[2] = ha;
+    Nyb[0] = fma(s.V, a[0], s.th * G1b);
+    Nyb[1] = s.V * a[1];
+    Nyb[2] = s.V * ha;
+    xb.r2 = fma(a[2], h.m[2], xb.r2);
+    xb.q3 = fma(ka, h.m[2], xb.q3);
+    yb.r2 = fma(v1b, h.m[1], fma(a[1], h.m[2], fma(ha, h.m[3], yb.r2)));
+    yb.q3 = fma(G1b, h.m[1], yb.q3);
+    mb.m[1] = fma(v1b, y.r2, fma(G1b, y.q3, mb.m[1]));
+    mb.m[2] = fma(a[2], x.r2, fma(ka, x.q3, fma(a[1], y.r2, mb.m[2])));
+    mb.m[3] = fma(ha, y.r2, mb.m[3]);
+    sb.V = fma(a[0], Ny[0], fma(a[1], Ny[1], fma(ha, Ny[2], fma(a[2], v1, fma(ka, G1, sb.V)))));
+    sb.th = fma(k3 * v1, a[3], fma(ka, Nx0, fma(G1b, Ny[0], sb.th)));
+}
+
+// euler_time_grad's reverse: t's adjoint (q3 included) to those of the gradients and the state
+DFK_HD void euler_time_grad_rev(const FlowState& s, const FlowGrad& x, const FlowGrad& y, const FlowGrad& t, const GradBar& tb,
+                                const SchemeConsts& S, GradBar& xb, GradBar& yb, FlowBar& sb) {
+    sb.th = fma(-t.r0, tb.q3, sb.th);
+    const Real s0 = fma(s.th, tb.q3, -tb.r0), s1 = -tb.r1, s2 = -tb.r2, s3 = -(tb.dp + tb.q3);
+    const Real gs = S.gamma * s3, div = x.r1 + y.r2, divb = fma(gs, s.th, s0);
+    sb.th = fma(gs, div, sb.th);
+    sb.U = fma(x.r0, s0, fma(x.r1, s1, fma(x.r2, s2, fma(x.dp, s3, sb.U))));
+    sb.V = fma(y.r0, s0, fma(y.r1, s1, fma(y.r2, s2, fma(y.dp, s3, sb.V))));
+    xb.r0 = fma(s.U, s0, xb.r0); yb.r0 = fma(s.V, s0, yb.r0);
+    xb.r1 = fma(s.U, s1, xb.r1 + divb); yb.r1 = fma(s.V, s1, yb.r1);
+    xb.r2 = fma(s.U, s2, xb.r2); yb.r2 = fma(s.V, s2, yb.r2 + divb);
+    xb.dp = fma(s.U, s3, xb.dp + s1); yb.dp = fma(s.V, s3, yb.dp + s2);
+}
+
+// one side (SIGN +1 left, -1 right) from the adjoints of its sums (the equilibrium state, its gradients, dg, g1,
+// g2) and of its pressure through tau_n
 template <int SIGN, class Tape>
-DFK_HD void tau_side_terms(const Tape& tp, const Maxw& s, double K, Mom& mF, double bA[4], double A[4]) {
-    double ax[4], ay[4], t1[4], t2[4];
-    tape_get_vec(tp, SIGN > 0 ? TG_ALX : TG_ARX, ax);
-    tape_get_vec(tp, SIGN > 0 ? TG_ALY : TG_ARY, ay);
-    fill_moments<0>(s, K, mF);
-    a_mom<1, 0>(mF, ax, t1);
-    a_mom<0, 1>(mF, ay, t2);
-    for (int i = 0; i < 4; ++i) bA[i] = -(t1[i] + t2[i]);
-    slope_solve(s, bA, A);
-}
-
-// reverse of one side's share of gks_flux (SIGN +1 left, -1 right): its half-space moment sums in
-// the flux, in the kinetic weighting of the equilibrium state and in its slopes, its slope
-// coefficients and (tau = tau_n) its extra terms; accumulates into the side's Maxwellian adjoint sb
-// and the Gauss-point state adjoint Pb.  The sides are reversed one after the other so that only
-// one side's moments and their adjoints are live at a time.
-template <int SIGN, class Tape>
-DFK_HD void gks_side_reverse(const Tape& tp, const GPState& P, const Maxw& s, const SchemeConsts& S,
-                             const double Wcb[4], const double Wcxb[4], const double Wcyb[4], const double M0b[4],
-                             const double M1b[4], const double M2b[4], MaxwBar& sb, GPStateBar& Pb) {
-    constexpr bool left = SIGN > 0;
-    Mom m;
-    tape_get_mom(tp, left ? TG_ML : TG_MR, m);
-    MomBar mb;
-    zero(mb);
-    double axb[4] = {0, 0, 0, 0}, ayb[4] = {0, 0, 0, 0};
-    if (S.tau_reading == 1) {
-        Mom mF;
-        double bA[4], A[4], Ab[4] = {0, 0, 0, 0}, bAb[4] = {0, 0, 0, 0}, nb[4], ax[4], ay[4];
-        tau_side_terms<SIGN>(tp, s, S.K, mF, bA, A);
-        a_mom_vjp<1, 0>(m, A, M2b, mb, Ab);
-        slope_solve_vjp(s, bA, Ab, bAb, sb);
-        for (int i = 0; i < 4; ++i) nb[i] = -bAb[i];
-        tape_get_vec(tp, left ? TG_ALX : TG_ARX, ax);
-        tape_get_vec(tp, left ? TG_ALY : TG_ARY, ay);
-        MomBar mFb;
-        zero(mFb);
-        a_mom_vjp<1, 0>(mF, ax, nb, mFb, axb);
-        a_mom_vjp<0, 1>(mF, ay, nb, mFb, ayb);
-        fill_moments_vjp<0>(s, S.K, mF, mFb, sb);
-    }
-    // flux moments <u psi> of the side's initial distribution
-    psi_mom_vjp<1, 0, 0>(m, M0b, mb);
-    // kinetic weighting of the equilibrium state and its slopes
-    double pb[4], tb[4];
-    const int tp0 = left ? TG_PL0 : TG_PR0, tx0 = left ? TG_LX0 : TG_RX0, ty0 = left ? TG_LY0 : TG_RY0;
-    for (int i = 0; i < 4; ++i) {
-        sb.rho += Wcb[i] * tp.get(tp0 + i) + Wcxb[i] * tp.get(tx0 + i) + Wcyb[i] * tp.get(ty0 + i);
-        pb[i] = Wcb[i] * s.rho;
-    }
-    psi_mom_vjp<0, 0, 0>(m, pb, mb);
-    // the side's moment sums of a_x (kinetic weighting, flux moment) and of a_y, each reversed as one
+DFK_HD void gks_side_reverse(const Tape& tp, const GPState& P, const SchemeConsts& S, const Real Wcb[4], const Real Wcxb[4],
+                             const Real Wcyb[4], const Real g0b[4], const Real g1b[4], const Real g2b[4], Real pb,
+                             GPStateBar& Pb) {
+    constexpr int base = SIGN > 0 ? TG_L : TG_R;
+    const Real k1 = 0.5 * (S.K + 1.0), k3 = 0.5 * (S.K + 3.0);
+    const Real W[4] = {Real::raw(P.W[0]), Real::raw(P.W[1]), Real::raw(P.W[2]), Real::raw(P.W[3])};
+    const FlowState s = flow_state_again(W, tape_real(tp, base), S);
+    const FlowGrad x = point_grad(s, P.Wn, S), y = point_grad(s, P.Wt, S);
+    const Real i2th = tape_real(tp, base + 3);
+    HalfMom h;
+    h.m[0] = tape_real(tp, base + 1);
+    h.e1[0] = tape_real(tp, base + 2);                    // phi
+    h.m[1] = fma(s.U, h.m[0], s.th * h.e1[0]);
+    h.e2[0] = -(h.e1[0] * s.U) * i2th;
+    h.e2[1] = 0.5 * h.e1[0];
+    finish_moments(s, h);
+    FlowBar sb;
+    zero(sb);
+    sb.p = pb;
+    MomAdj mb;
+    GradBar xb, yb;
+    zero(xb);
+    zero(yb);
+    const Real hV2 = 0.5 * s.V * s.V, kth = k1 * s.th;
+    // c = rho <psi> and dg = rho <u psi>
     {
-        double ax[4];
-        tape_get_vec(tp, left ? TG_ALX : TG_ARX, ax);
-        AMomRev<0, 4, 0, 2> X(m, ax);
-        for (int i = 0; i < 4; ++i) tb[i] = Wcxb[i] * s.rho;
-        X.out_vjp<0, 0>(m, tb, mb);
-        X.out_vjp<2, 0>(m, M1b, mb);
-        X.finish(m, ax, mb, axb);
+        Real a[4], b[4];
+        to_lab_rev(s.V, hV2, Wcb, s.rho * h.m[0], 0.0, a, sb.V);
+        to_lab_rev(s.V, hV2, g0b, s.rho * h.m[1], 0.0, b, sb.V);
+        const Real A0 = fma(kth, a[3], a[0]), A1 = fma(kth, b[3], a[1] + b[0]), A2 = fma(0.5, a[3], b[1]), A3 = 0.5 * b[3];
+        sb.rho = fma(A0, h.m[0], fma(A1, h.m[1], fma(A2, h.m[2], A3 * h.m[3])));
+        sb.th = (k1 * s.rho) * fma(h.m[0], a[3], h.m[1] * b[3]);
+        mb.m[0] = s.rho * A0; mb.m[1] = s.rho * A1; mb.m[2] = s.rho * A2; mb.m[3] = s.rho * A3;
+        mb.m[4] = 0.0; mb.phi = 0.0; mb.e = 0.0;
+    }
+    // the two gradients' sums and their transport
+    const Real Nx0 = grad_mom(h, x, 0), Nx2 = grad_mom(h, x, 2), Ny0 = grad_mom(h, y, 0);
+    const Real Ny[3] = {grad_mom(h, y, 1), grad_mom(h, y, 2), grad_mom(h, y, 3)};
+    Real Nxb[5], Nyb[4];
+    {
+        Real a[4];
+        const Real v1 = y.r2 * h.m[1];
+        const Real o0 = fma(s.V, Ny[0], Nx2) + v1, o2 = fma(s.V, v1, fma(x.r2, h.m[2], fma(s.th, Ny[0], y.q3 * h.m[1])));
+        to_lab_rev(s.V, hV2, g1b, o0, o2, a, sb.V);
+        transport_rev(s, h, x, y, Nx2, Ny, k1, k3, a, Nxb + 2, Nyb + 1, xb, yb, mb, sb);
     }
     {
-        double ay[4];
-        tape_get_vec(tp, left ? TG_ALY : TG_ARY, ay);
-        AMomRev<0, 3, 0, 3> Y(m, ay);
-        for (int i = 0; i < 4; ++i) tb[i] = Wcyb[i] * s.rho;
-        Y.out_vjp<0, 0>(m, tb, mb);
-        Y.out_vjp<1, 1>(m, M1b, mb);
-        Y.finish(m, ay, mb, ayb);
+        Real a[4];
+        const Real p = x.r2 * h.m[0];
+        to_lab_rev(s.V, hV2, Wcxb, Nx0, p, a, sb.V);
+        const Real ka = k1 * a[3];
+        Nxb[0] = fma(s.th, ka, a[0]);
+        Nxb[1] = a[1];
+        Nxb[2] = fma(0.5, a[3], Nxb[2]);
+        xb.r2 = fma(a[2], h.m[0], xb.r2);
+        xb.q3 = fma(ka, h.m[0], xb.q3);
+        mb.m[0] = fma(a[2], x.r2, fma(ka, x.q3, mb.m[0]));
+        sb.th = fma(ka, Nx0, sb.th);
     }
-    // slope coefficients from the side's normal and tangential slopes (b = W_n / rho, W_t / rho)
-    double b[4], bb[4] = {0, 0, 0, 0};
-    for (int i = 0; i < 4; ++i) b[i] = P.Wn[i] * s.ir;
-    slope_solve_vjp(s, b, axb, bb, sb);
-    for (int i = 0; i < 4; ++i) {
-        Pb.Wn[i] += bb[i] * s.ir;
-        sb.ir += bb[i] * P.Wn[i];
-        bb[i] = 0.0;
-        b[i] = P.Wt[i] * s.ir;
+    {
+        Real a[4];
+        const Real p = y.r2 * h.m[0];
+        to_lab_rev(s.V, hV2, Wcyb, Ny0, p, a, sb.V);
+        const Real ka = k1 * a[3];
+        Nyb[0] = fma(s.th, ka, a[0]);
+        Nyb[1] = Nyb[1] + a[1];
+        Nyb[2] = fma(0.5, a[3], Nyb[2]);
+        yb.r2 = fma(a[2], h.m[0], yb.r2);
+        yb.q3 = fma(ka, h.m[0], yb.q3);
+        mb.m[0] = fma(a[2], y.r2, fma(ka, y.q3, mb.m[0]));
+        sb.th = fma(ka, Ny0, sb.th);
     }
-    slope_solve_vjp(s, b, ayb, bb, sb);
-    for (int i = 0; i < 4; ++i) { Pb.Wt[i] += bb[i] * s.ir; sb.ir += bb[i] * P.Wt[i]; }
-    fill_moments_vjp<SIGN>(s, S.K, m, mb, sb);
-    maxw_of_vjp(P.W, S, s, sb, Pb.W);
+    grad_mom_rev<0, 4>(h, x, Nxb, xb, mb);
+    grad_mom_rev<0, 3>(h, y, Nyb, yb, mb);
+    if (S.tau_reading == 1) {                             // g2 = rho <u A psi>
+        const FlowGrad t = euler_time_grad(s, x, y, S);
+        GradBar tb;
+        zero(tb);
+        const Real N1 = grad_mom(h, t, 1), p = t.r2 * h.m[1];
+        Real a[4], Ntb[3];
+        to_lab_rev(s.V, hV2, g2b, N1, p, a, sb.V);
+        const Real ka = k1 * a[3];
+        Ntb[0] = fma(s.th, ka, a[0]);
+        Ntb[1] = a[1];
+        Ntb[2] = 0.5 * a[3];
+        tb.r2 = a[2] * h.m[1];
+        tb.q3 = ka * h.m[1];
+        mb.m[1] = fma(a[2], t.r2, fma(ka, t.q3, mb.m[1]));
+        sb.th = fma(ka, N1, sb.th);
+        grad_mom_rev<1, 3>(h, t, Ntb, tb, mb);
+        euler_time_grad_rev(s, x, y, t, tb, S, xb, yb, sb);
+    }
+    // moments to U and theta
+    {
+        const Real U2 = 2.0 * (s.U * s.U) * i2th;         // U^2 / theta
+        const Real psi = (h.e1[0] * i2th) * (U2 - 1.0);
+        Real u = fma(2.0 * mb.phi, h.e2[0], mb.e * psi), th = fma(mb.phi, psi, (mb.e * h.e2[0]) * (i2th * (U2 - 3.0)));
+#pragma unroll
+        for (int k = 0; k < 5; ++k) { u = fma(mb.m[k], h.e1[k], u); th = fma(mb.m[k], h.e2[k], th); }
+        sb.U = sb.U + u;
+        sb.th = sb.th + th;
+    }
+    Real d[4];
+    flow_grad_rev(s, x.r0, x, xb, S, d, sb);
+#pragma unroll
+    for (int i = 0; i < 4; ++i) Pb.Wn[i] = d[i].v;
+    flow_grad_rev(s, y.r0, y, yb, S, d, sb);
+#pragma unroll
+    for (int i = 0; i < 4; ++i) Pb.Wt[i] = d[i].v;
+    flow_state_rev(s, sb, S, d);
+#pragma unroll
+    for (int i = 0; i < 4; ++i) Pb.W[i] = d[i].v;
 }
 
-// reverse of gks_flux from its taped forward intermediates: given Fb, dFb (local frame) accumulates
-// into Lb, Rb.  The tau = tau_n reading's extra terms are recomputed from the tape.  Taped values
-// are read where they are used: the reverse holds many adjoint accumulators at once, and values
-// kept live from the start would spill.
+// reverse of the GKS flux from its tape: sets the Gauss-point state adjoints Lb, Rb for the adjoints Fb, dFb
+// (local frame) of F and dF
 template <class Tape>
-DFK_HD void gks_flux_reverse(const Tape& tp, const GPState& L, const GPState& R, double dt, const SchemeConsts& S,
-                             const double Fb[4], const double dFb[4], GPStateBar& Lb, GPStateBar& Rb) {
-    const double K = S.K;
-    const Maxw sl = tape_get_maxw(tp, TG_SL), sr = tape_get_maxw(tp, TG_SR), sc = tape_get_maxw(tp, TG_SC);
-    const double q = tp.get(TG_Q);
-    double rT = S.C1 + S.C2 * fabs(q);
-    TimeCoeffs tc = time_coeffs(rT, dt, S.tau_reading);
-    double Ml2[4] = {0, 0, 0, 0}, Mr2[4] = {0, 0, 0, 0};
-    if (S.tau_reading == 1) {
-        Mom m, mF;
-        double bA[4], A[4];
-        tau_side_terms<+1>(tp, sl, K, mF, bA, A);
-        tape_get_mom(tp, TG_ML, m);
-        a_mom<1, 0>(m, A, Ml2);
-        tau_side_terms<-1>(tp, sr, K, mF, bA, A);
-        tape_get_mom(tp, TG_MR, m);
-        a_mom<1, 0>(m, A, Mr2);
-    }
-    // ---- reverse of the final combination
-    MaxwBar slb, srb, scb;
-    zero(slb); zero(srb); zero(scb);
-    double Mc0b[4], Mc1b[4], Mc2b[4], Ml0b[4], Mr0b[4], Ml1b[4], Mr1b[4], Ml2b[4], Mr2b[4];
-    double rTb = 0.0;
-    for (int i = 0; i < 4; ++i) {
-        const double Mc0 = tp.get(TG_MC0 + i), Mc1 = tp.get(TG_MC1 + i), Mc2 = tp.get(TG_MC2 + i);
-        const double Ml0 = tp.get(TG_ML0 + i), Mr0 = tp.get(TG_MR0 + i);
-        const double Ml1 = tp.get(TG_ML1 + i), Mr1 = tp.get(TG_MR1 + i);
-        double c0 = sc.rho * Mc0, c1 = sc.rho * Mc1, c2 = sc.rho * Mc2;
-        double g0 = sl.rho * Ml0 + sr.rho * Mr0;
-        double g1 = sl.rho * Ml1 + sr.rho * Mr1;
-        double g2 = sl.rho * Ml2[i] + sr.rho * Mr2[i];
-        double c0b = Fb[i] * tc.gcF.v + dFb[i] * tc.gcD.v;
-        double c1b = Fb[i] * tc.acF.v + dFb[i] * tc.acD.v;
-        double c2b = Fb[i] * tc.AcF.v + dFb[i] * tc.AcD.v;
-        double g0b = Fb[i] * tc.glrF.v + dFb[i] * tc.glrD.v;
-        double g1b = Fb[i] * tc.alrF.v + dFb[i] * tc.alrD.v;
-        double g2b = Fb[i] * tc.AlrF.v + dFb[i] * tc.AlrD.v;
-        rTb += Fb[i] * (tc.gcF.d * c0 + tc.acF.d * c1 + tc.AcF.d * c2 + tc.glrF.d * g0 + tc.alrF.d * g1 + tc.AlrF.d * g2)
-             + dFb[i] * (tc.gcD.d * c0 + tc.acD.d * c1 + tc.AcD.d * c2 + tc.glrD.d * g0 + tc.alrD.d * g1 + tc.AlrD.d * g2);
-        scb.rho += c0b * Mc0 + c1b * Mc1 + c2b * Mc2;
-        Mc0b[i] = c0b * sc.rho; Mc1b[i] = c1b * sc.rho; Mc2b[i] = c2b * sc.rho;
-        slb.rho += g0b * Ml0 + g1b * Ml1 + g2b * Ml2[i];
-        srb.rho += g0b * Mr0 + g1b * Mr1 + g2b * Mr2[i];
-        Ml0b[i] = g0b * sl.rho; Ml1b[i] = g1b * sl.rho; Ml2b[i] = g2b * sl.rho;
-        Mr0b[i] = g0b * sr.rho; Mr1b[i] = g1b * sr.rho; Mr2b[i] = g2b * sr.rho;
-    }
-    // tau_n / dt = C1 + C2 |(pl - pr)/(pl + pr)|
+DFK_HD void gks_flux_reverse(const Tape& tp, const GPState& L, const GPState& R, const SchemeConsts& S, const double Fbv[4],
+                             const double dFbv[4], GPStateBar& Lb, GPStateBar& Rb) {
+    const Real k1 = 0.5 * (S.K + 1.0), k3 = 0.5 * (S.K + 3.0);
+    // the final combination and tau_n / dt
+    Real c0b[4], c1b[4], c2b[4], g0b[4], g1b[4], g2b[4], rTb = 0.0;
     {
-        double sg = q >= 0.0 ? 1.0 : -1.0;
-        double den = (sl.p + sr.p) * (sl.p + sr.p);
-        slb.p += rTb * S.C2 * sg * 2.0 * sr.p / den;
-        srb.p += rTb * S.C2 * sg * (-2.0) * sl.p / den;
-    }
-    // ---- the equilibrium state's part: its flux moments and the compatibility condition of A^c
-    // (the moment sums of a_x and of a_y reversed together: their outputs share P, Q terms), its
-    // slopes and its Maxwellian
-    double Wcb[4] = {0, 0, 0, 0}, Wcxb[4], Wcyb[4];
-    {
-        Mom mc;
-        tape_get_mom(tp, TG_MC, mc);
-        MomBar mcb;
-        zero(mcb);
-        double Acb[4] = {0, 0, 0, 0}, bctb[4] = {0, 0, 0, 0}, acxb[4] = {0, 0, 0, 0}, acyb[4] = {0, 0, 0, 0};
-        psi_mom_vjp<1, 0, 0>(mc, Mc0b, mcb);
-        {
-            double Ac[4];
-            tape_get_vec(tp, TG_AC, Ac);
-            a_mom_vjp<1, 0>(mc, Ac, Mc2b, mcb, Acb);
+        const Real gF = tape_real(tp, TG_GF), gD = tape_real(tp, TG_GD), aF = tape_real(tp, TG_AF), aD = tape_real(tp, TG_AD);
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            const Real Fb = Real::raw(Fbv[i]), Db = Real::raw(dFbv[i]);
+            g0b[i] = fma(Fb, gF, Db * gD);
+            c0b[i] = Fb - g0b[i];
+            c1b[i] = fma(Fb, aF, Db * aD);
+            g1b[i] = -c1b[i];
+            c2b[i] = Db;
+            rTb = fma(Fb, tape_real(tp, TG_FR + i), fma(Db, tape_real(tp, TG_DFR + i), rTb));
         }
-        {
-            double bct[4];
-            tape_get_vec(tp, TG_BCT, bct);
-            slope_solve_vjp(sc, bct, Acb, bctb, scb);
-        }
-        {
-            double acx[4], acy[4], nb[4];
-            tape_get_vec(tp, TG_ACX, acx);
-            tape_get_vec(tp, TG_ACY, acy);
-            for (int i = 0; i < 4; ++i) nb[i] = -bctb[i];
-            AMomRev<1, 4, 0, 2> Cx(mc, acx);
-            AMomRev<0, 3, 0, 3> Cy(mc, acy);
-            Cx.out_vjp<2, 0>(mc, Mc1b, mcb);
-            Cx.out_vjp<1, 0>(mc, nb, mcb);
-            Cx.finish(mc, acx, mcb, acxb);
-            Cy.out_vjp<1, 1>(mc, Mc1b, mcb);
-            Cy.out_vjp<0, 1>(mc, nb, mcb);
-            Cy.finish(mc, acy, mcb, acyb);
-        }
-        {
-            double Wcx[4], Wcy[4], bcx[4], bcy[4], bcxb[4] = {0, 0, 0, 0}, bcyb[4] = {0, 0, 0, 0};
-            tape_get_vec(tp, TG_WCX, Wcx);
-            tape_get_vec(tp, TG_WCY, Wcy);
-            for (int i = 0; i < 4; ++i) { bcx[i] = Wcx[i] * sc.ir; bcy[i] = Wcy[i] * sc.ir; }
-            slope_solve_vjp(sc, bcx, acxb, bcxb, scb);
-            slope_solve_vjp(sc, bcy, acyb, bcyb, scb);
+        if (S.tau_reading == 1) {
+            const Real T = tape_real(tp, TG_T), cF = tape_real(tp, TG_CF), cD = tape_real(tp, TG_CD), bF = tape_real(tp, TG_BF);
+#pragma unroll
             for (int i = 0; i < 4; ++i) {
-                Wcxb[i] = bcxb[i] * sc.ir;
-                Wcyb[i] = bcyb[i] * sc.ir;
-                scb.ir += bcxb[i] * Wcx[i] + bcyb[i] * Wcy[i];
+                const Real Fb = Real::raw(Fbv[i]), Db = Real::raw(dFbv[i]);
+                g1b[i] = fma(-Fb, T, g1b[i]);
+                c2b[i] = fma(-Db, cD, fma(Fb, cF, Db));
+                g2b[i] = fma(Fb, bF, Db * cD);
             }
         }
-        fill_moments_vjp<0>(sc, K, mc, mcb, scb);
-        double Wc[4];
-        tape_get_vec(tp, TG_WC, Wc);
-        maxw_of_vjp(Wc, S, sc, scb, Wcb);
     }
-    // ---- the two sides
-    gks_side_reverse<+1>(tp, L, sl, S, Wcb, Wcxb, Wcyb, Ml0b, Ml1b, Ml2b, slb, Lb);
-    gks_side_reverse<-1>(tp, R, sr, S, Wcb, Wcxb, Wcyb, Mr0b, Mr1b, Mr2b, srb, Rb);
+    // the equilibrium state
+    Real Wcb[4], Wcxb[4], Wcyb[4];
+    {
+        Real Wc[4], d[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) Wc[i] = tape_real(tp, TG_WC + i);
+        const FlowState c = flow_state_again(Wc, tape_real(tp, TG_IRC), S);
+#pragma unroll
+        for (int i = 0; i < 4; ++i) d[i] = tape_real(tp, TG_WCX + i);
+        const FlowGrad x = flow_grad(c, d, S);
+#pragma unroll
+        for (int i = 0; i < 4; ++i) d[i] = tape_real(tp, TG_WCY + i);
+        const FlowGrad y = flow_grad(c, d, S);
+        const FlowGrad t = euler_time_grad(c, x, y, S);
+        HalfMom h;
+        h.m[0] = 1.0; h.m[1] = c.U;
+        h.e1[0] = 0.0; h.e2[0] = 0.0; h.e2[1] = 0.0;
+        finish_moments(c, h);
+        const Real hV2 = 0.5 * c.V * c.V, hU2 = 0.5 * c.U * c.U, gg = 0.5 * (S.K + 4.0), ru = Wc[1];
+        FlowBar sb;
+        zero(sb);
+        Real rub, a[4];
+        to_lab_rev(c.V, hV2, c0b, ru, 0.0, a, sb.V);
+        {
+            const Real g3 = gg * a[3];
+            rub = fma(hU2, a[3], fma(c.U, a[1], a[0]));
+            sb.U = fma(ru, fma(c.U, a[3], a[1]), g3 * c.p);
+            sb.p = fma(g3, c.U, a[1]);
+        }
+        GradBar xb, yb, tb;
+        zero(xb); zero(yb); zero(tb);
+        const Real n1 = fma(c.U, t.r0, t.r1);
+        to_lab_rev(c.V, hV2, c2b, n1, c.U * t.r2, a, sb.V);
+        {
+            const Real g3 = gg * a[3], U1 = c.U * a[1], H = hU2 * a[3];
+            const Real n1b = a[0] + U1 + H;
+            tb.r0 = c.U * n1b;
+            tb.r1 = fma(2.0, H, U1) + fma(g3, c.th, n1b);
+            tb.r2 = c.U * a[2];
+            tb.dp = fma(g3, c.U, a[1]);
+            sb.U = fma(n1 + t.r1, a[1], fma(t.r2, a[2], fma(c.U * a[3], fma(2.0, t.r1, n1), fma(g3, t.dp, fma(t.r0, n1b, sb.U)))));
+            sb.th = fma(g3, t.r1, sb.th);
+        }
+        euler_time_grad_rev(c, x, y, t, tb, S, xb, yb, sb);
+        MomAdj mb;
+#pragma unroll
+        for (int k = 0; k < 5; ++k) mb.m[k] = 0.0;
+        mb.phi = 0.0; mb.e = 0.0;
+        const Real Nx2 = grad_mom(h, x, 2), Ny[3] = {fma(c.U, y.r0, y.r1), grad_mom(h, y, 2), grad_mom(h, y, 3)};
+        Real Nxb[3], Nyb[3];
+        const Real v1 = y.r2 * h.m[1];
+        const Real o0 = fma(c.V, Ny[0], Nx2) + v1, o2 = fma(c.V, v1, fma(x.r2, h.m[2], fma(c.th, Ny[0], y.q3 * h.m[1])));
+        to_lab_rev(c.V, hV2, c1b, o0, o2, a, sb.V);
+        transport_rev(c, h, x, y, Nx2, Ny, k1, k3, a, Nxb, Nyb, xb, yb, mb, sb);
+        grad_mom_rev<2, 4>(h, x, Nxb, xb, mb);
+        grad_mom_rev<1, 3>(h, y, Nyb, yb, mb);
+        sb.U = sb.U + mb.m[1];
+#pragma unroll
+        for (int k = 2; k < 5; ++k) { sb.U = fma(mb.m[k], h.e1[k], sb.U); sb.th = fma(mb.m[k], h.e2[k], sb.th); }
+        flow_grad_rev(c, x.r0, x, xb, S, Wcxb, sb);
+        flow_grad_rev(c, y.r0, y, yb, S, Wcyb, sb);
+        flow_state_rev(c, sb, S, Wcb);
+        Wcb[1] = Wcb[1] + rub;
+    }
+    gks_side_reverse<+1>(tp, L, S, Wcb, Wcxb, Wcyb, g0b, g1b, g2b, rTb * tape_real(tp, TG_PL), Lb);
+    gks_side_reverse<-1>(tp, R, S, Wcb, Wcxb, Wcyb, g0b, g1b, g2b, rTb * tape_real(tp, TG_PR), Rb);
 }
 
-// adjoint of gks_flux: the forward recomputed into a local tape, then its reverse
+// reverse of gks_flux: the forward evaluated again into a local tape, then its reverse; sets Lb, Rb
 DFK_HD void gks_flux_vjp(const GPState& L, const GPState& R, double dt, const SchemeConsts& S,
                          const double Fb[4], const double dFb[4], GPStateBar& Lb, GPStateBar& Rb) {
     double t[TG_COUNT], F[4], dF[4];
     ArrayTape tp{t};
-    gks_flux_t(L, R, dt, S, F, dF, tp);
-    gks_flux_reverse(tp, L, R, dt, S, Fb, dFb, Lb, Rb);
+    gks_flux_sides(L, R, side_state(L.W, S), side_state(R.W, S), dt, S, F, dF, tp);
+    gks_flux_reverse(tp, L, R, S, Fb, dFb, Lb, Rb);
 }
 
 // ------------------------------------------------------------------------------------------

@@ -475,20 +475,13 @@ DFK_HD void flux_point(int dir, const SchemeConsts& S, const FluxSite& site, con
     // always evaluated (the default path stays branch-free); the cell-average reading, when selected,
     // overwrites it with its face line's value
     double F[4], dF[4];
-    if constexpr (TAPE && FLUX == 0) {
-        Maxw sl, sr;
-        maxw_pair(L.W, R.W, S, sl, sr);
-        fr[FR_ALPHA * fs + e] = df_alpha_maxw(sl, sr, S);
-        if (S.df_states) fr[FR_ALPHA * fs + e] = lines[LR_DFC * ls + site.li];
-        gks_flux_t(L, R, sl, sr, dt, S, F, dF, PlaneTape{tape + e, fs});
-    } else {
-        const FlowState sl = side_state(L.W, S), sr = side_state(R.W, S);
-        fr[FR_ALPHA * fs + e] = df_alpha_sides(sl, sr, S).v;
-        if (S.df_states) fr[FR_ALPHA * fs + e] = lines[LR_DFC * ls + site.li];
-        if (ALPHA_ONLY) return;
-        if (FLUX == 0) gks_flux_sides(L, R, sl, sr, dt, S, F, dF);
-        else lf_flux(L, R, S, F, dF);
-    }
+    const FlowState sl = side_state(L.W, S), sr = side_state(R.W, S);
+    fr[FR_ALPHA * fs + e] = df_alpha_sides(sl, sr, S).v;
+    if (S.df_states) fr[FR_ALPHA * fs + e] = lines[LR_DFC * ls + site.li];
+    if (ALPHA_ONLY) return;
+    if constexpr (FLUX == 1) lf_flux(L, R, S, F, dF);
+    else if constexpr (TAPE) gks_flux_sides(L, R, sl, sr, dt, S, F, dF, PlaneTape{tape + e, fs});
+    else gks_flux_sides(L, R, sl, sr, dt, S, F, dF, NoTape{});
     if (dir == 1) { to_global<1>(F); to_global<1>(dF); }
 #pragma unroll
     for (int k = 0; k < 4; ++k) { fr[(FR_F + k) * fs + e] = F[k]; fr[(FR_DF + k) * fs + e] = dF[k]; }

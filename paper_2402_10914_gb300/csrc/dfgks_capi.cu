@@ -41,6 +41,7 @@ struct dfgks {
     double* adj_lines;     // reverse sweep: face-line record adjoints
     double* adj_gp;        // reverse sweep: Gauss-point record adjoints
     double* adj_Wg;        // reverse sweep: ghosted cell adjoints
+    double* adj_tape;      // reverse sweep: the GKS flux's tape of one direction (optional)
     // checkpointed forward pass kept for dfgks_adjoint_checkpointed
     double* ck_W;          // dense [nseg][4][ny][nx]: W at steps 0, k, 2k, ...
     double* ck_A;          // dense [nseg][ny][nx]: alpha at the same steps
@@ -122,7 +123,7 @@ static bool config_ok(const dfgks_config* c) {
 static void free_all(dfgks* h) {
     double* ptrs[] = {h->W[0], h->W[1], h->A[0], h->A[1], h->Ws, h->As, h->acc, h->B.lines, h->B.gp,
                       h->B.flux[0], h->B.flux[1], h->By.lines, h->By.gp, h->dt_scratch, h->dts, h->adj_lines,
-                      h->adj_gp, h->adj_Wg};
+                      h->adj_gp, h->adj_Wg, h->adj_tape};
     for (double* p : ptrs) if (p) cudaFree(p);
     if (h->seg_arena) cudaFree(h->seg_arena);
     if (h->ck_W) cudaFree(h->ck_W);
@@ -485,6 +486,16 @@ static dfgks_status ensure_adjoint_buffers(dfgks* h) {
     CK(dalloc(h, &h->adj_lines, (long long)LR_COUNT * h->B.line_stride));
     CK(dalloc(h, &h->adj_gp, (long long)GP_COUNT * h->B.gp_stride));
     CK(dalloc(h, &h->adj_Wg, 4 * h->mesh.plane));
+    // The GKS flux's tape of one direction, for reverse sweeps that evaluate their forward first: its reverse
+    // then does not evaluate the flux a second time.  Left out where it would take more than a quarter of the
+    // free memory.
+    const long long n = (long long)TG_COUNT * (h->B.flux_stride[0] > h->B.flux_stride[1] ? h->B.flux_stride[0] : h->B.flux_stride[1]);
+    size_t free_b = 0, total_b = 0;
+    cudaMemGetInfo(&free_b, &total_b);
+    if ((double)n * sizeof(double) <= 0.25 * (double)free_b && dalloc(h, &h->adj_tape, n) != cudaSuccess) {
+        cudaGetLastError();
+        h->adj_tape = nullptr;
+    }
     return DFGKS_OK;
 }
 
@@ -502,11 +513,13 @@ static dfgks_status adjoint_stage(dfgks* h, const double* W, const double* alpha
     launch_set_scalar(h->dt_scratch, dt, h->stream);
     CK(cudaMemsetAsync(h->adj_Wg, 0, sizeof(double) * 4 * h->mesh.plane, h->stream));
     AdjointArgs a = {L_bar, dtL_bar, dtLt_bar};
+    SweepBuffers own = h->B;
+    if (flux == DFGKS_FLUX_GKS) own.tape[0] = own.tape[1] = h->adj_tape;
     for (int d = 0; d < 2; ++d) {
         // the records of this direction, then its reverse sweep
         if (!rec)
-            launch_sweep(d, h->mesh, h->S, flux, false, h->Ws, h->As, h->dt_scratch, h->B, nullptr, nullptr, h->stream);
-        launch_adjoint_dir(d, h->mesh, h->S, flux, a, h->Ws, h->As, h->dt_scratch, rec ? rec[d] : h->B, h->adj_lines,
+            launch_sweep(d, h->mesh, h->S, flux, false, h->Ws, h->As, h->dt_scratch, own, nullptr, nullptr, h->stream);
+        launch_adjoint_dir(d, h->mesh, h->S, flux, a, h->Ws, h->As, h->dt_scratch, rec ? rec[d] : own, h->adj_lines,
                            h->adj_gp, h->adj_Wg, h->stream, h->timer->on ? h->timer : nullptr);
     }
     launch_adjoint_finish(h->mesh, h->adj_Wg, W_bar, h->stream);

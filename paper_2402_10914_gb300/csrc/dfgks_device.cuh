@@ -10,7 +10,7 @@
 //     fixes a0), so smoothness indicators (Eq. 38) and every evaluation point share them;
 //   * S2O4 flux coefficients (Eq. 27) combined analytically per kinetic term before the moments
 //     are summed, using E(dt) = E(dt/2)^2, which avoids the cancellation of 4(F(dt)-2F(dt/2));
-//   * the GKS slope system <a psi> = b (Sect. 2.2) solved in closed form.
+//   * GKS moments of slope polynomials (Sect. 2.2) as derivatives of the moments themselves.
 #pragma once
 #include <cuda_runtime.h>
 #include <math.h>
@@ -502,18 +502,9 @@ DFK_HD void df_at_gauss(const double q[5], double alpha, double val[2], double s
 }
 
 // ------------------------------------------------------------------------------------------
-// Gas-kinetic flux at one Gauss point in the local frame (Sect. 2.2, 3.4; Eqs. 25-27).
-// Maxwellian moments are normalised by rho.  <u^k v^l xi^{2c}> = mu[k] mv[l] mx[c].
+// A side's Maxwellian for the DF factor of two cell averages (df_alpha)
 // ------------------------------------------------------------------------------------------
-struct Mom {
-    double mu[7];   // <u^n>, full or half-space
-    double mv[6];   // <v^n>, full
-    double mx[3];   // <1>, <xi^2>, <xi^4>
-};
-
-// One Maxwellian: il2 = 1/(2 lambda) = p/rho, tl = 2 lambda, f4 = 4 lambda^2/(K+2),
-// qK = U^2 + V^2 + (K+2)/(2 lambda); the slope solves of a state share them.
-struct Maxw { double rho, ir, U, V, p, il2, tl, f4, qK, isl; };   // isl = 1/sqrt(lambda)
+struct Maxw { double rho, ir, U, V, p, tl, isl; };   // tl = 2 lambda = rho/p, isl = 1/sqrt(lambda)
 
 // velocities and pressure of W given ir = 1/rho
 DFK_HD void maxw_velocities(const double W[4], double ir, const SchemeConsts& S, Maxw& s) {
@@ -525,24 +516,14 @@ DFK_HD void maxw_velocities(const double W[4], double ir, const SchemeConsts& S,
 }
 
 // the rest given tl = 2 lambda = rho / p
-DFK_HD void maxw_finish(double tl, const SchemeConsts& S, Maxw& s) {
+DFK_HD void maxw_finish(double tl, Maxw& s) {
     s.tl = tl;
-    s.il2 = s.p * s.ir;
-    s.f4 = tl * tl * S.inv_K2;
-    s.qK = s.U * s.U + s.V * s.V + (S.K + 2.0) * s.il2;
-    s.isl = rsqrt(0.5 * tl);           // the half-space moments and the DF factor's 1/c need it
-}
-
-DFK_HD Maxw maxw_of(const double W[4], const SchemeConsts& S) {
-    Maxw s;
-    maxw_velocities(W, 1.0 / W[0], S, s);
-    maxw_finish(W[0] / s.p, S, s);
-    return s;
+    s.isl = rsqrt(0.5 * tl);
 }
 
 // the two sides' Maxwellians with two divisions instead of four: 1/(rho_l rho_r) gives both 1/rho
 // and 1/(p_l p_r) both rho/p.  A product outside [1e-150, 1e150] (non-physical or extreme states)
-// is divided side by side as in maxw_of.
+// is divided side by side.
 DFK_HD void maxw_pair(const double WL[4], const double WR[4], const SchemeConsts& S, Maxw& a, Maxw& b) {
     const double rr = WL[0] * WR[0];
     if (in_range(rr, 1e-150, 1e150)) {
@@ -556,287 +537,18 @@ DFK_HD void maxw_pair(const double WL[4], const double WR[4], const SchemeConsts
     const double pp = a.p * b.p;
     if (in_range(pp, 1e-150, 1e150)) {
         const double r = 1.0 / pp;
-        maxw_finish(WL[0] * b.p * r, S, a);
-        maxw_finish(WR[0] * a.p * r, S, b);
+        maxw_finish(WL[0] * b.p * r, a);
+        maxw_finish(WR[0] * a.p * r, b);
     } else {
-        maxw_finish(WL[0] / a.p, S, a);
-        maxw_finish(WR[0] / b.p, S, b);
+        maxw_finish(WL[0] / a.p, a);
+        maxw_finish(WR[0] / b.p, b);
     }
-}
-
-// half: 0 full, +1 u>0, -1 u<0
-template <int HALF>
-DFK_HD void fill_moments(const Maxw& s, double K, Mom& m) {
-    if (HALF == 0) {
-        m.mu[0] = 1.0;
-        m.mu[1] = s.U;
-    } else {
-        double lam = 0.5 * s.tl;
-        double isl = s.isl;                                   // 1/sqrt(lambda)
-        double x = lam * isl * s.U;                           // sqrt(lambda) U
-        double G = exp(-x * x);
-        double e = G * (0.28209479177387814347 * isl);        // exp(-lambda U^2) / (2 sqrt(pi lambda))
-        // erfc(|x|) / 2 from the scaled function erfcx(|x|) = exp(x^2) erfc(|x|) and the Gaussian
-        // above (one exponential for both); erfc(-|x|) = 2 - erfc(|x|)
-#ifdef __CUDA_ARCH__
-        double h = 0.5 * G * erfcx(fabs(x));
-#else
-        double h = 0.5 * erfc(fabs(x));
-#endif
-        const bool xpos = dbits(x) >= 0;                      // x >= +0 (at -0 both forms give 1/2)
-        if (HALF > 0) { m.mu[0] = xpos ? 1.0 - h : h; m.mu[1] = s.U * m.mu[0] + e; }   // erfc(-x) / 2
-        else          { m.mu[0] = xpos ? h : 1.0 - h; m.mu[1] = s.U * m.mu[0] - e; }   // erfc(x) / 2
-    }
-#pragma unroll
-    for (int n = 2; n < 7; ++n) m.mu[n] = s.U * m.mu[n - 1] + (double)(n - 1) * s.il2 * m.mu[n - 2];
-    m.mv[0] = 1.0;
-    m.mv[1] = s.V;
-#pragma unroll
-    for (int n = 2; n < 6; ++n) m.mv[n] = s.V * m.mv[n - 1] + (double)(n - 1) * s.il2 * m.mv[n - 2];
-    m.mx[0] = 1.0;
-    m.mx[1] = K * s.il2;
-    m.mx[2] = K * (K + 2.0) * s.il2 * s.il2;
-}
-
-template <int k, int l, int c>
-DFK_HD double M(const Mom& m) { return m.mu[k] * m.mv[l] * m.mx[c]; }
-
-// <u^k v^l xi^{2c} psi>, psi = (1, u, v, (u^2+v^2+xi^2)/2)
-template <int k, int l, int c>
-DFK_HD void psi_mom(const Mom& m, double out[4]) {
-    out[0] = M<k, l, c>(m);
-    out[1] = M<k + 1, l, c>(m);
-    out[2] = M<k, l + 1, c>(m);
-    out[3] = 0.5 * (M<k + 2, l, c>(m) + M<k, l + 2, c>(m) + M<k, l, c + 1>(m));
-}
-
-// <u^k v^l a psi> with a = a0 + a1 u + a2 v + a3 (u^2+v^2+xi^2)/2.  With h = a3/2 and the
-// factorised moments <u^k v^l xi^2c> = mu_k mv_l mx_c (mx_0 = 1):
-//   G(k,l,c) = <u^k v^l xi^2c a> = mx_c (mv_l P_k + mu_k Q_l) + h mu_k mv_l mx_{c+1},
-//   P_k = a0 mu_k + a1 mu_{k+1} + h mu_{k+2},   Q_l = a2 mv_{l+1} + h mv_{l+2},
-// and out = (G(k,l,0), G(k+1,l,0), G(k,l+1,0), [G(k+2,l,0) + G(k,l+2,0) + G(k,l,1)] / 2).
-// Qp_j = Q_{l+j} + h mx_1 mv_{l+j} folds the xi^2 term into the c = 0 forms.
-template <int k, int l>
-DFK_HD void a_mom(const Mom& m, const double a[4], double out[4]) {
-    const double h = 0.5 * a[3], hx1 = h * m.mx[1];
-    double P[3], Qp[3];
-#pragma unroll
-    for (int j = 0; j < 3; ++j) {
-        P[j] = a[0] * m.mu[k + j] + a[1] * m.mu[k + j + 1] + h * m.mu[k + j + 2];
-        Qp[j] = a[2] * m.mv[l + j + 1] + h * m.mv[l + j + 2] + hx1 * m.mv[l + j];
-    }
-    const double Ql = a[2] * m.mv[l + 1] + h * m.mv[l + 2];
-    const double G1 = m.mx[1] * (m.mv[l] * P[0] + m.mu[k] * Ql) + h * m.mu[k] * m.mv[l] * m.mx[2];
-    out[0] = m.mv[l] * P[0] + m.mu[k] * Qp[0];
-    out[1] = m.mv[l] * P[1] + m.mu[k + 1] * Qp[0];
-    out[2] = m.mv[l + 1] * P[0] + m.mu[k] * Qp[1];
-    out[3] = 0.5 * ((m.mv[l] * P[2] + m.mu[k + 2] * Qp[0]) + (m.mv[l + 2] * P[0] + m.mu[k] * Qp[2]) + G1);
-}
-
-// closed-form solution of <a psi> = b for a Maxwellian (U, V, lambda)
-DFK_HD void slope_solve(const Maxw& s, const double b[4], double a[4]) {
-    double R2 = b[1] - s.U * b[0], R3 = b[2] - s.V * b[0], R4 = 2.0 * b[3] - s.qK * b[0];
-    a[3] = s.f4 * (R4 - 2.0 * s.U * R2 - 2.0 * s.V * R3);
-    a[2] = s.tl * R3 - s.V * a[3];
-    a[1] = s.tl * R2 - s.U * a[3];
-    a[0] = b[0] - s.U * a[1] - s.V * a[2] - 0.5 * a[3] * s.qK;
 }
 
 struct GPState { double W[4], Wn[4], Wt[4]; };   // one side of one Gauss point, local frame
 
-// Forward intermediates of gks_flux that its reverse reads (the tau = 0 reading's part), as a
-// tape of doubles: the three Maxwellians (rho, 1/rho, U, V, p, 1/(2 lambda), 2 lambda, f4, qK),
-// their moments (mu[7], mv[6], mx[3]), the slope coefficients, the compatibility right-hand side,
-// the equilibrium state and slopes, the kinetic-weighting moments, the flux moments and the
-// pressure ratio of tau_n.  A reverse sweep can read them back instead of recomputing the flux.
-enum GksTapeField {
-    TG_SL = 0, TG_SR = 9, TG_SC = 18, TG_ML = 27, TG_MR = 43, TG_MC = 59,
-    TG_ALX = 75, TG_ALY = 79, TG_ARX = 83, TG_ARY = 87, TG_ACX = 91, TG_ACY = 95, TG_AC = 99, TG_BCT = 103,
-    TG_WC = 107, TG_WCX = 111, TG_WCY = 115,
-    TG_PL0 = 119, TG_PR0 = 123, TG_LX0 = 127, TG_RX0 = 131, TG_LY0 = 135, TG_RY0 = 139,
-    TG_MC0 = 143, TG_MC1 = 147, TG_MC2 = 151, TG_ML0 = 155, TG_MR0 = 159, TG_ML1 = 163, TG_MR1 = 167,
-    TG_Q = 171, TG_COUNT = 172
-};
-
-
-template <class Tape>
-DFK_HD void tape_maxw(const Tape& tp, int b, const Maxw& s) {
-    tp.put(b, s.rho); tp.put(b + 1, s.ir); tp.put(b + 2, s.U); tp.put(b + 3, s.V); tp.put(b + 4, s.p);
-    tp.put(b + 5, s.il2); tp.put(b + 6, s.tl); tp.put(b + 7, s.f4); tp.put(b + 8, s.qK);
-}
-template <class Tape>
-DFK_HD void tape_mom(const Tape& tp, int b, const Mom& m) {
-#pragma unroll
-    for (int n = 0; n < 7; ++n) tp.put(b + n, m.mu[n]);
-#pragma unroll
-    for (int n = 0; n < 6; ++n) tp.put(b + 7 + n, m.mv[n]);
-#pragma unroll
-    for (int n = 0; n < 3; ++n) tp.put(b + 13 + n, m.mx[n]);
-}
-template <class Tape>
-DFK_HD void tape_vec(const Tape& tp, int b, const double v[4]) {
-#pragma unroll
-    for (int i = 0; i < 4; ++i) tp.put(b + i, v[i]);
-}
-
-// sl, sr: the Maxwellians of L.W and R.W (maxw_pair)
-template <class Tape>
-DFK_HD void gks_flux_t(const GPState& L, const GPState& R, const Maxw& sl, const Maxw& sr, double dt,
-                       const SchemeConsts& S, double F[4], double dF[4], const Tape& tp) {
-    const double K = S.K;
-    Mom ml, mr;
-    fill_moments<+1>(sl, K, ml);
-    fill_moments<-1>(sr, K, mr);
-    double b[4], alx[4], aly[4], arx[4], ary[4];
-    const double irl = sl.ir, irr = sr.ir;
-#pragma unroll
-    for (int i = 0; i < 4; ++i) b[i] = L.Wn[i] * irl;
-    slope_solve(sl, b, alx);
-#pragma unroll
-    for (int i = 0; i < 4; ++i) b[i] = L.Wt[i] * irl;
-    slope_solve(sl, b, aly);
-#pragma unroll
-    for (int i = 0; i < 4; ++i) b[i] = R.Wn[i] * irr;
-    slope_solve(sr, b, arx);
-#pragma unroll
-    for (int i = 0; i < 4; ++i) b[i] = R.Wt[i] * irr;
-    slope_solve(sr, b, ary);
-    tape_maxw(tp, TG_SL, sl); tape_maxw(tp, TG_SR, sr);
-    tape_mom(tp, TG_ML, ml); tape_mom(tp, TG_MR, mr);
-    tape_vec(tp, TG_ALX, alx); tape_vec(tp, TG_ALY, aly); tape_vec(tp, TG_ARX, arx); tape_vec(tp, TG_ARY, ary);
-    // Sect. 3.4: equilibrium state and slopes by kinetic weighting
-    double Wc[4], Wcx[4], Wcy[4], t1[4], t2[4];
-    psi_mom<0, 0, 0>(ml, t1); psi_mom<0, 0, 0>(mr, t2);
-    tape_vec(tp, TG_PL0, t1); tape_vec(tp, TG_PR0, t2);
-#pragma unroll
-    for (int i = 0; i < 4; ++i) Wc[i] = sl.rho * t1[i] + sr.rho * t2[i];
-    a_mom<0, 0>(ml, alx, t1); a_mom<0, 0>(mr, arx, t2);
-    tape_vec(tp, TG_LX0, t1); tape_vec(tp, TG_RX0, t2);
-#pragma unroll
-    for (int i = 0; i < 4; ++i) Wcx[i] = sl.rho * t1[i] + sr.rho * t2[i];
-    a_mom<0, 0>(ml, aly, t1); a_mom<0, 0>(mr, ary, t2);
-    tape_vec(tp, TG_LY0, t1); tape_vec(tp, TG_RY0, t2);
-#pragma unroll
-    for (int i = 0; i < 4; ++i) Wcy[i] = sl.rho * t1[i] + sr.rho * t2[i];
-    tape_vec(tp, TG_WC, Wc); tape_vec(tp, TG_WCX, Wcx); tape_vec(tp, TG_WCY, Wcy);
-    // the equilibrium state's Maxwellian: 1/rho_c shares a division with 1/dt, and rho_c / p_c one
-    // with 1/(p_l + p_r) of the pressure ratio in tau_n (products outside [1e-150, 1e150] are
-    // divided separately)
-    Maxw sc;
-    double idt, ips;
-    {
-        const double a = Wc[0] * dt;
-        if (in_range(a, 1e-150, 1e150)) {
-            const double r = 1.0 / a;
-            maxw_velocities(Wc, dt * r, S, sc);
-            idt = Wc[0] * r;
-        } else {
-            maxw_velocities(Wc, 1.0 / Wc[0], S, sc);
-            idt = 1.0 / dt;
-        }
-        const double ps = sl.p + sr.p, b = sc.p * ps;
-        if (in_range(b, 1e-150, 1e150)) {
-            const double r = 1.0 / b;
-            maxw_finish(Wc[0] * ps * r, S, sc);
-            ips = sc.p * r;
-        } else {
-            maxw_finish(Wc[0] / sc.p, S, sc);
-            ips = 1.0 / ps;
-        }
-    }
-    Mom mc;
-    fill_moments<0>(sc, K, mc);
-    tape_maxw(tp, TG_SC, sc); tape_mom(tp, TG_MC, mc);
-    double acx[4], acy[4], Ac[4];
-    const double irc = sc.ir;
-#pragma unroll
-    for (int i = 0; i < 4; ++i) b[i] = Wcx[i] * irc;
-    slope_solve(sc, b, acx);
-#pragma unroll
-    for (int i = 0; i < 4; ++i) b[i] = Wcy[i] * irc;
-    slope_solve(sc, b, acy);
-    // compatibility <A + a_x u + a_y v> = 0
-    a_mom<1, 0>(mc, acx, t1); a_mom<0, 1>(mc, acy, t2);
-#pragma unroll
-    for (int i = 0; i < 4; ++i) b[i] = -(t1[i] + t2[i]);
-    slope_solve(sc, b, Ac);
-    tape_vec(tp, TG_ACX, acx); tape_vec(tp, TG_ACY, acy); tape_vec(tp, TG_AC, Ac); tape_vec(tp, TG_BCT, b);
-    // moments entering the flux
-    double Mc0[4], Mc1[4], Mc2[4], Ml0[4], Mr0[4], Ml1[4], Mr1[4];
-    psi_mom<1, 0, 0>(mc, Mc0);
-    a_mom<2, 0>(mc, acx, t1); a_mom<1, 1>(mc, acy, t2);
-#pragma unroll
-    for (int i = 0; i < 4; ++i) Mc1[i] = t1[i] + t2[i];
-    a_mom<1, 0>(mc, Ac, Mc2);
-    psi_mom<1, 0, 0>(ml, Ml0);
-    psi_mom<1, 0, 0>(mr, Mr0);
-    a_mom<2, 0>(ml, alx, t1); a_mom<1, 1>(ml, aly, t2);
-#pragma unroll
-    for (int i = 0; i < 4; ++i) Ml1[i] = t1[i] + t2[i];
-    a_mom<2, 0>(mr, arx, t1); a_mom<1, 1>(mr, ary, t2);
-#pragma unroll
-    for (int i = 0; i < 4; ++i) Mr1[i] = t1[i] + t2[i];
-    tape_vec(tp, TG_MC0, Mc0); tape_vec(tp, TG_MC1, Mc1); tape_vec(tp, TG_MC2, Mc2);
-    tape_vec(tp, TG_ML0, Ml0); tape_vec(tp, TG_MR0, Mr0); tape_vec(tp, TG_ML1, Ml1); tape_vec(tp, TG_MR1, Mr1);
-    // numerical collision time (Sect. 2.2) and the combined time coefficients of Eq. 27
-    const double q = (sl.p - sr.p) * ips;
-    tp.put(TG_Q, q);
-    double rT = S.C1 + S.C2 * fabs(q);   // tau_n / dt
-    double T = rT * dt;
-    double tau = (S.tau_reading == 1) ? T : 0.0;
-    double E2 = 0.0, r = 0.0;
-    if (dbits(rT) > 0) { E2 = exp(-0.5 / rT); r = rT; }   // rT >= 0
-    double E1 = E2 * E2;
-    double om = 1.0 - E2;
-    double S3 = om * (3.0 - E2);                       // 3 - 4 E2 + E1
-    // F-coefficients (4 G(dt/2) - G(dt)) / dt and dF-coefficients 4 (G(dt) - 2 G(dt/2)) / dt^2
-    double glrF = r * S3, glrD = -4.0 * r * om * om * idt;
-    double gcF = 1.0 - glrF, gcD = -glrD;
-    double TT = T * T + T * tau;
-    double acF = TT * S3 * idt - 2.0 * T * E2 + T * E1 - tau;
-    double acD = 4.0 * (-TT * om * om + T * dt * E2 * om) * idt * idt;
-    double AcF = -tau + tau * r * S3;
-    double AcD = 1.0 - 4.0 * T * tau * om * om * idt * idt;
-    double alrF = -acF - tau, alrD = -acD;
-    double AlrF = -T * tau * S3 * idt, AlrD = 4.0 * T * tau * om * om * idt * idt;
-    double Ml2[4] = {0, 0, 0, 0}, Mr2[4] = {0, 0, 0, 0};
-    if (S.tau_reading == 1) {
-        Mom mlF, mrF;
-        fill_moments<0>(sl, K, mlF);
-        fill_moments<0>(sr, K, mrF);
-        double Al[4], Ar[4];
-        a_mom<1, 0>(mlF, alx, t1); a_mom<0, 1>(mlF, aly, t2);
-#pragma unroll
-        for (int i = 0; i < 4; ++i) b[i] = -(t1[i] + t2[i]);
-        slope_solve(sl, b, Al);
-        a_mom<1, 0>(mrF, arx, t1); a_mom<0, 1>(mrF, ary, t2);
-#pragma unroll
-        for (int i = 0; i < 4; ++i) b[i] = -(t1[i] + t2[i]);
-        slope_solve(sr, b, Ar);
-        a_mom<1, 0>(ml, Al, Ml2);
-        a_mom<1, 0>(mr, Ar, Mr2);
-    }
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-        double c0 = sc.rho * Mc0[i], c1 = sc.rho * Mc1[i], c2 = sc.rho * Mc2[i];
-        double g0 = sl.rho * Ml0[i] + sr.rho * Mr0[i];
-        double g1 = sl.rho * Ml1[i] + sr.rho * Mr1[i];
-        double g2 = sl.rho * Ml2[i] + sr.rho * Mr2[i];
-        F[i] = gcF * c0 + acF * c1 + AcF * c2 + glrF * g0 + alrF * g1 + AlrF * g2;
-        dF[i] = gcD * c0 + acD * c1 + AcD * c2 + glrD * g0 + alrD * g1 + AlrD * g2;
-    }
-}
-
-template <class Tape>
-DFK_HD void gks_flux_t(const GPState& L, const GPState& R, double dt, const SchemeConsts& S,
-                       double F[4], double dF[4], const Tape& tp) {
-    Maxw sl, sr;
-    maxw_pair(L.W, R.W, S, sl, sr);
-    gks_flux_t(L, R, sl, sr, dt, S, F, dF, tp);
-}
-
 // ------------------------------------------------------------------------------------------
-// The same flux in gradient form, for the forward sweeps.
+// Gas-kinetic flux at one Gauss point in the local frame (Sect. 2.2, 3.4; Eqs. 25-27), in gradient form.
 //
 // rho <a phi> with the slope polynomial a of a Maxwellian g (a g = the derivative of g along W') is the
 // derivative of the moment rho <phi> itself, so no slope coefficients are needed: with the primitive
@@ -853,6 +565,16 @@ DFK_HD void gks_flux_t(const GPState& L, const GPState& R, double dt, const Sche
 // slope coefficients and general products of moments, on a kernel bound by the FP64 units: 2.38 -> 1.38 ms
 // per 400 x 400 step (1.09 with vector-register operands and the tables below), 158 instead of 250 registers.
 // ------------------------------------------------------------------------------------------
+
+// What the flux's reverse (gks_flux_reverse) reads of its forward: per side 1/rho, m_0, the boundary value
+// phi (signed) and 1/(2 theta); the equilibrium state, its 1/rho and its two gradients; the time coefficients
+// of Eq. 27 (the last four under the tau = tau_n reading only); the derivatives of F and dF by tau_n/dt; and
+// that ratio's by the two pressures.  39 values: what costs a transcendental, a division or a sum over both
+// sides.  States, gradients and moments are cheaper to form again than to keep.
+enum GksTapeField {
+    TG_L = 0, TG_R = 4, TG_WC = 8, TG_IRC = 12, TG_WCX = 13, TG_WCY = 17,
+    TG_GF = 21, TG_GD, TG_AF, TG_AD, TG_T, TG_CF, TG_CD, TG_BF, TG_FR = 29, TG_DFR = 33, TG_PL = 37, TG_PR = 38, TG_COUNT = 39
+};
 
 // rcp() where its range holds, a division elsewhere (negative, zero, extreme)
 DFK_HD Real rcp_or_div(Real x) { return in_range(x, 1e-300, 1e300) ? rcp(x) : Real::raw(1.0 / x.v); }
@@ -1102,9 +824,22 @@ DFK_HD void side_time_sum(const FlowState& s, const FlowGrad& x, const FlowGrad&
     for (int i = 0; i < 4; ++i) g2[i] = g2[i] + o[i];
 }
 
+template <class Tape>
+DFK_HD void tape_side(const Tape& tp, int b, const FlowState& s, const HalfMom& h) {
+    if constexpr (Tape::active) { tp.put(b, s.ir.v); tp.put(b + 1, h.m[0].v); tp.put(b + 2, h.e1[0].v); tp.put(b + 3, Real(s.rs * s.rs).v); }
+}
+template <class Tape>
+DFK_HD void tape_vec(const Tape& tp, int b, const Real v[4]) {
+    if constexpr (Tape::active) {
+#pragma unroll
+        for (int i = 0; i < 4; ++i) tp.put(b + i, v[i].v);
+    }
+}
+
 // sl, sr: side_state of L.W and R.W
+template <class Tape>
 DFK_HD void gks_flux_sides(const GPState& L, const GPState& Rt, const FlowState& sl, const FlowState& sr, double dtv,
-                           const SchemeConsts& S, double F[4], double dF[4]) {
+                           const SchemeConsts& S, double F[4], double dF[4], const Tape& tp) {
     const Real dt = dtv;
     const Real k1 = 0.5 * (S.K + 1.0), k3 = 0.5 * (S.K + 3.0);
     // Sect. 3.4: the equilibrium state and its slopes by kinetic weighting, and the sides' flux moments
@@ -1113,6 +848,7 @@ DFK_HD void gks_flux_sides(const GPState& L, const GPState& Rt, const FlowState&
         const FlowGrad x = point_grad(sl, L.Wn, S), y = point_grad(sl, L.Wt, S);
         HalfMom h;
         half_moments<+1>(sl, h);
+        tape_side(tp, TG_L, sl, h);
         side_sums<+1>(sl, x, y, h, k1, k3, Wc, Wcx, Wcy, dg, g1);
         if (S.tau_reading == 1) side_time_sum(sl, x, y, h, S, k1, g2);
     }
@@ -1120,11 +856,14 @@ DFK_HD void gks_flux_sides(const GPState& L, const GPState& Rt, const FlowState&
         const FlowGrad x = point_grad(sr, Rt.Wn, S), y = point_grad(sr, Rt.Wt, S);
         HalfMom h;
         half_moments<-1>(sr, h);
+        tape_side(tp, TG_R, sr, h);
         side_sums<-1>(sr, x, y, h, k1, k3, Wc, Wcx, Wcy, dg, g1);
         if (S.tau_reading == 1) side_time_sum(sr, x, y, h, S, k1, g2);
     }
     // the equilibrium state: c0 = rho <u psi>, c1 = rho <u^2 a_x psi> + rho <u v a_y psi>, c2 = rho <u A psi>
     const FlowState c = flow_state(Wc, S);
+    tape_vec(tp, TG_WC, Wc); tape_vec(tp, TG_WCX, Wcx); tape_vec(tp, TG_WCY, Wcy);
+    if constexpr (Tape::active) tp.put(TG_IRC, c.ir.v);
     Real c0[4], c1[4], c2[4];
     {
         const FlowGrad x = flow_grad(c, Wcx, S), y = flow_grad(c, Wcy, S), t = euler_time_grad(c, x, y, S);
@@ -1152,36 +891,72 @@ DFK_HD void gks_flux_sides(const GPState& L, const GPState& Rt, const FlowState&
     }
     // numerical collision time (Sect. 2.2) and the time coefficients of Eq. 27 (4 G(dt/2) - G(dt)) / dt and
     // 4 (G(dt) - 2 G(dt/2)) / dt^2, combined with E(dt) = E(dt/2)^2
-    const Real q = (sl.p - sr.p) * rcp_or_div(sl.p + sr.p);
+    const Real ips = rcp_or_div(sl.p + sr.p), q = (sl.p - sr.p) * ips;
     const Real rT = fma(S.C2, fabs(q), S.C1);        // tau_n / dt
-    Real E2 = 0.0, r = 0.0;
-    if (dbits(rT.v) > 0) { E2 = exp_neg(0.5 * rcp_or_div(rT)); r = rT; }   // rT >= 0
-    const Real om = 1.0 - E2, om2 = om * om, rom = r * om;
-    const Real gF = rom * (3.0 - E2), gD = -4.0 * (r * om2) * rcp_or_div(dt);
-    if (S.tau_reading == 1) {
-        const Real T = r * dt, E1 = E2 * E2, idt = Real::raw(1.0 / dt.v), TT = 2.0 * T * T, S3 = om * (3.0 - E2);
-        const Real aF = TT * S3 * idt - 2.0 * T * E2 + T * E1 - T;
-        const Real aD = 4.0 * (-TT * om2 + T * dt * E2 * om) * idt * idt;
-        const Real AF = -T + T * gF, AD = 4.0 * T * T * om2 * idt * idt, BF = -T * T * S3 * idt;
+    Real E2 = 0.0, r = 0.0, h = 0.0;
+    const bool viscous = dbits(rT.v) > 0;            // rT >= 0
+    if (viscous) {
+        h = 0.5 * rcp_or_div(rT);
+        E2 = exp_neg(h);
+        r = rT;
+    }
+    const Real om = 1.0 - E2, om2 = om * om, rom = r * om, idt = rcp_or_div(dt);
+    const Real gF = rom * (3.0 - E2), gD = -4.0 * (r * om2) * idt;
+    const Real aF = (r * dt) * (gF + (om2 - 1.0)), aD = 4.0 * rom * (E2 - rom);
+    // their derivatives by r, with r E2' = h E2 (h = 1/(2 r))
+    [[maybe_unused]] Real hE, gFr, gDr, aFr, aDr;
+    if constexpr (Tape::active) {
+        hE = h * E2;
+        gFr = viscous ? fma(om, 3.0 - E2, -2.0 * hE * (2.0 - E2)) : Real(0.0);
+        gDr = viscous ? Real(-4.0 * (om * fma(-2.0, hE, om)) * idt) : Real(0.0);
+        aFr = dt * fma(r, gFr, fma(-2.0 * om, hE, gF + (om2 - 1.0)));
+        aDr = 4.0 * fma(om, E2, fma(hE, fma(2.0, rom, om - E2), -2.0 * rom * om));
+        tp.put(TG_GF, gF.v); tp.put(TG_GD, gD.v);
+        const Real k2 = (Real(2.0 * S.C2) * ips) * ips, kl = k2 * sr.p, kr = k2 * sl.p;
+        tp.put(TG_PL, dbits(q.v) >= 0 ? kl.v : -kl.v);
+        tp.put(TG_PR, dbits(q.v) >= 0 ? -kr.v : kr.v);
+    }
+    if (S.tau_reading == 1) {                        // tau = tau_n: aF, aD as below with r (..) for tau = 0 added
+        const Real T = r * dt, E1 = E2 * E2, TT = 2.0 * T * T, S3 = om * (3.0 - E2);
+        const Real bF = TT * S3 * idt - 2.0 * T * E2 + T * E1 - T;
+        const Real bD = 4.0 * (-TT * om2 + T * dt * E2 * om) * idt * idt;
+        const Real cF = -T + T * gF, cD = 4.0 * T * T * om2 * idt * idt, dF1 = -T * T * S3 * idt;
+        if constexpr (Tape::active) {
+            tp.put(TG_AF, bF.v); tp.put(TG_AD, bD.v); tp.put(TG_T, T.v); tp.put(TG_CF, cF.v); tp.put(TG_CD, cD.v); tp.put(TG_BF, dF1.v);
+        }
+        // derivatives by r: (r^2 S3)' = r (gF + r S3')..., S3' = -2 E2' (2 - E2), r E2' = hE
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
             const Real d = dg[i] - c0[i];
-            F[i] = (c0[i] + gF * d + aF * (c1[i] - g1[i]) - T * g1[i] + AF * c2[i] + BF * g2[i]).v;
-            dF[i] = (c2[i] + gD * d + aD * (c1[i] - g1[i]) + AD * (g2[i] - c2[i])).v;
+            F[i] = (c0[i] + gF * d + bF * (c1[i] - g1[i]) - T * g1[i] + cF * c2[i] + dF1 * g2[i]).v;
+            dF[i] = (c2[i] + gD * d + bD * (c1[i] - g1[i]) + cD * (g2[i] - c2[i])).v;
+            if constexpr (Tape::active) {
+                const Real rS = fma(-2.0 * hE, 2.0 - E2, 2.0 * S3);            // (r^2 S3)' / r
+                const Real bFr = dt * (2.0 * r * rS - 2.0 * (E2 + hE) + E1 + 2.0 * hE * E2 - 1.0);
+                const Real oo = 2.0 * rom * (om - hE);                          // (r^2 om^2)'
+                const Real bDr = 4.0 * (-2.0 * oo + E2 * om + hE * (om - E2));
+                const Real cFr = dt * (-1.0 + gF + r * gFr), cDr = 4.0 * oo, dFr = -dt * (r * rS);
+                tp.put(TG_FR + i, (gFr * d + bFr * (c1[i] - g1[i]) - dt * g1[i] + cFr * c2[i] + dFr * g2[i]).v);
+                tp.put(TG_DFR + i, (gDr * d + bDr * (c1[i] - g1[i]) + cDr * (g2[i] - c2[i])).v);
+            }
         }
         return;
     }
-    const Real aF = (r * dt) * (gF + (om2 - 1.0)), aD = 4.0 * rom * (E2 - rom);
+    if constexpr (Tape::active) { tp.put(TG_AF, aF.v); tp.put(TG_AD, aD.v); }
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
         const Real d = dg[i] - c0[i], e = c1[i] - g1[i];
         F[i] = fma(gF, d, fma(aF, e, c0[i])).v;
         dF[i] = fma(gD, d, fma(aD, e, c2[i])).v;
+        if constexpr (Tape::active) {
+            tp.put(TG_FR + i, fma(gFr, d, aFr * e).v);
+            tp.put(TG_DFR + i, fma(gDr, d, aDr * e).v);
+        }
     }
 }
 
 DFK_HD void gks_flux(const GPState& L, const GPState& R, double dt, const SchemeConsts& S, double F[4], double dF[4]) {
-    gks_flux_sides(L, R, side_state(L.W, S), side_state(R.W, S), dt, S, F, dF);
+    gks_flux_sides(L, R, side_state(L.W, S), side_state(R.W, S), dt, S, F, dF, NoTape{});
 }
 
 // ------------------------------------------------------------------------------------------
