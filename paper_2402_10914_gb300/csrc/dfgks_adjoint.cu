@@ -7,8 +7,8 @@
 //              Gauss-point record adjoints, and the time-limiter weight's adjoint.  When the
 //              forward sweep taped the GKS flux's intermediates, its reverse reads them instead
 //              of recomputing the flux.
-//   ka_faces : one thread per face side.  Evaluates each tangential reconstruction once, with its
-//              intermediates kept for its reverse (or reads them from the forward sweep's tape),
+//   ka_faces : one thread per face side.  Evaluates the ratios of each tangential reconstruction
+//              (or reads them from the forward sweep's tape), reverses it in differences,
 //              and scatters (atomically) into the adjoints of
 //              the five face lines and of the face basis; a Gauss point that fell back to the cell
 //              average (flagged in the forward record) sends its adjoint to that cell.
@@ -24,7 +24,7 @@ namespace dfk {
 
 DFK_HD void aadd(double* p, double v) {
 #ifdef __CUDA_ARCH__
-    if (v != 0.0) atomicAdd(p, v);
+    if (dbits(v) << 1) atomicAdd(p, v);         // not +-0, tested off the FP64 units
 #else
     *p += v;
 #endif
@@ -97,7 +97,16 @@ DFK_HD void ka_flux_body(const Mesh& m, const SchemeConsts& S, const AdjointArgs
     }
 }
 
-// TAPED: the tangential reconstructions' intermediates are read from the tape the forward sweep wrote
+// the face basis of a line record
+DFK_HD CharBasis line_basis(const double* __restrict__ lines, long long ls, long long l) {
+    CharBasis B;
+    B.u = lines[LR_U * ls + l]; B.v = lines[LR_V * ls + l]; B.c = lines[LR_C * ls + l];
+    B.ic = lines[LR_IC * ls + l]; B.H = lines[LR_H * ls + l]; B.b1 = lines[LR_B1 * ls + l];
+    B.b2 = lines[LR_B2 * ls + l]; B.q2 = lines[LR_Q2 * ls + l];
+    return B;
+}
+
+// TAPED: the tangential reconstructions' ratios are read from the tape the forward sweep wrote
 template <int DIR, bool TAPED = false>
 DFK_HD void ka_faces_body(const Mesh& m, const SchemeConsts& S, const double* __restrict__ alpha,
                           const double* __restrict__ lines, long long ls, const double* __restrict__ gp,
@@ -108,100 +117,185 @@ DFK_HD void ka_faces_body(const Mesh& m, const SchemeConsts& S, const double* __
     int t = DIR == 0 ? ay : ax;
     if (f > g.nn || t >= g.nt) return;
     const long long l0 = g.line(f, t);
-    CharBasis B;
-    B.u = lines[LR_U * ls + l0]; B.v = lines[LR_V * ls + l0]; B.c = lines[LR_C * ls + l0];
-    B.ic = lines[LR_IC * ls + l0]; B.H = lines[LR_H * ls + l0]; B.b1 = lines[LR_B1 * ls + l0];
-    B.b2 = lines[LR_B2 * ls + l0]; B.q2 = lines[LR_Q2 * ls + l0];
+    const DiffBasis D = diff_basis(line_basis(lines, ls, l0));
     const int wbase = side == 0 ? LR_WL : LR_WR;
     const int nbase = side == 0 ? LR_WLN : LR_WRN;
-    double Wl[5][4], Q[5][4];
-    for (int b = 0; b < 5; ++b) {
-        long long lbb = g.line(f, t + Geo<DIR>::sigma * (b - 2));
-        for (int k = 0; k < 4; ++k) Wl[b][k] = lines[(wbase + k) * ls + lbb];
-        project(B, Wl[b], Q[b]);
-    }
     const int ncell = f - 1 + side;
     double al[3];
+#pragma unroll
     for (int b = 0; b < 3; ++b) al[b] = alpha[g.cell(m, ncell, t + Geo<DIR>::sigma * (b - 1))];
     const bool df = nn_less(nn_max(nn_max(al[0], al[1]), al[2]), S.alpha_thres);
-    const double idt = g.idtan;
+    const Real idt = g.idtan;
     const long long e = (long long)side * g.nfaces() + g.face(f, t);
     const int fbits = (int)gp[GP_FB * gs + e];
-    // Gauss-point adjoints -> characteristic value and tangential-slope adjoints (R^T, independent
-    // of the reconstruction); a Gauss point that used the cell average sends its adjoint there
-    double wb[2][4], wtb[2][4], qvb[2][4], slb[2][4];
+    Real dW[4][4], F[4][4];
+    {
+        Real prev[4];
+#pragma unroll
+        for (int b = 0; b < 5; ++b) {
+            const long long lbb = g.line(f, t + Geo<DIR>::sigma * (b - 2));
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                const Real w = Real::raw(lines[(wbase + k) * ls + lbb]);
+                if (b > 0) dW[b - 1][k] = w - prev[k];
+                prev[k] = w;
+            }
+            if (b > 0) project_diff(D, dW[b - 1], F[b - 1]);
+        }
+    }
+    // Gauss-point adjoints -> characteristic value and tangential-slope adjoints (R^T, independent of the
+    // reconstruction); a Gauss point that used the cell average sends its adjoint there.  The face line's normal
+    // slope adjoint has no other contribution, so it is stored.
+    Real wb[2][4], wtb[2][4], qvb[2][4], qtb[2][4], nb[4], centre[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) nb[k] = centre[k] = 0.0;
+#pragma unroll
     for (int mm = 0; mm < 2; ++mm) {
+#pragma unroll
         for (int k = 0; k < 4; ++k) {
-            wb[mm][k] = gb[(mm * 12 + k) * gs + e];
-            wtb[mm][k] = gb[(mm * 12 + 8 + k) * gs + e];
-            qvb[mm][k] = 0.0;
-            slb[mm][k] = 0.0;
+            wb[mm][k] = Real::raw(gb[(mm * 12 + k) * gs + e]);
+            wtb[mm][k] = idt * Real::raw(gb[(mm * 12 + 8 + k) * gs + e]);
         }
         if ((fbits >> mm) & 1) {
-            double wg[4] = {wb[mm][0], wb[mm][1], wb[mm][2], wb[mm][3]};
+            double wg[4] = {wb[mm][0].v, wb[mm][1].v, wb[mm][2].v, wb[mm][3].v};
             to_global<DIR>(wg);
             const long long c = g.cell(m, ncell, t);
-            for (int k = 0; k < 4; ++k) { aadd(&Wb[k * m.plane + c], wg[k]); wb[mm][k] = 0.0; wtb[mm][k] = 0.0; }
-            continue;
+#pragma unroll
+            for (int k = 0; k < 4; ++k) { aadd(&Wb[k * m.plane + c], wg[k]); wb[mm][k] = wtb[mm][k] = 0.0; }
+        } else {
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                nb[k] = nb[k] + Real::raw(gb[(mm * 12 + 4 + k) * gs + e]);
+                centre[k] = centre[k] + wb[mm][k];
+            }
         }
-        double qtb[4] = {0, 0, 0, 0};
-        back_project_T(B, wb[mm], qvb[mm]);
-        back_project_T(B, wtb[mm], qtb);
-        for (int k = 0; k < 4; ++k) {
-            slb[mm][k] = qtb[k] * idt;
-            aadd(&lb[(nbase + k) * ls + l0], gb[(mm * 12 + 4 + k) * gs + e]);   // normal slope copied from the line
-        }
+        back_project_diff_T(D, wb[mm], qvb[mm]);
+        back_project_diff_T(D, wtb[mm], qtb[mm]);
     }
-    // per characteristic component: the reconstruction once, then its reverse
-    double qv[2][4], qt[2][4], Qb[5][4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) lb[(nbase + k) * ls + l0] = nb[k].v;
+    // per characteristic component: the coefficients, the evaluation's and the weights' reverse
+    Real qv[2][4], qt[2][4], Fb[4][4];
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
-        double sq[5] = {Q[0][k], Q[1][k], Q[2][k], Q[3][k], Q[4][k]};
-        double vb[2] = {qvb[0][k], qvb[1][k]}, sb[2] = {slb[0][k], slb[1][k]};
-        double v[2], sl[2], qb[5] = {0, 0, 0, 0, 0};
+        const Real gg = kGaussEta;
+        const Real s0 = F[1][k] - F[0][k], s1 = F[2][k] - F[1][k], s2 = F[3][k] - F[2][k];
+        const Real a11 = fma(0.5, s1, F[1][k]);
+        const Real Ob = gg * (qvb[1][k] - qvb[0][k]), Esb = qtb[0][k] + qtb[1][k], Osb = gg * (qtb[1][k] - qtb[0][k]);
+        Real v[2], sl[2];
+        AODiffBar b;
+        b.fb = b.ff = b.s0 = b.s2 = b.to = b.ti = 0.0;
         if (df) {
-            df_at_gauss(sq, al[1], v, sl);
-            df_at_gauss_vjp(al[1], vb, sb, qb);
-        } else if (TAPED) {
-            const PlaneTape T{ftape + e, gs};
-            AO o = ao_from_tape(T, k * AT_COUNT, S);
-            ao_at_gauss(o, sq[2], v, sl);
-            AOBar ob;
-            ao_bar_zero(ob);
-            ao_at_gauss_vjp(vb, sb, qb[2], ob);
-            weno_ao_rev(T, k * AT_COUNT, S, ob, qb);
+            const Real alpha1 = Real::raw(al[1]);
+            df_diff_at_gauss(a11, s1, alpha1, v, sl);
+            const Real a11b = alpha1 * (Ob + Esb);
+            b.fb = a11b;
+            b.s1 = fma(0.5, a11b, alpha1 * Osb);
         } else {
-            double tb[AT_COUNT];
-            const ArrayTape T{tb};
-            AO o = weno_ao_t(sq, S, T, 0);
-            ao_at_gauss(o, sq[2], v, sl);
-            AOBar ob;
-            ao_bar_zero(ob);
-            ao_at_gauss_vjp(vb, sb, qb[2], ob);
-            weno_ao_rev(T, 0, S, ob, qb);
+            const Real t1 = s1 - s0, t2 = s2 - s1, T = t1 + t2, U = t2 - t1;
+            AORatios q;
+            if constexpr (TAPED) q = tape_get_ratios(PlaneTape{ftape + e, gs}, k * RT_COUNT);
+            else {
+                const Real eps = (k == 0 || k == 3) ? Real(4.0 * S.eps) : Real(S.eps);
+                q = ao_ratios(ao_weights<+1>(F[1][k], F[2][k], s0, s1, s2, second_difference_energy(s0, eps),
+                                             second_difference_energy(s1, eps), second_difference_energy(s2, eps), a11, T, U,
+                                             eps, S));
+            }
+            const AOCoeffs c = ao_coeffs(q);
+            const Real dp = S.d[0] * c.p0, dr = S.d[0] * c.p2, p = dp * t1, r = dr * t2, c3T = c.c3 * T, c3U = c.c3 * U;
+            {   // the values, for the basis (ao_diff_at_gauss)
+                const Real B = fma(-0.5, p + r, a11);
+                const Real O = gg * fma(-7.0 / 72.0, c3T, B), Es = fma(-1.0 / 12.0, c3T, B);
+                const Real Os = gg * fma(-1.0 / 9.0, c3U, s1 - (p - r)), E = (-1.0 / 4320.0) * c3U;
+                v[0] = E - O; v[1] = E + O;
+                sl[0] = Es - Os; sl[1] = Es + Os;
+            }
+            const Real Eb = qvb[0][k] + qvb[1][k], Bb = Ob + Esb;
+            const Real c3Tb = fma(-7.0 / 72.0, Ob, (-1.0 / 12.0) * Esb), c3Ub = fma(-1.0 / 4320.0, Eb, (-1.0 / 9.0) * Osb);
+            const Real pb = fma(-0.5, Bb, -Osb), rb = fma(-0.5, Bb, Osb);
+            b.a11 = Bb;
+            b.s1 = Osb;
+            b.to = dp * pb;
+            b.ti = dr * rb;
+            Real zb[4];
+            ao_coeffs_rev(c, q, fma(c3Tb, T, c3Ub * U), (S.d[0] * t1) * pb, (S.d[0] * t2) * rb, S, zb);
+            ao_ratios_rev<+1>(q, c, zb, F[1][k], F[2][k], s0, s1, s2, a11, T, U, c.c3 * c3Tb, c.c3 * c3Ub, b);
         }
+        // third differences to second, second to first
+        const Real s0b = b.s0 - b.to, s1b = b.s1 + (b.to - b.ti), s2b = b.s2 + b.ti;
+        Fb[0][k] = -s0b;
+        Fb[1][k] = b.fb + (s0b - s1b);
+        Fb[2][k] = b.ff + (s1b - s2b);
+        Fb[3][k] = s2b;
         qv[0][k] = v[0]; qv[1][k] = v[1];
-        qt[0][k] = sl[0] * idt; qt[1][k] = sl[1] * idt;
-        for (int b = 0; b < 5; ++b) Qb[b][k] = qb[b];
+        qt[0][k] = sl[0]; qt[1][k] = sl[1];
     }
-    BasisBar Bb;
-    basis_bar_zero(Bb);
+    DiffBasisBar Bb;
+    zero(Bb);
+#pragma unroll
     for (int mm = 0; mm < 2; ++mm) {          // zero adjoints (fallback) add nothing
-        back_project_basis_vjp(B, qv[mm], wb[mm], Bb);
-        back_project_basis_vjp(B, qt[mm], wtb[mm], Bb);
+        back_project_diff_basis_rev(qv[mm], wb[mm], Bb);
+        back_project_diff_basis_rev(qt[mm], wtb[mm], Bb);
     }
+    Real left[4];                             // adjoint of line b from the difference below it
+#pragma unroll
+    for (int k = 0; k < 4; ++k) left[k] = 0.0;
+#pragma unroll
     for (int b = 0; b < 5; ++b) {
-        double wl[4] = {0, 0, 0, 0};
-        project_vjp(B, Wl[b], Qb[b], wl, Bb);
-        long long lbb = g.line(f, t + Geo<DIR>::sigma * (b - 2));
-        for (int k = 0; k < 4; ++k) aadd(&lb[(wbase + k) * ls + lbb], wl[k]);
+        Real w[4];
+        if (b < 4) project_diff_rev(D, dW[b], Fb[b], w, Bb);
+        const long long lbb = g.line(f, t + Geo<DIR>::sigma * (b - 2));
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            Real x = left[k];
+            if (b < 4) x = b == 0 ? -w[k] : x - w[k];
+            if (b == 2) x = x + centre[k];
+            aadd(&lb[(wbase + k) * ls + lbb], x.v);
+            if (b < 4) left[k] = w[k];
+        }
     }
-    aadd(&lb[LR_U * ls + l0], Bb.u); aadd(&lb[LR_V * ls + l0], Bb.v); aadd(&lb[LR_C * ls + l0], Bb.c);
-    aadd(&lb[LR_IC * ls + l0], Bb.ic); aadd(&lb[LR_H * ls + l0], Bb.H); aadd(&lb[LR_B1 * ls + l0], Bb.b1);
-    aadd(&lb[LR_B2 * ls + l0], Bb.b2); aadd(&lb[LR_Q2 * ls + l0], Bb.q2);
+    const BasisAdj o = diff_basis_rev(D, Bb);
+    aadd(&lb[LR_U * ls + l0], o.u.v); aadd(&lb[LR_V * ls + l0], o.v.v); aadd(&lb[LR_C * ls + l0], o.c.v);
+    aadd(&lb[LR_IC * ls + l0], o.ic.v); aadd(&lb[LR_H * ls + l0], o.H.v); aadd(&lb[LR_B1 * ls + l0], o.b1.v);
+    aadd(&lb[LR_B2 * ls + l0], o.b2.v); aadd(&lb[LR_Q2 * ls + l0], o.q2.v);
 }
 
-// TAPED: the normal reconstructions' intermediates are read from the tape the forward sweep wrote
+// one normal reconstruction's reverse (SGN +1: cell f-1's value at its right edge, -1: cell f's at its left): value
+// and slope adjoints vb, sb (the slope per cell), limiter weight adjoint wb (0 unless this one set it); sets the
+// value minus the cell average and the slope, and adds to b
+template <int SGN>
+DFK_HD void edge_reverse(const AORatios& q, bool df, Real alpha, Real vb, Real sb, double wb, Real fb, Real ff, Real s0, Real s1,
+                         Real s2, Real to, Real ti, const SchemeConsts& S, Real& v, Real& sl, AODiffBar& b) {
+    const Real base = SGN > 0 ? fma(-1.0 / 6.0, s1, 0.5 * ff) : fma(-1.0 / 6.0, s1, -0.5 * ff);
+    const Real a = df ? alpha : Real(1.0), ab = a * vb;
+    b.ff = fma(a, sb, fma(0.5 * SGN, ab, b.ff));
+    b.s1 = fma(-1.0 / 6.0, ab, b.s1);
+    v = a * base;
+    sl = a * ff;
+    const bool lim = (dbits(wb) << 1) != 0;
+    if (df && !lim) return;
+    const AOCoeffs c = ao_coeffs(q);
+    const Real T = to + ti, U = SGN > 0 ? ti - to : to - ti, a11 = fma(0.5 * SGN, s1, fb);
+    Real zb[4];
+    if (!df) {
+        const Real d0 = S.d[0], dp = d0 * c.p0, dr = (1.0 / 6.0) * (d0 * c.p2), h12 = (1.0 / 12.0) * ti;
+        const Real w = fma(1.0 / 30.0, to, (1.0 / 20.0) * ti), p = dp * to;
+        const Real x = fma(c.c3, w, fma(dr, ti, (1.0 / 3.0) * p));
+        v = SGN > 0 ? v - x : v + x;
+        sl = sl - fma(c.c3, h12, p);
+        const Real xb = SGN > 0 ? -vb : vb, yb = fma(1.0 / 3.0, xb, -sb);
+        b.to = fma(dp, yb, fma((1.0 / 30.0) * c.c3, xb, b.to));
+        b.ti = fma(dr, xb, fma(c.c3, fma(1.0 / 20.0, xb, (-1.0 / 12.0) * sb), b.ti));
+        ao_coeffs_rev(c, q, fma(xb, w, -(sb * h12)), (d0 * to) * yb, (d0 * ti) * ((1.0 / 6.0) * xb), S, zb);
+    } else {
+        zb[0] = zb[1] = zb[2] = zb[3] = 0.0;
+    }
+    if (lim) ao_limiter_rev(q, c, Real::raw(wb), zb);
+    b.a11 = 0.0;
+    ao_ratios_rev<SGN>(q, c, zb, fb, ff, s0, s1, s2, a11, T, U, 0.0, 0.0, b);
+}
+
+// TAPED: the normal reconstructions' ratios are read from the tape the forward sweep wrote
 template <int DIR, bool TAPED = false>
 DFK_HD void ka_lines_body(const Mesh& m, const SchemeConsts& S, const double* __restrict__ W,
                           const double* __restrict__ alpha, const double* __restrict__ lines,
@@ -213,91 +307,116 @@ DFK_HD void ka_lines_body(const Mesh& m, const SchemeConsts& S, const double* __
     if (f > g.nn || tt >= g.nt + 4) return;
     const int t = tt - 2;
     const long long li = g.line(f, t);
-    double Wc[6][4], al[6];
-    for (int s = 0; s < 6; ++s) {
-        long long c = g.cell(m, f - 3 + s, t);
-        for (int k = 0; k < 4; ++k) Wc[s][k] = W[k * m.plane + c];
-        to_local<DIR>(Wc[s]);
-        al[s] = alpha[c];
+    const CharBasis B = line_basis(lines, ls, li);
+    const DiffBasis D = diff_basis(B);
+    Real dW[5][4], F[5][4];
+    Real density = 0.0;
+    double al[6];
+    {
+        Real prev[4];
+#pragma unroll
+        for (int s = 0; s < 6; ++s) {
+            const long long c = g.cell(m, f - 3 + s, t);
+            double w[4];
+#pragma unroll
+            for (int k = 0; k < 4; ++k) w[k] = W[k * m.plane + c];
+            to_local<DIR>(w);
+            al[s] = alpha[c];
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                const Real x = Real::raw(w[k]);
+                if (s > 0) dW[s - 1][k] = x - prev[k];
+                prev[k] = x;
+            }
+            if (s == 2 || s == 3) density = fma(0.5, prev[0], density);
+            if (s > 0) project_diff(D, dW[s - 1], F[s - 1]);
+        }
     }
-    CharBasis B = make_basis(Wc[2], Wc[3], S);
-    double Q[6][4];
-    for (int s = 0; s < 6; ++s) project(B, Wc[s], Q[s]);
     const bool dfL = nn_less(nn_max(nn_max(al[1], al[2]), al[3]), S.alpha_thres);
     const bool dfR = nn_less(nn_max(nn_max(al[2], al[3]), al[4]), S.alpha_thres);
-    const double idn = g.idn;
+    const Real idn = g.idn;
     // the reconstruction that set the limiter weight in the forward pass (2k + side) and the
     // weight's adjoint
     const int tlk = S.time_limiter ? (int)lines[LR_TLK * ls + li] : -1;
     const double tlb = S.time_limiter ? lb[LR_TL * ls + li] : 0.0;
-    BasisBar Bb;
-    Bb.u = lb[LR_U * ls + li]; Bb.v = lb[LR_V * ls + li]; Bb.c = lb[LR_C * ls + li]; Bb.ic = lb[LR_IC * ls + li];
-    Bb.H = lb[LR_H * ls + li]; Bb.b1 = lb[LR_B1 * ls + li]; Bb.b2 = lb[LR_B2 * ls + li]; Bb.q2 = lb[LR_Q2 * ls + li];
-    double WLb[4], WLnb[4], WRb[4], WRnb[4];
+    Real WLb[4], WLnb[4], WRb[4], WRnb[4], qLb[4], qLnb[4], qRb[4], qRnb[4];
+#pragma unroll
     for (int k = 0; k < 4; ++k) {
-        WLb[k] = lb[(LR_WL + k) * ls + li]; WLnb[k] = lb[(LR_WLN + k) * ls + li];
-        WRb[k] = lb[(LR_WR + k) * ls + li]; WRnb[k] = lb[(LR_WRN + k) * ls + li];
+        WLb[k] = Real::raw(lb[(LR_WL + k) * ls + li]); WLnb[k] = idn * Real::raw(lb[(LR_WLN + k) * ls + li]);
+        WRb[k] = Real::raw(lb[(LR_WR + k) * ls + li]); WRnb[k] = idn * Real::raw(lb[(LR_WRN + k) * ls + li]);
     }
-    double qLb[4] = {0, 0, 0, 0}, qLnb[4] = {0, 0, 0, 0}, qRb[4] = {0, 0, 0, 0}, qRnb[4] = {0, 0, 0, 0};
-    back_project_T(B, WLb, qLb);
-    back_project_T(B, WLnb, qLnb);
-    back_project_T(B, WRb, qRb);
-    back_project_T(B, WRnb, qRnb);
-    double qL[4], qLn[4], qR[4], qRn[4], Qb[6][4];
-    for (int s = 0; s < 6; ++s) for (int k = 0; k < 4; ++k) Qb[s][k] = 0.0;
+    back_project_diff_T(D, WLb, qLb);
+    back_project_diff_T(D, WLnb, qLnb);
+    back_project_diff_T(D, WRb, qRb);
+    back_project_diff_T(D, WRnb, qRnb);
+    Real qL[4], qLn[4], qR[4], qRn[4], Fb[5][4];
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
-#pragma unroll
-        for (int sd = 0; sd < 2; ++sd) {
-            // side 0: cell f-1, value at xi = +1/2; side 1: cell f, mirrored stencil, slope sign reversed
-            double sq[5];
-            for (int i = 0; i < 5; ++i) sq[i] = sd == 0 ? Q[i][k] : Q[5 - i][k];
-            const bool dfs = sd == 0 ? dfL : dfR;
-            const double as = sd == 0 ? al[2] : al[3];
-            const double sgn = sd == 0 ? 1.0 : -1.0;
-            const double vb = sd == 0 ? qLb[k] : qRb[k];
-            const double sb = sgn * (sd == 0 ? qLnb[k] : qRnb[k]) * idn;
-            const bool lim = tlk == 2 * k + sd && tlb != 0.0;
-            double v = 0.0, sl = 0.0, qb[5] = {0, 0, 0, 0, 0};
-            if (!dfs || lim) {
-                double tb[AT_COUNT];
-                const int base = TAPED ? (2 * k + sd) * AT_COUNT : 0;
-                const PlaneTape PT{ltape + (TAPED ? li : 0), ls};
-                const ArrayTape AT{tb};
-                AO o = TAPED ? ao_from_tape(PT, base, S) : weno_ao_t(sq, S, AT, 0);
-                AOBar ob;
-                ao_bar_zero(ob);
-                if (!dfs) {
-                    ao_at_right_edge(o, sq[2], v, sl);
-                    ao_at_right_edge_vjp(vb, sb, qb[2], ob);
-                }
-                if (lim) limiter_alpha_vjp(o, tlb, ob);
-                if (TAPED) weno_ao_rev(PT, base, S, ob, qb);
-                else weno_ao_rev(AT, 0, S, ob, qb);
-            }
-            if (dfs) {
-                df_at_right_edge(sq, as, v, sl);
-                df_at_right_edge_vjp(as, vb, sb, qb);
-            }
-            if (sd == 0) { qL[k] = v; qLn[k] = sl * idn; }
-            else { qR[k] = v; qRn[k] = -sl * idn; }
-            for (int i = 0; i < 5; ++i) Qb[sd == 0 ? i : 5 - i][k] += qb[i];
+        const Real f3 = F[2][k];
+        const Real s1 = F[1][k] - F[0][k], s2 = f3 - F[1][k], s3 = F[3][k] - f3, s4 = F[4][k] - F[3][k];
+        const Real t1 = s2 - s1, t2 = s3 - s2, t3 = s4 - s3;
+        AORatios L, R;
+        if constexpr (TAPED) {
+            const PlaneTape T{ltape + li, ls};
+            L = tape_get_ratios(T, 2 * k * RT_COUNT);
+            R = tape_get_ratios(T, (2 * k + 1) * RT_COUNT);
+        } else {
+            const Real eps = (k == 0 || k == 3) ? Real(4.0 * S.eps) : Real(S.eps);
+            const Real w1 = second_difference_energy(s1, eps), w2 = second_difference_energy(s2, eps);
+            const Real w3 = second_difference_energy(s3, eps), w4 = second_difference_energy(s4, eps);
+            L = ao_ratios(ao_weights<+1>(F[1][k], f3, s1, s2, s3, w1, w2, w3, fma(0.5, s2, F[1][k]), t1 + t2, t2 - t1, eps, S));
+            R = ao_ratios(ao_weights<-1>(F[3][k], f3, s4, s3, s2, w4, w3, w2, fma(-0.5, s3, F[3][k]), t2 + t3, t3 - t2, eps, S));
         }
+        AODiffBar l, r;                       // adjoints of F1, f3; s1, s2, s3; t1, t2 and of F3, f3; s4, s3, s2; t3, t2
+        l.fb = l.ff = l.s0 = l.s1 = l.s2 = l.to = l.ti = 0.0;
+        r = l;
+        edge_reverse<+1>(L, dfL, Real::raw(al[2]), qLb[k], qLnb[k], tlk == 2 * k ? tlb : 0.0, F[1][k], f3, s1, s2, s3, t1, t2, S,
+                         qL[k], qLn[k], l);
+        edge_reverse<-1>(R, dfR, Real::raw(al[3]), qRb[k], qRnb[k], tlk == 2 * k + 1 ? tlb : 0.0, F[3][k], f3, s4, s3, s2, t3, t2,
+                         S, qR[k], qRn[k], r);
+        const Real tib = l.ti + r.ti;
+        const Real s1b = l.s0 - l.to, s2b = (l.s1 + r.s2) + (l.to - tib), s3b = (l.s2 + r.s1) + (tib - r.to), s4b = r.s0 + r.to;
+        Fb[0][k] = -s1b;
+        Fb[1][k] = l.fb + (s1b - s2b);
+        Fb[2][k] = (l.ff + r.ff) + (s2b - s3b);
+        Fb[3][k] = r.fb + (s3b - s4b);
+        Fb[4][k] = s4b;
     }
-    back_project_basis_vjp(B, qL, WLb, Bb);
-    back_project_basis_vjp(B, qLn, WLnb, Bb);
-    back_project_basis_vjp(B, qR, WRb, Bb);
-    back_project_basis_vjp(B, qRn, WRnb, Bb);
-    double Wcb[6][4];
-    for (int s = 0; s < 6; ++s) {
-        for (int k = 0; k < 4; ++k) Wcb[s][k] = 0.0;
-        project_vjp(B, Wc[s], Qb[s], Wcb[s], Bb);
+    DiffBasisBar Bb;
+    zero(Bb);
+    back_project_diff_basis_rev(qL, WLb, Bb);
+    back_project_diff_basis_rev(qLn, WLnb, Bb);
+    back_project_diff_basis_rev(qR, WRb, Bb);
+    back_project_diff_basis_rev(qRn, WRnb, Bb);
+    Real Wcb[6][4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) Wcb[0][k] = 0.0;
+#pragma unroll
+    for (int s = 0; s < 5; ++s) {
+        Real w[4];
+        project_diff_rev(D, dW[s], Fb[s], w, Bb);
+#pragma unroll
+        for (int k = 0; k < 4; ++k) { Wcb[s][k] = s == 0 ? -w[k] : Wcb[s][k] - w[k]; Wcb[s + 1][k] = w[k]; }
     }
-    make_basis_vjp(Wc[2], Wc[3], S, Bb, Wcb[2], Wcb[3]);
+    BasisAdj o = diff_basis_rev(D, Bb);
+    o.u = o.u + Real::raw(lb[LR_U * ls + li]); o.v = o.v + Real::raw(lb[LR_V * ls + li]);
+    o.c = o.c + Real::raw(lb[LR_C * ls + li]); o.ic = o.ic + Real::raw(lb[LR_IC * ls + li]);
+    o.H = o.H + Real::raw(lb[LR_H * ls + li]); o.b1 = o.b1 + Real::raw(lb[LR_B1 * ls + li]);
+    o.b2 = o.b2 + Real::raw(lb[LR_B2 * ls + li]); o.q2 = o.q2 + Real::raw(lb[LR_Q2 * ls + li]);
+    Real gm[4];
+    make_basis_rev(B, density, o, S, gm);
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        Wcb[2][k] = Wcb[2][k] + (gm[k] + WLb[k]);
+        Wcb[3][k] = Wcb[3][k] + (gm[k] + WRb[k]);
+    }
+#pragma unroll
     for (int s = 0; s < 6; ++s) {
-        to_global<DIR>(Wcb[s]);                                // the rotation is orthogonal
-        long long c = g.cell(m, f - 3 + s, t);
-        for (int k = 0; k < 4; ++k) aadd(&Wb[k * m.plane + c], Wcb[s][k]);
+        double w[4] = {Wcb[s][0].v, Wcb[s][1].v, Wcb[s][2].v, Wcb[s][3].v};
+        to_global<DIR>(w);                                     // the rotation is orthogonal
+        const long long c = g.cell(m, f - 3 + s, t);
+#pragma unroll
+        for (int k = 0; k < 4; ++k) aadd(&Wb[k * m.plane + c], w[k]);
     }
 }
 

@@ -199,107 +199,73 @@ DFK_HD int lines_body(const Mesh& m, const SchemeConsts& S, const double* __rest
         double tn = 1.0, td = 1.0;
         int tlk = -1;                                     // the reconstruction that set it
         double out[16];
-        if constexpr (!TAPE) {
-            const DiffBasis D = diff_basis(B);
-            const Real idn = g.idn;
-            Real F[5][4];                               // first differences of the characteristic variables
+        const DiffBasis D = diff_basis(B);
+        const Real idn = g.idn;
+        Real F[5][4];                               // first differences of the characteristic variables
 #pragma unroll
-            for (int s = 0; s < 5; ++s) {
-                Real dW[4];
+        for (int s = 0; s < 5; ++s) {
+            Real dW[4];
 #pragma unroll
-                for (int k = 0; k < 4; ++k) dW[k] = Real::raw(Wc[s + 1][k]) - Real::raw(Wc[s][k]);
-                project_diff(D, dW, F[s]);
-            }
-            Real qL[4], qLn[4], qR[4], qRn[4];          // face value minus cell value, slope
-            Real xhi = 1.0, xlo = 1.0;                  // limiter: (1 + rmax^2) / (1 + rmin^2), the largest so far
-#pragma unroll
-            for (int k = 0; k < 4; ++k) {
-                const Real s1 = F[1][k] - F[0][k], s2 = F[2][k] - F[1][k], s3 = F[3][k] - F[2][k], s4 = F[4][k] - F[3][k];
-                const Real f3 = F[2][k], hf = 0.5 * f3;
-                // both sides' central quadratics at the face: cell f-1 at xi = +1/2, cell f mirrored
-                const Real baseL = fma(-1.0 / 6.0, s2, hf), baseR = fma(-1.0 / 6.0, s3, -hf);
-                if (!dfL || !dfR || S.time_limiter) {
-                    const Real eps = (k == 0 || k == 3) ? Real(4.0 * S.eps) : Real(S.eps);
-                    const Real t1 = s2 - s1, t2 = s3 - s2, t3 = s4 - s3;
-                    const Real w1 = second_difference_energy(s1, eps), w2 = second_difference_energy(s2, eps);
-                    const Real w3 = second_difference_energy(s3, eps), w4 = second_difference_energy(s4, eps);
-                    const AOWeights L = ao_weights<+1>(F[1][k], f3, s1, s2, s3, w1, w2, w3, fma(0.5, s2, F[1][k]), t1 + t2,
-                                                       t2 - t1, eps, S);
-                    const AOWeights R = ao_weights<-1>(F[3][k], f3, s4, s3, s2, w4, w3, w2, fma(-0.5, s3, F[3][k]), t2 + t3,
-                                                       t3 - t2, eps, S);
-                    if (S.time_limiter) {
-                        if (nn_less(xhi * L.xmin, L.xmax * xlo)) { xhi = L.xmax; xlo = L.xmin; tlk = 2 * k; }
-                        if (nn_less(xhi * R.xmin, R.xmax * xlo)) { xhi = R.xmax; xlo = R.xmin; tlk = 2 * k + 1; }
-                    }
-                    const Real h2 = 0.5 * t2, h12 = (1.0 / 12.0) * t2, h20 = (1.0 / 20.0) * t2, d03 = (1.0 / 3.0) * S.d[0];
-                    if (!dfL) {
-                        const Real iv = ao_inverse_sum(L), p = L.y0 * t1;
-                        const Real v = fma(d03, fma(h2, L.y2, p), L.x3 * fma(1.0 / 30.0, t1, h20));
-                        qL[k] = fma(-iv, v, baseL);
-                        qLn[k] = idn * fma(-iv, fma(S.d[0], p, L.x3 * h12), f3);
-                    }
-                    if (!dfR) {
-                        const Real iv = ao_inverse_sum(R), p = R.y0 * t3;
-                        const Real v = fma(d03, fma(h2, R.y2, p), R.x3 * fma(1.0 / 30.0, t3, h20));
-                        qR[k] = fma(iv, v, baseR);
-                        qRn[k] = idn * fma(-iv, fma(S.d[0], p, R.x3 * h12), f3);
-                    }
-                }
-                if (dfL) { qL[k] = Real::raw(al[2]) * baseL; qLn[k] = idn * (Real::raw(al[2]) * f3); }
-                if (dfR) { qR[k] = Real::raw(al[3]) * baseR; qRn[k] = idn * (Real::raw(al[3]) * f3); }
-            }
-            tn = Real(2.0 * xlo).v;
-            td = (xhi + xlo).v;
-            Real w[16];
-            back_project_diff(D, qL, w + LR_WL);
-            back_project_diff(D, qLn, w + LR_WLN);
-            back_project_diff(D, qR, w + LR_WR);
-            back_project_diff(D, qRn, w + LR_WRN);
-#pragma unroll
-            for (int k = 0; k < 4; ++k) {
-                w[LR_WL + k] = w[LR_WL + k] + Real::raw(Wc[2][k]);
-                w[LR_WR + k] = w[LR_WR + k] + Real::raw(Wc[3][k]);
-            }
-#pragma unroll
-            for (int k = 0; k < 16; ++k) out[k] = w[k].v;
-        } else {
-            const double idn = g.idn;
-            double Q[6][4], qL[4], qLn[4], qR[4], qRn[4];
-#pragma unroll
-            for (int s = 0; s < 6; ++s) project(B, Wc[s], Q[s]);
-#pragma unroll
-            for (int k = 0; k < 4; ++k) {
-                double sL[5] = {Q[0][k], Q[1][k], Q[2][k], Q[3][k], Q[4][k]};
-                double sR[5] = {Q[5][k], Q[4][k], Q[3][k], Q[2][k], Q[1][k]};   // mirrored about cell f
-                double v, sl;
-                if (!dfL || S.time_limiter) {
-                    AO o = weno_ao_t(sL, S, PlaneTape{ltape + li, ls}, 2 * k * AT_COUNT);
-                    if (S.time_limiter) {
-                        double n, d;
-                        limiter_fraction(o, n, d);
-                        if (nn_less(n * td, tn * d)) { tn = n; td = d; tlk = 2 * k; }
-                    }
-                    if (!dfL) ao_at_right_edge(o, sL[2], v, sl);
-                }
-                if (dfL) df_at_right_edge(sL, al[2], v, sl);
-                qL[k] = v; qLn[k] = sl * idn;
-                if (!dfR || S.time_limiter) {
-                    AO o = weno_ao_t(sR, S, PlaneTape{ltape + li, ls}, (2 * k + 1) * AT_COUNT);
-                    if (S.time_limiter) {
-                        double n, d;
-                        limiter_fraction(o, n, d);
-                        if (nn_less(n * td, tn * d)) { tn = n; td = d; tlk = 2 * k + 1; }
-                    }
-                    if (!dfR) ao_at_right_edge(o, sR[2], v, sl);
-                }
-                if (dfR) df_at_right_edge(sR, al[3], v, sl);
-                qR[k] = v; qRn[k] = -sl * idn;
-            }
-            back_project(B, qL, out + LR_WL);
-            back_project(B, qLn, out + LR_WLN);
-            back_project(B, qR, out + LR_WR);
-            back_project(B, qRn, out + LR_WRN);
+            for (int k = 0; k < 4; ++k) dW[k] = Real::raw(Wc[s + 1][k]) - Real::raw(Wc[s][k]);
+            project_diff(D, dW, F[s]);
         }
+        Real qL[4], qLn[4], qR[4], qRn[4];          // face value minus cell value, slope
+        Real xhi = 1.0, xlo = 1.0;                  // limiter: (1 + rmax^2) / (1 + rmin^2), the largest so far
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            const Real s1 = F[1][k] - F[0][k], s2 = F[2][k] - F[1][k], s3 = F[3][k] - F[2][k], s4 = F[4][k] - F[3][k];
+            const Real f3 = F[2][k], hf = 0.5 * f3;
+            // both sides' central quadratics at the face: cell f-1 at xi = +1/2, cell f mirrored
+            const Real baseL = fma(-1.0 / 6.0, s2, hf), baseR = fma(-1.0 / 6.0, s3, -hf);
+            if (!dfL || !dfR || S.time_limiter) {
+                const Real eps = (k == 0 || k == 3) ? Real(4.0 * S.eps) : Real(S.eps);
+                const Real t1 = s2 - s1, t2 = s3 - s2, t3 = s4 - s3;
+                const Real w1 = second_difference_energy(s1, eps), w2 = second_difference_energy(s2, eps);
+                const Real w3 = second_difference_energy(s3, eps), w4 = second_difference_energy(s4, eps);
+                const AOWeights L = ao_weights<+1>(F[1][k], f3, s1, s2, s3, w1, w2, w3, fma(0.5, s2, F[1][k]), t1 + t2,
+                                                   t2 - t1, eps, S);
+                const AOWeights R = ao_weights<-1>(F[3][k], f3, s4, s3, s2, w4, w3, w2, fma(-0.5, s3, F[3][k]), t2 + t3,
+                                                   t3 - t2, eps, S);
+                if constexpr (TAPE) {
+                    const PlaneTape T{ltape + li, ls};
+                    tape_ratios(T, 2 * k * RT_COUNT, ao_ratios(L));
+                    tape_ratios(T, (2 * k + 1) * RT_COUNT, ao_ratios(R));
+                }
+                if (S.time_limiter) {
+                    if (nn_less(xhi * L.xmin, L.xmax * xlo)) { xhi = L.xmax; xlo = L.xmin; tlk = 2 * k; }
+                    if (nn_less(xhi * R.xmin, R.xmax * xlo)) { xhi = R.xmax; xlo = R.xmin; tlk = 2 * k + 1; }
+                }
+                const Real h2 = 0.5 * t2, h12 = (1.0 / 12.0) * t2, h20 = (1.0 / 20.0) * t2, d03 = (1.0 / 3.0) * S.d[0];
+                if (!dfL) {
+                    const Real iv = ao_inverse_sum(L), p = L.y0 * t1;
+                    const Real v = fma(d03, fma(h2, L.y2, p), L.x3 * fma(1.0 / 30.0, t1, h20));
+                    qL[k] = fma(-iv, v, baseL);
+                    qLn[k] = idn * fma(-iv, fma(S.d[0], p, L.x3 * h12), f3);
+                }
+                if (!dfR) {
+                    const Real iv = ao_inverse_sum(R), p = R.y0 * t3;
+                    const Real v = fma(d03, fma(h2, R.y2, p), R.x3 * fma(1.0 / 30.0, t3, h20));
+                    qR[k] = fma(iv, v, baseR);
+                    qRn[k] = idn * fma(-iv, fma(S.d[0], p, R.x3 * h12), f3);
+                }
+            }
+            if (dfL) { qL[k] = Real::raw(al[2]) * baseL; qLn[k] = idn * (Real::raw(al[2]) * f3); }
+            if (dfR) { qR[k] = Real::raw(al[3]) * baseR; qRn[k] = idn * (Real::raw(al[3]) * f3); }
+        }
+        tn = Real(2.0 * xlo).v;
+        td = (xhi + xlo).v;
+        Real w[16];
+        back_project_diff(D, qL, w + LR_WL);
+        back_project_diff(D, qLn, w + LR_WLN);
+        back_project_diff(D, qR, w + LR_WR);
+        back_project_diff(D, qRn, w + LR_WRN);
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            w[LR_WL + k] = w[LR_WL + k] + Real::raw(Wc[2][k]);
+            w[LR_WR + k] = w[LR_WR + k] + Real::raw(Wc[3][k]);
+        }
+#pragma unroll
+        for (int k = 0; k < 16; ++k) out[k] = w[k].v;
 #pragma unroll
         for (int q = 0; q < 16; ++q) lines[q * ls + li] = out[q];
         lines[LR_TL * ls + li] = tn / td;
@@ -353,61 +319,41 @@ DFK_HD int faces_body(const Mesh& m, const SchemeConsts& S, const double* __rest
 #pragma unroll
             for (int k = 0; k < 4; ++k) Wl[b][k] = lines[(wbase + k) * ls + lb];
         }
-        if constexpr (!TAPE) {
-            const DiffBasis D = diff_basis(B);
-            const Real idt = g.idtan;
-            Real F[4][4], qv[2][4], qt[2][4];
+        const DiffBasis D = diff_basis(B);
+        const Real idt = g.idtan;
+        Real F[4][4], qv[2][4], qt[2][4];
 #pragma unroll
-            for (int b = 0; b < 4; ++b) {
-                Real dW[4];
+        for (int b = 0; b < 4; ++b) {
+            Real dW[4];
 #pragma unroll
-                for (int k = 0; k < 4; ++k) dW[k] = Real::raw(Wl[b + 1][k]) - Real::raw(Wl[b][k]);
-                project_diff(D, dW, F[b]);
+            for (int k = 0; k < 4; ++k) dW[k] = Real::raw(Wl[b + 1][k]) - Real::raw(Wl[b][k]);
+            project_diff(D, dW, F[b]);
+        }
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            const Real s0 = F[1][k] - F[0][k], s1 = F[2][k] - F[1][k], s2 = F[3][k] - F[2][k];
+            const Real a11 = fma(0.5, s1, F[1][k]);
+            Real v[2], s[2];
+            if (df) df_diff_at_gauss(a11, s1, Real::raw(al[1]), v, s);
+            else {
+                const Real eps = (k == 0 || k == 3) ? Real(4.0 * S.eps) : Real(S.eps);
+                const Real t1 = s1 - s0, t2 = s2 - s1, T = t1 + t2, U = t2 - t1;
+                const AOWeights o = ao_weights<+1>(F[1][k], F[2][k], s0, s1, s2, second_difference_energy(s0, eps),
+                                                   second_difference_energy(s1, eps), second_difference_energy(s2, eps),
+                                                   a11, T, U, eps, S);
+                if constexpr (TAPE) tape_ratios(PlaneTape{ftape + e, gs}, k * RT_COUNT, ao_ratios(o));
+                ao_diff_at_gauss(o, a11, s1, t1, t2, T, U, S, v, s);
             }
+            qv[0][k] = v[0]; qv[1][k] = v[1];
+            qt[0][k] = s[0] * idt; qt[1][k] = s[1] * idt;
+        }
 #pragma unroll
-            for (int k = 0; k < 4; ++k) {
-                const Real s0 = F[1][k] - F[0][k], s1 = F[2][k] - F[1][k], s2 = F[3][k] - F[2][k];
-                const Real a11 = fma(0.5, s1, F[1][k]);
-                Real v[2], s[2];
-                if (df) df_diff_at_gauss(a11, s1, Real::raw(al[1]), v, s);
-                else {
-                    const Real eps = (k == 0 || k == 3) ? Real(4.0 * S.eps) : Real(S.eps);
-                    const Real t1 = s1 - s0, t2 = s2 - s1, T = t1 + t2, U = t2 - t1;
-                    const AOWeights o = ao_weights<+1>(F[1][k], F[2][k], s0, s1, s2, second_difference_energy(s0, eps),
-                                                       second_difference_energy(s1, eps), second_difference_energy(s2, eps),
-                                                       a11, T, U, eps, S);
-                    ao_diff_at_gauss(o, a11, s1, t1, t2, T, U, S, v, s);
-                }
-                qv[0][k] = v[0]; qv[1][k] = v[1];
-                qt[0][k] = s[0] * idt; qt[1][k] = s[1] * idt;
-            }
+        for (int mm = 0; mm < 2; ++mm) {
+            Real w[4], d[4];
+            back_project_diff(D, qv[mm], w);
+            back_project_diff(D, qt[mm], d);
 #pragma unroll
-            for (int mm = 0; mm < 2; ++mm) {
-                Real w[4], d[4];
-                back_project_diff(D, qv[mm], w);
-                back_project_diff(D, qt[mm], d);
-#pragma unroll
-                for (int k = 0; k < 4; ++k) { Wv[mm][k] = (w[k] + Real::raw(Wl[2][k])).v; Wd[mm][k] = d[k].v; }
-            }
-        } else {
-            const double idt = g.idtan;
-            double Q[5][4], qv[2][4], qt[2][4];
-#pragma unroll
-            for (int b = 0; b < 5; ++b) project(B, Wl[b], Q[b]);
-#pragma unroll
-            for (int k = 0; k < 4; ++k) {
-                double sq[5] = {Q[0][k], Q[1][k], Q[2][k], Q[3][k], Q[4][k]};
-                double v[2], s[2];
-                if (df) df_at_gauss(sq, al[1], v, s);
-                else {
-                    AO o = weno_ao_t(sq, S, PlaneTape{ftape + e, gs}, k * AT_COUNT);
-                    ao_at_gauss(o, sq[2], v, s);
-                }
-                qv[0][k] = v[0]; qv[1][k] = v[1];
-                qt[0][k] = s[0] * idt; qt[1][k] = s[1] * idt;
-            }
-#pragma unroll
-            for (int mm = 0; mm < 2; ++mm) { back_project(B, qv[mm], Wv[mm]); back_project(B, qt[mm], Wd[mm]); }
+            for (int k = 0; k < 4; ++k) { Wv[mm][k] = (w[k] + Real::raw(Wl[2][k])).v; Wd[mm][k] = d[k].v; }
         }
         const int nbase = side == 0 ? LR_WLN : LR_WRN;
         int fbits = 0;

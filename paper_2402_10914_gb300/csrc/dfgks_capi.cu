@@ -41,7 +41,7 @@ struct dfgks {
     double* adj_lines;     // reverse sweep: face-line record adjoints
     double* adj_gp;        // reverse sweep: Gauss-point record adjoints
     double* adj_Wg;        // reverse sweep: ghosted cell adjoints
-    double* adj_tape;      // reverse sweep: the GKS flux's tape of one direction (optional)
+    double* adj_tape;      // reverse sweep: one direction's tapes (optional)
     // checkpointed forward pass kept for dfgks_adjoint_checkpointed
     double* ck_W;          // dense [nseg][4][ny][nx]: W at steps 0, k, 2k, ...
     double* ck_A;          // dense [nseg][ny][nx]: alpha at the same steps
@@ -486,10 +486,12 @@ static dfgks_status ensure_adjoint_buffers(dfgks* h) {
     CK(dalloc(h, &h->adj_lines, (long long)LR_COUNT * h->B.line_stride));
     CK(dalloc(h, &h->adj_gp, (long long)GP_COUNT * h->B.gp_stride));
     CK(dalloc(h, &h->adj_Wg, 4 * h->mesh.plane));
-    // The GKS flux's tape of one direction, for reverse sweeps that evaluate their forward first: its reverse
-    // then does not evaluate the flux a second time.  Left out where it would take more than a quarter of the
+    // One direction's tapes, for reverse sweeps that evaluate their forward first: the reverse then does not
+    // evaluate fluxes and weights a second time.  Left out where they would take more than a quarter of the
     // free memory.
-    const long long n = (long long)TG_COUNT * (h->B.flux_stride[0] > h->B.flux_stride[1] ? h->B.flux_stride[0] : h->B.flux_stride[1]);
+    const long long nflux = (long long)TG_COUNT * (h->B.flux_stride[0] > h->B.flux_stride[1] ? h->B.flux_stride[0] : h->B.flux_stride[1]);
+    const long long nlines = (long long)8 * RT_COUNT * h->B.line_stride, nfaces = (long long)4 * RT_COUNT * h->B.gp_stride;
+    const long long n = nflux + nlines + nfaces;
     size_t free_b = 0, total_b = 0;
     cudaMemGetInfo(&free_b, &total_b);
     if ((double)n * sizeof(double) <= 0.25 * (double)free_b && dalloc(h, &h->adj_tape, n) != cudaSuccess) {
@@ -514,7 +516,11 @@ static dfgks_status adjoint_stage(dfgks* h, const double* W, const double* alpha
     CK(cudaMemsetAsync(h->adj_Wg, 0, sizeof(double) * 4 * h->mesh.plane, h->stream));
     AdjointArgs a = {L_bar, dtL_bar, dtLt_bar};
     SweepBuffers own = h->B;
-    if (flux == DFGKS_FLUX_GKS) own.tape[0] = own.tape[1] = h->adj_tape;
+    if (h->adj_tape) {
+        own.ltape = h->adj_tape;
+        own.ftape = own.ltape + (long long)8 * RT_COUNT * own.line_stride;
+        if (flux == DFGKS_FLUX_GKS) own.tape[0] = own.tape[1] = own.ftape + (long long)4 * RT_COUNT * own.gp_stride;
+    }
     for (int d = 0; d < 2; ++d) {
         // the records of this direction, then its reverse sweep
         if (!rec)
@@ -538,8 +544,8 @@ extern "C" dfgks_status dfgks_adjoint_residual(dfgks* h, const double* W, const 
 // fluxes, and (tape) the reconstructions' intermediates and, for GKS, the flux's intermediates
 static long long record_doubles_per_step(const dfgks* h, bool tape, bool gks) {
     const SweepBuffers& B = h->B;
-    long long per_dir = (long long)(LR_COUNT + (tape ? 8 * AT_COUNT : 0)) * B.line_stride
-                      + (long long)(GP_COUNT + (tape ? 4 * AT_COUNT : 0)) * B.gp_stride;
+    long long per_dir = (long long)(LR_COUNT + (tape ? 8 * RT_COUNT : 0)) * B.line_stride
+                      + (long long)(GP_COUNT + (tape ? 4 * RT_COUNT : 0)) * B.gp_stride;
     long long flux = (long long)(FR_COUNT + (tape && gks ? TG_COUNT : 0)) * (B.flux_stride[0] + B.flux_stride[1]);
     return 2 * (2 * per_dir + flux);
 }
@@ -557,8 +563,8 @@ static void record_sets(const dfgks* h, double* base, bool tape, bool gks, Sweep
         rec[q].tape[0] = rec[q].tape[1] = nullptr;
         rec[q].ltape = rec[q].ftape = nullptr;
         if (tape) {
-            rec[q].ltape = p; p += (long long)8 * AT_COUNT * B.line_stride;
-            rec[q].ftape = p; p += (long long)4 * AT_COUNT * B.gp_stride;
+            rec[q].ltape = p; p += (long long)8 * RT_COUNT * B.line_stride;
+            rec[q].ftape = p; p += (long long)4 * RT_COUNT * B.gp_stride;
             if (gks) { rec[q].tape[d] = p; p += (long long)TG_COUNT * B.flux_stride[d]; }
         }
     }

@@ -350,7 +350,11 @@ DFK_HD Real rcp(Real x) {
 
 // weights of one reconstruction: c_3 = x3 / sum, c_0 = d0 y0 / sum, c_2 = d0 y2 / sum, and the extreme
 // x_k, all carried scaled by (3 prod)^2, prod = the product of the four beta_k + eps (the scale cancels)
-struct AOWeights { Real x3, y0, y2, sum, xmax, xmin; };
+struct AOWeights {
+    Real x3, y0, y2, sum, xmax, xmin;
+    Real e[4], tau3, prod, p2;             // beta_k + eps, 3 tau, the scale: for ao_ratios
+    bool scaled;
+};
 
 // 13/12 s^2 + eps, shared by the reconstructions that use the second difference s
 DFK_HD Real second_difference_energy(Real s, Real eps) { return fma((13.0 / 12.0) * s, s, eps); }
@@ -375,7 +379,8 @@ DFK_HD AOWeights ao_weights(Real fb, Real ff, Real s0, Real s1, Real s2, Real w0
     Real t0 = e1 * g23, t1 = e0 * g23, t2 = e3 * g01, t3 = e2 * g01;
     Real p2;
     const Real tm = nn_max(nn_max(t0, t1), nn_max(t2, t3));
-    if (in_range(prod, 1e-75, 1e75) && nn_less(tm.v, 1e75)) {
+    const bool scaled = in_range(prod, 1e-75, 1e75) && nn_less(tm.v, 1e75);
+    if (scaled) {
         const Real p3 = 3.0 * prod;
         p2 = p3 * p3;
     } else {                                       // extreme data: the ratios themselves
@@ -393,11 +398,49 @@ DFK_HD AOWeights ao_weights(Real fb, Real ff, Real s0, Real s1, Real s2, Real w0
     o.sum = fma(S.d[0], o.y0 + o.y2, fma(S.d[1], y1, o.x3));
     o.xmax = fma(tmax, tmax, p2);                  // the time limiter's; dropped where it is not used
     o.xmin = fma(tmin, tmin, p2);
+    o.e[0] = e0; o.e[1] = e1; o.e[2] = e2; o.e[3] = e3;
+    o.tau3 = tau3; o.prod = prod; o.p2 = p2; o.scaled = scaled;
     return o;
 }
 
 // 1/sum: a positive normal number unless the data overflow
 DFK_HD Real ao_inverse_sum(const AOWeights& o) { return in_range(o.sum, 1e-300, 1e300) ? rcp(o.sum) : Real::raw(1.0 / o.sum.v); }
+
+// What a reconstruction's reverse needs beside its differences: 1/(beta_k + eps), tau and the unscaled 1/sum.
+// Taped (6 planes) where a reverse sweep follows its own forward; the weights cost more than a third of the
+// reverse, what they are made from is cheaper to form again.
+struct AORatios { Real ie[4], tau, iv; };
+enum AORatioField { RT_IE = 0, RT_TAU = 4, RT_IV = 5, RT_COUNT = 6 };
+
+DFK_HD AORatios ao_ratios(const AOWeights& o) {
+    AORatios a;
+    if (o.scaled) {
+        const Real ip = rcp(o.prod), i01 = (o.e[2] * o.e[3]) * ip, i23 = (o.e[0] * o.e[1]) * ip;   // 1/(e0 e1), 1/(e2 e3)
+        a.ie[0] = o.e[1] * i01; a.ie[1] = o.e[0] * i01; a.ie[2] = o.e[3] * i23; a.ie[3] = o.e[2] * i23;
+    } else {
+#pragma unroll
+        for (int k = 0; k < 4; ++k) a.ie[k] = Real::raw(1.0 / o.e[k].v);
+    }
+    a.tau = (1.0 / 3.0) * o.tau3;
+    a.iv = ao_inverse_sum(o) * o.p2;
+    return a;
+}
+template <class Tape>
+DFK_HD void tape_ratios(const Tape& tp, int b, const AORatios& a) {
+#pragma unroll
+    for (int k = 0; k < 4; ++k) tp.put(b + RT_IE + k, a.ie[k].v);
+    tp.put(b + RT_TAU, a.tau.v);
+    tp.put(b + RT_IV, a.iv.v);
+}
+template <class Tape>
+DFK_HD AORatios tape_get_ratios(const Tape& tp, int b) {
+    AORatios a;
+#pragma unroll
+    for (int k = 0; k < 4; ++k) a.ie[k] = Real::raw(tp.get(b + RT_IE + k));
+    a.tau = Real::raw(tp.get(b + RT_TAU));
+    a.iv = Real::raw(tp.get(b + RT_IV));
+    return a;
+}
 
 // values minus q0 and d/deta (unscaled) at the two Gauss points eta = -g (m=1), +g (m=2), g = sqrt(3)/6
 DFK_HD void ao_diff_at_gauss(const AOWeights& o, Real a11, Real s1, Real t1, Real t2, Real T, Real U,

@@ -109,8 +109,8 @@ struct SweepBuffers {
     // optional, per direction: the GKS flux's forward intermediates (TG_COUNT planes of
     // flux_stride[dir]), written by the forward sweep when set and read by the reverse sweep
     double* tape[2] = {nullptr, nullptr};
-    // optional: the WENO-AO intermediates of the face lines' 8 reconstructions (8 x AT_COUNT planes
-    // of line_stride, reconstruction 2k + side) and of the face sides' 4 tangential ones (4 x AT_COUNT
+    // optional: the WENO-AO ratios (AORatios) of the face lines' 8 reconstructions (8 x RT_COUNT planes
+    // of line_stride, reconstruction 2k + side) and of the face sides' 4 tangential ones (4 x RT_COUNT
     // planes of gp_stride), written by the forward sweep when set and read by the reverse sweep
     double* ltape = nullptr;
     double* ftape = nullptr;
