@@ -83,7 +83,6 @@ DFK_HD void ka_flux_body(const Mesh& m, const SchemeConsts& S, const AdjointArgs
         R.Wt[k] = gp[(mm * 12 + 8 + k) * gs + eR];
     }
     GPStateBar Lbar, Rbar;
-    for (int k = 0; k < 4; ++k) { Lbar.W[k] = Lbar.Wn[k] = Lbar.Wt[k] = Rbar.W[k] = Rbar.Wn[k] = Rbar.Wt[k] = 0.0; }
     if (FLUX == 0 && TAPED) gks_flux_reverse(PlaneTape{tape + (long long)mm * nf + fid, fs}, L, R, S, Fb, dFb, Lbar, Rbar);
     else if (FLUX == 0) gks_flux_vjp(L, R, dt, S, Fb, dFb, Lbar, Rbar);
     else lf_flux_vjp(L, R, S, Fb, dFb, Lbar, Rbar);

@@ -164,8 +164,10 @@ DFK_HD void ghost_y_body(const Mesh& m, double* W, double* alpha, int i, int gr)
 }
 
 // one face line (normal reconstruction of both sides); returns the number of DF branches taken
-// TAPE: also write the reconstructions' intermediates for a reverse sweep (ltape, see SweepBuffers)
-template <int DIR, bool TAPE = false>
+// TAPE: also write the reconstructions' ratios for a reverse sweep (ltape, see SweepBuffers)
+// VALUES: the face values alone, for sweeps whose consumers use neither slopes nor the limiter weight: the DF
+// factors (alpha_only) and the L-F flux of the Runge-Kutta stages.  The slope and limiter fields stay unwritten.
+template <int DIR, bool TAPE = false, bool VALUES = false>
 DFK_HD int lines_body(const Mesh& m, const SchemeConsts& S, const double* __restrict__ W,
                                           const double* __restrict__ alpha, double* __restrict__ lines,
                                           long long ls, int ax, int ay, double* __restrict__ ltape = nullptr) {
@@ -198,7 +200,6 @@ DFK_HD int lines_body(const Mesh& m, const SchemeConsts& S, const double* __rest
         // compared by cross-multiplication, one division at the end
         double tn = 1.0, td = 1.0;
         int tlk = -1;                                     // the reconstruction that set it
-        double out[16];
         const DiffBasis D = diff_basis(B);
         const Real idn = g.idn;
         Real F[5][4];                               // first differences of the characteristic variables
@@ -217,7 +218,8 @@ DFK_HD int lines_body(const Mesh& m, const SchemeConsts& S, const double* __rest
             const Real f3 = F[2][k], hf = 0.5 * f3;
             // both sides' central quadratics at the face: cell f-1 at xi = +1/2, cell f mirrored
             const Real baseL = fma(-1.0 / 6.0, s2, hf), baseR = fma(-1.0 / 6.0, s3, -hf);
-            if (!dfL || !dfR || S.time_limiter) {
+            const bool limit = !VALUES && S.time_limiter;
+            if (!dfL || !dfR || limit) {
                 const Real eps = (k == 0 || k == 3) ? Real(4.0 * S.eps) : Real(S.eps);
                 const Real t1 = s2 - s1, t2 = s3 - s2, t3 = s4 - s3;
                 const Real w1 = second_difference_energy(s1, eps), w2 = second_difference_energy(s2, eps);
@@ -231,7 +233,7 @@ DFK_HD int lines_body(const Mesh& m, const SchemeConsts& S, const double* __rest
                     tape_ratios(T, 2 * k * RT_COUNT, ao_ratios(L));
                     tape_ratios(T, (2 * k + 1) * RT_COUNT, ao_ratios(R));
                 }
-                if (S.time_limiter) {
+                if (limit) {
                     if (nn_less(xhi * L.xmin, L.xmax * xlo)) { xhi = L.xmax; xlo = L.xmin; tlk = 2 * k; }
                     if (nn_less(xhi * R.xmin, R.xmax * xlo)) { xhi = R.xmax; xlo = R.xmin; tlk = 2 * k + 1; }
                 }
@@ -256,20 +258,23 @@ DFK_HD int lines_body(const Mesh& m, const SchemeConsts& S, const double* __rest
         td = (xhi + xlo).v;
         Real w[16];
         back_project_diff(D, qL, w + LR_WL);
-        back_project_diff(D, qLn, w + LR_WLN);
         back_project_diff(D, qR, w + LR_WR);
-        back_project_diff(D, qRn, w + LR_WRN);
+        if constexpr (!VALUES) {
+            back_project_diff(D, qLn, w + LR_WLN);
+            back_project_diff(D, qRn, w + LR_WRN);
+        }
 #pragma unroll
         for (int k = 0; k < 4; ++k) {
             w[LR_WL + k] = w[LR_WL + k] + Real::raw(Wc[2][k]);
             w[LR_WR + k] = w[LR_WR + k] + Real::raw(Wc[3][k]);
         }
 #pragma unroll
-        for (int k = 0; k < 16; ++k) out[k] = w[k].v;
-#pragma unroll
-        for (int q = 0; q < 16; ++q) lines[q * ls + li] = out[q];
-        lines[LR_TL * ls + li] = tn / td;
-        lines[LR_TLK * ls + li] = (double)tlk;
+        for (int q = 0; q < 16; ++q)
+            if (!VALUES || (q & 4) == 0) lines[q * ls + li] = w[q].v;       // LR_WLN, LR_WRN have bit 2
+        if constexpr (!VALUES) {
+            lines[LR_TL * ls + li] = tn / td;
+            lines[LR_TLK * ls + li] = (double)tlk;
+        }
         lines[LR_U * ls + li] = B.u;
         lines[LR_V * ls + li] = B.v;
         lines[LR_C * ls + li] = B.c;
@@ -284,8 +289,9 @@ DFK_HD int lines_body(const Mesh& m, const SchemeConsts& S, const double* __rest
 
 // one face side (tangential reconstruction at both Gauss points, fallback); returns the number of
 // DF branches taken and sets nfb to the number of fallbacks
-// TAPE: also write the reconstructions' intermediates for a reverse sweep (ftape, see SweepBuffers)
-template <int DIR, bool TAPE = false>
+// TAPE: also write the reconstructions' ratios for a reverse sweep (ftape, see SweepBuffers)
+// VALUES: the Gauss-point values alone, without the two slopes (see lines_body)
+template <int DIR, bool TAPE = false, bool VALUES = false>
 DFK_HD int faces_body(const Mesh& m, const SchemeConsts& S, const double* __restrict__ W,
                                           const double* __restrict__ alpha, const double* __restrict__ lines,
                                           long long ls, double* __restrict__ gp, long long gs,
@@ -351,9 +357,12 @@ DFK_HD int faces_body(const Mesh& m, const SchemeConsts& S, const double* __rest
         for (int mm = 0; mm < 2; ++mm) {
             Real w[4], d[4];
             back_project_diff(D, qv[mm], w);
-            back_project_diff(D, qt[mm], d);
+            if constexpr (!VALUES) back_project_diff(D, qt[mm], d);
 #pragma unroll
-            for (int k = 0; k < 4; ++k) { Wv[mm][k] = (w[k] + Real::raw(Wl[2][k])).v; Wd[mm][k] = d[k].v; }
+            for (int k = 0; k < 4; ++k) {
+                Wv[mm][k] = (w[k] + Real::raw(Wl[2][k])).v;
+                if constexpr (!VALUES) Wd[mm][k] = d[k].v;
+            }
         }
         const int nbase = side == 0 ? LR_WLN : LR_WRN;
         int fbits = 0;
@@ -361,11 +370,17 @@ DFK_HD int faces_body(const Mesh& m, const SchemeConsts& S, const double* __rest
         for (int mm = 0; mm < 2; ++mm) {
             double Wg[4], Wt[4], Wn[4];
 #pragma unroll
-            for (int k = 0; k < 4; ++k) { Wg[k] = Wv[mm][k]; Wt[k] = Wd[mm][k]; Wn[k] = lines[(nbase + k) * ls + l0]; }
+            for (int k = 0; k < 4; ++k) {
+                Wg[k] = Wv[mm][k];
+                if constexpr (!VALUES) { Wt[k] = Wd[mm][k]; Wn[k] = lines[(nbase + k) * ls + l0]; }
+            }
             if (S.gp_fallback && !physical_state(Wg, S.gm1)) {
                 long long c = g.cell(m, ncell, t);
 #pragma unroll
-                for (int k = 0; k < 4; ++k) { Wg[k] = W[k * m.plane + c]; Wn[k] = 0.0; Wt[k] = 0.0; }
+                for (int k = 0; k < 4; ++k) {
+                    Wg[k] = W[k * m.plane + c];
+                    if constexpr (!VALUES) { Wn[k] = 0.0; Wt[k] = 0.0; }
+                }
                 to_local<DIR>(Wg);
                 ++nfb;
                 fbits |= 1 << mm;
@@ -373,8 +388,10 @@ DFK_HD int faces_body(const Mesh& m, const SchemeConsts& S, const double* __rest
 #pragma unroll
             for (int k = 0; k < 4; ++k) {
                 gp[(mm * 12 + k) * gs + e] = Wg[k];
-                gp[(mm * 12 + 4 + k) * gs + e] = Wn[k];
-                gp[(mm * 12 + 8 + k) * gs + e] = Wt[k];
+                if constexpr (!VALUES) {
+                    gp[(mm * 12 + 4 + k) * gs + e] = Wn[k];
+                    gp[(mm * 12 + 8 + k) * gs + e] = Wt[k];
+                }
             }
         }
         gp[GP_FB * gs + e] = (double)fbits;
@@ -402,19 +419,23 @@ DFK_HD FluxSite flux_site(const Mesh& m, int ax, int ay, int mm) {
 }
 
 // one Gauss point (flux, time derivative, DF factor, omega^t) of direction dir at a site
-template <int FLUX, bool ALPHA_ONLY, bool TAPE = false>
+// VALUES (L-F): the flux and the DF factor alone, from records without slopes
+template <int FLUX, bool ALPHA_ONLY, bool TAPE = false, bool VALUES = false>
 DFK_HD void flux_point(int dir, const SchemeConsts& S, const FluxSite& site, const double* __restrict__ lines,
                        long long ls, const double* __restrict__ gp, long long gs, double* __restrict__ fr,
                        long long fs, double dt, int mm, double* __restrict__ tape = nullptr) {
+    static_assert(!VALUES || FLUX == 1, "the GKS flux uses the slopes");
     GPState L, R;
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
         L.W[k] = gp[(mm * 12 + k) * gs + site.eL];
-        L.Wn[k] = gp[(mm * 12 + 4 + k) * gs + site.eL];
-        L.Wt[k] = gp[(mm * 12 + 8 + k) * gs + site.eL];
         R.W[k] = gp[(mm * 12 + k) * gs + site.eR];
-        R.Wn[k] = gp[(mm * 12 + 4 + k) * gs + site.eR];
-        R.Wt[k] = gp[(mm * 12 + 8 + k) * gs + site.eR];
+        if constexpr (!VALUES && !ALPHA_ONLY) {
+            L.Wn[k] = gp[(mm * 12 + 4 + k) * gs + site.eL];
+            L.Wt[k] = gp[(mm * 12 + 8 + k) * gs + site.eL];
+            R.Wn[k] = gp[(mm * 12 + 4 + k) * gs + site.eR];
+            R.Wt[k] = gp[(mm * 12 + 8 + k) * gs + site.eR];
+        }
     }
     const long long e = site.e;
     // the two sides' states serve the DF factor and the GKS flux.  The Gauss-point reading of Eq. 33 is
@@ -425,13 +446,18 @@ DFK_HD void flux_point(int dir, const SchemeConsts& S, const FluxSite& site, con
     fr[FR_ALPHA * fs + e] = df_alpha_sides(sl, sr, S).v;
     if (S.df_states) fr[FR_ALPHA * fs + e] = lines[LR_DFC * ls + site.li];
     if (ALPHA_ONLY) return;
-    if constexpr (FLUX == 1) lf_flux(L, R, S, F, dF);
+    if constexpr (FLUX == 1) lf_flux_sides<VALUES>(L, R, sl, sr, S, F, dF);
     else if constexpr (TAPE) gks_flux_sides(L, R, sl, sr, dt, S, F, dF, PlaneTape{tape + e, fs});
     else gks_flux_sides(L, R, sl, sr, dt, S, F, dF, NoTape{});
-    if (dir == 1) { to_global<1>(F); to_global<1>(dF); }
+    if (dir == 1) to_global<1>(F);
 #pragma unroll
-    for (int k = 0; k < 4; ++k) { fr[(FR_F + k) * fs + e] = F[k]; fr[(FR_DF + k) * fs + e] = dF[k]; }
-    fr[FR_OMEGA * fs + e] = S.time_limiter ? lines[LR_TL * ls + site.li] : 1.0;
+    for (int k = 0; k < 4; ++k) fr[(FR_F + k) * fs + e] = F[k];
+    if constexpr (!VALUES) {
+        if (dir == 1) to_global<1>(dF);
+#pragma unroll
+        for (int k = 0; k < 4; ++k) fr[(FR_DF + k) * fs + e] = dF[k];
+        fr[FR_OMEGA * fs + e] = S.time_limiter ? lines[LR_TL * ls + site.li] : 1.0;
+    }
 }
 
 // one Gauss point (flux, time derivative, DF factor, omega^t)

@@ -269,7 +269,7 @@ static dfgks_status compute_alpha0(dfgks* h, double* Wg, double* Ag) {
     launch_fill_value(Ag, h->mesh.plane, 1.0, h->stream);
     launch_fill_ghosts(h->mesh, Wg, nullptr, nullptr, h->stream);
     launch_set_scalar(h->dt_scratch, 1.0, h->stream);
-    launch_sweep_xy(h->mesh, h->S, 1, true, Wg, Ag, h->dt_scratch, h->B, h->By, nullptr, nullptr, h->stream);
+    launch_sweep_xy(h->mesh, h->S, 1, SWEEP_ALPHA, Wg, Ag, h->dt_scratch, h->B, h->By, nullptr, nullptr, h->stream);
     UpdateArgs a;
     memset(&a, 0, sizeof(a));
     a.alpha_out = Ag;
@@ -364,26 +364,26 @@ static void enqueue_step(dfgks* h, int s, double dt, int flux, double t_end, int
                 Bu[q].flux[0] = rec[2 * q].flux[0]; Bu[q].flux_stride[0] = rec[2 * q].flux_stride[0];
                 Bu[q].flux[1] = rec[2 * q + 1].flux[1]; Bu[q].flux_stride[1] = rec[2 * q + 1].flux_stride[1];
             }
-        if (rec) launch_sweep_xy(m, S, flux, false, in, ain, dtp, rec[0], rec[1], h->st, halt, st, T);
-        else launch_sweep_xy(m, S, flux, false, in, ain, dtp, h->B, h->By, h->st, halt, st, T);
+        if (rec) launch_sweep_xy(m, S, flux, SWEEP_FULL, in, ain, dtp, rec[0], rec[1], h->st, halt, st, T);
+        else launch_sweep_xy(m, S, flux, SWEEP_FULL, in, ain, dtp, h->B, h->By, h->st, halt, st, T);
         a.Win = in; a.Wout = h->Ws; a.acc = h->acc;
         launch_update(UM_S2O4_1, m, S, a, Bu[0], dtp, h->st, halt, st, T);
         if (Wstar_store) launch_ghosted_to_dense(m, h->Ws, 4, Wstar_store, st);
         launch_fill_ghosts(m, h->Ws, nullptr, halt, st, T);
-        if (rec) launch_sweep_xy(m, S, flux, false, h->Ws, ain, dtp, rec[2], rec[3], h->st, halt, st, T);
-        else launch_sweep_xy(m, S, flux, false, h->Ws, ain, dtp, h->B, h->By, h->st, halt, st, T);
+        if (rec) launch_sweep_xy(m, S, flux, SWEEP_FULL, h->Ws, ain, dtp, rec[2], rec[3], h->st, halt, st, T);
+        else launch_sweep_xy(m, S, flux, SWEEP_FULL, h->Ws, ain, dtp, h->B, h->By, h->st, halt, st, T);
         a.Win = h->Ws; a.Wout = out; a.alpha_out = aout;
         launch_update(UM_S2O4_2, m, S, a, Bu[1], dtp, h->st, halt, st, T);
     } else {
-        launch_sweep_xy(m, S, flux, false, in, ain, dtp, h->B, h->By, h->st, halt, st, T);
+        launch_sweep_xy(m, S, flux, SWEEP_VALUES, in, ain, dtp, h->B, h->By, h->st, halt, st, T);
         a.Win = in; a.Wout = h->Ws;
         launch_update(UM_RK_1, m, S, a, h->B, dtp, h->st, halt, st, T);
         launch_fill_ghosts(m, h->Ws, nullptr, halt, st, T);
-        launch_sweep_xy(m, S, flux, false, h->Ws, ain, dtp, h->B, h->By, h->st, halt, st, T);
+        launch_sweep_xy(m, S, flux, SWEEP_VALUES, h->Ws, ain, dtp, h->B, h->By, h->st, halt, st, T);
         a.Wn = in; a.Win = h->Ws; a.Wout = out;
         launch_update(UM_RK_2, m, S, a, h->B, dtp, h->st, halt, st, T);
         launch_fill_ghosts(m, out, nullptr, halt, st, T);
-        launch_sweep_xy(m, S, flux, false, out, ain, dtp, h->B, h->By, h->st, halt, st, T);
+        launch_sweep_xy(m, S, flux, SWEEP_VALUES, out, ain, dtp, h->B, h->By, h->st, halt, st, T);
         a.Wn = in; a.Win = out; a.Wout = out; a.alpha_out = aout;
         launch_update(UM_RK_3, m, S, a, h->B, dtp, h->st, halt, st, T);
     }
@@ -393,7 +393,7 @@ static void enqueue_step(dfgks* h, int s, double dt, int flux, double t_end, int
         // of alpha^0 on the new state, overwriting the last stage's product.  No counters (no flux
         // comes from it); a halted step skips it.
         launch_fill_ghosts(m, out, ain, halt, st, T);
-        launch_sweep_xy(m, S, DFGKS_FLUX_LF, true, out, ain, dtp, h->B, h->By, nullptr, halt, st, T);
+        launch_sweep_xy(m, S, DFGKS_FLUX_LF, SWEEP_ALPHA, out, ain, dtp, h->B, h->By, nullptr, halt, st, T);
         UpdateArgs aa;
         memset(&aa, 0, sizeof(aa));
         aa.alpha_out = aout;

@@ -325,7 +325,7 @@ extern "C" DFGKS_API dfgks_status dfgks_decomp_set_ic(dfgks_decomp* d, const dou
     for (Block& b : d->blk) launch_fill_value(b.A[0], b.m.plane, 1.0, d->stream);
     DCK(halo(d, 0, 0, false));
     for (Block& b : d->blk) {
-        launch_sweep_xy(b.m, d->S, 1, true, b.W[0], b.A[0], d->one, b.B, b.By, nullptr, nullptr, d->stream);
+        launch_sweep_xy(b.m, d->S, 1, SWEEP_ALPHA, b.W[0], b.A[0], d->one, b.B, b.By, nullptr, nullptr, d->stream);
         UpdateArgs a;
         memset(&a, 0, sizeof(a));
         a.alpha_out = b.A[0];
@@ -350,7 +350,7 @@ static cudaError_t enqueue_decomp_step(dfgks_decomp* d, int s, int in, int flux,
     cudaError_t e = halo(d, 0, in, true);
     if (e != cudaSuccess) return e;
     for (Block& b : d->blk) {
-        launch_sweep_xy(b.m, d->S, flux, false, b.W[in], b.A[in], dtp, b.B, b.By, ds, halt, st);
+        launch_sweep_xy(b.m, d->S, flux, SWEEP_FULL, b.W[in], b.A[in], dtp, b.B, b.By, ds, halt, st);
         UpdateArgs a;
         memset(&a, 0, sizeof(a));
         a.Win = b.W[in]; a.Wout = b.Ws; a.acc = b.acc;
@@ -359,7 +359,7 @@ static cudaError_t enqueue_decomp_step(dfgks_decomp* d, int s, int in, int flux,
     e = halo(d, 1, in, false);
     if (e != cudaSuccess) return e;
     for (Block& b : d->blk) {
-        launch_sweep_xy(b.m, d->S, flux, false, b.Ws, b.A[in], dtp, b.B, b.By, ds, halt, st);
+        launch_sweep_xy(b.m, d->S, flux, SWEEP_FULL, b.Ws, b.A[in], dtp, b.B, b.By, ds, halt, st);
         UpdateArgs a;
         memset(&a, 0, sizeof(a));
         a.Win = b.Ws; a.Wout = b.W[out]; a.acc = b.acc; a.alpha_out = b.A[out];

@@ -1006,56 +1006,50 @@ DFK_HD void gks_flux(const GPState& L, const GPState& R, double dt, const Scheme
 // Lax-Friedrichs flux (Sect. 2.3) and its time derivative with frozen wave speed and
 // W_t = -(A W_n + B W_t) on each side (Cauchy-Kovalevskaya)
 // ------------------------------------------------------------------------------------------
-struct EulerPt { double u, v, p, c, H, q; };
-
-DFK_HD EulerPt euler_pt(const double W[4], const SchemeConsts& S) {
-    EulerPt e;
-    double ir = 1.0 / W[0];
-    e.u = W[1] * ir;
-    e.v = W[2] * ir;
-    e.q = 0.5 * (e.u * e.u + e.v * e.v);
-    e.p = S.gm1 * (W[3] - W[0] * e.q);
-    e.c = sqrt(S.gamma * e.p * ir);
-    e.H = (W[3] + e.p) * ir;
-    return e;
+// W_t from the primitive time derivative; 1/(gamma - 1) = (K + 2)/2
+DFK_HD void lf_time(const FlowState& s, const FlowGrad& t, const SchemeConsts& S, Real T[4]) {
+    T[0] = t.r0;
+    T[1] = fma(s.U, t.r0, t.r1);
+    T[2] = fma(s.V, t.r0, t.r2);
+    T[3] = fma(0.5 * (S.K + 2.0), t.dp, fma(s.hq, t.r0, fma(s.U, t.r1, s.V * t.r2)));
 }
 
-// A X (x-flux Jacobian) and B X (y-flux Jacobian) at a state
-DFK_HD void jac_x(const EulerPt& e, double gm1, const double X[4], double Y[4]) {
-    double dp = gm1 * (X[3] - e.u * X[1] - e.v * X[2] + e.q * X[0]);
-    Y[0] = X[1];
-    Y[1] = 2.0 * e.u * X[1] - e.u * e.u * X[0] + dp;
-    Y[2] = e.v * X[1] + e.u * X[2] - e.u * e.v * X[0];
-    Y[3] = e.u * (X[3] + dp) + e.H * (X[1] - e.u * X[0]);
+// One side's flux (F) and, unless VALUES, W_t (T) and the flux's derivative along it (D), in gradient form as
+// the GKS flux: primitive gradients, the Euler equations' time derivative, back to conserved variables.
+// sl, sr: side_state of L.W and R.W, which the DF factor shares; c = c^2 / c needs no root
+template <bool VALUES>
+DFK_HD Real lf_side(const FlowState& s, const GPState& P, const SchemeConsts& S, Real F[4], Real T[4], Real D[4]) {
+    const Real m = Real::raw(P.W[1]), E = Real::raw(P.W[3]), Ep = E + s.p;
+    F[0] = m;
+    F[1] = fma(m, s.U, s.p);
+    F[2] = m * s.V;
+    F[3] = s.U * Ep;
+    if constexpr (!VALUES) {
+        const FlowGrad t = euler_time_grad(s, point_grad(s, P.Wn, S), point_grad(s, P.Wt, S), S);
+        lf_time(s, t, S, T);
+        D[0] = T[1];
+        D[1] = fma(s.U, T[1] + t.r1, t.dp);
+        D[2] = fma(s.V, T[1], s.U * t.r2);
+        D[3] = fma(Ep * s.ir, t.r1, s.U * (T[3] + t.dp));
+    }
+    return fma(S.gamma * s.th, S.r2g * s.rs, fabs(s.U));
 }
-DFK_HD void jac_y(const EulerPt& e, double gm1, const double X[4], double Y[4]) {
-    double dp = gm1 * (X[3] - e.u * X[1] - e.v * X[2] + e.q * X[0]);
-    Y[0] = X[2];
-    Y[1] = e.v * X[1] + e.u * X[2] - e.u * e.v * X[0];
-    Y[2] = 2.0 * e.v * X[2] - e.v * e.v * X[0] + dp;
-    Y[3] = e.v * (X[3] + dp) + e.H * (X[2] - e.v * X[0]);
-}
-
-DFK_HD void lf_flux(const GPState& L, const GPState& R, const SchemeConsts& S,
-                                        double F[4], double dF[4]) {
-    EulerPt el = euler_pt(L.W, S), er = euler_pt(R.W, S);
-    double FL[4] = {L.W[1], L.W[1] * el.u + el.p, L.W[1] * el.v, el.u * (L.W[3] + el.p)};
-    double FR[4] = {R.W[1], R.W[1] * er.u + er.p, R.W[1] * er.v, er.u * (R.W[3] + er.p)};
-    double s = nn_max(fabs(el.u) + el.c, fabs(er.u) + er.c);
-    double t1[4], t2[4], WtL[4], WtR[4], AL[4], AR[4];
-    jac_x(el, S.gm1, L.Wn, t1); jac_y(el, S.gm1, L.Wt, t2);
-#pragma unroll
-    for (int i = 0; i < 4; ++i) WtL[i] = -(t1[i] + t2[i]);
-    jac_x(er, S.gm1, R.Wn, t1); jac_y(er, S.gm1, R.Wt, t2);
-#pragma unroll
-    for (int i = 0; i < 4; ++i) WtR[i] = -(t1[i] + t2[i]);
-    jac_x(el, S.gm1, WtL, AL);
-    jac_x(er, S.gm1, WtR, AR);
+// VALUES: F alone (the Runge-Kutta stages use no time derivative); the slopes are not read
+template <bool VALUES>
+DFK_HD void lf_flux_sides(const GPState& L, const GPState& R, const FlowState& sl, const FlowState& sr, const SchemeConsts& S,
+                          double F[4], double dF[4]) {
+    Real Fl[4], Tl[4], Dl[4], Fr[4], Tr[4], Dr[4];
+    const Real al = lf_side<VALUES>(sl, L, S, Fl, Tl, Dl), ar = lf_side<VALUES>(sr, R, S, Fr, Tr, Dr);
+    const Real h = 0.5 * nn_max(al, ar);
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
-        F[i] = 0.5 * (FL[i] + FR[i]) - 0.5 * s * (R.W[i] - L.W[i]);
-        dF[i] = 0.5 * (AL[i] + AR[i]) - 0.5 * s * (WtR[i] - WtL[i]);
+        F[i] = fma(0.5, Fl[i] + Fr[i], -h * (Real::raw(R.W[i]) - Real::raw(L.W[i]))).v;
+        if constexpr (!VALUES) dF[i] = fma(0.5, Dl[i] + Dr[i], -h * (Tr[i] - Tl[i])).v;
     }
+}
+
+DFK_HD void lf_flux(const GPState& L, const GPState& R, const SchemeConsts& S, double F[4], double dF[4]) {
+    lf_flux_sides<false>(L, R, side_state(L.W, S), side_state(R.W, S), S, F, dF);
 }
 
 // DF factor of one Gauss point (Sect. 3.2, Eq. 33) from the Maxwellians of its two local-frame

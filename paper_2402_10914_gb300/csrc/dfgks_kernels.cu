@@ -105,7 +105,7 @@ void launch_end_step(DevState* st, double t_end, cudaStream_t s, KernelTimer* T)
 // DIR 1: y-faces in the frame rotated by pi/2: normal = +y, tangential = -x, so the local
 // tangential offset b maps to global column t - b.  Face f lies between normal cells f-1, f.
 // ---------------------------------------------------------------------------------------------
-template <int DIR, bool TAPE = false>
+template <int DIR, bool TAPE = false, bool VALUES = false>
 __global__ void __launch_bounds__(128, 3) k_lines(Mesh m, SchemeConsts S, const double* __restrict__ W,
                                                const double* __restrict__ alpha, double* __restrict__ lines,
                                                long long ls, DevState* st, const int* halt,
@@ -113,11 +113,11 @@ __global__ void __launch_bounds__(128, 3) k_lines(Mesh m, SchemeConsts S, const 
     if (halted(halt)) return;
     int ax, ay;
     sweep_xy(lines_lx<DIR>(m), ax, ay);
-    int ndf = lines_body<DIR, TAPE>(m, S, W, alpha, lines, ls, ax, ay, ltape);
+    int ndf = lines_body<DIR, TAPE, VALUES>(m, S, W, alpha, lines, ls, ax, ay, ltape);
     if (st) warp_count_add(&st->df_normal, ndf);
 }
 
-template <int DIR, bool TAPE = false>
+template <int DIR, bool TAPE = false, bool VALUES = false>
 __global__ void __launch_bounds__(128) k_faces(Mesh m, SchemeConsts S, const double* __restrict__ W,
                                                const double* __restrict__ alpha, const double* __restrict__ lines,
                                                long long ls, double* __restrict__ gp, long long gs,
@@ -125,7 +125,7 @@ __global__ void __launch_bounds__(128) k_faces(Mesh m, SchemeConsts S, const dou
     if (halted(halt)) return;
     int nfb, ax, ay;
     sweep_xy(faces_lx<DIR>(m), ax, ay);
-    int ndf = faces_body<DIR, TAPE>(m, S, W, alpha, lines, ls, gp, gs, ax, ay, blockIdx.y, nfb, ftape);
+    int ndf = faces_body<DIR, TAPE, VALUES>(m, S, W, alpha, lines, ls, gp, gs, ax, ay, blockIdx.y, nfb, ftape);
     if (st) { warp_count_add(&st->df_tangential, ndf); warp_count_add(&st->fallbacks, nfb); }
 }
 
@@ -153,7 +153,7 @@ __device__ __forceinline__ void sweep_at(int b, int lx, int& ax, int& ay) {
     ay = i / lx;
 }
 
-template <bool TAPE>
+template <bool TAPE, bool VALUES = false>
 __global__ void __launch_bounds__(128, 3) k_lines_xy(Mesh m, SchemeConsts S, const double* __restrict__ W,
                                                   const double* __restrict__ alpha, double* __restrict__ lines0,
                                                   double* __restrict__ lines1, long long ls, double* __restrict__ ltape0,
@@ -162,15 +162,15 @@ __global__ void __launch_bounds__(128, 3) k_lines_xy(Mesh m, SchemeConsts S, con
     int ax, ay, ndf;
     if ((int)blockIdx.x < nb0) {
         sweep_at(blockIdx.x, lines_lx<0>(m), ax, ay);
-        ndf = lines_body<0, TAPE>(m, S, W, alpha, lines0, ls, ax, ay, ltape0);
+        ndf = lines_body<0, TAPE, VALUES>(m, S, W, alpha, lines0, ls, ax, ay, ltape0);
     } else {
         sweep_at(blockIdx.x - nb0, lines_lx<1>(m), ax, ay);
-        ndf = lines_body<1, TAPE>(m, S, W, alpha, lines1, ls, ax, ay, ltape1);
+        ndf = lines_body<1, TAPE, VALUES>(m, S, W, alpha, lines1, ls, ax, ay, ltape1);
     }
     if (st) warp_count_add(&st->df_normal, ndf);
 }
 
-template <bool TAPE>
+template <bool TAPE, bool VALUES = false>
 __global__ void __launch_bounds__(128) k_faces_xy(Mesh m, SchemeConsts S, const double* __restrict__ W,
                                                const double* __restrict__ alpha, const double* __restrict__ lines0,
                                                const double* __restrict__ lines1, long long ls, double* __restrict__ gp0,
@@ -180,15 +180,15 @@ __global__ void __launch_bounds__(128) k_faces_xy(Mesh m, SchemeConsts S, const 
     int nfb, ax, ay, ndf;
     if ((int)blockIdx.x < nb0) {
         sweep_at(blockIdx.x, faces_lx<0>(m), ax, ay);
-        ndf = faces_body<0, TAPE>(m, S, W, alpha, lines0, ls, gp0, gs, ax, ay, blockIdx.y, nfb, ftape0);
+        ndf = faces_body<0, TAPE, VALUES>(m, S, W, alpha, lines0, ls, gp0, gs, ax, ay, blockIdx.y, nfb, ftape0);
     } else {
         sweep_at(blockIdx.x - nb0, faces_lx<1>(m), ax, ay);
-        ndf = faces_body<1, TAPE>(m, S, W, alpha, lines1, ls, gp1, gs, ax, ay, blockIdx.y, nfb, ftape1);
+        ndf = faces_body<1, TAPE, VALUES>(m, S, W, alpha, lines1, ls, gp1, gs, ax, ay, blockIdx.y, nfb, ftape1);
     }
     if (st) { warp_count_add(&st->df_tangential, ndf); warp_count_add(&st->fallbacks, nfb); }
 }
 
-template <int FLUX, bool ALPHA_ONLY, bool TAPE = false>
+template <int FLUX, bool ALPHA_ONLY, bool TAPE = false, bool VALUES = false>
 __global__ void __launch_bounds__(128) k_flux_xy(Mesh m, SchemeConsts S, const double* __restrict__ lines0,
                                               const double* __restrict__ lines1, long long ls,
                                               const double* __restrict__ gp0, const double* __restrict__ gp1,
@@ -210,21 +210,26 @@ __global__ void __launch_bounds__(128) k_flux_xy(Mesh m, SchemeConsts S, const d
         dir = 1;
     }
     if (!site.ok) return;
-    flux_point<FLUX, ALPHA_ONLY, TAPE>(dir, S, site, dir == 0 ? lines0 : lines1, ls, dir == 0 ? gp0 : gp1, gs,
+    flux_point<FLUX, ALPHA_ONLY, TAPE, VALUES>(dir, S, site, dir == 0 ? lines0 : lines1, ls, dir == 0 ? gp0 : gp1, gs,
                                        dir == 0 ? fr0 : fr1, dir == 0 ? fs0 : fs1, dt, blockIdx.y,
                                        dir == 0 ? tape0 : tape1);
 }
 
-void launch_sweep_xy(const Mesh& m, const SchemeConsts& S, int flux, bool alpha_only, const double* W,
+void launch_sweep_xy(const Mesh& m, const SchemeConsts& S, int flux, SweepWhat what, const double* W,
                      const double* alpha, const double* dtp, const SweepBuffers& Bx, const SweepBuffers& By,
                      DevState* st, const int* halt, cudaStream_t s, KernelTimer* T) {
     const dim3 blk(kSweepThreads);
     const int nl0 = (int)sweep_blocks(lines_lx<0>(m), lines_ly<0>(m)), nl1 = (int)sweep_blocks(lines_lx<1>(m), lines_ly<1>(m));
     const int nf0 = (int)sweep_blocks(faces_lx<0>(m), faces_ly<0>(m)), nf1 = (int)sweep_blocks(faces_lx<1>(m), faces_ly<1>(m));
     const bool tape = Bx.ltape != nullptr;      // both directions' record sets carry tapes or neither
+    // without slopes and limiter weight where nothing reads them
+    const bool alpha_only = what == SWEEP_ALPHA, values = alpha_only || (what == SWEEP_VALUES && flux != 0);
     const long long ls = Bx.line_stride, gs = Bx.gp_stride;
     if (T) T->begin(KK_LINES);
-    if (tape)
+    if (values)
+        k_lines_xy<false, true><<<dim3(nl0 + nl1), blk, 0, s>>>(m, S, W, alpha, Bx.lines, By.lines, ls, nullptr, nullptr, nl0,
+                                                                st, halt);
+    else if (tape)
         k_lines_xy<true><<<dim3(nl0 + nl1), blk, 0, s>>>(m, S, W, alpha, Bx.lines, By.lines, ls, Bx.ltape, By.ltape, nl0,
                                                          st, halt);
     else
@@ -233,7 +238,10 @@ void launch_sweep_xy(const Mesh& m, const SchemeConsts& S, int flux, bool alpha_
     if (T) T->end(KK_LINES, 1);
     const dim3 gf(nf0 + nf1, 2);
     if (T) T->begin(KK_FACES);
-    if (tape)
+    if (values)
+        k_faces_xy<false, true><<<gf, blk, 0, s>>>(m, S, W, alpha, Bx.lines, By.lines, ls, Bx.gp, By.gp, gs, nullptr,
+                                                   nullptr, nf0, st, halt);
+    else if (tape)
         k_faces_xy<true><<<gf, blk, 0, s>>>(m, S, W, alpha, Bx.lines, By.lines, ls, Bx.gp, By.gp, gs, Bx.ftape,
                                             By.ftape, nf0, st, halt);
     else
@@ -247,6 +255,9 @@ void launch_sweep_xy(const Mesh& m, const SchemeConsts& S, int flux, bool alpha_
     if (alpha_only)
         k_flux_xy<1, true><<<gf, blk, 0, s>>>(m, S, Bx.lines, By.lines, ls, Bx.gp, By.gp, gs, f0, fs0, f1, fs1,
                                                nullptr, nullptr, dtp, nf0, halt);
+    else if (values)
+        k_flux_xy<1, false, false, true><<<gf, blk, 0, s>>>(m, S, Bx.lines, By.lines, ls, Bx.gp, By.gp, gs, f0, fs0, f1, fs1,
+                                                            nullptr, nullptr, dtp, nf0, halt);
     else if (flux == 0 && Bx.tape[0])        // GKS forward that also tapes its intermediates for a reverse sweep
         k_flux_xy<0, false, true><<<gf, blk, 0, s>>>(m, S, Bx.lines, By.lines, ls, Bx.gp, By.gp, gs, f0, fs0, f1, fs1,
                                                      Bx.tape[0], By.tape[1], dtp, nf0, halt);
@@ -268,12 +279,15 @@ static void sweep_dir(const Mesh& m, const SchemeConsts& S, int flux, bool alpha
     const dim3 blk(kSweepThreads);
     const dim3 gl(sweep_blocks(lines_lx<DIR>(m), lines_ly<DIR>(m)));
     if (T) T->begin(KK_LINES);
-    if (B.ltape) k_lines<DIR, true><<<gl, blk, 0, s>>>(m, S, W, alpha, B.lines, B.line_stride, st, halt, B.ltape);
+    if (alpha_only) k_lines<DIR, false, true><<<gl, blk, 0, s>>>(m, S, W, alpha, B.lines, B.line_stride, st, halt);
+    else if (B.ltape) k_lines<DIR, true><<<gl, blk, 0, s>>>(m, S, W, alpha, B.lines, B.line_stride, st, halt, B.ltape);
     else k_lines<DIR><<<gl, blk, 0, s>>>(m, S, W, alpha, B.lines, B.line_stride, st, halt);
     if (T) T->end(KK_LINES, 1);
     const dim3 gf(sweep_blocks(faces_lx<DIR>(m), faces_ly<DIR>(m)), 2);
     if (T) T->begin(KK_FACES);
-    if (B.ftape)
+    if (alpha_only)
+        k_faces<DIR, false, true><<<gf, blk, 0, s>>>(m, S, W, alpha, B.lines, B.line_stride, B.gp, B.gp_stride, st, halt);
+    else if (B.ftape)
         k_faces<DIR, true><<<gf, blk, 0, s>>>(m, S, W, alpha, B.lines, B.line_stride, B.gp, B.gp_stride, st, halt, B.ftape);
     else
         k_faces<DIR><<<gf, blk, 0, s>>>(m, S, W, alpha, B.lines, B.line_stride, B.gp, B.gp_stride, st, halt);
