@@ -23,11 +23,54 @@
 #include <vector>
 
 #include "../../include/dfgks.h"
-#include "dfgks_internal.h"
+#include "dfgks_bodies.cuh"
 
 using namespace dfk;
 
 namespace {
+
+// A block as the ghost-fill kernel sees it: its fields and, per side shared with another block, that block and
+// the first cells of the two windows (halo_window)
+struct HaloBlock {
+    Mesh m;
+    double* W[3];         // W[0], W[1], Ws
+    double* A[2];
+    int neighbour[4], di[4], dj[4], si[4], sj[4];
+};
+
+// One pass of the ghost fill of all blocks (grid x: block): 0 the ghost columns of the interior rows, 1 the ghost
+// rows of all columns.  A pass reads no cell that it writes, so physical sides and copies go together.  One launch
+// instead of a launch and up to ten strided copies per block, each of which took longer than this kernel:
+// 3 x 2 periodic blocks of 100 x 100, see Helpers below.
+__global__ void k_halo(const HaloBlock* __restrict__ H, int pass, int field, int alpha, const int* halt) {
+    if (*(volatile const int*)halt != 0) return;
+    const HaloBlock& b = H[blockIdx.x];
+    const int idx = blockIdx.y * blockDim.x + threadIdx.x;
+    const Mesh& m = b.m;
+    double* W = b.W[field];
+    double* A = alpha >= 0 ? b.A[alpha] : nullptr;
+    int i, j, g;                                          // cell and ghost layer
+    if (pass == 0) {
+        g = idx % (2 * G); j = idx / (2 * G);
+        if (j >= m.ny) return;
+        i = g < G ? g - G : m.nx + g - G;
+    } else {
+        i = idx % (m.nx + 2 * G) - G; g = idx / (m.nx + 2 * G);
+        if (g >= 2 * G) return;
+        j = g < G ? g - G : m.ny + g - G;
+    }
+    const int side = 2 * pass + (g < G ? 0 : 1), nb = b.neighbour[side];
+    if (nb < 0) {
+        if (pass == 0) ghost_x_body(m, W, A, g, j);
+        else ghost_y_body(m, W, A, i, g);
+        return;
+    }
+    const HaloBlock& a = H[nb];
+    const long long d = gid(m, i, j), o = gid(a.m, b.si[side] + (i - b.di[side]), b.sj[side] + (j - b.dj[side]));
+#pragma unroll
+    for (int k = 0; k < 4; ++k) W[k * m.plane + d] = a.W[field][k * a.m.plane + o];
+    if (A) A[d] = a.A[alpha][o];
+}
 
 struct Block {
     dfgks_block_plan plan;
@@ -100,6 +143,14 @@ struct dfgks_decomp {
     double* stage;           // dense [4][ny][nx] of the whole mesh: transfers
     int cur;
     std::vector<void*> allocs;
+    HaloBlock* halo;         // device
+    int halo_tiles[2];       // 128-thread tiles of the largest block's ghost cells per pass
+    // Helpers: the blocks' kernels between two ghost fills are independent and a block alone leaves part of the
+    // chip idle, so block b runs on stream b mod their number.  With the fused ghost fill, 4 steps of 3 x 2 blocks
+    // of 100 x 100 11.8 -> 5.6 ms.
+    std::vector<cudaStream_t> streams;
+    std::vector<cudaEvent_t> done;
+    cudaEvent_t ready;
 };
 
 static dfgks_status dstat(cudaError_t e) {
@@ -118,20 +169,10 @@ static void free_decomp(dfgks_decomp* d) {
     for (void* p : d->allocs) cudaFree(p);
     if (d->st_host) cudaFreeHost(d->st_host);
     if (d->flag_host) cudaFreeHost(d->flag_host);
+    for (cudaEvent_t e : d->done) cudaEventDestroy(e);
+    if (d->ready) cudaEventDestroy(d->ready);
+    for (cudaStream_t s : d->streams) cudaStreamDestroy(s);
     if (d->own_stream && d->stream) cudaStreamDestroy(d->stream);
-}
-
-// copy a width x height window (doubles x rows) of ncomp planes between two ghosted fields
-static cudaError_t copy_window(const Block& dst, double* dfield, int di, int dj, const Block& src,
-                               const double* sfield, int si, int sj, int width, int height, int ncomp,
-                               cudaStream_t s) {
-    for (int k = 0; k < ncomp; ++k) {
-        cudaError_t e = cudaMemcpy2DAsync(dfield + k * dst.m.plane + gid(dst.m, di, dj), (size_t)dst.m.P * sizeof(double),
-                                          sfield + k * src.m.plane + gid(src.m, si, sj), (size_t)src.m.P * sizeof(double),
-                                          (size_t)width * sizeof(double), (size_t)height, cudaMemcpyDeviceToDevice, s);
-        if (e != cudaSuccess) return e;
-    }
-    return cudaSuccess;
 }
 
 // The halo copy of side `side` of block b from its neighbour a: the window of b's ghosted field
@@ -152,25 +193,58 @@ static void halo_window(const dfgks_block_plan& b, const dfgks_block_plan& a, in
 
 // ghost layers of every block: field 0 = W[in] (with alpha[in] when with_alpha), 1 = Ws
 static cudaError_t halo(dfgks_decomp* d, int field, int in, bool with_alpha) {
-    const int* halt = &d->st->halt;
-    auto Wof = [&](Block& b) { return field == 0 ? b.W[in] : b.Ws; };
-    for (int pass = 0; pass < 2; ++pass) {
-        for (Block& b : d->blk) launch_ghost_pass(pass, b.m, Wof(b), with_alpha ? b.A[in] : nullptr, halt, d->stream);
-        for (Block& b : d->blk) {
-            for (int side = 2 * pass; side < 2 * pass + 2; ++side) {
-                const int nb = b.plan.neighbour[side];
-                if (nb < 0) continue;
-                Block& a = d->blk[nb];
-                dfgks_halo_window hw;
-                halo_window(b.plan, a.plan, side, &hw);
-                cudaError_t e = copy_window(b, Wof(b), hw.di, hw.dj, a, Wof(a), hw.si, hw.sj, hw.w, hw.h, 4, d->stream);
-                if (e == cudaSuccess && with_alpha)
-                    e = copy_window(b, b.A[in], hw.di, hw.dj, a, a.A[in], hw.si, hw.sj, hw.w, hw.h, 1, d->stream);
-                if (e != cudaSuccess) return e;
-            }
-        }
+    for (int pass = 0; pass < 2; ++pass)
+        k_halo<<<dim3((unsigned)d->blk.size(), d->halo_tiles[pass]), 128, 0, d->stream>>>(
+            d->halo, pass, field == 0 ? in : 2, with_alpha ? in : -1, &d->st->halt);
+    return cudaGetLastError();
+}
+
+// the blocks' streams after the handle's stream, and the handle's stream after theirs
+static cudaError_t fork(dfgks_decomp* d) {
+    cudaError_t e = d->streams.empty() ? cudaSuccess : cudaEventRecord(d->ready, d->stream);
+    for (size_t q = 0; q < d->streams.size() && e == cudaSuccess; ++q) e = cudaStreamWaitEvent(d->streams[q], d->ready, 0);
+    return e;
+}
+static cudaError_t join(dfgks_decomp* d) {
+    cudaError_t e = cudaSuccess;
+    for (size_t q = 0; q < d->streams.size() && e == cudaSuccess; ++q) {
+        e = cudaEventRecord(d->done[q], d->streams[q]);
+        if (e == cudaSuccess) e = cudaStreamWaitEvent(d->stream, d->done[q], 0);
     }
-    return cudaSuccess;
+    return e;
+}
+static cudaStream_t stream_of(const dfgks_decomp* d, size_t b) { return d->streams.empty() ? d->stream : d->streams[b % d->streams.size()]; }
+
+static cudaError_t create_halo(dfgks_decomp* d) {
+    std::vector<HaloBlock> H(d->blk.size());
+    int rows = 0, cols = 0;
+    for (size_t b = 0; b < H.size(); ++b) {
+        const Block& k = d->blk[b];
+        HaloBlock& h = H[b];
+        h.m = k.m;
+        h.W[0] = k.W[0]; h.W[1] = k.W[1]; h.W[2] = k.Ws; h.A[0] = k.A[0]; h.A[1] = k.A[1];
+        for (int s = 0; s < 4; ++s) {
+            dfgks_halo_window w = {};
+            h.neighbour[s] = k.plan.neighbour[s];
+            if (h.neighbour[s] >= 0) halo_window(k.plan, d->blk[h.neighbour[s]].plan, s, &w);
+            h.di[s] = w.di; h.dj[s] = w.dj; h.si[s] = w.si; h.sj[s] = w.sj;
+        }
+        if (k.m.ny > rows) rows = k.m.ny;
+        if (k.m.nx + 2 * G > cols) cols = k.m.nx + 2 * G;
+    }
+    d->halo_tiles[0] = (2 * G * rows + 127) / 128;
+    d->halo_tiles[1] = (2 * G * cols + 127) / 128;
+    cudaError_t e = dalloc(d, &d->halo, (long long)H.size());
+    if (e == cudaSuccess) e = cudaMemcpy(d->halo, H.data(), H.size() * sizeof(HaloBlock), cudaMemcpyHostToDevice);
+    const size_t n = H.size() < 2 ? 0 : (H.size() < 8 ? H.size() : 8);
+    if (e == cudaSuccess && n) e = cudaEventCreateWithFlags(&d->ready, cudaEventDisableTiming);
+    for (size_t q = 0; q < n && e == cudaSuccess; ++q) {
+        cudaStream_t st;
+        cudaEvent_t ev;
+        if ((e = cudaStreamCreateWithFlags(&st, cudaStreamNonBlocking)) == cudaSuccess) d->streams.push_back(st);
+        if (e == cudaSuccess && (e = cudaEventCreateWithFlags(&ev, cudaEventDisableTiming)) == cudaSuccess) d->done.push_back(ev);
+    }
+    return e;
 }
 
 static dfgks_status reset_state(dfgks_decomp* d, double t, long long step) {
@@ -282,6 +356,7 @@ extern "C" DFGKS_API dfgks_status dfgks_decomp_create(const dfgks_config* cfg, i
     if (e == cudaSuccess) e = dalloc(d, &d->stage, 4LL * cfg->nx * cfg->ny);
     if (e == cudaSuccess) e = cudaMallocHost((void**)&d->st_host, sizeof(DevState));
     if (e == cudaSuccess) e = cudaMallocHost((void**)&d->flag_host, sizeof(int));
+    if (e == cudaSuccess) e = create_halo(d);
     if (e == cudaSuccess) launch_set_scalar(d->one, 1.0, d->stream);
     dfgks_status r = dstat(e);
     if (r == DFGKS_OK) r = reset_state(d, 0.0, 0);
@@ -324,13 +399,16 @@ extern "C" DFGKS_API dfgks_status dfgks_decomp_set_ic(dfgks_decomp* d, const dou
     if (r != DFGKS_OK) return r;
     for (Block& b : d->blk) launch_fill_value(b.A[0], b.m.plane, 1.0, d->stream);
     DCK(halo(d, 0, 0, false));
-    for (Block& b : d->blk) {
-        launch_sweep_xy(b.m, d->S, 1, SWEEP_ALPHA, b.W[0], b.A[0], d->one, b.B, b.By, nullptr, nullptr, d->stream);
+    DCK(fork(d));
+    for (size_t q = 0; q < d->blk.size(); ++q) {
+        Block& b = d->blk[q];
+        launch_sweep_xy(b.m, d->S, 1, SWEEP_ALPHA, b.W[0], b.A[0], d->one, b.B, b.By, nullptr, nullptr, stream_of(d, q));
         UpdateArgs a;
         memset(&a, 0, sizeof(a));
         a.alpha_out = b.A[0];
-        launch_update(UM_ALPHA, b.m, d->S, a, b.B, d->one, nullptr, nullptr, d->stream);
+        launch_update(UM_ALPHA, b.m, d->S, a, b.B, d->one, nullptr, nullptr, stream_of(d, q));
     }
+    DCK(join(d));
     DCK(cudaGetLastError());
     DCK(cudaStreamSynchronize(d->stream));
     return DFGKS_OK;
@@ -338,32 +416,40 @@ extern "C" DFGKS_API dfgks_status dfgks_decomp_set_ic(dfgks_decomp* d, const dou
 
 // one S2O4 step (Eq. 24 with the time limiter) of all blocks from buffer `in` to `in ^ 1`; every
 // kernel returns at once once the shared halt flag is set, so a queue of steps drains without
-// work and the state stays at the last good step (the halo copies then touch ghost cells only)
+// work and the state stays at the last good step
 static cudaError_t enqueue_decomp_step(dfgks_decomp* d, int s, int in, int flux, double t_end) {
     cudaStream_t st = d->stream;
     DevState* ds = d->st;
     const int* halt = &ds->halt;
     const double* dtp = &ds->dt;
     const int out = in ^ 1;
-    for (Block& b : d->blk) launch_cfl_min(b.m, b.W[in], d->S.gamma, ds, st);     // minimum over all blocks
+    cudaError_t e = fork(d);
+    if (e != cudaSuccess) return e;
+    for (size_t q = 0; q < d->blk.size(); ++q)                                    // minimum over all blocks
+        launch_cfl_min(d->blk[q].m, d->blk[q].W[in], d->S.gamma, ds, stream_of(d, q));
+    if ((e = join(d)) != cudaSuccess) return e;
     launch_begin_step(ds, d->cfg.cfl, 0.0, t_end, d->dts, s, st);
-    cudaError_t e = halo(d, 0, in, true);
-    if (e != cudaSuccess) return e;
-    for (Block& b : d->blk) {
-        launch_sweep_xy(b.m, d->S, flux, SWEEP_FULL, b.W[in], b.A[in], dtp, b.B, b.By, ds, halt, st);
-        UpdateArgs a;
-        memset(&a, 0, sizeof(a));
-        a.Win = b.W[in]; a.Wout = b.Ws; a.acc = b.acc;
-        launch_update(UM_S2O4_1, b.m, d->S, a, b.B, dtp, ds, halt, st);
-    }
-    e = halo(d, 1, in, false);
-    if (e != cudaSuccess) return e;
-    for (Block& b : d->blk) {
-        launch_sweep_xy(b.m, d->S, flux, SWEEP_FULL, b.Ws, b.A[in], dtp, b.B, b.By, ds, halt, st);
-        UpdateArgs a;
-        memset(&a, 0, sizeof(a));
-        a.Win = b.Ws; a.Wout = b.W[out]; a.acc = b.acc; a.alpha_out = b.A[out];
-        launch_update(UM_S2O4_2, b.m, d->S, a, b.B, dtp, ds, halt, st);
+    for (int stage = 0; stage < 2; ++stage) {
+        e = halo(d, stage, in, stage == 0);
+        if (e == cudaSuccess) e = fork(d);
+        if (e != cudaSuccess) return e;
+        for (size_t q = 0; q < d->blk.size(); ++q) {
+            Block& b = d->blk[q];
+            launch_sweep_xy(b.m, d->S, flux, SWEEP_FULL, stage == 0 ? b.W[in] : b.Ws, b.A[in], dtp, b.B, b.By, ds, halt,
+                            stream_of(d, q));
+        }
+        // an update that loses positivity halts all that start later: none starts before every sweep has ended
+        if ((e = join(d)) != cudaSuccess || (e = fork(d)) != cudaSuccess) return e;
+        for (size_t q = 0; q < d->blk.size(); ++q) {
+            Block& b = d->blk[q];
+            UpdateArgs a;
+            memset(&a, 0, sizeof(a));
+            a.acc = b.acc;
+            if (stage == 0) { a.Win = b.W[in]; a.Wout = b.Ws; }
+            else { a.Win = b.Ws; a.Wout = b.W[out]; a.alpha_out = b.A[out]; }
+            launch_update(stage == 0 ? UM_S2O4_1 : UM_S2O4_2, b.m, d->S, a, b.B, dtp, ds, halt, stream_of(d, q));
+        }
+        if ((e = join(d)) != cudaSuccess) return e;
     }
     launch_end_step(ds, t_end, st);
     return cudaGetLastError();
