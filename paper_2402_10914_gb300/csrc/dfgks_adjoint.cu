@@ -1,7 +1,7 @@
 // dfgks_adjoint.cu -- reverse (vector-Jacobian product) of the single-stage operator.
 //
-// With the forward records of one direction in place (face lines, Gauss-point states, fluxes),
-// three kernels walk that direction's sweep backwards:
+// With the forward records in place (face lines, Gauss-point states, fluxes), three kernels walk the
+// sweeps backwards, both directions in one launch each where there is memory for both's adjoints:
 //   ka_flux  : one thread per Gauss point.  Face adjoints from the cells' L, dL/dt and limited
 //              dL/dt adjoints (Eq. 2 with A_m = 1/2), then the GKS / L-F flux adjoint into the
 //              Gauss-point record adjoints, and the time-limiter weight's adjoint.  When the
@@ -419,34 +419,51 @@ DFK_HD void ka_lines_body(const Mesh& m, const SchemeConsts& S, const double* __
     }
 }
 
-// Reverse of the ghost fill: the y pass (all columns) first, then the x pass (interior rows).
-DFK_HD void ka_fold_y_body(const Mesh& m, double* Wb, int i) {
-    if (i >= m.nx + G) return;
-    for (int gr = 2 * G - 1; gr >= 0; --gr) {
-        int j = gr < G ? gr - G : m.ny + gr - G;
-        bool mir;
-        int s = ghost_src(j, m.ny, m.bc[2], m.bc[3], mir);
-        long long d = gid(m, i, j), o = gid(m, i, s);
-        for (int k = 0; k < 4; ++k) {
-            double v = Wb[k * m.plane + d];
-            Wb[k * m.plane + d] = 0.0;
-            Wb[k * m.plane + o] += (mir && k == 2) ? -v : v;
-        }
+// Reverse of the ghost fill: the y pass (all columns) first, then the x pass (interior rows).  Components
+// [k0, k1): the kernels take one each, with the six ghost values loaded before they are added, as one thread's
+// chain of dependent loads and stores is all the time there is (20 us a pass for four components in turn).
+DFK_HD void fold_add(double* W, const long long d[2 * G], const long long o[2 * G], const bool neg[2 * G]) {
+    double v[2 * G];
+#pragma unroll
+    for (int q = 0; q < 2 * G; ++q) v[q] = W[d[q]];
+#pragma unroll
+    for (int q = 2 * G - 1; q >= 0; --q) {
+        W[d[q]] = 0.0;
+        W[o[q]] += neg[q] ? -v[q] : v[q];
     }
 }
 
-DFK_HD void ka_fold_x_body(const Mesh& m, double* Wb, int j) {
-    if (j >= m.ny) return;
-    for (int gc = 2 * G - 1; gc >= 0; --gc) {
-        int i = gc < G ? gc - G : m.nx + gc - G;
-        bool mir;
-        int s = ghost_src(i, m.nx, m.bc[0], m.bc[1], mir);
-        long long d = gid(m, i, j), o = gid(m, s, j);
-        for (int k = 0; k < 4; ++k) {
-            double v = Wb[k * m.plane + d];
-            Wb[k * m.plane + d] = 0.0;
-            Wb[k * m.plane + o] += (mir && k == 1) ? -v : v;
+DFK_HD void ka_fold_y_body(const Mesh& m, double* Wb, int i, int k0 = 0, int k1 = 4) {
+    if (i >= m.nx + G) return;
+    for (int k = k0; k < k1; ++k) {
+        long long d[2 * G], o[2 * G];
+        bool neg[2 * G];
+#pragma unroll
+        for (int gr = 0; gr < 2 * G; ++gr) {
+            const int j = gr < G ? gr - G : m.ny + gr - G;
+            bool mir;
+            o[gr] = gid(m, i, ghost_src(j, m.ny, m.bc[2], m.bc[3], mir));
+            d[gr] = gid(m, i, j);
+            neg[gr] = mir && k == 2;
         }
+        fold_add(Wb + k * m.plane, d, o, neg);
+    }
+}
+
+DFK_HD void ka_fold_x_body(const Mesh& m, double* Wb, int j, int k0 = 0, int k1 = 4) {
+    if (j >= m.ny) return;
+    for (int k = k0; k < k1; ++k) {
+        long long d[2 * G], o[2 * G];
+        bool neg[2 * G];
+#pragma unroll
+        for (int gc = 0; gc < 2 * G; ++gc) {
+            const int i = gc < G ? gc - G : m.nx + gc - G;
+            bool mir;
+            o[gc] = gid(m, ghost_src(i, m.nx, m.bc[0], m.bc[1], mir), j);
+            d[gc] = gid(m, i, j);
+            neg[gc] = mir && k == 1;
+        }
+        fold_add(Wb + k * m.plane, d, o, neg);
     }
 }
 
@@ -456,86 +473,98 @@ DFK_HD void ka_accumulate_body(const Mesh& m, const double* __restrict__ Wbg, do
     for (int k = 0; k < 4; ++k) out[k * dp + (long long)j * m.nx + i] += Wbg[k * m.plane + gid(m, i, j)];
 }
 
-// ---- kernels: one thread per body invocation ----
-template <int DIR, int FLUX, bool TAPED = false>
-__global__ void __launch_bounds__(128) ka_flux(Mesh m, SchemeConsts S, AdjointArgs a, const double* __restrict__ gp,
-                                               long long gs, const double* __restrict__ fr, long long fs,
-                                               const double* dtp, double* __restrict__ lb, long long ls,
-                                               double* __restrict__ gb, double* __restrict__ tape = nullptr) {
-    int ax, ay;
-    sweep_xy(faces_lx<DIR>(m), ax, ay);
-    ka_flux_body<DIR, FLUX, TAPED>(m, S, a, gp, gs, fr, fs, *dtp, lb, ls, gb, ax, ay, blockIdx.y, tape);
+// ---- kernels: one thread per body invocation; blocks [0, nb0) take the x sweep, the rest the y sweep ----
+struct ReverseDir {
+    const double* lines; const double* gp; const double* fr; long long fs;
+    double* lb; double* gb; double* tape; double* ltape; double* ftape;
+};
+
+__device__ __forceinline__ void reverse_at(int b, int lx, int& ax, int& ay) {
+    const int i = b * (int)blockDim.x + (int)threadIdx.x;
+    ax = i % lx;
+    ay = i / lx;
 }
 
-template <int DIR, bool TAPED>
-__global__ void __launch_bounds__(128) ka_faces(Mesh m, SchemeConsts S, const double* __restrict__ alpha,
-                                                const double* __restrict__ lines, long long ls,
-                                                const double* __restrict__ gp, const double* __restrict__ gb,
-                                                long long gs, double* __restrict__ lb, double* __restrict__ Wb,
-                                                double* __restrict__ ftape) {
+template <int FLUX, bool TAPED>
+__global__ void __launch_bounds__(128) ka_flux(Mesh m, SchemeConsts S, AdjointArgs a, ReverseDir X, ReverseDir Y, long long ls,
+                                               long long gs, const double* dtp, int nb0) {
     int ax, ay;
-    sweep_xy(faces_lx<DIR>(m), ax, ay);
-    ka_faces_body<DIR, TAPED>(m, S, alpha, lines, ls, gp, gb, gs, lb, Wb, ax, ay, blockIdx.y, ftape);
+    const int b = blockIdx.x;
+    if (b < nb0) {
+        reverse_at(b, faces_lx<0>(m), ax, ay);
+        ka_flux_body<0, FLUX, TAPED>(m, S, a, X.gp, gs, X.fr, X.fs, *dtp, X.lb, ls, X.gb, ax, ay, blockIdx.y, X.tape);
+    } else {
+        reverse_at(b - nb0, faces_lx<1>(m), ax, ay);
+        ka_flux_body<1, FLUX, TAPED>(m, S, a, Y.gp, gs, Y.fr, Y.fs, *dtp, Y.lb, ls, Y.gb, ax, ay, blockIdx.y, Y.tape);
+    }
 }
 
-template <int DIR, bool TAPED>
-__global__ void __launch_bounds__(128) ka_lines(Mesh m, SchemeConsts S, const double* __restrict__ W,
-                                                const double* __restrict__ alpha, const double* __restrict__ lines,
-                                                const double* __restrict__ lb, long long ls, double* __restrict__ Wb,
-                                                double* __restrict__ ltape) {
+template <bool TAPED>
+__global__ void __launch_bounds__(128) ka_faces(Mesh m, SchemeConsts S, const double* __restrict__ alpha, ReverseDir X, ReverseDir Y,
+                                                long long ls, long long gs, double* __restrict__ Wb, int nb0) {
     int ax, ay;
-    sweep_xy(lines_lx<DIR>(m), ax, ay);
-    ka_lines_body<DIR, TAPED>(m, S, W, alpha, lines, lb, ls, Wb, ax, ay, ltape);
+    const int b = blockIdx.x;
+    if (b < nb0) {
+        reverse_at(b, faces_lx<0>(m), ax, ay);
+        ka_faces_body<0, TAPED>(m, S, alpha, X.lines, ls, X.gp, X.gb, gs, X.lb, Wb, ax, ay, blockIdx.y, X.ftape);
+    } else {
+        reverse_at(b - nb0, faces_lx<1>(m), ax, ay);
+        ka_faces_body<1, TAPED>(m, S, alpha, Y.lines, ls, Y.gp, Y.gb, gs, Y.lb, Wb, ax, ay, blockIdx.y, Y.ftape);
+    }
 }
 
-__global__ void ka_fold_y(Mesh m, double* Wb) { ka_fold_y_body(m, Wb, blockIdx.x * blockDim.x + threadIdx.x - G); }
-__global__ void ka_fold_x(Mesh m, double* Wb) { ka_fold_x_body(m, Wb, blockIdx.x * blockDim.x + threadIdx.x); }
+template <bool TAPED>
+__global__ void __launch_bounds__(128) ka_lines(Mesh m, SchemeConsts S, const double* __restrict__ W, const double* __restrict__ alpha,
+                                                ReverseDir X, ReverseDir Y, long long ls, double* __restrict__ Wb, int nb0) {
+    int ax, ay;
+    const int b = blockIdx.x;
+    if (b < nb0) {
+        reverse_at(b, lines_lx<0>(m), ax, ay);
+        ka_lines_body<0, TAPED>(m, S, W, alpha, X.lines, X.lb, ls, Wb, ax, ay, X.ltape);
+    } else {
+        reverse_at(b - nb0, lines_lx<1>(m), ax, ay);
+        ka_lines_body<1, TAPED>(m, S, W, alpha, Y.lines, Y.lb, ls, Wb, ax, ay, Y.ltape);
+    }
+}
+
+__global__ void ka_fold_y(Mesh m, double* Wb) { ka_fold_y_body(m, Wb, blockIdx.x * blockDim.x + threadIdx.x - G, blockIdx.y, blockIdx.y + 1); }
+__global__ void ka_fold_x(Mesh m, double* Wb) { ka_fold_x_body(m, Wb, blockIdx.x * blockDim.x + threadIdx.x, blockIdx.y, blockIdx.y + 1); }
 __global__ void ka_accumulate_dense(Mesh m, const double* __restrict__ Wbg, double* __restrict__ out) {
     ka_accumulate_body(m, Wbg, out, blockIdx.x * blockDim.x + threadIdx.x, blockIdx.y * blockDim.y + threadIdx.y);
 }
 
-template <int DIR>
-static void adjoint_dir(const Mesh& m, const SchemeConsts& S, int flux, const AdjointArgs& a, const double* W,
-                        const double* alpha, const double* dtp, const SweepBuffers& B, double* lb, double* gbuf,
-                        double* Wb, cudaStream_t s, KernelTimer* T) {
+void launch_adjoint(int dirs, const Mesh& m, const SchemeConsts& S, int flux, const AdjointArgs& a, const double* W,
+                    const double* alpha, const double* dtp, const SweepBuffers B[2], double* const lb[2],
+                    double* const gbuf[2], double* Wb, cudaStream_t s, KernelTimer* T) {
     // the forward sweep's 1-D grids (sweep_xy)
     const dim3 blk(kSweepThreads);
-    const dim3 gf(sweep_blocks(faces_lx<DIR>(m), faces_ly<DIR>(m)), 2);
-    const dim3 gl(sweep_blocks(lines_lx<DIR>(m), lines_ly<DIR>(m)));
-    cudaMemsetAsync(lb, 0, sizeof(double) * LR_COUNT * B.line_stride, s);
+    const bool dx = dirs & 1, dy = dirs & 2;
+    const int nf0 = dx ? (int)sweep_blocks(faces_lx<0>(m), faces_ly<0>(m)) : 0, nf1 = dy ? (int)sweep_blocks(faces_lx<1>(m), faces_ly<1>(m)) : 0;
+    const int nl0 = dx ? (int)sweep_blocks(lines_lx<0>(m), lines_ly<0>(m)) : 0, nl1 = dy ? (int)sweep_blocks(lines_lx<1>(m), lines_ly<1>(m)) : 0;
+    const dim3 gf(nf0 + nf1, 2), gl(nl0 + nl1);
+    ReverseDir R[2];
+    for (int d = 0; d < 2; ++d) {
+        R[d] = {B[d].lines, B[d].gp, B[d].flux[d], B[d].flux_stride[d], lb[d], gbuf[d], B[d].tape[d], B[d].ltape, B[d].ftape};
+        if (dirs & (1 << d)) cudaMemsetAsync(lb[d], 0, sizeof(double) * LR_COUNT * B[d].line_stride, s);
+    }
+    const int d0 = dx ? 0 : 1;
+    const long long ls = B[d0].line_stride, gs = B[d0].gp_stride;
     if (T) T->begin(KK_FLUX);
-    if (flux == 0 && B.tape[DIR])
-        ka_flux<DIR, 0, true><<<gf, blk, 0, s>>>(m, S, a, B.gp, B.gp_stride, B.flux[DIR], B.flux_stride[DIR], dtp, lb,
-                                                 B.line_stride, gbuf, B.tape[DIR]);
-    else if (flux == 0)
-        ka_flux<DIR, 0><<<gf, blk, 0, s>>>(m, S, a, B.gp, B.gp_stride, B.flux[DIR], B.flux_stride[DIR], dtp, lb,
-                                           B.line_stride, gbuf);
-    else
-        ka_flux<DIR, 1><<<gf, blk, 0, s>>>(m, S, a, B.gp, B.gp_stride, B.flux[DIR], B.flux_stride[DIR], dtp, lb,
-                                           B.line_stride, gbuf);
+    if (flux == 0 && B[d0].tape[d0]) ka_flux<0, true><<<gf, blk, 0, s>>>(m, S, a, R[0], R[1], ls, gs, dtp, nf0);
+    else if (flux == 0) ka_flux<0, false><<<gf, blk, 0, s>>>(m, S, a, R[0], R[1], ls, gs, dtp, nf0);
+    else ka_flux<1, false><<<gf, blk, 0, s>>>(m, S, a, R[0], R[1], ls, gs, dtp, nf0);
     if (T) { T->end(KK_FLUX, 1); T->begin(KK_FACES); }
-    if (B.ftape)
-        ka_faces<DIR, true><<<gf, blk, 0, s>>>(m, S, alpha, B.lines, B.line_stride, B.gp, gbuf, B.gp_stride, lb, Wb, B.ftape);
-    else
-        ka_faces<DIR, false><<<gf, blk, 0, s>>>(m, S, alpha, B.lines, B.line_stride, B.gp, gbuf, B.gp_stride, lb, Wb, nullptr);
+    if (B[d0].ftape) ka_faces<true><<<gf, blk, 0, s>>>(m, S, alpha, R[0], R[1], ls, gs, Wb, nf0);
+    else ka_faces<false><<<gf, blk, 0, s>>>(m, S, alpha, R[0], R[1], ls, gs, Wb, nf0);
     if (T) { T->end(KK_FACES, 1); T->begin(KK_LINES); }
-    if (B.ltape)
-        ka_lines<DIR, true><<<gl, blk, 0, s>>>(m, S, W, alpha, B.lines, lb, B.line_stride, Wb, B.ltape);
-    else
-        ka_lines<DIR, false><<<gl, blk, 0, s>>>(m, S, W, alpha, B.lines, lb, B.line_stride, Wb, nullptr);
+    if (B[d0].ltape) ka_lines<true><<<gl, blk, 0, s>>>(m, S, W, alpha, R[0], R[1], ls, Wb, nl0);
+    else ka_lines<false><<<gl, blk, 0, s>>>(m, S, W, alpha, R[0], R[1], ls, Wb, nl0);
     if (T) T->end(KK_LINES, 1);
 }
 
-void launch_adjoint_dir(int dir, const Mesh& m, const SchemeConsts& S, int flux, const AdjointArgs& a,
-                        const double* W, const double* alpha, const double* dtp, const SweepBuffers& B,
-                        double* lb, double* gbuf, double* Wb, cudaStream_t s, KernelTimer* T) {
-    if (dir == 0) adjoint_dir<0>(m, S, flux, a, W, alpha, dtp, B, lb, gbuf, Wb, s, T);
-    else adjoint_dir<1>(m, S, flux, a, W, alpha, dtp, B, lb, gbuf, Wb, s, T);
-}
-
 void launch_adjoint_finish(const Mesh& m, double* Wbg, double* Wb_dense, cudaStream_t s) {
-    ka_fold_y<<<(m.nx + 2 * G + 127) / 128, 128, 0, s>>>(m, Wbg);
-    ka_fold_x<<<(m.ny + 127) / 128, 128, 0, s>>>(m, Wbg);
+    ka_fold_y<<<dim3((m.nx + 2 * G + 31) / 32, 4), 32, 0, s>>>(m, Wbg);
+    ka_fold_x<<<dim3((m.ny + 31) / 32, 4), 32, 0, s>>>(m, Wbg);
     dim3 blk(32, 8), grd((m.nx + 31) / 32, (m.ny + 7) / 8);
     ka_accumulate_dense<<<grd, blk, 0, s>>>(m, Wbg, Wb_dense);
 }

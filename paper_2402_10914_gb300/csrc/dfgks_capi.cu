@@ -38,10 +38,12 @@ struct dfgks {
     long long fail_step;
     int fail_i, fail_j;
     KernelTimer* timer;    // per-kernel-class event timing and launch counts
-    double* adj_lines;     // reverse sweep: face-line record adjoints
-    double* adj_gp;        // reverse sweep: Gauss-point record adjoints
-    double* adj_Wg;        // reverse sweep: ghosted cell adjoints
-    double* adj_tape;      // reverse sweep: one direction's tapes (optional)
+    // reverse sweep: face-line and Gauss-point record adjoints (the second set, for both directions at once,
+    // optional), ghosted cell adjoints, and the tapes of one direction (or of both, with the second set; optional)
+    double* adj_lines[2];
+    double* adj_gp[2];
+    double* adj_Wg;
+    double* adj_tape;
     // checkpointed forward pass kept for dfgks_adjoint_checkpointed
     double* ck_W;          // dense [nseg][4][ny][nx]: W at steps 0, k, 2k, ...
     double* ck_A;          // dense [nseg][ny][nx]: alpha at the same steps
@@ -122,8 +124,8 @@ static bool config_ok(const dfgks_config* c) {
 
 static void free_all(dfgks* h) {
     double* ptrs[] = {h->W[0], h->W[1], h->A[0], h->A[1], h->Ws, h->As, h->acc, h->B.lines, h->B.gp,
-                      h->B.flux[0], h->B.flux[1], h->By.lines, h->By.gp, h->dt_scratch, h->dts, h->adj_lines,
-                      h->adj_gp, h->adj_Wg, h->adj_tape};
+                      h->B.flux[0], h->B.flux[1], h->By.lines, h->By.gp, h->dt_scratch, h->dts, h->adj_lines[0],
+                      h->adj_lines[1], h->adj_gp[0], h->adj_gp[1], h->adj_Wg, h->adj_tape};
     for (double* p : ptrs) if (p) cudaFree(p);
     if (h->seg_arena) cudaFree(h->seg_arena);
     if (h->ck_W) cudaFree(h->ck_W);
@@ -447,8 +449,7 @@ static dfgks_status run_stage_operator(dfgks* h, const double* W, const double* 
     launch_dense_to_ghosted(h->mesh, alpha, 1, h->As, h->stream);
     launch_fill_ghosts(h->mesh, h->Ws, h->As, nullptr, h->stream);
     launch_set_scalar(h->dt_scratch, dt, h->stream);
-    for (int d = 0; d < 2; ++d)
-        launch_sweep(d, h->mesh, h->S, flux, false, h->Ws, h->As, h->dt_scratch, h->B, nullptr, nullptr, h->stream);
+    launch_sweep_xy(h->mesh, h->S, flux, SWEEP_FULL, h->Ws, h->As, h->dt_scratch, h->B, h->By, nullptr, nullptr, h->stream);
     CK_LAUNCH();
     return DFGKS_OK;
 }
@@ -481,24 +482,47 @@ extern "C" dfgks_status dfgks_face_records(dfgks* h, const double* W, const doub
     return DFGKS_OK;
 }
 
+// one direction's tapes: reconstruction ratios of face lines and face sides, GKS flux
+static long long tape_doubles(const dfgks* h) {
+    const SweepBuffers& B = h->B;
+    return (long long)TG_COUNT * (B.flux_stride[0] > B.flux_stride[1] ? B.flux_stride[0] : B.flux_stride[1])
+         + (long long)8 * RT_COUNT * B.line_stride + (long long)4 * RT_COUNT * B.gp_stride;
+}
+
 static dfgks_status ensure_adjoint_buffers(dfgks* h) {
-    if (h->adj_lines) return DFGKS_OK;
-    CK(dalloc(h, &h->adj_lines, (long long)LR_COUNT * h->B.line_stride));
-    CK(dalloc(h, &h->adj_gp, (long long)GP_COUNT * h->B.gp_stride));
+    if (h->adj_Wg) return DFGKS_OK;
+    const SweepBuffers& B = h->B;
+    const long long nl = (long long)LR_COUNT * B.line_stride, ng = (long long)GP_COUNT * B.gp_stride;
+    if (!h->adj_lines[0]) CK(dalloc(h, &h->adj_lines[0], nl));
+    if (!h->adj_gp[0]) CK(dalloc(h, &h->adj_gp[0], ng));
     CK(dalloc(h, &h->adj_Wg, 4 * h->mesh.plane));
-    // One direction's tapes, for reverse sweeps that evaluate their forward first: the reverse then does not
-    // evaluate fluxes and weights a second time.  Left out where they would take more than a quarter of the
-    // free memory.
-    const long long nflux = (long long)TG_COUNT * (h->B.flux_stride[0] > h->B.flux_stride[1] ? h->B.flux_stride[0] : h->B.flux_stride[1]);
-    const long long nlines = (long long)8 * RT_COUNT * h->B.line_stride, nfaces = (long long)4 * RT_COUNT * h->B.gp_stride;
-    const long long n = nflux + nlines + nfaces;
+    // With a second set both directions are reversed at once: the launches are twice as large, so small meshes
+    // fill more of the chip and the last round of blocks weighs less (67 x 83 GKS stage with its forward 483 ->
+    // 302 us, 400 x 400 L-F 3.67 -> 3.48 ms, the latter by the last round and faster folds).  The tapes are for reverse sweeps that
+    // evaluate their forward first: the reverse then does not evaluate fluxes and weights a second time.  Each is
+    // left out where it would take more than a quarter of the free memory.
+    const long long n = tape_doubles(h);
     size_t free_b = 0, total_b = 0;
     cudaMemGetInfo(&free_b, &total_b);
-    if ((double)n * sizeof(double) <= 0.25 * (double)free_b && dalloc(h, &h->adj_tape, n) != cudaSuccess) {
-        cudaGetLastError();
-        h->adj_tape = nullptr;
-    }
+    const double quarter = 0.25 * (double)free_b / sizeof(double);
+    if ((double)(nl + ng + 2 * n) <= quarter && dalloc(h, &h->adj_lines[1], nl) == cudaSuccess
+        && dalloc(h, &h->adj_gp[1], ng) == cudaSuccess && dalloc(h, &h->adj_tape, 2 * n) == cudaSuccess)
+        return DFGKS_OK;
+    for (double** q : {&h->adj_lines[1], &h->adj_gp[1], &h->adj_tape})
+        if (*q) { cudaFree(*q); h->bytes -= sizeof(double) * (unsigned long long)(q == &h->adj_gp[1] ? ng : q == &h->adj_tape ? 2 * n : nl); *q = nullptr; }
+    if ((double)n <= quarter && dalloc(h, &h->adj_tape, n) != cudaSuccess) h->adj_tape = nullptr;
+    cudaGetLastError();
     return DFGKS_OK;
+}
+
+// h's records with set k of the tapes (none if there are none)
+static SweepBuffers taped_records(const dfgks* h, const SweepBuffers& B, int k, int flux) {
+    SweepBuffers t = B;
+    if (!h->adj_tape) return t;
+    t.ltape = h->adj_tape + k * tape_doubles(h);
+    t.ftape = t.ltape + (long long)8 * RT_COUNT * t.line_stride;
+    if (flux == DFGKS_FLUX_GKS) t.tape[0] = t.tape[1] = t.ftape + (long long)4 * RT_COUNT * t.gp_stride;
+    return t;
 }
 
 // reverse sweep of the stage operator at (W, alpha, dt); W_bar (dense, device) += J^T (L_bar, ...)
@@ -515,18 +539,23 @@ static dfgks_status adjoint_stage(dfgks* h, const double* W, const double* alpha
     launch_set_scalar(h->dt_scratch, dt, h->stream);
     CK(cudaMemsetAsync(h->adj_Wg, 0, sizeof(double) * 4 * h->mesh.plane, h->stream));
     AdjointArgs a = {L_bar, dtL_bar, dtLt_bar};
-    SweepBuffers own = h->B;
-    if (h->adj_tape) {
-        own.ltape = h->adj_tape;
-        own.ftape = own.ltape + (long long)8 * RT_COUNT * own.line_stride;
-        if (flux == DFGKS_FLUX_GKS) own.tape[0] = own.tape[1] = own.ftape + (long long)4 * RT_COUNT * own.gp_stride;
-    }
-    for (int d = 0; d < 2; ++d) {
-        // the records of this direction, then its reverse sweep
+    KernelTimer* T = h->timer->on ? h->timer : nullptr;
+    const bool both = h->adj_lines[1] != nullptr;
+    const SweepBuffers own[2] = {taped_records(h, h->B, 0, flux), taped_records(h, both ? h->By : h->B, both ? 1 : 0, flux)};
+    const SweepBuffers* R = rec ? rec : own;
+    if (both) {
         if (!rec)
-            launch_sweep(d, h->mesh, h->S, flux, false, h->Ws, h->As, h->dt_scratch, own, nullptr, nullptr, h->stream);
-        launch_adjoint_dir(d, h->mesh, h->S, flux, a, h->Ws, h->As, h->dt_scratch, rec ? rec[d] : own, h->adj_lines,
-                           h->adj_gp, h->adj_Wg, h->stream, h->timer->on ? h->timer : nullptr);
+            launch_sweep_xy(h->mesh, h->S, flux, SWEEP_FULL, h->Ws, h->As, h->dt_scratch, own[0], own[1], nullptr, nullptr, h->stream);
+        launch_adjoint(3, h->mesh, h->S, flux, a, h->Ws, h->As, h->dt_scratch, R, h->adj_lines, h->adj_gp, h->adj_Wg, h->stream, T);
+    } else {
+        double* const lb[2] = {h->adj_lines[0], h->adj_lines[0]};
+        double* const gb[2] = {h->adj_gp[0], h->adj_gp[0]};
+        for (int d = 0; d < 2; ++d) {
+            // the records of this direction, then its reverse sweep
+            if (!rec)
+                launch_sweep(d, h->mesh, h->S, flux, false, h->Ws, h->As, h->dt_scratch, own[d], nullptr, nullptr, h->stream);
+            launch_adjoint(1 << d, h->mesh, h->S, flux, a, h->Ws, h->As, h->dt_scratch, R, lb, gb, h->adj_Wg, h->stream, T);
+        }
     }
     launch_adjoint_finish(h->mesh, h->adj_Wg, W_bar, h->stream);
     CK_LAUNCH();

@@ -162,9 +162,10 @@ void launch_set_scalar(double* p, double v, cudaStream_t s);
 void launch_pack_faces(int dir, const Mesh& m, const SweepBuffers& B, double* out, cudaStream_t s);
 
 // ---- reverse sweep (dfgks_adjoint.cu) -------------------------------------------------------
-void launch_adjoint_dir(int dir, const Mesh& m, const SchemeConsts& S, int flux, const AdjointArgs& a,
-                        const double* W, const double* alpha, const double* dtp, const SweepBuffers& B,
-                        double* lb, double* gbuf, double* Wb, cudaStream_t s, KernelTimer* T = nullptr);
+// dirs: 1 the x sweep, 2 the y sweep, 3 both at once; B, lb, gbuf per direction (distinct for 3)
+void launch_adjoint(int dirs, const Mesh& m, const SchemeConsts& S, int flux, const AdjointArgs& a,
+                    const double* W, const double* alpha, const double* dtp, const SweepBuffers B[2],
+                    double* const lb[2], double* const gbuf[2], double* Wb, cudaStream_t s, KernelTimer* T = nullptr);
 void launch_adjoint_finish(const Mesh& m, double* Wbg, double* Wb_dense, cudaStream_t s);
 void launch_axpby(long long n, double a, const double* x, double b, double* y, cudaStream_t s);
 
