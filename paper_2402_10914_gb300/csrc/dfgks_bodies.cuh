@@ -163,6 +163,45 @@ DFK_HD void ghost_y_body(const Mesh& m, double* W, double* alpha, int i, int gr)
     if (alpha) alpha[d] = alpha[o];
 }
 
+// One characteristic variable of a face line from its first differences f: both sides' value (relative to the cell
+// average) and slope, q = qL, qLn, qR, qRn, and their weights where they are used (L, R)
+template <bool VALUES>
+DFK_HD void line_component(const Real f[5], bool acoustic, bool dfL, bool dfR, double alL, double alR, Real idn,
+                           const SchemeConsts& S, Real q[4], AOWeights& L, AOWeights& R) {
+    const Real s1 = f[1] - f[0], s2 = f[2] - f[1], s3 = f[3] - f[2], s4 = f[4] - f[3];
+    const Real f3 = f[2], hf = 0.5 * f3;
+    // both sides' central quadratics at the face: cell f-1 at xi = +1/2, cell f mirrored
+    const Real baseL = fma(-1.0 / 6.0, s2, hf), baseR = fma(-1.0 / 6.0, s3, -hf);
+    if (!dfL || !dfR || (!VALUES && S.time_limiter)) {
+        const Real eps = acoustic ? Real(4.0 * S.eps) : Real(S.eps);
+        const Real t1 = s2 - s1, t2 = s3 - s2, t3 = s4 - s3;
+        const Real w1 = second_difference_energy(s1, eps), w2 = second_difference_energy(s2, eps);
+        const Real w3 = second_difference_energy(s3, eps), w4 = second_difference_energy(s4, eps);
+        L = ao_weights<+1>(f[1], f3, s1, s2, s3, w1, w2, w3, fma(0.5, s2, f[1]), t1 + t2, t2 - t1, eps, S);
+        R = ao_weights<-1>(f[3], f3, s4, s3, s2, w4, w3, w2, fma(-0.5, s3, f[3]), t2 + t3, t3 - t2, eps, S);
+        const Real h2 = 0.5 * t2, h12 = (1.0 / 12.0) * t2, h20 = (1.0 / 20.0) * t2, d03 = (1.0 / 3.0) * S.d[0];
+        if (!dfL) {
+            const Real iv = ao_inverse_sum(L), p = L.y0 * t1;
+            const Real v = fma(d03, fma(h2, L.y2, p), L.x3 * fma(1.0 / 30.0, t1, h20));
+            q[0] = fma(-iv, v, baseL);
+            q[1] = idn * fma(-iv, fma(S.d[0], p, L.x3 * h12), f3);
+        }
+        if (!dfR) {
+            const Real iv = ao_inverse_sum(R), p = R.y0 * t3;
+            const Real v = fma(d03, fma(h2, R.y2, p), R.x3 * fma(1.0 / 30.0, t3, h20));
+            q[2] = fma(iv, v, baseR);
+            q[3] = idn * fma(-iv, fma(S.d[0], p, R.x3 * h12), f3);
+        }
+    }
+    if (dfL) { q[0] = Real::raw(alL) * baseL; q[1] = idn * (Real::raw(alL) * f3); }
+    if (dfR) { q[2] = Real::raw(alR) * baseR; q[3] = idn * (Real::raw(alR) * f3); }
+}
+
+// the limiter fraction so far, (1 + rmax^2) / (1 + rmin^2) = hi / lo at its largest, and the reconstruction it is of
+DFK_HD void limiter_update(Real xmax, Real xmin, int which, Real& hi, Real& lo, int& tlk) {
+    if (nn_less(hi * xmin, xmax * lo)) { hi = xmax; lo = xmin; tlk = which; }
+}
+
 // one face line (normal reconstruction of both sides); returns the number of DF branches taken
 // TAPE: also write the reconstructions' ratios for a reverse sweep (ltape, see SweepBuffers)
 // VALUES: the face values alone, for sweeps whose consumers use neither slopes nor the limiter weight: the DF
@@ -214,45 +253,22 @@ DFK_HD int lines_body(const Mesh& m, const SchemeConsts& S, const double* __rest
         Real xhi = 1.0, xlo = 1.0;                  // limiter: (1 + rmax^2) / (1 + rmin^2), the largest so far
 #pragma unroll
         for (int k = 0; k < 4; ++k) {
-            const Real s1 = F[1][k] - F[0][k], s2 = F[2][k] - F[1][k], s3 = F[3][k] - F[2][k], s4 = F[4][k] - F[3][k];
-            const Real f3 = F[2][k], hf = 0.5 * f3;
-            // both sides' central quadratics at the face: cell f-1 at xi = +1/2, cell f mirrored
-            const Real baseL = fma(-1.0 / 6.0, s2, hf), baseR = fma(-1.0 / 6.0, s3, -hf);
-            const bool limit = !VALUES && S.time_limiter;
-            if (!dfL || !dfR || limit) {
-                const Real eps = (k == 0 || k == 3) ? Real(4.0 * S.eps) : Real(S.eps);
-                const Real t1 = s2 - s1, t2 = s3 - s2, t3 = s4 - s3;
-                const Real w1 = second_difference_energy(s1, eps), w2 = second_difference_energy(s2, eps);
-                const Real w3 = second_difference_energy(s3, eps), w4 = second_difference_energy(s4, eps);
-                const AOWeights L = ao_weights<+1>(F[1][k], f3, s1, s2, s3, w1, w2, w3, fma(0.5, s2, F[1][k]), t1 + t2,
-                                                   t2 - t1, eps, S);
-                const AOWeights R = ao_weights<-1>(F[3][k], f3, s4, s3, s2, w4, w3, w2, fma(-0.5, s3, F[3][k]), t2 + t3,
-                                                   t3 - t2, eps, S);
-                if constexpr (TAPE) {
+            const Real fk[5] = {F[0][k], F[1][k], F[2][k], F[3][k], F[4][k]};
+            Real q[4];
+            AOWeights L, R;
+            line_component<VALUES>(fk, k == 0 || k == 3, dfL, dfR, al[2], al[3], idn, S, q, L, R);
+            if constexpr (TAPE) {
+                if (!dfL || !dfR || S.time_limiter) {
                     const PlaneTape T{ltape + li, ls};
                     tape_ratios(T, 2 * k * RT_COUNT, ao_ratios(L));
                     tape_ratios(T, (2 * k + 1) * RT_COUNT, ao_ratios(R));
                 }
-                if (limit) {
-                    if (nn_less(xhi * L.xmin, L.xmax * xlo)) { xhi = L.xmax; xlo = L.xmin; tlk = 2 * k; }
-                    if (nn_less(xhi * R.xmin, R.xmax * xlo)) { xhi = R.xmax; xlo = R.xmin; tlk = 2 * k + 1; }
-                }
-                const Real h2 = 0.5 * t2, h12 = (1.0 / 12.0) * t2, h20 = (1.0 / 20.0) * t2, d03 = (1.0 / 3.0) * S.d[0];
-                if (!dfL) {
-                    const Real iv = ao_inverse_sum(L), p = L.y0 * t1;
-                    const Real v = fma(d03, fma(h2, L.y2, p), L.x3 * fma(1.0 / 30.0, t1, h20));
-                    qL[k] = fma(-iv, v, baseL);
-                    qLn[k] = idn * fma(-iv, fma(S.d[0], p, L.x3 * h12), f3);
-                }
-                if (!dfR) {
-                    const Real iv = ao_inverse_sum(R), p = R.y0 * t3;
-                    const Real v = fma(d03, fma(h2, R.y2, p), R.x3 * fma(1.0 / 30.0, t3, h20));
-                    qR[k] = fma(iv, v, baseR);
-                    qRn[k] = idn * fma(-iv, fma(S.d[0], p, R.x3 * h12), f3);
-                }
             }
-            if (dfL) { qL[k] = Real::raw(al[2]) * baseL; qLn[k] = idn * (Real::raw(al[2]) * f3); }
-            if (dfR) { qR[k] = Real::raw(al[3]) * baseR; qRn[k] = idn * (Real::raw(al[3]) * f3); }
+            if (!VALUES && S.time_limiter) {
+                limiter_update(L.xmax, L.xmin, 2 * k, xhi, xlo, tlk);
+                limiter_update(R.xmax, R.xmin, 2 * k + 1, xhi, xlo, tlk);
+            }
+            qL[k] = q[0]; qLn[k] = q[1]; qR[k] = q[2]; qRn[k] = q[3];
         }
         tn = Real(2.0 * xlo).v;
         td = (xhi + xlo).v;
@@ -285,6 +301,28 @@ DFK_HD int lines_body(const Mesh& m, const SchemeConsts& S, const double* __rest
         lines[LR_Q2 * ls + li] = B.q2;
     }
     return ndf;
+}
+
+// One characteristic variable of a face side from its first differences f: values (relative to the line's) and
+// scaled slopes at the two Gauss points, q = v0, v1, slope0, slope1
+template <class Tape>
+DFK_HD void face_component(const Real f[4], bool acoustic, bool df, double alpha, Real idt, const SchemeConsts& S, Real q[4],
+                           const Tape& tp, int base) {
+    const Real s0 = f[1] - f[0], s1 = f[2] - f[1], s2 = f[3] - f[2];
+    const Real a11 = fma(0.5, s1, f[1]);
+    Real v[2], s[2];
+    if (df) df_diff_at_gauss(a11, s1, Real::raw(alpha), v, s);
+    else {
+        const Real eps = acoustic ? Real(4.0 * S.eps) : Real(S.eps);
+        const Real t1 = s1 - s0, t2 = s2 - s1, T = t1 + t2, U = t2 - t1;
+        const AOWeights o = ao_weights<+1>(f[1], f[2], s0, s1, s2, second_difference_energy(s0, eps),
+                                           second_difference_energy(s1, eps), second_difference_energy(s2, eps),
+                                           a11, T, U, eps, S);
+        if constexpr (Tape::active) tape_ratios(tp, base, ao_ratios(o));
+        ao_diff_at_gauss(o, a11, s1, t1, t2, T, U, S, v, s);
+    }
+    q[0] = v[0]; q[1] = v[1];
+    q[2] = s[0] * idt; q[3] = s[1] * idt;
 }
 
 // one face side (tangential reconstruction at both Gauss points, fallback); returns the number of
@@ -337,21 +375,12 @@ DFK_HD int faces_body(const Mesh& m, const SchemeConsts& S, const double* __rest
         }
 #pragma unroll
         for (int k = 0; k < 4; ++k) {
-            const Real s0 = F[1][k] - F[0][k], s1 = F[2][k] - F[1][k], s2 = F[3][k] - F[2][k];
-            const Real a11 = fma(0.5, s1, F[1][k]);
-            Real v[2], s[2];
-            if (df) df_diff_at_gauss(a11, s1, Real::raw(al[1]), v, s);
-            else {
-                const Real eps = (k == 0 || k == 3) ? Real(4.0 * S.eps) : Real(S.eps);
-                const Real t1 = s1 - s0, t2 = s2 - s1, T = t1 + t2, U = t2 - t1;
-                const AOWeights o = ao_weights<+1>(F[1][k], F[2][k], s0, s1, s2, second_difference_energy(s0, eps),
-                                                   second_difference_energy(s1, eps), second_difference_energy(s2, eps),
-                                                   a11, T, U, eps, S);
-                if constexpr (TAPE) tape_ratios(PlaneTape{ftape + e, gs}, k * RT_COUNT, ao_ratios(o));
-                ao_diff_at_gauss(o, a11, s1, t1, t2, T, U, S, v, s);
-            }
-            qv[0][k] = v[0]; qv[1][k] = v[1];
-            qt[0][k] = s[0] * idt; qt[1][k] = s[1] * idt;
+            const Real fk[4] = {F[0][k], F[1][k], F[2][k], F[3][k]};
+            Real q[4];
+            if constexpr (TAPE) face_component(fk, k == 0 || k == 3, df, al[1], idt, S, q, PlaneTape{ftape + e, gs}, k * RT_COUNT);
+            else face_component(fk, k == 0 || k == 3, df, al[1], idt, S, q, NoTape{}, 0);
+            qv[0][k] = q[0]; qv[1][k] = q[1];
+            qt[0][k] = q[2]; qt[1][k] = q[3];
         }
 #pragma unroll
         for (int mm = 0; mm < 2; ++mm) {
@@ -398,6 +427,177 @@ DFK_HD int faces_body(const Mesh& m, const SchemeConsts& S, const double* __rest
     }
     return ndf;
 }
+
+// ------------------------------------------------------------------------------------------
+// Four threads per face line and per face side, one per characteristic variable, for meshes so small that a
+// launch takes as long as one thread: a warp alone on its scheduler takes 12.7 cycles per instruction, 31 us for a
+// line and 19 us for a side, whatever the mesh.  Differences and basis are formed by each thread of a quad; the
+// results change hands in one 4 x 4 transposition, after which thread j back-projects the j-th vector.  The
+// arithmetic is that of lines_body and faces_body operation by operation, so the results are the same bits.
+// All 32 lanes take part in the exchanges: a quad past the end works on item 0 and writes nothing.
+// 8 GKS steps of 100 x 4 1.77 -> 1.31 ms, 20 L-F steps of 40 x 40 3.82 -> 2.75 ms.
+// ------------------------------------------------------------------------------------------
+#ifdef __CUDACC__
+// component k of project_diff
+__device__ __forceinline__ Real project_diff_component(const DiffBasis& D, const Real W[4], int k) {
+    const Real kk = fma(D.b1, W[3], fma(-D.b1v, W[2], fma(-D.b1u, W[1], D.b2 * W[0])));
+    const Real mm = fma(-D.ic, W[1], D.uic * W[0]);
+    const Real A = k == 2 ? -D.v : (k == 1 ? W[0] : kk), M = k == 2 ? W[0] : Real(1.0);
+    const Real C = k == 2 ? W[2] : (k == 1 ? -kk : (k == 3 ? -mm : mm));
+    return fma(A, M, C);
+}
+__device__ __forceinline__ Real pick(const Real q[4], int j) { return (j & 2) ? ((j & 1) ? q[3] : q[2]) : ((j & 1) ? q[1] : q[0]); }
+// thread j of a quad holds q[0..3] of component j and gets the four components of q[j]
+__device__ __forceinline__ void quad_transpose(Real q[4], int j) {
+    Real r[4];
+#pragma unroll
+    for (int x = 0; x < 4; ++x) r[x] = Real::raw(__shfl_xor_sync(0xffffffffu, pick(q, j ^ x).v, x));   // component j ^ x
+#pragma unroll
+    for (int c = 0; c < 4; ++c) q[c] = pick(r, c ^ j);
+}
+__device__ __forceinline__ Real quad_get(Real v, int c) { return Real::raw(__shfl_sync(0xffffffffu, v.v, ((int)threadIdx.x & 28) + c)); }
+
+template <int DIR, bool VALUES>
+__device__ __forceinline__ int lines_quad(const Mesh& m, const SchemeConsts& S, const double* __restrict__ W,
+                                          const double* __restrict__ alpha, double* __restrict__ lines, long long ls,
+                                          int ax, int ay) {
+    Geo<DIR> g(m);
+    const int j = threadIdx.x & 3;
+    int f = DIR == 0 ? ax : ay, tt = DIR == 0 ? ay : ax;
+    const bool active = f <= g.nn && tt < g.nt + 4;
+    if (!active) f = tt = 0;
+    const int t = tt - 2;
+    double Wc[6][4], al[6];
+#pragma unroll
+    for (int s = 0; s < 6; ++s) {
+        const long long c = g.cell(m, f - 3 + s, t);
+#pragma unroll
+        for (int k = 0; k < 4; ++k) Wc[s][k] = W[k * m.plane + c];
+        to_local<DIR>(Wc[s]);
+        al[s] = alpha[c];
+    }
+    const CharBasis B = make_basis(Wc[2], Wc[3], S);
+    const bool dfL = nn_less(nn_max(nn_max(al[1], al[2]), al[3]), S.alpha_thres);
+    const bool dfR = nn_less(nn_max(nn_max(al[2], al[3]), al[4]), S.alpha_thres);
+    const long long li = g.line(f, t);
+    if (S.df_states && active && j == 2) lines[LR_DFC * ls + li] = df_alpha(Wc[2], Wc[3], S);
+    const DiffBasis D = diff_basis(B);
+    Real F[5], q[4];
+#pragma unroll
+    for (int s = 0; s < 5; ++s) {
+        Real dW[4];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) dW[k] = Real::raw(Wc[s + 1][k]) - Real::raw(Wc[s][k]);
+        F[s] = project_diff_component(D, dW, j);
+    }
+    AOWeights L, R;
+    line_component<VALUES>(F, j == 0 || j == 3, dfL, dfR, al[2], al[3], g.idn, S, q, L, R);
+    Real xhi = 1.0, xlo = 1.0;
+    int tlk = -1;
+    if (!VALUES && S.time_limiter) {
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            limiter_update(quad_get(L.xmax, k), quad_get(L.xmin, k), 2 * k, xhi, xlo, tlk);
+            limiter_update(quad_get(R.xmax, k), quad_get(R.xmin, k), 2 * k + 1, xhi, xlo, tlk);
+        }
+    }
+    quad_transpose(q, j);
+    if (!active) return 0;
+    if (!VALUES || (j & 1) == 0) {
+        Real w[4];
+        back_project_diff(D, q, w);
+        if ((j & 1) == 0) {
+#pragma unroll
+            for (int k = 0; k < 4; ++k) w[k] = w[k] + Real::raw(j == 0 ? Wc[2][k] : Wc[3][k]);
+        }
+#pragma unroll
+        for (int k = 0; k < 4; ++k) lines[(4 * j + k) * ls + li] = w[k].v;      // LR_WL, LR_WLN, LR_WR, LR_WRN
+    }
+    if (j == 0) {
+        if (!VALUES) {
+            lines[LR_TL * ls + li] = Real(2.0 * xlo).v / (xhi + xlo).v;
+            lines[LR_TLK * ls + li] = (double)tlk;
+        }
+        return (int)dfL + (int)dfR;
+    }
+    if (j == 1) {
+        lines[LR_U * ls + li] = B.u; lines[LR_V * ls + li] = B.v; lines[LR_C * ls + li] = B.c; lines[LR_IC * ls + li] = B.ic;
+    } else if (j == 3) {
+        lines[LR_H * ls + li] = B.H; lines[LR_B1 * ls + li] = B.b1; lines[LR_B2 * ls + li] = B.b2; lines[LR_Q2 * ls + li] = B.q2;
+    }
+    return 0;
+}
+
+template <int DIR, bool VALUES>
+__device__ __forceinline__ int faces_quad(const Mesh& m, const SchemeConsts& S, const double* __restrict__ W,
+                                          const double* __restrict__ alpha, const double* __restrict__ lines, long long ls,
+                                          double* __restrict__ gp, long long gs, int ax, int ay, int side, int& nfb) {
+    Geo<DIR> g(m);
+    const int j = threadIdx.x & 3;
+    int f = DIR == 0 ? ax : ay, t = DIR == 0 ? ay : ax;
+    const bool active = f <= g.nn && t < g.nt;
+    if (!active) f = t = 0;
+    nfb = 0;
+    const long long l0 = g.line(f, t);
+    CharBasis B;
+    B.u = lines[LR_U * ls + l0]; B.v = lines[LR_V * ls + l0]; B.c = lines[LR_C * ls + l0];
+    B.ic = lines[LR_IC * ls + l0]; B.H = lines[LR_H * ls + l0]; B.b1 = lines[LR_B1 * ls + l0];
+    B.b2 = lines[LR_B2 * ls + l0]; B.q2 = lines[LR_Q2 * ls + l0];
+    const int wbase = side == 0 ? LR_WL : LR_WR, nbase = side == 0 ? LR_WLN : LR_WRN, ncell = f - 1 + side;
+    double al[3];
+#pragma unroll
+    for (int b = 0; b < 3; ++b) al[b] = alpha[g.cell(m, ncell, t + Geo<DIR>::sigma * (b - 1))];
+    const bool df = nn_less(nn_max(nn_max(al[0], al[1]), al[2]), S.alpha_thres);
+    const long long e = (long long)side * g.nfaces() + g.face(f, t);
+    double Wl[5][4];
+#pragma unroll
+    for (int b = 0; b < 5; ++b) {
+        const long long lb = g.line(f, t + Geo<DIR>::sigma * (b - 2));
+#pragma unroll
+        for (int k = 0; k < 4; ++k) Wl[b][k] = lines[(wbase + k) * ls + lb];
+    }
+    const DiffBasis D = diff_basis(B);
+    Real F[4], q[4], w[4];
+#pragma unroll
+    for (int b = 0; b < 4; ++b) {
+        Real dW[4];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) dW[k] = Real::raw(Wl[b + 1][k]) - Real::raw(Wl[b][k]);
+        F[b] = project_diff_component(D, dW, j);
+    }
+    face_component(F, j == 0 || j == 3, df, al[1], g.idtan, S, q, NoTape{}, 0);
+    quad_transpose(q, j);                      // threads 0, 1: the values at the two Gauss points; 2, 3: the slopes
+    back_project_diff(D, q, w);
+    double Wg[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) Wg[k] = j < 2 ? (w[k] + Real::raw(Wl[2][k])).v : w[k].v;
+    const int bad = j < 2 && S.gp_fallback && !physical_state(Wg, S.gm1);
+    const int b0 = __shfl_sync(0xffffffffu, bad, threadIdx.x & 28), b1 = __shfl_sync(0xffffffffu, bad, (threadIdx.x & 28) + 1);
+    if (!active) return 0;
+    const int mm = j & 1;
+    const bool fell = mm == 0 ? b0 : b1;
+    if (j < 2) {
+        if (fell) {
+            const long long c = g.cell(m, ncell, t);
+#pragma unroll
+            for (int k = 0; k < 4; ++k) Wg[k] = W[k * m.plane + c];
+            to_local<DIR>(Wg);
+            nfb = 1;
+        }
+#pragma unroll
+        for (int k = 0; k < 4; ++k) gp[(mm * 12 + k) * gs + e] = Wg[k];
+    } else if (!VALUES) {
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            gp[(mm * 12 + 4 + k) * gs + e] = fell ? 0.0 : lines[(nbase + k) * ls + l0];
+            gp[(mm * 12 + 8 + k) * gs + e] = fell ? 0.0 : Wg[k];
+        }
+    }
+    if (j != 0) return 0;
+    gp[GP_FB * gs + e] = (double)(b0 | (b1 << 1));
+    return (int)df;
+}
+#endif
 
 // where one Gauss point's records live: side records eL / eR, its flux record e, its face line li
 struct FluxSite { long long eL, eR, e, li; bool ok; };

@@ -188,6 +188,46 @@ __global__ void __launch_bounds__(128) k_faces_xy(Mesh m, SchemeConsts S, const 
     if (st) { warp_count_add(&st->df_tangential, ndf); warp_count_add(&st->fallbacks, nfb); }
 }
 
+// the same with four threads per line and per side (blocks of one warp: eight items)
+__device__ __forceinline__ void quad_at(int b, int lx, int& ax, int& ay) {
+    const int i = (b * (int)blockDim.x + (int)threadIdx.x) >> 2;
+    ax = i % lx;
+    ay = i / lx;
+}
+
+template <bool VALUES>
+__global__ void __launch_bounds__(32) k_lines_quad(Mesh m, SchemeConsts S, const double* __restrict__ W,
+                                                   const double* __restrict__ alpha, double* __restrict__ lines0,
+                                                   double* __restrict__ lines1, long long ls, int nb0, DevState* st, const int* halt) {
+    if (halted(halt)) return;
+    int ax, ay, ndf;
+    if ((int)blockIdx.x < nb0) {
+        quad_at(blockIdx.x, lines_lx<0>(m), ax, ay);
+        ndf = lines_quad<0, VALUES>(m, S, W, alpha, lines0, ls, ax, ay);
+    } else {
+        quad_at(blockIdx.x - nb0, lines_lx<1>(m), ax, ay);
+        ndf = lines_quad<1, VALUES>(m, S, W, alpha, lines1, ls, ax, ay);
+    }
+    if (st) warp_count_add(&st->df_normal, ndf);
+}
+
+template <bool VALUES>
+__global__ void __launch_bounds__(32) k_faces_quad(Mesh m, SchemeConsts S, const double* __restrict__ W,
+                                                   const double* __restrict__ alpha, const double* __restrict__ lines0,
+                                                   const double* __restrict__ lines1, long long ls, double* __restrict__ gp0,
+                                                   double* __restrict__ gp1, long long gs, int nb0, DevState* st, const int* halt) {
+    if (halted(halt)) return;
+    int nfb, ax, ay, ndf;
+    if ((int)blockIdx.x < nb0) {
+        quad_at(blockIdx.x, faces_lx<0>(m), ax, ay);
+        ndf = faces_quad<0, VALUES>(m, S, W, alpha, lines0, ls, gp0, gs, ax, ay, blockIdx.y, nfb);
+    } else {
+        quad_at(blockIdx.x - nb0, faces_lx<1>(m), ax, ay);
+        ndf = faces_quad<1, VALUES>(m, S, W, alpha, lines1, ls, gp1, gs, ax, ay, blockIdx.y, nfb);
+    }
+    if (st) { warp_count_add(&st->df_tangential, ndf); warp_count_add(&st->fallbacks, nfb); }
+}
+
 template <int FLUX, bool ALPHA_ONLY, bool TAPE = false, bool VALUES = false>
 __global__ void __launch_bounds__(128) k_flux_xy(Mesh m, SchemeConsts S, const double* __restrict__ lines0,
                                               const double* __restrict__ lines1, long long ls,
@@ -215,6 +255,8 @@ __global__ void __launch_bounds__(128) k_flux_xy(Mesh m, SchemeConsts S, const d
                                        dir == 0 ? tape0 : tape1);
 }
 
+constexpr int kSMs = 152;
+
 void launch_sweep_xy(const Mesh& m, const SchemeConsts& S, int flux, SweepWhat what, const double* W,
                      const double* alpha, const double* dtp, const SweepBuffers& Bx, const SweepBuffers& By,
                      DevState* st, const int* halt, cudaStream_t s, KernelTimer* T) {
@@ -226,7 +268,17 @@ void launch_sweep_xy(const Mesh& m, const SchemeConsts& S, int flux, SweepWhat w
     const bool alpha_only = what == SWEEP_ALPHA, values = alpha_only || (what == SWEEP_VALUES && flux != 0);
     const long long ls = Bx.line_stride, gs = Bx.gp_stride;
     if (T) T->begin(KK_LINES);
-    if (values)
+    // Four threads per item where whole items are at most two (three) warps per SM.  A line's 740 FP64 instructions
+    // keep an SM's units 6 us per warp, a side's 430 3.5; the quads' 1200 and 620 take 10 and 5, against the 31 and
+    // 19 us that one thread takes however few there are: the quads win below three warps of lines and four of sides.
+    const bool quad_lines = !tape && nl0 + nl1 <= 2 * kSMs, quad_faces = !tape && 2 * (nf0 + nf1) <= 3 * kSMs;
+    const int ql0 = (int)sweep_blocks(lines_lx<0>(m), lines_ly<0>(m), kSweepThreads / 4), ql1 = (int)sweep_blocks(lines_lx<1>(m), lines_ly<1>(m), kSweepThreads / 4);
+    const int qf0 = (int)sweep_blocks(faces_lx<0>(m), faces_ly<0>(m), kSweepThreads / 4), qf1 = (int)sweep_blocks(faces_lx<1>(m), faces_ly<1>(m), kSweepThreads / 4);
+    if (quad_lines && values)
+        k_lines_quad<true><<<ql0 + ql1, blk, 0, s>>>(m, S, W, alpha, Bx.lines, By.lines, ls, ql0, st, halt);
+    else if (quad_lines)
+        k_lines_quad<false><<<ql0 + ql1, blk, 0, s>>>(m, S, W, alpha, Bx.lines, By.lines, ls, ql0, st, halt);
+    else if (values)
         k_lines_xy<false, true><<<dim3(nl0 + nl1), blk, 0, s>>>(m, S, W, alpha, Bx.lines, By.lines, ls, nullptr, nullptr, nl0,
                                                                 st, halt);
     else if (tape)
@@ -238,7 +290,11 @@ void launch_sweep_xy(const Mesh& m, const SchemeConsts& S, int flux, SweepWhat w
     if (T) T->end(KK_LINES, 1);
     const dim3 gf(nf0 + nf1, 2);
     if (T) T->begin(KK_FACES);
-    if (values)
+    if (quad_faces && values)
+        k_faces_quad<true><<<dim3(qf0 + qf1, 2), blk, 0, s>>>(m, S, W, alpha, Bx.lines, By.lines, ls, Bx.gp, By.gp, gs, qf0, st, halt);
+    else if (quad_faces)
+        k_faces_quad<false><<<dim3(qf0 + qf1, 2), blk, 0, s>>>(m, S, W, alpha, Bx.lines, By.lines, ls, Bx.gp, By.gp, gs, qf0, st, halt);
+    else if (values)
         k_faces_xy<false, true><<<gf, blk, 0, s>>>(m, S, W, alpha, Bx.lines, By.lines, ls, Bx.gp, By.gp, gs, nullptr,
                                                    nullptr, nf0, st, halt);
     else if (tape)
