@@ -163,6 +163,24 @@ DFK_HD void ghost_y_body(const Mesh& m, double* W, double* alpha, int i, int gr)
     if (alpha) alpha[d] = alpha[o];
 }
 
+// one ghost cell of the y pass on a whole mesh (no side BC_EXTERNAL), from the interior cell that the two passes
+// lead to: column i in [-G, nx+G), ghost row gr
+DFK_HD void ghost_corner_body(const Mesh& m, double* W, double* alpha, int i, int gr) {
+    if (i >= m.nx + G || gr >= 2 * G) return;
+    const int j = gr < G ? gr - G : m.ny + gr - G;
+    bool mx, my;
+    const int si = ghost_src(i, m.nx, m.bc[0], m.bc[1], mx), sj = ghost_src(j, m.ny, m.bc[2], m.bc[3], my);
+    const long long d = gid(m, i, j), o = gid(m, si, sj);
+    if (W) {
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            const double v = W[k * m.plane + o];
+            W[k * m.plane + d] = (k == 1 && mx) || (k == 2 && my) ? -v : v;
+        }
+    }
+    if (alpha) alpha[d] = alpha[o];
+}
+
 // One characteristic variable of a face line from its first differences f: both sides' value (relative to the cell
 // average) and slope, q = qL, qLn, qR, qRn, and their weights where they are used (L, R)
 template <bool VALUES>

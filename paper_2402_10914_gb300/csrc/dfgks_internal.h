@@ -132,8 +132,6 @@ struct AdjointArgs { const double* Lb; const double* dtLb; const double* dtLtb; 
 
 // ---- launchers (dfgks_kernels.cu) -----------------------------------------------------------
 void launch_fill_ghosts(const Mesh& m, double* W, double* alpha, const int* halt, cudaStream_t s, KernelTimer* T = nullptr);
-// one pass of the ghost fill: 0 = ghost columns of the interior rows, 1 = ghost rows of all columns
-void launch_ghost_pass(int dir, const Mesh& m, double* W, double* alpha, const int* halt, cudaStream_t s);
 void launch_cfl_min(const Mesh& m, const double* W, double gamma, DevState* st, cudaStream_t s, KernelTimer* T = nullptr);
 void launch_begin_step(DevState* st, double cfl, double dt_fixed, double t_end, double* dts, int idx, cudaStream_t s,
                        KernelTimer* T = nullptr);

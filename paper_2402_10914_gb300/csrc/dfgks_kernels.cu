@@ -14,36 +14,31 @@
 
 namespace dfk {
 
+constexpr int kSMs = 152;
+
 __device__ __forceinline__ bool halted(const int* halt) { return halt != nullptr && *(volatile const int*)halt != 0; }
 
 // ---------------------------------------------------------------------------------------------
 // Ghost fill: x pass over interior rows, then y pass over all columns (corners included)
 // ---------------------------------------------------------------------------------------------
-__global__ void k_ghost_x(Mesh m, double* W, double* alpha, const int* halt) {
+// Both passes in one launch: a ghost row's cells in the ghost columns are what pass 1 would copy of pass 0's, so
+// they are copied from the interior cell both lead to.  Blocks [0, nbx) take the ghost columns, the rest the rows.
+__global__ void k_ghosts(Mesh m, double* W, double* alpha, int nbx, const int* halt) {
     if (halted(halt)) return;
-    ghost_x_body(m, W, alpha, threadIdx.x, blockIdx.x * blockDim.y + threadIdx.y);
-}
-
-__global__ void k_ghost_y(Mesh m, double* W, double* alpha, const int* halt) {
-    if (halted(halt)) return;
-    ghost_y_body(m, W, alpha, blockIdx.x * blockDim.x + threadIdx.x - G, blockIdx.y);
-}
-
-void launch_ghost_pass(int dir, const Mesh& m, double* W, double* alpha, const int* halt, cudaStream_t s) {
-    if (dir == 0) {
-        dim3 bx(2 * G, 32), gx((m.ny + 31) / 32);
-        k_ghost_x<<<gx, bx, 0, s>>>(m, W, alpha, halt);
+    if ((int)blockIdx.x < nbx) {
+        const int idx = blockIdx.x * blockDim.x + threadIdx.x;
+        ghost_x_body(m, W, alpha, idx % (2 * G), idx / (2 * G));
     } else {
-        dim3 by(128), gy((m.nx + 2 * G + 127) / 128, 2 * G);
-        k_ghost_y<<<gy, by, 0, s>>>(m, W, alpha, halt);
+        const int idx = (blockIdx.x - nbx) * blockDim.x + threadIdx.x, w = m.nx + 2 * G;
+        ghost_corner_body(m, W, alpha, idx % w - G, idx / w);
     }
 }
 
 void launch_fill_ghosts(const Mesh& m, double* W, double* alpha, const int* halt, cudaStream_t s, KernelTimer* T) {
+    const int nbx = (2 * G * m.ny + 63) / 64, nby = (2 * G * (m.nx + 2 * G) + 63) / 64;
     if (T) T->begin(KK_OTHER);
-    launch_ghost_pass(0, m, W, alpha, halt, s);
-    launch_ghost_pass(1, m, W, alpha, halt, s);
-    if (T) T->end(KK_OTHER, 2);
+    k_ghosts<<<nbx + nby, 64, 0, s>>>(m, W, alpha, nbx, halt);
+    if (T) T->end(KK_OTHER, 1);
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -62,11 +57,12 @@ __global__ void k_cfl_min(Mesh m, const double* W, double gamma, DevState* st) {
 }
 
 void launch_cfl_min(const Mesh& m, const double* W, double gamma, DevState* st, cudaStream_t s, KernelTimer* T) {
-    int n = m.nx * m.ny;
-    int blocks = (n + 255) / 256;
-    if (blocks > 4 * 152) blocks = 4 * 152;
+    // one warp per block, as the sweeps: a block of eight keeps one SM's FP64 units busy while others idle
+    const int n = m.nx * m.ny;
+    int blocks = (n + 31) / 32;
+    if (blocks > 32 * kSMs) blocks = 32 * kSMs;
     if (T) T->begin(KK_OTHER);
-    k_cfl_min<<<blocks, 256, 0, s>>>(m, W, gamma, st);
+    k_cfl_min<<<blocks, 32, 0, s>>>(m, W, gamma, st);
     if (T) T->end(KK_OTHER, 1);
 }
 
@@ -255,8 +251,6 @@ __global__ void __launch_bounds__(128) k_flux_xy(Mesh m, SchemeConsts S, const d
                                        dir == 0 ? tape0 : tape1);
 }
 
-constexpr int kSMs = 152;
-
 void launch_sweep_xy(const Mesh& m, const SchemeConsts& S, int flux, SweepWhat what, const double* W,
                      const double* alpha, const double* dtp, const SweepBuffers& Bx, const SweepBuffers& By,
                      DevState* st, const int* halt, cudaStream_t s, KernelTimer* T) {
@@ -378,13 +372,15 @@ __global__ void __launch_bounds__(256) k_update(Mesh m, SchemeConsts S, UpdateAr
                                                 const double* dtp, DevState* st, const int* halt) {
     if (halted(halt)) return;
     const double dt = (MODE == UM_RESIDUAL || MODE == UM_ALPHA) ? 0.0 : *dtp;
-    update_body<MODE>(m, S, a, frx, fsx, fry, fsy, dt, st, blockIdx.x * blockDim.x + threadIdx.x,
-                      blockIdx.y * blockDim.y + threadIdx.y);
+    int i, j;
+    sweep_xy(m.nx, i, j);
+    update_body<MODE>(m, S, a, frx, fsx, fry, fsy, dt, st, i, j);
 }
 
 void launch_update(int mode, const Mesh& m, const SchemeConsts& S, const UpdateArgs& a, const SweepBuffers& B,
                    const double* dtp, DevState* st, const int* halt, cudaStream_t s, KernelTimer* T) {
-    dim3 blk(32, 8), grd((m.nx + 31) / 32, (m.ny + 7) / 8);
+    // one warp per block, as the sweeps: blocks of eight left most SMs of a small mesh idle
+    const dim3 blk(32), grd(((long long)m.nx * m.ny + 31) / 32);
     if (T) T->begin(KK_UPDATE);
     const double* fx = B.flux[0];
     const double* fy = B.flux[1];
