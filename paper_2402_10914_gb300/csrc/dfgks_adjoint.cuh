@@ -612,16 +612,18 @@ DFK_HD AOCoeffs ao_coeffs(const AORatios& q) {
     return c;
 }
 
-// adjoints of z_k for those of c_3, p_0, p_2
+// four times the adjoints of z_k for those of c_3, p_0, p_2 (the factors 2 of z = r^2 and of the squares in the
+// smoothness indicators, once)
 DFK_HD void ao_coeffs_rev(const AOCoeffs& c, const AORatios& q, Real c3b, Real p0b, Real p2b, const SchemeConsts& S, Real zb[4]) {
     const Real n = fma(c3b, c.c3, fma(p0b, c.p0, p2b * c.p2));          // minus the sum's adjoint times the sum
-    zb[0] = q.iv * fma(-S.d[0], n, p0b);
-    zb[1] = q.iv * (Real(-S.d[1]) * n);
-    zb[2] = q.iv * fma(-S.d[0], n, p2b);
-    zb[3] = q.iv * (fma(-S.d[3], n, c3b) - (p0b + p2b));
+    const Real iv = 4.0 * q.iv;
+    zb[0] = iv * fma(-S.d[0], n, p0b);
+    zb[1] = iv * (Real(-S.d[1]) * n);
+    zb[2] = iv * fma(-S.d[0], n, p2b);
+    zb[3] = iv * (fma(-S.d[3], n, c3b) - (p0b + p2b));
 }
 
-// the limiter weight 2 (1 + z_min) / ((1 + z_max) + (1 + z_min)): adds to the adjoints of the z it was made of
+// the limiter weight 2 (1 + z_min) / ((1 + z_max) + (1 + z_min)): adds to (four times) the adjoints of the z it was made of
 // (the first attaining k, as the ratios' order is that of 1/(beta_k + eps))
 DFK_HD void ao_limiter_rev(const AORatios& q, const AOCoeffs& c, Real wb, Real zb[4]) {
     int kmax = 0, kmin = 0;
@@ -632,7 +634,7 @@ DFK_HD void ao_limiter_rev(const AORatios& q, const AOCoeffs& c, Real wb, Real z
         if (nn_less(q.ie[k], lo)) { lo = q.ie[k]; kmin = k; rl = c.r[k]; }
     }
     const Real xh = fma(rh, rh, 1.0), xl = fma(rl, rl, 1.0), den = xh + xl;
-    const Real g = wb * Real::raw(2.0 / Real(den * den).v);
+    const Real g = wb * Real::raw(8.0 / Real(den * den).v);
     const Real hb = -(g * xl), lb = g * xh;
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
@@ -641,25 +643,25 @@ DFK_HD void ao_limiter_rev(const AORatios& q, const AOCoeffs& c, Real wb, Real z
     }
 }
 
-// adjoints zb of the z_k, and those of T, U so far, to the differences (b accumulates; b.a11 holds the
+// four times the adjoints of the z_k, and those of T, U so far, to the differences (b accumulates; b.a11 holds the
 // evaluation's share of the adjoint of a11 = fb + SGN s1/2)
 template <int SGN>
 DFK_HD void ao_ratios_rev(const AORatios& q, const AOCoeffs& c, const Real zb[4], Real fb, Real ff, Real s0, Real s1, Real s2,
                           Real a11, Real T, Real U, Real Tb, Real Ub, AODiffBar& b) {
-    // r_k = tau / e_k
+    // r_k = tau / e_k; eb: twice the adjoints of e_k
     Real eb[4], g[4];
 #pragma unroll
-    for (int k = 0; k < 4; ++k) { g[k] = (2.0 * zb[k]) * c.r[k] * q.ie[k]; eb[k] = -(g[k] * c.r[k]); }
-    const Real t3 = (1.0 / 3.0) * ((g[0] + g[1]) + (g[2] + g[3]));       // the adjoint of 3 tau
+    for (int k = 0; k < 4; ++k) { g[k] = zb[k] * c.r[k] * q.ie[k]; eb[k] = -(g[k] * c.r[k]); }
+    const Real t3 = (1.0 / 3.0) * ((g[0] + g[1]) + (g[2] + g[3]));       // twice the adjoint of 3 tau
     // 3 tau = sum_k |e_3 - e_k|, the sign that of e_3 - e_k: e_3 >= e_k where 1/e_k >= 1/e_3
+    int below = 0;
 #pragma unroll
     for (int k = 0; k < 3; ++k) {
-        const Real t = nn_less(q.ie[k], q.ie[3]) ? -t3 : t3;
-        eb[3] = eb[3] + t;
-        eb[k] = eb[k] - t;
+        const bool neg = nn_less(q.ie[k], q.ie[3]);
+        below += neg;
+        eb[k] = eb[k] - (neg ? -t3 : t3);
     }
-#pragma unroll
-    for (int k = 0; k < 4; ++k) eb[k] = 2.0 * eb[k];
+    eb[3] = fma(t3, below < 2 ? (below ? Real(1.0) : Real(3.0)) : (below == 2 ? Real(-1.0) : Real(-3.0)), eb[3]);
     const Real h = 0.5 * SGN;
     const Real a10b = eb[0] * fma(h, s0, fb), a12b = eb[2] * fma(-h, s2, ff);
     const Real m1b = eb[3] * fma(-1.0 / 12.0, T, a11), m2b = (13.0 / 12.0) * eb[3] * fma(-11.0 / 130.0, U, s1);
