@@ -801,7 +801,7 @@ DFK_HD void lf_flux_vjp(const GPState& L, const GPState& R, const SchemeConsts& 
     const FlowState sl = side_state(L.W, S), sr = side_state(R.W, S);
     const FlowGrad xl = point_grad(sl, L.Wn, S), yl = point_grad(sl, L.Wt, S), xr = point_grad(sr, R.Wn, S), yr = point_grad(sr, R.Wt, S);
     const FlowGrad tl = euler_time_grad(sl, xl, yl, S), tr = euler_time_grad(sr, xr, yr, S);
-    const Real al = fma(S.gamma * sl.th, S.r2g * sl.rs, fabs(sl.U)), ar = fma(S.gamma * sr.th, S.r2g * sr.rs, fabs(sr.U));
+    const Real al = fabs(sl.U) + sound_speed(sl, S), ar = fabs(sr.U) + sound_speed(sr, S);
     const bool left = !nn_less(al, ar);           // the left speed on a tie (both >= 0)
     const Real h = 0.5 * (left ? al : ar);
     Real Tl[4], Tr[4];

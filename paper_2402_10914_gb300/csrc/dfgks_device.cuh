@@ -1014,9 +1014,15 @@ DFK_HD void lf_time(const FlowState& s, const FlowGrad& t, const SchemeConsts& S
     T[3] = fma(0.5 * (S.K + 2.0), t.dp, fma(s.hq, t.r0, fma(s.U, t.r1, s.V * t.r2)));
 }
 
+// c = c^2 / c; zero at zero pressure, where 1/c is infinite
+DFK_HD Real sound_speed(const FlowState& s, const SchemeConsts& S) {
+    const Real c = (S.gamma * s.th) * (S.r2g * s.rs);
+    return (dbits(s.th.v) << 1) == 0 ? Real(0.0) : c;
+}
+
 // One side's flux (F) and, unless VALUES, W_t (T) and the flux's derivative along it (D), in gradient form as
 // the GKS flux: primitive gradients, the Euler equations' time derivative, back to conserved variables.
-// sl, sr: side_state of L.W and R.W, which the DF factor shares; c = c^2 / c needs no root
+// sl, sr: side_state of L.W and R.W, which the DF factor shares
 template <bool VALUES>
 DFK_HD Real lf_side(const FlowState& s, const GPState& P, const SchemeConsts& S, Real F[4], Real T[4], Real D[4]) {
     const Real m = Real::raw(P.W[1]), E = Real::raw(P.W[3]), Ep = E + s.p;
@@ -1032,7 +1038,7 @@ DFK_HD Real lf_side(const FlowState& s, const GPState& P, const SchemeConsts& S,
         D[2] = fma(s.V, T[1], s.U * t.r2);
         D[3] = fma(Ep * s.ir, t.r1, s.U * (T[3] + t.dp));
     }
-    return fma(S.gamma * s.th, S.r2g * s.rs, fabs(s.U));
+    return fabs(s.U) + sound_speed(s, S);
 }
 // VALUES: F alone (the Runge-Kutta stages use no time derivative); the slopes are not read
 template <bool VALUES>
