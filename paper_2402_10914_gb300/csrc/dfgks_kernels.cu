@@ -16,6 +16,30 @@ namespace dfk {
 
 constexpr int kSMs = 152;
 
+// The kernels of a step follow one another on a stream, each reading what the one before wrote.  They are launched
+// ahead of that one's end (programmatic dependent launch), so their launch and first instructions overlap its last
+// blocks, and wait in follow() until it has ended and its writes are visible before they touch memory; by then the
+// next launch may be set up in turn.  Nothing else differs from launches one after the other.  8 GKS steps of 100 x 4
+// 1.24 -> 1.04 ms, 20 L-F steps of 40 x 40 2.51 -> 1.96, 4 GKS steps of 400 x 400 12.74 -> 12.64.
+__device__ __forceinline__ void follow() {
+    cudaGridDependencySynchronize();
+    cudaTriggerProgrammaticLaunchCompletion();
+}
+
+template <class... P, class... A>
+static void launch(void (*kernel)(P...), dim3 grid, dim3 block, cudaStream_t s, A... args) {
+    cudaLaunchConfig_t c = {};
+    c.gridDim = grid;
+    c.blockDim = block;
+    c.stream = s;
+    cudaLaunchAttribute a[1];
+    a[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    a[0].val.programmaticStreamSerializationAllowed = 1;
+    c.attrs = a;
+    c.numAttrs = 1;
+    cudaLaunchKernelEx(&c, kernel, P(args)...);
+}
+
 __device__ __forceinline__ bool halted(const int* halt) { return halt != nullptr && *(volatile const int*)halt != 0; }
 
 // ---------------------------------------------------------------------------------------------
@@ -24,6 +48,7 @@ __device__ __forceinline__ bool halted(const int* halt) { return halt != nullptr
 // Both passes in one launch: a ghost row's cells in the ghost columns are what pass 1 would copy of pass 0's, so
 // they are copied from the interior cell both lead to.  Blocks [0, nbx) take the ghost columns, the rest the rows.
 __global__ void k_ghosts(Mesh m, double* W, double* alpha, int nbx, const int* halt) {
+    follow();
     if (halted(halt)) return;
     if ((int)blockIdx.x < nbx) {
         const int idx = blockIdx.x * blockDim.x + threadIdx.x;
@@ -37,7 +62,7 @@ __global__ void k_ghosts(Mesh m, double* W, double* alpha, int nbx, const int* h
 void launch_fill_ghosts(const Mesh& m, double* W, double* alpha, const int* halt, cudaStream_t s, KernelTimer* T) {
     const int nbx = (2 * G * m.ny + 63) / 64, nby = (2 * G * (m.nx + 2 * G) + 63) / 64;
     if (T) T->begin(KK_OTHER);
-    k_ghosts<<<nbx + nby, 64, 0, s>>>(m, W, alpha, nbx, halt);
+    launch(k_ghosts, nbx + nby, 64, s, m, W, alpha, nbx, halt);
     if (T) T->end(KK_OTHER, 1);
 }
 
@@ -45,6 +70,7 @@ void launch_fill_ghosts(const Mesh& m, double* W, double* alpha, const int* halt
 // CFL time step (Algorithm 1, first line): min over cells of min(dx/(|U|+c), dy/(|V|+c))
 // ---------------------------------------------------------------------------------------------
 __global__ void k_cfl_min(Mesh m, const double* W, double gamma, DevState* st) {
+    follow();
     if (st->halt) return;
     double best = DBL_MAX;
     const int n = m.nx * m.ny;
@@ -62,11 +88,12 @@ void launch_cfl_min(const Mesh& m, const double* W, double gamma, DevState* st, 
     int blocks = (n + 31) / 32;
     if (blocks > 32 * kSMs) blocks = 32 * kSMs;
     if (T) T->begin(KK_OTHER);
-    k_cfl_min<<<blocks, 32, 0, s>>>(m, W, gamma, st);
+    launch(k_cfl_min, blocks, 32, s, m, W, gamma, st);
     if (T) T->end(KK_OTHER, 1);
 }
 
 __global__ void k_begin_step(DevState* st, double cfl, double dt_fixed, double t_end, double* dts, int idx) {
+    follow();
     // consume and reset the CFL accumulator first, so a halted step leaves it clean
     const double dtmin = __longlong_as_double((long long)st->dtmin_bits);
     st->dtmin_bits = (unsigned long long)__double_as_longlong(DBL_MAX);
@@ -81,6 +108,7 @@ __global__ void k_begin_step(DevState* st, double cfl, double dt_fixed, double t
 }
 
 __global__ void k_end_step(DevState* st, double t_end) {
+    follow();
     if (st->halt) return;
     st->t = st->clipped ? t_end : st->t + st->dt;
     st->step += 1;
@@ -88,11 +116,11 @@ __global__ void k_end_step(DevState* st, double t_end) {
 
 void launch_begin_step(DevState* st, double cfl, double dt_fixed, double t_end, double* dts, int idx, cudaStream_t s,
                        KernelTimer* T) {
-    k_begin_step<<<1, 1, 0, s>>>(st, cfl, dt_fixed, t_end, dts, idx);
+    launch(k_begin_step, 1, 1, s, st, cfl, dt_fixed, t_end, dts, idx);
     if (T) T->end(KK_OTHER, 1);
 }
 void launch_end_step(DevState* st, double t_end, cudaStream_t s, KernelTimer* T) {
-    k_end_step<<<1, 1, 0, s>>>(st, t_end);
+    launch(k_end_step, 1, 1, s, st, t_end);
     if (T) T->end(KK_OTHER, 1);
 }
 
@@ -106,6 +134,7 @@ __global__ void __launch_bounds__(128, 3) k_lines(Mesh m, SchemeConsts S, const 
                                                const double* __restrict__ alpha, double* __restrict__ lines,
                                                long long ls, DevState* st, const int* halt,
                                                double* __restrict__ ltape = nullptr) {
+    follow();
     if (halted(halt)) return;
     int ax, ay;
     sweep_xy(lines_lx<DIR>(m), ax, ay);
@@ -118,6 +147,7 @@ __global__ void __launch_bounds__(128) k_faces(Mesh m, SchemeConsts S, const dou
                                                const double* __restrict__ alpha, const double* __restrict__ lines,
                                                long long ls, double* __restrict__ gp, long long gs,
                                                DevState* st, const int* halt, double* __restrict__ ftape = nullptr) {
+    follow();
     if (halted(halt)) return;
     int nfb, ax, ay;
     sweep_xy(faces_lx<DIR>(m), ax, ay);
@@ -130,6 +160,7 @@ __global__ void __launch_bounds__(128) k_flux(Mesh m, SchemeConsts S, const doub
                                               long long ls, const double* __restrict__ gp, long long gs,
                                               double* __restrict__ fr, long long fs, const double* dtp,
                                               const int* halt, double* __restrict__ tape = nullptr) {
+    follow();
     if (halted(halt)) return;
     int ax, ay;
     sweep_xy(faces_lx<DIR>(m), ax, ay);
@@ -154,6 +185,7 @@ __global__ void __launch_bounds__(128, 3) k_lines_xy(Mesh m, SchemeConsts S, con
                                                   const double* __restrict__ alpha, double* __restrict__ lines0,
                                                   double* __restrict__ lines1, long long ls, double* __restrict__ ltape0,
                                                   double* __restrict__ ltape1, int nb0, DevState* st, const int* halt) {
+    follow();
     if (halted(halt)) return;
     int ax, ay, ndf;
     if ((int)blockIdx.x < nb0) {
@@ -172,6 +204,7 @@ __global__ void __launch_bounds__(128) k_faces_xy(Mesh m, SchemeConsts S, const 
                                                const double* __restrict__ lines1, long long ls, double* __restrict__ gp0,
                                                double* __restrict__ gp1, long long gs, double* __restrict__ ftape0,
                                                double* __restrict__ ftape1, int nb0, DevState* st, const int* halt) {
+    follow();
     if (halted(halt)) return;
     int nfb, ax, ay, ndf;
     if ((int)blockIdx.x < nb0) {
@@ -195,6 +228,7 @@ template <bool VALUES>
 __global__ void __launch_bounds__(32) k_lines_quad(Mesh m, SchemeConsts S, const double* __restrict__ W,
                                                    const double* __restrict__ alpha, double* __restrict__ lines0,
                                                    double* __restrict__ lines1, long long ls, int nb0, DevState* st, const int* halt) {
+    follow();
     if (halted(halt)) return;
     int ax, ay, ndf;
     if ((int)blockIdx.x < nb0) {
@@ -212,6 +246,7 @@ __global__ void __launch_bounds__(32) k_faces_quad(Mesh m, SchemeConsts S, const
                                                    const double* __restrict__ alpha, const double* __restrict__ lines0,
                                                    const double* __restrict__ lines1, long long ls, double* __restrict__ gp0,
                                                    double* __restrict__ gp1, long long gs, int nb0, DevState* st, const int* halt) {
+    follow();
     if (halted(halt)) return;
     int nfb, ax, ay, ndf;
     if ((int)blockIdx.x < nb0) {
@@ -231,6 +266,7 @@ __global__ void __launch_bounds__(128) k_flux_xy(Mesh m, SchemeConsts S, const d
                                               long long gs, double* __restrict__ fr0, long long fs0,
                                               double* __restrict__ fr1, long long fs1, double* __restrict__ tape0,
                                               double* __restrict__ tape1, const double* dtp, int nb0, const int* halt) {
+    follow();
     if (halted(halt)) return;
     const double dt = ALPHA_ONLY ? 0.0 : *dtp;
     // the direction selects the records and the index map; the flux arithmetic is inlined once
@@ -269,33 +305,33 @@ void launch_sweep_xy(const Mesh& m, const SchemeConsts& S, int flux, SweepWhat w
     const int ql0 = (int)sweep_blocks(lines_lx<0>(m), lines_ly<0>(m), kSweepThreads / 4), ql1 = (int)sweep_blocks(lines_lx<1>(m), lines_ly<1>(m), kSweepThreads / 4);
     const int qf0 = (int)sweep_blocks(faces_lx<0>(m), faces_ly<0>(m), kSweepThreads / 4), qf1 = (int)sweep_blocks(faces_lx<1>(m), faces_ly<1>(m), kSweepThreads / 4);
     if (quad_lines && values)
-        k_lines_quad<true><<<ql0 + ql1, blk, 0, s>>>(m, S, W, alpha, Bx.lines, By.lines, ls, ql0, st, halt);
+        launch(k_lines_quad<true>, ql0 + ql1, blk, s, m, S, W, alpha, Bx.lines, By.lines, ls, ql0, st, halt);
     else if (quad_lines)
-        k_lines_quad<false><<<ql0 + ql1, blk, 0, s>>>(m, S, W, alpha, Bx.lines, By.lines, ls, ql0, st, halt);
+        launch(k_lines_quad<false>, ql0 + ql1, blk, s, m, S, W, alpha, Bx.lines, By.lines, ls, ql0, st, halt);
     else if (values)
-        k_lines_xy<false, true><<<dim3(nl0 + nl1), blk, 0, s>>>(m, S, W, alpha, Bx.lines, By.lines, ls, nullptr, nullptr, nl0,
+        launch(k_lines_xy<false, true>, dim3(nl0 + nl1), blk, s, m, S, W, alpha, Bx.lines, By.lines, ls, nullptr, nullptr, nl0,
                                                                 st, halt);
     else if (tape)
-        k_lines_xy<true><<<dim3(nl0 + nl1), blk, 0, s>>>(m, S, W, alpha, Bx.lines, By.lines, ls, Bx.ltape, By.ltape, nl0,
+        launch(k_lines_xy<true>, dim3(nl0 + nl1), blk, s, m, S, W, alpha, Bx.lines, By.lines, ls, Bx.ltape, By.ltape, nl0,
                                                          st, halt);
     else
-        k_lines_xy<false><<<dim3(nl0 + nl1), blk, 0, s>>>(m, S, W, alpha, Bx.lines, By.lines, ls, nullptr, nullptr, nl0,
+        launch(k_lines_xy<false>, dim3(nl0 + nl1), blk, s, m, S, W, alpha, Bx.lines, By.lines, ls, nullptr, nullptr, nl0,
                                                           st, halt);
     if (T) T->end(KK_LINES, 1);
     const dim3 gf(nf0 + nf1, 2);
     if (T) T->begin(KK_FACES);
     if (quad_faces && values)
-        k_faces_quad<true><<<dim3(qf0 + qf1, 2), blk, 0, s>>>(m, S, W, alpha, Bx.lines, By.lines, ls, Bx.gp, By.gp, gs, qf0, st, halt);
+        launch(k_faces_quad<true>, dim3(qf0 + qf1, 2), blk, s, m, S, W, alpha, Bx.lines, By.lines, ls, Bx.gp, By.gp, gs, qf0, st, halt);
     else if (quad_faces)
-        k_faces_quad<false><<<dim3(qf0 + qf1, 2), blk, 0, s>>>(m, S, W, alpha, Bx.lines, By.lines, ls, Bx.gp, By.gp, gs, qf0, st, halt);
+        launch(k_faces_quad<false>, dim3(qf0 + qf1, 2), blk, s, m, S, W, alpha, Bx.lines, By.lines, ls, Bx.gp, By.gp, gs, qf0, st, halt);
     else if (values)
-        k_faces_xy<false, true><<<gf, blk, 0, s>>>(m, S, W, alpha, Bx.lines, By.lines, ls, Bx.gp, By.gp, gs, nullptr,
+        launch(k_faces_xy<false, true>, gf, blk, s, m, S, W, alpha, Bx.lines, By.lines, ls, Bx.gp, By.gp, gs, nullptr,
                                                    nullptr, nf0, st, halt);
     else if (tape)
-        k_faces_xy<true><<<gf, blk, 0, s>>>(m, S, W, alpha, Bx.lines, By.lines, ls, Bx.gp, By.gp, gs, Bx.ftape,
+        launch(k_faces_xy<true>, gf, blk, s, m, S, W, alpha, Bx.lines, By.lines, ls, Bx.gp, By.gp, gs, Bx.ftape,
                                             By.ftape, nf0, st, halt);
     else
-        k_faces_xy<false><<<gf, blk, 0, s>>>(m, S, W, alpha, Bx.lines, By.lines, ls, Bx.gp, By.gp, gs, nullptr,
+        launch(k_faces_xy<false>, gf, blk, s, m, S, W, alpha, Bx.lines, By.lines, ls, Bx.gp, By.gp, gs, nullptr,
                                              nullptr, nf0, st, halt);
     if (T) T->end(KK_FACES, 1);
     double* f0 = Bx.flux[0];
@@ -303,19 +339,19 @@ void launch_sweep_xy(const Mesh& m, const SchemeConsts& S, int flux, SweepWhat w
     const long long fs0 = Bx.flux_stride[0], fs1 = By.flux_stride[1];
     if (T) T->begin(KK_FLUX);
     if (alpha_only)
-        k_flux_xy<1, true><<<gf, blk, 0, s>>>(m, S, Bx.lines, By.lines, ls, Bx.gp, By.gp, gs, f0, fs0, f1, fs1,
+        launch(k_flux_xy<1, true>, gf, blk, s, m, S, Bx.lines, By.lines, ls, Bx.gp, By.gp, gs, f0, fs0, f1, fs1,
                                                nullptr, nullptr, dtp, nf0, halt);
     else if (values)
-        k_flux_xy<1, false, false, true><<<gf, blk, 0, s>>>(m, S, Bx.lines, By.lines, ls, Bx.gp, By.gp, gs, f0, fs0, f1, fs1,
+        launch(k_flux_xy<1, false, false, true>, gf, blk, s, m, S, Bx.lines, By.lines, ls, Bx.gp, By.gp, gs, f0, fs0, f1, fs1,
                                                             nullptr, nullptr, dtp, nf0, halt);
     else if (flux == 0 && Bx.tape[0])        // GKS forward that also tapes its intermediates for a reverse sweep
-        k_flux_xy<0, false, true><<<gf, blk, 0, s>>>(m, S, Bx.lines, By.lines, ls, Bx.gp, By.gp, gs, f0, fs0, f1, fs1,
+        launch(k_flux_xy<0, false, true>, gf, blk, s, m, S, Bx.lines, By.lines, ls, Bx.gp, By.gp, gs, f0, fs0, f1, fs1,
                                                      Bx.tape[0], By.tape[1], dtp, nf0, halt);
     else if (flux == 0)
-        k_flux_xy<0, false><<<gf, blk, 0, s>>>(m, S, Bx.lines, By.lines, ls, Bx.gp, By.gp, gs, f0, fs0, f1, fs1,
+        launch(k_flux_xy<0, false>, gf, blk, s, m, S, Bx.lines, By.lines, ls, Bx.gp, By.gp, gs, f0, fs0, f1, fs1,
                                                 nullptr, nullptr, dtp, nf0, halt);
     else
-        k_flux_xy<1, false><<<gf, blk, 0, s>>>(m, S, Bx.lines, By.lines, ls, Bx.gp, By.gp, gs, f0, fs0, f1, fs1,
+        launch(k_flux_xy<1, false>, gf, blk, s, m, S, Bx.lines, By.lines, ls, Bx.gp, By.gp, gs, f0, fs0, f1, fs1,
                                                 nullptr, nullptr, dtp, nf0, halt);
     if (T) T->end(KK_FLUX, 1);
 }
@@ -329,28 +365,28 @@ static void sweep_dir(const Mesh& m, const SchemeConsts& S, int flux, bool alpha
     const dim3 blk(kSweepThreads);
     const dim3 gl(sweep_blocks(lines_lx<DIR>(m), lines_ly<DIR>(m)));
     if (T) T->begin(KK_LINES);
-    if (alpha_only) k_lines<DIR, false, true><<<gl, blk, 0, s>>>(m, S, W, alpha, B.lines, B.line_stride, st, halt);
-    else if (B.ltape) k_lines<DIR, true><<<gl, blk, 0, s>>>(m, S, W, alpha, B.lines, B.line_stride, st, halt, B.ltape);
-    else k_lines<DIR><<<gl, blk, 0, s>>>(m, S, W, alpha, B.lines, B.line_stride, st, halt);
+    if (alpha_only) launch(k_lines<DIR, false, true>, gl, blk, s, m, S, W, alpha, B.lines, B.line_stride, st, halt, (double*)nullptr);
+    else if (B.ltape) launch(k_lines<DIR, true>, gl, blk, s, m, S, W, alpha, B.lines, B.line_stride, st, halt, B.ltape);
+    else launch(k_lines<DIR>, gl, blk, s, m, S, W, alpha, B.lines, B.line_stride, st, halt, (double*)nullptr);
     if (T) T->end(KK_LINES, 1);
     const dim3 gf(sweep_blocks(faces_lx<DIR>(m), faces_ly<DIR>(m)), 2);
     if (T) T->begin(KK_FACES);
     if (alpha_only)
-        k_faces<DIR, false, true><<<gf, blk, 0, s>>>(m, S, W, alpha, B.lines, B.line_stride, B.gp, B.gp_stride, st, halt);
+        launch(k_faces<DIR, false, true>, gf, blk, s, m, S, W, alpha, B.lines, B.line_stride, B.gp, B.gp_stride, st, halt, (double*)nullptr);
     else if (B.ftape)
-        k_faces<DIR, true><<<gf, blk, 0, s>>>(m, S, W, alpha, B.lines, B.line_stride, B.gp, B.gp_stride, st, halt, B.ftape);
+        launch(k_faces<DIR, true>, gf, blk, s, m, S, W, alpha, B.lines, B.line_stride, B.gp, B.gp_stride, st, halt, B.ftape);
     else
-        k_faces<DIR><<<gf, blk, 0, s>>>(m, S, W, alpha, B.lines, B.line_stride, B.gp, B.gp_stride, st, halt);
+        launch(k_faces<DIR>, gf, blk, s, m, S, W, alpha, B.lines, B.line_stride, B.gp, B.gp_stride, st, halt, (double*)nullptr);
     if (T) T->end(KK_FACES, 1);
     double* fr = B.flux[DIR];
     long long fs = B.flux_stride[DIR];
     if (T) T->begin(KK_FLUX);
-    if (alpha_only) k_flux<DIR, 1, true><<<gf, blk, 0, s>>>(m, S, B.lines, B.line_stride, B.gp, B.gp_stride, fr, fs, dtp, halt);
+    if (alpha_only) launch(k_flux<DIR, 1, true>, gf, blk, s, m, S, B.lines, B.line_stride, B.gp, B.gp_stride, fr, fs, dtp, halt, (double*)nullptr);
     else if (flux == 0 && B.tape[DIR])      // GKS forward that also tapes its intermediates for a reverse sweep
-        k_flux<DIR, 0, false, true><<<gf, blk, 0, s>>>(m, S, B.lines, B.line_stride, B.gp, B.gp_stride, fr, fs, dtp, halt,
+        launch(k_flux<DIR, 0, false, true>, gf, blk, s, m, S, B.lines, B.line_stride, B.gp, B.gp_stride, fr, fs, dtp, halt,
                                                        B.tape[DIR]);
-    else if (flux == 0) k_flux<DIR, 0, false><<<gf, blk, 0, s>>>(m, S, B.lines, B.line_stride, B.gp, B.gp_stride, fr, fs, dtp, halt);
-    else k_flux<DIR, 1, false><<<gf, blk, 0, s>>>(m, S, B.lines, B.line_stride, B.gp, B.gp_stride, fr, fs, dtp, halt);
+    else if (flux == 0) launch(k_flux<DIR, 0, false>, gf, blk, s, m, S, B.lines, B.line_stride, B.gp, B.gp_stride, fr, fs, dtp, halt, (double*)nullptr);
+    else launch(k_flux<DIR, 1, false>, gf, blk, s, m, S, B.lines, B.line_stride, B.gp, B.gp_stride, fr, fs, dtp, halt, (double*)nullptr);
     if (T) T->end(KK_FLUX, 1);
 }
 
@@ -370,6 +406,7 @@ __global__ void __launch_bounds__(256) k_update(Mesh m, SchemeConsts S, UpdateAr
                                                 const double* __restrict__ frx, long long fsx,
                                                 const double* __restrict__ fry, long long fsy,
                                                 const double* dtp, DevState* st, const int* halt) {
+    follow();
     if (halted(halt)) return;
     const double dt = (MODE == UM_RESIDUAL || MODE == UM_ALPHA) ? 0.0 : *dtp;
     int i, j;
@@ -386,13 +423,13 @@ void launch_update(int mode, const Mesh& m, const SchemeConsts& S, const UpdateA
     const double* fy = B.flux[1];
     long long sx = B.flux_stride[0], sy = B.flux_stride[1];
     switch (mode) {
-        case UM_RESIDUAL: k_update<UM_RESIDUAL><<<grd, blk, 0, s>>>(m, S, a, fx, sx, fy, sy, dtp, st, halt); break;
-        case UM_S2O4_1: k_update<UM_S2O4_1><<<grd, blk, 0, s>>>(m, S, a, fx, sx, fy, sy, dtp, st, halt); break;
-        case UM_S2O4_2: k_update<UM_S2O4_2><<<grd, blk, 0, s>>>(m, S, a, fx, sx, fy, sy, dtp, st, halt); break;
-        case UM_RK_1: k_update<UM_RK_1><<<grd, blk, 0, s>>>(m, S, a, fx, sx, fy, sy, dtp, st, halt); break;
-        case UM_RK_2: k_update<UM_RK_2><<<grd, blk, 0, s>>>(m, S, a, fx, sx, fy, sy, dtp, st, halt); break;
-        case UM_RK_3: k_update<UM_RK_3><<<grd, blk, 0, s>>>(m, S, a, fx, sx, fy, sy, dtp, st, halt); break;
-        default: k_update<UM_ALPHA><<<grd, blk, 0, s>>>(m, S, a, fx, sx, fy, sy, dtp, st, halt); break;
+        case UM_RESIDUAL: launch(k_update<UM_RESIDUAL>, grd, blk, s, m, S, a, fx, sx, fy, sy, dtp, st, halt); break;
+        case UM_S2O4_1: launch(k_update<UM_S2O4_1>, grd, blk, s, m, S, a, fx, sx, fy, sy, dtp, st, halt); break;
+        case UM_S2O4_2: launch(k_update<UM_S2O4_2>, grd, blk, s, m, S, a, fx, sx, fy, sy, dtp, st, halt); break;
+        case UM_RK_1: launch(k_update<UM_RK_1>, grd, blk, s, m, S, a, fx, sx, fy, sy, dtp, st, halt); break;
+        case UM_RK_2: launch(k_update<UM_RK_2>, grd, blk, s, m, S, a, fx, sx, fy, sy, dtp, st, halt); break;
+        case UM_RK_3: launch(k_update<UM_RK_3>, grd, blk, s, m, S, a, fx, sx, fy, sy, dtp, st, halt); break;
+        default: launch(k_update<UM_ALPHA>, grd, blk, s, m, S, a, fx, sx, fy, sy, dtp, st, halt); break;
     }
     if (T) T->end(KK_UPDATE, 1);
 }
