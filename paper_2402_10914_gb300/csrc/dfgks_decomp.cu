@@ -39,9 +39,8 @@ struct HaloBlock {
 };
 
 // One pass of the ghost fill of all blocks (grid x: block): 0 the ghost columns of the interior rows, 1 the ghost
-// rows of all columns.  A pass reads no cell that it writes, so physical sides and copies go together.  One launch
-// instead of a launch and up to ten strided copies per block, each of which took longer than this kernel:
-// 3 x 2 periodic blocks of 100 x 100, see Helpers below.
+// rows of all columns.  A pass reads no cell that it writes, so physical sides and copies go together: one launch
+// instead of a launch and up to ten strided copies per block (measured with the blocks' streams, see Helpers below).
 __global__ void k_halo(const HaloBlock* __restrict__ H, int pass, int field, int alpha, const int* halt) {
     if (*(volatile const int*)halt != 0) return;
     const HaloBlock& b = H[blockIdx.x];
