@@ -19,8 +19,11 @@ constexpr int kSMs = 152;
 // The kernels of a step follow one another on a stream, each reading what the one before wrote.  They are launched
 // ahead of that one's end (programmatic dependent launch), so their launch and first instructions overlap its last
 // blocks, and wait in follow() until it has ended and its writes are visible before they touch memory; by then the
-// next launch may be set up in turn.  Nothing else differs from launches one after the other.  8 GKS steps of 100 x 4
-// 1.24 -> 1.04 ms, 20 L-F steps of 40 x 40 2.51 -> 1.96, 4 GKS steps of 400 x 400 12.74 -> 12.64.
+// next launch may be set up in turn.  Their inputs are plain pointers to const, not __restrict__ ones: those may be
+// read by non-coherent loads, which are defined only for memory that nothing writes from a kernel's start to its
+// end, and the kernel before still writes after the start.  Nothing else differs from launches one after the other.
+// 8 GKS steps of 100 x 4 1.24 -> 1.04 ms, 20 L-F steps of 40 x 40 2.51 -> 1.96, 4 GKS steps of 400 x 400
+// 12.74 -> 12.64.
 __device__ __forceinline__ void follow() {
     cudaGridDependencySynchronize();
     cudaTriggerProgrammaticLaunchCompletion();
@@ -130,8 +133,8 @@ void launch_end_step(DevState* st, double t_end, cudaStream_t s, KernelTimer* T)
 // tangential offset b maps to global column t - b.  Face f lies between normal cells f-1, f.
 // ---------------------------------------------------------------------------------------------
 template <int DIR, bool TAPE = false, bool VALUES = false>
-__global__ void __launch_bounds__(128, 3) k_lines(Mesh m, SchemeConsts S, const double* __restrict__ W,
-                                               const double* __restrict__ alpha, double* __restrict__ lines,
+__global__ void __launch_bounds__(128, 3) k_lines(Mesh m, SchemeConsts S, const double* W,
+                                               const double* alpha, double* __restrict__ lines,
                                                long long ls, DevState* st, const int* halt,
                                                double* __restrict__ ltape = nullptr) {
     follow();
@@ -143,8 +146,8 @@ __global__ void __launch_bounds__(128, 3) k_lines(Mesh m, SchemeConsts S, const 
 }
 
 template <int DIR, bool TAPE = false, bool VALUES = false>
-__global__ void __launch_bounds__(128) k_faces(Mesh m, SchemeConsts S, const double* __restrict__ W,
-                                               const double* __restrict__ alpha, const double* __restrict__ lines,
+__global__ void __launch_bounds__(128) k_faces(Mesh m, SchemeConsts S, const double* W,
+                                               const double* alpha, const double* lines,
                                                long long ls, double* __restrict__ gp, long long gs,
                                                DevState* st, const int* halt, double* __restrict__ ftape = nullptr) {
     follow();
@@ -156,8 +159,8 @@ __global__ void __launch_bounds__(128) k_faces(Mesh m, SchemeConsts S, const dou
 }
 
 template <int DIR, int FLUX, bool ALPHA_ONLY, bool TAPE = false>
-__global__ void __launch_bounds__(128) k_flux(Mesh m, SchemeConsts S, const double* __restrict__ lines,
-                                              long long ls, const double* __restrict__ gp, long long gs,
+__global__ void __launch_bounds__(128) k_flux(Mesh m, SchemeConsts S, const double* lines,
+                                              long long ls, const double* gp, long long gs,
                                               double* __restrict__ fr, long long fs, const double* dtp,
                                               const int* halt, double* __restrict__ tape = nullptr) {
     follow();
@@ -181,8 +184,8 @@ __device__ __forceinline__ void sweep_at(int b, int lx, int& ax, int& ay) {
 }
 
 template <bool TAPE, bool VALUES = false>
-__global__ void __launch_bounds__(128, 3) k_lines_xy(Mesh m, SchemeConsts S, const double* __restrict__ W,
-                                                  const double* __restrict__ alpha, double* __restrict__ lines0,
+__global__ void __launch_bounds__(128, 3) k_lines_xy(Mesh m, SchemeConsts S, const double* W,
+                                                  const double* alpha, double* __restrict__ lines0,
                                                   double* __restrict__ lines1, long long ls, double* __restrict__ ltape0,
                                                   double* __restrict__ ltape1, int nb0, DevState* st, const int* halt) {
     follow();
@@ -199,9 +202,9 @@ __global__ void __launch_bounds__(128, 3) k_lines_xy(Mesh m, SchemeConsts S, con
 }
 
 template <bool TAPE, bool VALUES = false>
-__global__ void __launch_bounds__(128) k_faces_xy(Mesh m, SchemeConsts S, const double* __restrict__ W,
-                                               const double* __restrict__ alpha, const double* __restrict__ lines0,
-                                               const double* __restrict__ lines1, long long ls, double* __restrict__ gp0,
+__global__ void __launch_bounds__(128) k_faces_xy(Mesh m, SchemeConsts S, const double* W,
+                                               const double* alpha, const double* lines0,
+                                               const double* lines1, long long ls, double* __restrict__ gp0,
                                                double* __restrict__ gp1, long long gs, double* __restrict__ ftape0,
                                                double* __restrict__ ftape1, int nb0, DevState* st, const int* halt) {
     follow();
@@ -225,8 +228,8 @@ __device__ __forceinline__ void quad_at(int b, int lx, int& ax, int& ay) {
 }
 
 template <bool VALUES>
-__global__ void __launch_bounds__(32) k_lines_quad(Mesh m, SchemeConsts S, const double* __restrict__ W,
-                                                   const double* __restrict__ alpha, double* __restrict__ lines0,
+__global__ void __launch_bounds__(32) k_lines_quad(Mesh m, SchemeConsts S, const double* W,
+                                                   const double* alpha, double* __restrict__ lines0,
                                                    double* __restrict__ lines1, long long ls, int nb0, DevState* st, const int* halt) {
     follow();
     if (halted(halt)) return;
@@ -242,9 +245,9 @@ __global__ void __launch_bounds__(32) k_lines_quad(Mesh m, SchemeConsts S, const
 }
 
 template <bool VALUES>
-__global__ void __launch_bounds__(32) k_faces_quad(Mesh m, SchemeConsts S, const double* __restrict__ W,
-                                                   const double* __restrict__ alpha, const double* __restrict__ lines0,
-                                                   const double* __restrict__ lines1, long long ls, double* __restrict__ gp0,
+__global__ void __launch_bounds__(32) k_faces_quad(Mesh m, SchemeConsts S, const double* W,
+                                                   const double* alpha, const double* lines0,
+                                                   const double* lines1, long long ls, double* __restrict__ gp0,
                                                    double* __restrict__ gp1, long long gs, int nb0, DevState* st, const int* halt) {
     follow();
     if (halted(halt)) return;
@@ -260,9 +263,9 @@ __global__ void __launch_bounds__(32) k_faces_quad(Mesh m, SchemeConsts S, const
 }
 
 template <int FLUX, bool ALPHA_ONLY, bool TAPE = false, bool VALUES = false>
-__global__ void __launch_bounds__(128) k_flux_xy(Mesh m, SchemeConsts S, const double* __restrict__ lines0,
-                                              const double* __restrict__ lines1, long long ls,
-                                              const double* __restrict__ gp0, const double* __restrict__ gp1,
+__global__ void __launch_bounds__(128) k_flux_xy(Mesh m, SchemeConsts S, const double* lines0,
+                                              const double* lines1, long long ls,
+                                              const double* gp0, const double* gp1,
                                               long long gs, double* __restrict__ fr0, long long fs0,
                                               double* __restrict__ fr1, long long fs1, double* __restrict__ tape0,
                                               double* __restrict__ tape1, const double* dtp, int nb0, const int* halt) {
@@ -403,8 +406,8 @@ void launch_sweep(int dir, const Mesh& m, const SchemeConsts& S, int flux, bool 
 // ---------------------------------------------------------------------------------------------
 template <int MODE>
 __global__ void __launch_bounds__(256) k_update(Mesh m, SchemeConsts S, UpdateArgs a,
-                                                const double* __restrict__ frx, long long fsx,
-                                                const double* __restrict__ fry, long long fsy,
+                                                const double* frx, long long fsx,
+                                                const double* fry, long long fsy,
                                                 const double* dtp, DevState* st, const int* halt) {
     follow();
     if (halted(halt)) return;
