@@ -234,7 +234,10 @@ static cudaError_t create_halo(dfgks_decomp* d) {
     d->halo_tiles[0] = (2 * G * rows + 127) / 128;
     d->halo_tiles[1] = (2 * G * cols + 127) / 128;
     cudaError_t e = dalloc(d, &d->halo, (long long)H.size());
-    if (e == cudaSuccess) e = cudaMemcpy(d->halo, H.data(), H.size() * sizeof(HaloBlock), cudaMemcpyHostToDevice);
+    // on the handle's stream, which k_halo runs on: a plain cudaMemcpy goes to the legacy stream, may return before the
+    // data has reached the device, and a non-blocking stream does not wait for it
+    if (e == cudaSuccess) e = cudaMemcpyAsync(d->halo, H.data(), H.size() * sizeof(HaloBlock), cudaMemcpyHostToDevice, d->stream);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(d->stream);          // H ends here
     const size_t n = H.size() < 2 ? 0 : (H.size() < 8 ? H.size() : 8);
     if (e == cudaSuccess && n) e = cudaEventCreateWithFlags(&d->ready, cudaEventDisableTiming);
     for (size_t q = 0; q < n && e == cudaSuccess; ++q) {
