@@ -775,7 +775,8 @@ DFK_HD void lf_side_reverse(const FlowState& s, const GPState& P, const FlowGrad
     sb.V = fma(T[1], Db[2], fma(t.r0, Tb[2], fma(t.r2, T3b, m * Fb[2])));
     sb.hq = t.r0 * T3b;
     sb.p = Fb[1] + Epb;
-    sb.U = sb.U + (dbits(s.U.v) >= 0 ? ab : -ab);
+    // |U|'s slope: +1 at both zeros (the pattern of -0 is the smallest of the negative ones)
+    sb.U = sb.U + ((unsigned long long)dbits(s.U.v) <= 1ULL << 63 ? ab : -ab);
     sb.th = (0.5 * S.gamma) * (S.r2g * s.rs) * ab;                      // dc/dtheta = gamma / (2 c)
     euler_time_grad_rev(s, x, y, t, tb, S, xb, yb, sb);
     Real d[4];
