@@ -39,11 +39,13 @@ struct dfgks {
     int fail_i, fail_j;
     KernelTimer* timer;    // per-kernel-class event timing and launch counts
     // reverse sweep: face-line and Gauss-point record adjoints (the second set, for both directions at once,
-    // optional), ghosted cell adjoints, and the tapes of one direction (or of both, with the second set; optional)
+    // optional), ghosted cell adjoints, and the tapes of one direction (or of both, with the second set; optional):
+    // the reconstructions' ratios and the GKS flux's intermediates
     double* adj_lines[2];
     double* adj_gp[2];
     double* adj_Wg;
-    double* adj_tape;
+    double* adj_ratios;
+    double* adj_gks;
     // checkpointed forward pass kept for dfgks_adjoint_checkpointed
     double* ck_W;          // dense [nseg][4][ny][nx]: W at steps 0, k, 2k, ...
     double* ck_A;          // dense [nseg][ny][nx]: alpha at the same steps
@@ -125,7 +127,7 @@ static bool config_ok(const dfgks_config* c) {
 static void free_all(dfgks* h) {
     double* ptrs[] = {h->W[0], h->W[1], h->A[0], h->A[1], h->Ws, h->As, h->acc, h->B.lines, h->B.gp,
                       h->B.flux[0], h->B.flux[1], h->By.lines, h->By.gp, h->dt_scratch, h->dts, h->adj_lines[0],
-                      h->adj_lines[1], h->adj_gp[0], h->adj_gp[1], h->adj_Wg, h->adj_tape};
+                      h->adj_lines[1], h->adj_gp[0], h->adj_gp[1], h->adj_Wg, h->adj_ratios, h->adj_gks};
     for (double* p : ptrs) if (p) cudaFree(p);
     if (h->seg_arena) cudaFree(h->seg_arena);
     if (h->ck_W) cudaFree(h->ck_W);
@@ -482,57 +484,96 @@ extern "C" dfgks_status dfgks_face_records(dfgks* h, const double* W, const doub
     return DFGKS_OK;
 }
 
-// one direction's tapes: reconstruction ratios of face lines and face sides, GKS flux
-static long long tape_doubles(const dfgks* h) {
-    const SweepBuffers& B = h->B;
-    return (long long)TG_COUNT * (B.flux_stride[0] > B.flux_stride[1] ? B.flux_stride[0] : B.flux_stride[1])
-         + (long long)8 * RT_COUNT * B.line_stride + (long long)4 * RT_COUNT * B.gp_stride;
+// one direction's tapes: reconstruction ratios of face lines and face sides, and the GKS flux's intermediates
+static long long ratio_doubles(const dfgks* h) {
+    return (long long)8 * RT_COUNT * h->B.line_stride + (long long)4 * RT_COUNT * h->B.gp_stride;
+}
+static long long gks_doubles(const dfgks* h) {
+    const long long* s = h->B.flux_stride;
+    return (long long)TG_COUNT * (s[0] > s[1] ? s[0] : s[1]);
 }
 
-static dfgks_status ensure_adjoint_buffers(dfgks* h) {
-    if (h->adj_Wg) return DFGKS_OK;
+static void dfree(dfgks* h, double** p, long long n) {
+    if (!*p) return;
+    cudaFree(*p);
+    h->bytes -= (unsigned long long)n * sizeof(double);
+    *p = nullptr;
+}
+
+// The reverse sweep's buffers; tapes: for a reverse that evaluates its forward first, which then does not evaluate
+// fluxes and weights a second time (a reverse from kept records reads none of these tapes).
+// With a second set of adjoints both directions are reversed at once: the launches are twice as large, so small
+// meshes fill more of the chip and the last round of blocks weighs less.  Second set and tapes are left out where
+// they would take more than a quarter of the free memory.  They are kept for the calls that follow, and what is
+// missing is asked for again by the next call that would use it, unless that call is being captured.
+static dfgks_status ensure_adjoint_buffers(dfgks* h, bool tapes, int flux) {
     const SweepBuffers& B = h->B;
     const long long nl = (long long)LR_COUNT * B.line_stride, ng = (long long)GP_COUNT * B.gp_stride;
     if (!h->adj_lines[0]) CK(dalloc(h, &h->adj_lines[0], nl));
     if (!h->adj_gp[0]) CK(dalloc(h, &h->adj_gp[0], ng));
-    CK(dalloc(h, &h->adj_Wg, 4 * h->mesh.plane));
-    // With a second set both directions are reversed at once: the launches are twice as large, so small meshes
-    // fill more of the chip and the last round of blocks weighs less (67 x 83 GKS stage with its forward 483 ->
-    // 302 us, 400 x 400 L-F 3.67 -> 3.48 ms, the latter by the last round and faster folds).  The tapes are for reverse sweeps that
-    // evaluate their forward first: the reverse then does not evaluate fluxes and weights a second time.  Each is
-    // left out where it would take more than a quarter of the free memory.
-    const long long n = tape_doubles(h);
+    if (!h->adj_Wg) CK(dalloc(h, &h->adj_Wg, 4 * h->mesh.plane));
+    const bool gks = tapes && flux == DFGKS_FLUX_GKS;
+    const long long nr = ratio_doubles(h), nk = gks_doubles(h);
+    if (h->adj_lines[1] && (!tapes || h->adj_ratios) && (!gks || h->adj_gks)) return DFGKS_OK;
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(h->stream, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone) {
+        cudaGetLastError();
+        return DFGKS_OK;
+    }
     size_t free_b = 0, total_b = 0;
     cudaMemGetInfo(&free_b, &total_b);
     const double quarter = 0.25 * (double)free_b / sizeof(double);
-    if ((double)(nl + ng + 2 * n) <= quarter && dalloc(h, &h->adj_lines[1], nl) == cudaSuccess
-        && dalloc(h, &h->adj_gp[1], ng) == cudaSuccess && dalloc(h, &h->adj_tape, 2 * n) == cudaSuccess)
-        return DFGKS_OK;
-    for (double** q : {&h->adj_lines[1], &h->adj_gp[1], &h->adj_tape})
-        if (*q) { cudaFree(*q); h->bytes -= sizeof(double) * (unsigned long long)(q == &h->adj_gp[1] ? ng : q == &h->adj_tape ? 2 * n : nl); *q = nullptr; }
-    if ((double)n <= quarter && dalloc(h, &h->adj_tape, n) != cudaSuccess) h->adj_tape = nullptr;
-    cudaGetLastError();
+    // both directions: a single direction's tapes are too small for it and make room
+    const long long held = h->adj_lines[1] ? 0 : (h->adj_ratios ? nr : 0) + (h->adj_gks ? nk : 0);
+    const long long pair = h->adj_lines[1] ? 0 : nl + ng;
+    const bool have_r = h->adj_lines[1] && h->adj_ratios, have_k = h->adj_lines[1] && h->adj_gks;
+    const long long both = pair + (tapes && !have_r ? 2 * nr : 0) + (gks && !have_k ? 2 * nk : 0);
+    if ((double)(both - held) <= quarter) {
+        if (held) {
+            CK(cudaStreamSynchronize(h->stream));
+            dfree(h, &h->adj_ratios, nr);
+            dfree(h, &h->adj_gks, nk);
+        }
+        const bool new_l = !h->adj_lines[1], new_r = tapes && !h->adj_ratios, new_k = gks && !h->adj_gks;
+        if ((!new_l || (dalloc(h, &h->adj_lines[1], nl) == cudaSuccess && dalloc(h, &h->adj_gp[1], ng) == cudaSuccess))
+            && (!new_r || dalloc(h, &h->adj_ratios, 2 * nr) == cudaSuccess)
+            && (!new_k || dalloc(h, &h->adj_gks, 2 * nk) == cudaSuccess))
+            return DFGKS_OK;
+        if (new_k) dfree(h, &h->adj_gks, 2 * nk);
+        if (new_r) dfree(h, &h->adj_ratios, 2 * nr);
+        if (new_l) {
+            dfree(h, &h->adj_gp[1], ng);
+            dfree(h, &h->adj_lines[1], nl);
+        }
+        cudaGetLastError();
+    }
+    // one direction at a time
+    const bool one_r = tapes && !h->adj_ratios, one_k = gks && !h->adj_gks;
+    if (!h->adj_lines[1] && (one_r || one_k) && (double)((one_r ? nr : 0) + (one_k ? nk : 0)) <= quarter) {
+        if (one_r && dalloc(h, &h->adj_ratios, nr) != cudaSuccess) h->adj_ratios = nullptr;
+        if (one_k && h->adj_ratios && dalloc(h, &h->adj_gks, nk) != cudaSuccess) h->adj_gks = nullptr;
+        cudaGetLastError();
+    }
     return DFGKS_OK;
 }
 
 // h's records with set k of the tapes (none if there are none)
 static SweepBuffers taped_records(const dfgks* h, const SweepBuffers& B, int k, int flux) {
     SweepBuffers t = B;
-    if (!h->adj_tape) return t;
-    t.ltape = h->adj_tape + k * tape_doubles(h);
+    if (!h->adj_ratios) return t;
+    t.ltape = h->adj_ratios + k * ratio_doubles(h);
     t.ftape = t.ltape + (long long)8 * RT_COUNT * t.line_stride;
-    if (flux == DFGKS_FLUX_GKS) t.tape[0] = t.tape[1] = t.ftape + (long long)4 * RT_COUNT * t.gp_stride;
+    if (flux == DFGKS_FLUX_GKS && h->adj_gks) t.tape[0] = t.tape[1] = h->adj_gks + k * gks_doubles(h);
     return t;
 }
 
-// reverse sweep of the stage operator at (W, alpha, dt); W_bar (dense, device) += J^T (L_bar, ...)
+// reverse sweep of the stage operator at (W, alpha, dt); W_bar (dense, device) += J^T (L_bar, ...).  The buffers are
+// there (ensure_adjoint_buffers).
 // rec (optional): the stage's forward records per direction, kept by the forward pass; without
 // them each direction's forward sweep is recomputed first
 static dfgks_status adjoint_stage(dfgks* h, const double* W, const double* alpha, double dt, int flux,
                                   const double* L_bar, const double* dtL_bar, const double* dtLt_bar, double* W_bar,
                                   const SweepBuffers* rec = nullptr) {
-    dfgks_status r = ensure_adjoint_buffers(h);
-    if (r) return r;
     launch_dense_to_ghosted(h->mesh, W, 4, h->Ws, h->stream);
     launch_dense_to_ghosted(h->mesh, alpha, 1, h->As, h->stream);
     launch_fill_ghosts(h->mesh, h->Ws, h->As, nullptr, h->stream);
@@ -566,6 +607,8 @@ extern "C" dfgks_status dfgks_adjoint_residual(dfgks* h, const double* W, const 
                                                const double* L_bar, const double* dtL_bar, const double* dtLt_bar,
                                                double* W_bar) {
     if (!h || !W || !alpha || !W_bar || !(dt > 0.0) || (flux != 0 && flux != 1)) return DFGKS_EINVAL;
+    dfgks_status r = ensure_adjoint_buffers(h, true, flux);
+    if (r) return r;
     return adjoint_stage(h, W, alpha, dt, flux, L_bar, dtL_bar, dtLt_bar, W_bar);
 }
 
@@ -769,7 +812,7 @@ static dfgks_status backward_checkpointed(dfgks* h, const double* WT_bar, double
     if (bufs.size() != 7) r = DFGKS_ENOMEM;
     auto cleanup = [&]() { cudaStreamSynchronize(h->stream); for (double* p : bufs) if (p) cudaFree(p); };
     if (r) { cleanup(); return r; }
-    r = ensure_adjoint_buffers(h);
+    r = ensure_adjoint_buffers(h, a.recs == nullptr, flux);
     if (r) { cleanup(); return r; }
     // the passes; a CUDA error returns from this lambda, and the scratch is freed either way
     auto passes = [&]() -> dfgks_status {
