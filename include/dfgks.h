@@ -277,8 +277,8 @@ DFGKS_API dfgks_status dfgks_decomp_step(dfgks_decomp* d, int n, int flux, doubl
  * NULL; host memory if on_device == 0), time and step count. */
 DFGKS_API dfgks_status dfgks_decomp_get_state(dfgks_decomp* d, double* W, double* alpha, double* t, long* step,
                                               int on_device);
-/* Error flag (0 or DFGKS_ENONPOS), the first failing cell (whole-mesh indices, -1 if none) and the
- * branch counters summed over the blocks.  Any pointer may be NULL. */
+/* Error flag (0 or DFGKS_ENONPOS), the first failing cell of the first failing block (whole-mesh
+ * indices, -1 if none) and the branch counters summed over the blocks.  Any pointer may be NULL. */
 DFGKS_API dfgks_status dfgks_decomp_status(dfgks_decomp* d, int* err, int* fail_i, int* fail_j, dfgks_counters* counters);
 
 /* Per-face intermediates of one stage, for diagnostics and kernel-by-kernel comparison.

@@ -92,7 +92,7 @@ DFK_HD void report_fail(DevState* st, long long key) {
 #endif
 }
 
-// linear index j*nx + i of cell (i, j) in the enclosing mesh (the mesh itself unless a block)
+// number of cell (i, j) in positivity failures: j*nx + i in a whole mesh (Mesh::gi0)
 DFK_HD long long fail_key(const Mesh& m, int i, int j) {
     const long long gnx = m.gnx > 0 ? m.gnx : m.nx;
     return (long long)(j + m.gj0) * gnx + (i + m.gi0);

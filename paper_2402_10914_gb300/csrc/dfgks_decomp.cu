@@ -41,8 +41,11 @@ struct HaloBlock {
 // One pass of the ghost fill of all blocks (grid x: block): 0 the ghost columns of the interior rows, 1 the ghost
 // rows of all columns.  A pass reads no cell that it writes, so physical sides and copies go together: one launch
 // instead of a launch and up to ten strided copies per block (measured with the blocks' streams, see Helpers below).
-__global__ void k_halo(const HaloBlock* __restrict__ H, int pass, int field, int alpha, const int* halt) {
-    if (*(volatile const int*)halt != 0) return;
+// The last pass also notes the halt flag for the updates that follow (hold, see enqueue_decomp_step).
+__global__ void k_halo(const HaloBlock* __restrict__ H, int pass, int field, int alpha, const int* halt, int* hold) {
+    const int halted = *(volatile const int*)halt;
+    if (pass == 1 && blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) *hold = halted;
+    if (halted != 0) return;
     const HaloBlock& b = H[blockIdx.x];
     const int idx = blockIdx.y * blockDim.x + threadIdx.x;
     const Mesh& m = b.m;
@@ -143,6 +146,7 @@ struct dfgks_decomp {
     int cur;
     std::vector<void*> allocs;
     HaloBlock* halo;         // device
+    int* hold;               // device: the halt flag as the stage's ghost fill saw it
     int halo_tiles[2];       // 128-thread tiles of the largest block's ghost cells per pass
     // Helpers: the blocks' kernels between two ghost fills are independent and a block alone leaves part of the
     // chip idle, so block b runs on stream b mod their number.  With the fused ghost fill, 4 steps of 3 x 2 blocks
@@ -194,7 +198,7 @@ static void halo_window(const dfgks_block_plan& b, const dfgks_block_plan& a, in
 static cudaError_t halo(dfgks_decomp* d, int field, int in, bool with_alpha) {
     for (int pass = 0; pass < 2; ++pass)
         k_halo<<<dim3((unsigned)d->blk.size(), d->halo_tiles[pass]), 128, 0, d->stream>>>(
-            d->halo, pass, field == 0 ? in : 2, with_alpha ? in : -1, &d->st->halt);
+            d->halo, pass, field == 0 ? in : 2, with_alpha ? in : -1, &d->st->halt, d->hold);
     return cudaGetLastError();
 }
 
@@ -309,6 +313,7 @@ extern "C" DFGKS_API dfgks_status dfgks_decomp_create(const dfgks_config* cfg, i
     S.df_states = cfg->df_states;
     const double dx = (cfg->x1 - cfg->x0) / cfg->nx, dy = (cfg->y1 - cfg->y0) / cfg->ny;
     cudaError_t e = cudaSuccess;
+    long long cells = 0;
     d->blk.resize((size_t)px * py);
     for (int b = 0; b < px * py && e == cudaSuccess; ++b) {
         Block& k = d->blk[b];
@@ -323,7 +328,10 @@ extern "C" DFGKS_API dfgks_status dfgks_decomp_create(const dfgks_config* cfg, i
         m.rdx = 1.0 / dx; m.rdy = 1.0 / dy;
         for (int s = 0; s < 4; ++s) m.bc[s] = k.plan.bc[s];
         m.dt_rule = cfg->dt_rule;
-        m.gi0 = k.plan.i0; m.gj0 = k.plan.j0; m.gnx = cfg->nx;
+        // a failing cell's key: the cells of the blocks before, then row by row in its block (failing_cell), so the
+        // smallest key is in the first failing block.  (2^31 cells would take terabytes.)
+        m.gi0 = (int)cells; m.gj0 = 0; m.gnx = m.nx;
+        cells += (long long)m.nx * m.ny;
         const long long nfx = (long long)(m.nx + 1) * m.ny, nfy = (long long)(m.ny + 1) * m.nx;
         const long long nlx = (long long)(m.nx + 1) * (m.ny + 4), nly = (long long)(m.ny + 1) * (m.nx + 4);
         k.B.line_stride = round4(nlx > nly ? nlx : nly);
@@ -353,6 +361,7 @@ extern "C" DFGKS_API dfgks_status dfgks_decomp_create(const dfgks_config* cfg, i
     }
     if (e == cudaSuccess) e = dalloc(d, &d->st, 1);
     if (e == cudaSuccess) e = dalloc(d, &d->flag, 1);
+    if (e == cudaSuccess) e = dalloc(d, &d->hold, 1);
     if (e == cudaSuccess) { d->dts_cap = 1024; e = dalloc(d, &d->dts, d->dts_cap); }
     if (e == cudaSuccess) e = dalloc(d, &d->one, 4);
     if (e == cudaSuccess) e = dalloc(d, &d->stage, 4LL * cfg->nx * cfg->ny);
@@ -440,7 +449,10 @@ static cudaError_t enqueue_decomp_step(dfgks_decomp* d, int s, int in, int flux,
             launch_sweep_xy(b.m, d->S, flux, SWEEP_FULL, stage == 0 ? b.W[in] : b.Ws, b.A[in], dtp, b.B, b.By, ds, halt,
                             stream_of(d, q));
         }
-        // an update that loses positivity halts all that start later: none starts before every sweep has ended
+        // An update that loses positivity halts all that starts later.  The updates of one stage run side by side, so
+        // they go by the flag as the stage's ghost fill saw it (d->hold): each of them looks at all its cells, and the
+        // cell reported is the first one of the first failing block, whichever update came first.  None starts before
+        // every sweep has ended, as those go by the flag itself.
         if ((e = join(d)) != cudaSuccess || (e = fork(d)) != cudaSuccess) return e;
         for (size_t q = 0; q < d->blk.size(); ++q) {
             Block& b = d->blk[q];
@@ -449,7 +461,7 @@ static cudaError_t enqueue_decomp_step(dfgks_decomp* d, int s, int in, int flux,
             a.acc = b.acc;
             if (stage == 0) { a.Win = b.W[in]; a.Wout = b.Ws; }
             else { a.Win = b.Ws; a.Wout = b.W[out]; a.alpha_out = b.A[out]; }
-            launch_update(stage == 0 ? UM_S2O4_1 : UM_S2O4_2, b.m, d->S, a, b.B, dtp, ds, halt, stream_of(d, q));
+            launch_update(stage == 0 ? UM_S2O4_1 : UM_S2O4_2, b.m, d->S, a, b.B, dtp, ds, d->hold, stream_of(d, q));
         }
         if ((e = join(d)) != cudaSuccess) return e;
     }
@@ -514,6 +526,20 @@ extern "C" DFGKS_API dfgks_status dfgks_decomp_get_state(dfgks_decomp* d, double
     return DFGKS_OK;
 }
 
+// the whole mesh's indices of the cell that a key names (Mesh::gi0)
+static void failing_cell(const dfgks_decomp* d, unsigned long long key, int* i, int* j) {
+    *i = *j = -1;
+    for (const Block& b : d->blk) {
+        const unsigned long long n = (unsigned long long)b.m.nx * b.m.ny;
+        if (key < n) {
+            *i = b.plan.i0 + (int)(key % (unsigned long long)b.m.nx);
+            *j = b.plan.j0 + (int)(key / (unsigned long long)b.m.nx);
+            return;
+        }
+        key -= n;
+    }
+}
+
 extern "C" DFGKS_API dfgks_status dfgks_decomp_status(dfgks_decomp* d, int* err, int* fail_i, int* fail_j,
                                                       dfgks_counters* counters) {
     if (!d) return DFGKS_EINVAL;
@@ -521,9 +547,10 @@ extern "C" DFGKS_API dfgks_status dfgks_decomp_status(dfgks_decomp* d, int* err,
     DCK(cudaStreamSynchronize(d->stream));
     const DevState& h = *d->st_host;
     if (err) *err = h.err;
-    const bool failed = h.err != 0;
-    if (fail_i) *fail_i = failed ? (int)(h.fail_key % (unsigned long long)d->cfg.nx) : -1;
-    if (fail_j) *fail_j = failed ? (int)(h.fail_key / (unsigned long long)d->cfg.nx) : -1;
+    int i = -1, j = -1;
+    if (h.err != 0) failing_cell(d, h.fail_key, &i, &j);
+    if (fail_i) *fail_i = i;
+    if (fail_j) *fail_j = j;
     if (counters) {
         counters->fallbacks = h.fallbacks;
         counters->df_normal = h.df_normal;

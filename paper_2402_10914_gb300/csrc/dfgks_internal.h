@@ -59,8 +59,8 @@ struct Mesh {
     double rdx, rdy;    // 1/dx and 1/dy, divided once on the host (the same correctly rounded values)
     int bc[4];          // x-low, x-high, y-low, y-high; BC_EXTERNAL: ghosts written by a halo copy
     int dt_rule;        // CFL bound per cell: 0 per-direction minimum, 1 summed inverse
-    int gi0, gj0, gnx;  // a block of a larger mesh: its first cell there and that mesh's nx
-                        // (0, 0, nx for a whole mesh); positivity failures report that mesh's index
+    int gi0, gj0, gnx;  // numbering of the cells in positivity failures: cell (i, j) is (j + gj0) gnx + i + gi0
+                        // (0, 0, nx for a whole mesh; the blocks of a decomposition number theirs one after the other)
 };
 
 // boundary code of a block side whose ghost layers a neighbouring block's halo copy fills
