@@ -173,6 +173,13 @@ DFGKS_API dfgks_status dfgks_adjoint_residual(dfgks* h, const double* W, const d
                                               const double* L_bar, const double* dtL_bar, const double* dtLt_bar,
                                               double* W_bar);
 
+/* The most device memory, in bytes, that reverse sweeps of this handle may hold beyond what they
+ * cannot do without: a second direction's adjoints (both directions at once) and tapes of the
+ * forward's intermediates (no second evaluation).  Negative (the start): whatever is at most a
+ * quarter of the free memory when it is first wanted.  Results agree to rounding; 0 is the least
+ * memory and the slowest.  Memory held beyond a new limit is given back (synchronises). */
+DFGKS_API dfgks_status dfgks_set_reverse_memory(dfgks* h, long long max_bytes);
+
 /* Forward pass for a later gradient: sets the state to W0 (device, dense; alpha^0 computed from W0
  * as in dfgks_set_ic, t = 0) and advances n S2O4 steps of flux `flux`, with the step sizes dts_in[n]
  * (host) or, if dts_in is NULL, the CFL rule; dts_out[n] (host, may be NULL) receives them.  Keeps W

@@ -66,6 +66,7 @@ SIGNATURES = {
     "dfgks_step": [_V, C.c_int, C.c_double, C.c_int, C.c_double, _D, C.POINTER(C.c_int)],
     "dfgks_residual": [_V, _V, _V, C.c_double, C.c_int, _V, _V, _V, _V],
     "dfgks_adjoint_residual": [_V, _V, _V, C.c_double, C.c_int, _V, _V, _V, _V],
+    "dfgks_set_reverse_memory": [_V, C.c_longlong],
     "dfgks_face_records": [_V, _V, _V, C.c_double, C.c_int, C.c_int, _V],
     "dfgks_get_counters": [_V, C.POINTER(Counters)],
     "dfgks_last_error_detail": [_V, C.POINTER(C.c_long), C.POINTER(C.c_int), C.POINTER(C.c_int)],

@@ -46,6 +46,7 @@ struct dfgks {
     double* adj_Wg;
     double* adj_ratios;
     double* adj_gks;
+    long long adj_limit;   // bytes that the optional ones may take, -1: a quarter of the free memory
     // checkpointed forward pass kept for dfgks_adjoint_checkpointed
     double* ck_W;          // dense [nseg][4][ny][nx]: W at steps 0, k, 2k, ...
     double* ck_A;          // dense [nseg][ny][nx]: alpha at the same steps
@@ -242,6 +243,7 @@ extern "C" dfgks_status dfgks_create(const dfgks_config* cfg, void* stream, dfgk
     launch_fill_value(h->A[1], m.plane, 1.0, h->stream);
     launch_fill_value(h->As, m.plane, 1.0, h->stream);
     h->cur = 0;
+    h->adj_limit = -1;
     h->fail_step = -1; h->fail_i = -1; h->fail_j = -1;
     h->timer = new (std::nothrow) KernelTimer();
     if (!h->timer) { free_all(h); delete h; return DFGKS_ENOMEM; }
@@ -493,6 +495,13 @@ static long long gks_doubles(const dfgks* h) {
     return (long long)TG_COUNT * (s[0] > s[1] ? s[0] : s[1]);
 }
 
+// doubles that the reverse sweep holds beyond one direction's adjoints
+static long long adjoint_optional_doubles(const dfgks* h) {
+    const bool both = h->adj_lines[1] != nullptr;
+    const long long pair = (long long)LR_COUNT * h->B.line_stride + (long long)GP_COUNT * h->B.gp_stride;
+    return (both ? pair : 0) + (both ? 2 : 1) * ((h->adj_ratios ? ratio_doubles(h) : 0) + (h->adj_gks ? gks_doubles(h) : 0));
+}
+
 static void dfree(dfgks* h, double** p, long long n) {
     if (!*p) return;
     cudaFree(*p);
@@ -504,8 +513,9 @@ static void dfree(dfgks* h, double** p, long long n) {
 // fluxes and weights a second time (a reverse from kept records reads none of these tapes).
 // With a second set of adjoints both directions are reversed at once: the launches are twice as large, so small
 // meshes fill more of the chip and the last round of blocks weighs less.  Second set and tapes are left out where
-// they would take more than a quarter of the free memory.  They are kept for the calls that follow, and what is
-// missing is asked for again by the next call that would use it, unless that call is being captured.
+// they would take more than a quarter of the free memory, or than the handle's limit (dfgks_set_reverse_memory).
+// They are kept for the calls that follow, and what is missing is asked for again by the next call that would use
+// it, unless that call is being captured.
 static dfgks_status ensure_adjoint_buffers(dfgks* h, bool tapes, int flux) {
     const SweepBuffers& B = h->B;
     const long long nl = (long long)LR_COUNT * B.line_stride, ng = (long long)GP_COUNT * B.gp_stride;
@@ -520,15 +530,20 @@ static dfgks_status ensure_adjoint_buffers(dfgks* h, bool tapes, int flux) {
         cudaGetLastError();
         return DFGKS_OK;
     }
-    size_t free_b = 0, total_b = 0;
-    cudaMemGetInfo(&free_b, &total_b);
-    const double quarter = 0.25 * (double)free_b / sizeof(double);
+    double room;                                           // doubles that may be added
+    if (h->adj_limit >= 0) {
+        room = (double)h->adj_limit / sizeof(double) - (double)adjoint_optional_doubles(h);
+    } else {
+        size_t free_b = 0, total_b = 0;
+        cudaMemGetInfo(&free_b, &total_b);
+        room = 0.25 * (double)free_b / sizeof(double);
+    }
     // both directions: a single direction's tapes are too small for it and make room
     const long long held = h->adj_lines[1] ? 0 : (h->adj_ratios ? nr : 0) + (h->adj_gks ? nk : 0);
     const long long pair = h->adj_lines[1] ? 0 : nl + ng;
     const bool have_r = h->adj_lines[1] && h->adj_ratios, have_k = h->adj_lines[1] && h->adj_gks;
     const long long both = pair + (tapes && !have_r ? 2 * nr : 0) + (gks && !have_k ? 2 * nk : 0);
-    if ((double)(both - held) <= quarter) {
+    if ((double)(both - held) <= room) {
         if (held) {
             CK(cudaStreamSynchronize(h->stream));
             dfree(h, &h->adj_ratios, nr);
@@ -549,11 +564,24 @@ static dfgks_status ensure_adjoint_buffers(dfgks* h, bool tapes, int flux) {
     }
     // one direction at a time
     const bool one_r = tapes && !h->adj_ratios, one_k = gks && !h->adj_gks;
-    if (!h->adj_lines[1] && (one_r || one_k) && (double)((one_r ? nr : 0) + (one_k ? nk : 0)) <= quarter) {
+    if (!h->adj_lines[1] && (one_r || one_k) && (double)((one_r ? nr : 0) + (one_k ? nk : 0)) <= room) {
         if (one_r && dalloc(h, &h->adj_ratios, nr) != cudaSuccess) h->adj_ratios = nullptr;
         if (one_k && h->adj_ratios && dalloc(h, &h->adj_gks, nk) != cudaSuccess) h->adj_gks = nullptr;
         cudaGetLastError();
     }
+    return DFGKS_OK;
+}
+
+extern "C" dfgks_status dfgks_set_reverse_memory(dfgks* h, long long max_bytes) {
+    if (!h) return DFGKS_EINVAL;
+    h->adj_limit = max_bytes < 0 ? -1 : max_bytes;
+    if (h->adj_limit < 0 || adjoint_optional_doubles(h) * (long long)sizeof(double) <= h->adj_limit) return DFGKS_OK;
+    CK(cudaStreamSynchronize(h->stream));
+    const int n = h->adj_lines[1] ? 2 : 1;
+    dfree(h, &h->adj_ratios, n * ratio_doubles(h));
+    dfree(h, &h->adj_gks, n * gks_doubles(h));
+    dfree(h, &h->adj_lines[1], (long long)LR_COUNT * h->B.line_stride);
+    dfree(h, &h->adj_gp[1], (long long)GP_COUNT * h->B.gp_stride);
     return DFGKS_OK;
 }
 

@@ -173,6 +173,12 @@ class Solver:
         _lib.check(_lib.lib().dfgks_device_bytes(self._h, C.byref(b)), "dfgks_device_bytes")
         return b.value
 
+    def set_reverse_memory(self, max_bytes: int | None) -> None:
+        """Limit what reverse sweeps hold beyond the least they need (dfgks_set_reverse_memory); None: the
+        default, at most a quarter of the free device memory."""
+        _lib.check(_lib.lib().dfgks_set_reverse_memory(self._h, -1 if max_bytes is None else int(max_bytes)),
+                   "dfgks_set_reverse_memory")
+
     # -- stage operator ------------------------------------------------------------------
     def residual(self, W: torch.Tensor, alpha: torch.Tensor, dt: float, flux: int | None = None):
         """(L, dL/dt, limited dL/dt, alpha_next) as new CUDA tensors."""
