@@ -69,6 +69,22 @@ template <int DIR> DFK_HD int faces_ly(const Mesh& m) { return DIR == 0 ? m.ny :
 // 0.84 -> 0.77 ms, a 97 x 61 stage 0.177 -> 0.172 ms, a 400 x 400 step the same.
 constexpr int kSweepThreads = 32;
 inline unsigned sweep_blocks(int lx, int ly, int threads = kSweepThreads) { return (unsigned)(((long long)lx * ly + threads - 1) / threads); }
+
+// Which sweep kernels take four threads per item (lines_quad, faces_quad) on a mesh that `beside` meshes of its size
+// are swept at the same time as (itself included, the blocks of a decomposition on their streams): those whose whole
+// items, of all these meshes, are at most two (lines) or three (sides) warps per SM.  A line's 740 FP64 instructions
+// keep an SM's units 6 us per warp, a side's 430 3.5; the quads' 1200 and 620 take 10 and 5, against the 31 and
+// 19 us that one thread takes however few there are: the quads win below three warps of lines and four of sides.
+// Counting each block of a decomposition by itself costs 14 % in 4 x 4 blocks of 60 x 60 (1374 us a step, 1208 by the
+// warps of eight) and 23 % in 2 x 2 of 50 x 50 (398, 323); blocks of 20 x 20 take the quads either way (433).
+constexpr int kSMs = 152;
+struct QuadSweeps { bool lines, faces; };
+inline QuadSweeps quad_sweeps(const Mesh& m, int beside) {
+    const long long nl = (long long)sweep_blocks(lines_lx<0>(m), lines_ly<0>(m)) + sweep_blocks(lines_lx<1>(m), lines_ly<1>(m));
+    const long long nf = (long long)sweep_blocks(faces_lx<0>(m), faces_ly<0>(m)) + sweep_blocks(faces_lx<1>(m), faces_ly<1>(m));
+    return {beside * nl <= 2 * kSMs, beside * 2 * nf <= 3 * kSMs};
+}
+
 __device__ __forceinline__ void sweep_xy(int lx, int& ax, int& ay) {
     const int i = (int)(blockIdx.x * blockDim.x + threadIdx.x);
     ax = i % lx;

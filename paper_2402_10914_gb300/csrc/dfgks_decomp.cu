@@ -218,6 +218,9 @@ static cudaError_t join(dfgks_decomp* d) {
 }
 static cudaStream_t stream_of(const dfgks_decomp* d, size_t b) { return d->streams.empty() ? d->stream : d->streams[b % d->streams.size()]; }
 
+// blocks (all of about one size) whose kernels run side by side
+static int blocks_beside(const dfgks_decomp* d) { return d->streams.empty() ? 1 : (int)d->streams.size(); }
+
 static cudaError_t create_halo(dfgks_decomp* d) {
     std::vector<HaloBlock> H(d->blk.size());
     int rows = 0, cols = 0;
@@ -413,7 +416,8 @@ extern "C" DFGKS_API dfgks_status dfgks_decomp_set_ic(dfgks_decomp* d, const dou
     DCK(fork(d));
     for (size_t q = 0; q < d->blk.size(); ++q) {
         Block& b = d->blk[q];
-        launch_sweep_xy(b.m, d->S, 1, SWEEP_ALPHA, b.W[0], b.A[0], d->one, b.B, b.By, nullptr, nullptr, stream_of(d, q));
+        launch_sweep_xy(b.m, d->S, 1, SWEEP_ALPHA, b.W[0], b.A[0], d->one, b.B, b.By, nullptr, nullptr, stream_of(d, q),
+                        nullptr, blocks_beside(d));
         UpdateArgs a;
         memset(&a, 0, sizeof(a));
         a.alpha_out = b.A[0];
@@ -447,7 +451,7 @@ static cudaError_t enqueue_decomp_step(dfgks_decomp* d, int s, int in, int flux,
         for (size_t q = 0; q < d->blk.size(); ++q) {
             Block& b = d->blk[q];
             launch_sweep_xy(b.m, d->S, flux, SWEEP_FULL, stage == 0 ? b.W[in] : b.Ws, b.A[in], dtp, b.B, b.By, ds, halt,
-                            stream_of(d, q));
+                            stream_of(d, q), nullptr, blocks_beside(d));
         }
         // An update that loses positivity halts all that starts later.  The updates of one stage run side by side, so
         // they go by the flag as the stage's ghost fill saw it (d->hold): each of them looks at all its cells, and the

@@ -141,7 +141,7 @@ void launch_sweep(int dir, const Mesh& m, const SchemeConsts& S, int flux, bool 
                   DevState* st, const int* halt, cudaStream_t s, KernelTimer* T = nullptr);
 // both directions in one launch per kernel class: the x-faces use Bx's face-line and Gauss-point
 // records, flux[0] and tapes, the y-faces By's records, flux[1] and tapes (with tapes in both or
-// in neither)
+// in neither).  beside: meshes of this size swept at the same time, this one included (quad_sweeps)
 // SWEEP_ALPHA: the DF factors alone; SWEEP_VALUES: no time derivatives are used, so an L-F sweep leaves slopes,
 // limiter weights and dF out (a GKS flux needs the slopes all the same).  L-F with SSP-RK3 on 333 x 217, 4 steps:
 // 7.54 -> 5.73 ms, half of it from the L-F flux in gradient form; loading a state of 2048 x 2048 and one step
@@ -149,7 +149,7 @@ void launch_sweep(int dir, const Mesh& m, const SchemeConsts& S, int flux, bool 
 enum SweepWhat { SWEEP_FULL = 0, SWEEP_ALPHA, SWEEP_VALUES };
 void launch_sweep_xy(const Mesh& m, const SchemeConsts& S, int flux, SweepWhat what, const double* W,
                      const double* alpha, const double* dtp, const SweepBuffers& Bx, const SweepBuffers& By,
-                     DevState* st, const int* halt, cudaStream_t s, KernelTimer* T = nullptr);
+                     DevState* st, const int* halt, cudaStream_t s, KernelTimer* T = nullptr, int beside = 1);
 void launch_update(int mode, const Mesh& m, const SchemeConsts& S, const UpdateArgs& a, const SweepBuffers& B,
                    const double* dtp, DevState* st, const int* halt, cudaStream_t s, KernelTimer* T = nullptr);
 void launch_dense_to_ghosted(const Mesh& m, const double* dense, int ncomp, double* ghosted, cudaStream_t s);

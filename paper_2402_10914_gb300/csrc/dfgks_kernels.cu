@@ -14,8 +14,6 @@
 
 namespace dfk {
 
-constexpr int kSMs = 152;
-
 // The kernels of a step follow one another on a stream, each reading what the one before wrote.  They are launched
 // ahead of that one's end (programmatic dependent launch), so their launch and first instructions overlap its last
 // blocks, and wait in follow() until it has ended and its writes are visible before they touch memory; by then the
@@ -292,7 +290,7 @@ __global__ void __launch_bounds__(128) k_flux_xy(Mesh m, SchemeConsts S, const d
 
 void launch_sweep_xy(const Mesh& m, const SchemeConsts& S, int flux, SweepWhat what, const double* W,
                      const double* alpha, const double* dtp, const SweepBuffers& Bx, const SweepBuffers& By,
-                     DevState* st, const int* halt, cudaStream_t s, KernelTimer* T) {
+                     DevState* st, const int* halt, cudaStream_t s, KernelTimer* T, int beside) {
     const dim3 blk(kSweepThreads);
     const int nl0 = (int)sweep_blocks(lines_lx<0>(m), lines_ly<0>(m)), nl1 = (int)sweep_blocks(lines_lx<1>(m), lines_ly<1>(m));
     const int nf0 = (int)sweep_blocks(faces_lx<0>(m), faces_ly<0>(m)), nf1 = (int)sweep_blocks(faces_lx<1>(m), faces_ly<1>(m));
@@ -301,10 +299,8 @@ void launch_sweep_xy(const Mesh& m, const SchemeConsts& S, int flux, SweepWhat w
     const bool alpha_only = what == SWEEP_ALPHA, values = alpha_only || (what == SWEEP_VALUES && flux != 0);
     const long long ls = Bx.line_stride, gs = Bx.gp_stride;
     if (T) T->begin(KK_LINES);
-    // Four threads per item where whole items are at most two (three) warps per SM.  A line's 740 FP64 instructions
-    // keep an SM's units 6 us per warp, a side's 430 3.5; the quads' 1200 and 620 take 10 and 5, against the 31 and
-    // 19 us that one thread takes however few there are: the quads win below three warps of lines and four of sides.
-    const bool quad_lines = !tape && nl0 + nl1 <= 2 * kSMs, quad_faces = !tape && 2 * (nf0 + nf1) <= 3 * kSMs;
+    const QuadSweeps quads = quad_sweeps(m, beside);
+    const bool quad_lines = !tape && quads.lines, quad_faces = !tape && quads.faces;
     const int ql0 = (int)sweep_blocks(lines_lx<0>(m), lines_ly<0>(m), kSweepThreads / 4), ql1 = (int)sweep_blocks(lines_lx<1>(m), lines_ly<1>(m), kSweepThreads / 4);
     const int qf0 = (int)sweep_blocks(faces_lx<0>(m), faces_ly<0>(m), kSweepThreads / 4), qf1 = (int)sweep_blocks(faces_lx<1>(m), faces_ly<1>(m), kSweepThreads / 4);
     if (quad_lines && values)
