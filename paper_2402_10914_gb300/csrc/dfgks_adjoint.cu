@@ -183,8 +183,9 @@ DFK_HD void ka_faces_body(const Mesh& m, const SchemeConsts& S, const double* __
         const Real Ob = gg * (qvb[1][k] - qvb[0][k]), Esb = qtb[0][k] + qtb[1][k], Osb = gg * (qtb[1][k] - qtb[0][k]);
         Real v[2], sl[2];
         AODiffBar b;
-        b.fb = b.ff = b.s0 = b.s2 = b.to = b.ti = 0.0;
+        b.fb = b.ff = b.to = b.ti = 0.0;
         if (df) {
+            b.s0 = b.s2 = 0.0;
             const Real alpha1 = Real::raw(al[1]);
             df_diff_at_gauss(a11, s1, alpha1, v, sl);
             const Real a11b = alpha1 * (Ob + Esb);
@@ -200,25 +201,23 @@ DFK_HD void ka_faces_body(const Mesh& m, const SchemeConsts& S, const double* __
                                              second_difference_energy(s1, eps), second_difference_energy(s2, eps), a11, T, U,
                                              eps, S));
             }
-            const AOCoeffs c = ao_coeffs(q);
-            const Real dp = S.d[0] * c.p0, dr = S.d[0] * c.p2, p = dp * t1, r = dr * t2, c3T = c.c3 * T, c3U = c.c3 * U;
+            const AOCoeffs c = ao_coeffs(q, S);
+            const Real a10 = fma(0.5, s0, F[1][k]), a12 = fma(-0.5, s2, F[2][k]);
+            const Real c3T = c.c3 * T, c3U = c.c3 * U;
             {   // the values, for the basis (ao_diff_at_gauss)
-                const Real B = fma(-0.5, p + r, a11);
+                const Real B = fma(c.c0, a10, fma(c.cm, a11, c.c2 * a12)), E2 = fma(c.c0, s0, fma(c.cm, s1, c.c2 * s2));
                 const Real O = gg * fma(-7.0 / 72.0, c3T, B), Es = fma(-1.0 / 12.0, c3T, B);
-                const Real Os = gg * fma(-1.0 / 9.0, c3U, s1 - (p - r)), E = (-1.0 / 4320.0) * c3U;
+                const Real Os = gg * fma(-1.0 / 9.0, c3U, E2), E = (-1.0 / 4320.0) * c3U;
                 v[0] = E - O; v[1] = E + O;
                 sl[0] = Es - Os; sl[1] = Es + Os;
             }
             const Real Eb = qvb[0][k] + qvb[1][k], Bb = Ob + Esb;
             const Real c3Tb = fma(-7.0 / 72.0, Ob, (-1.0 / 12.0) * Esb), c3Ub = fma(-1.0 / 4320.0, Eb, (-1.0 / 9.0) * Osb);
-            const Real pb = fma(-0.5, Bb, -Osb), rb = fma(-0.5, Bb, Osb);
-            b.a11 = Bb;
-            b.s1 = Osb;
-            b.to = dp * pb;
-            b.ti = dr * rb;
+            b.a10 = c.c0 * Bb; b.a11 = c.cm * Bb; b.a12 = c.c2 * Bb;
+            b.s0 = c.c0 * Osb; b.s1 = c.cm * Osb; b.s2 = c.c2 * Osb;
             Real zb[4];
-            ao_coeffs_rev(c, q, fma(c3Tb, T, c3Ub * U), (S.d[0] * t1) * pb, (S.d[0] * t2) * rb, S, zb);
-            ao_ratios_rev<+1>(q, c, zb, F[1][k], F[2][k], s0, s1, s2, a11, T, U, c.c3 * c3Tb, c.c3 * c3Ub, b);
+            ao_coeffs_rev(c, q, fma(Bb, a10, Osb * s0), fma(Bb, a11, Osb * s1), fma(Bb, a12, Osb * s2), fma(c3Tb, T, c3Ub * U), S, zb);
+            ao_ratios_rev<+1>(q, c, zb, s0, s1, s2, a10, a11, a12, T, U, c.c3 * c3Tb, c.c3 * c3Ub, b);
         }
         // third differences to second, second to first
         const Real s0b = b.s0 - b.to, s1b = b.s1 + (b.to - b.ti), s2b = b.s2 + b.ti;
@@ -265,33 +264,39 @@ DFK_HD void ka_faces_body(const Mesh& m, const SchemeConsts& S, const double* __
 template <int SGN>
 DFK_HD void edge_reverse(const AORatios& q, bool df, Real alpha, Real vb, Real sb, double wb, Real fb, Real ff, Real s0, Real s1,
                          Real s2, Real to, Real ti, const SchemeConsts& S, Real& v, Real& sl, AODiffBar& b) {
-    const Real base = SGN > 0 ? fma(-1.0 / 6.0, s1, 0.5 * ff) : fma(-1.0 / 6.0, s1, -0.5 * ff);
-    const Real a = df ? alpha : Real(1.0), ab = a * vb;
-    b.ff = fma(a, sb, fma(0.5 * SGN, ab, b.ff));
-    b.s1 = fma(-1.0 / 6.0, ab, b.s1);
-    v = a * base;
-    sl = a * ff;
     const bool lim = (dbits(wb) << 1) != 0;
-    if (df && !lim) return;
-    const AOCoeffs c = ao_coeffs(q);
-    const Real T = to + ti, U = SGN > 0 ? ti - to : to - ti, a11 = fma(0.5 * SGN, s1, fb);
+    constexpr double h = 0.5 * SGN;
+    if (df) {
+        const Real ab = alpha * vb;
+        b.ff = fma(alpha, sb, fma(h, ab, b.ff));
+        b.s1 = fma(-1.0 / 6.0, ab, b.s1);
+        v = alpha * fma(-1.0 / 6.0, s1, h * ff);
+        sl = alpha * ff;
+        if (!lim) return;
+    }
+    const AOCoeffs c = ao_coeffs(q, S);
+    const Real a10 = fma(h, s0, fb), a11 = fma(h, s1, fb), a12 = fma(-h, s2, ff);
+    const Real T = to + ti, U = SGN > 0 ? ti - to : to - ti;
     Real zb[4];
     if (!df) {
-        const Real d0 = S.d[0], dp = d0 * c.p0, dr = (1.0 / 6.0) * (d0 * c.p2), h12 = (1.0 / 12.0) * ti;
-        const Real w = fma(1.0 / 30.0, to, (1.0 / 20.0) * ti), p = dp * to;
-        const Real x = fma(c.c3, w, fma(dr, ti, (1.0 / 3.0) * p));
-        v = SGN > 0 ? v - x : v + x;
-        sl = sl - fma(c.c3, h12, p);
-        const Real xb = SGN > 0 ? -vb : vb, yb = fma(1.0 / 3.0, xb, -sb);
-        b.to = fma(dp, yb, fma((1.0 / 30.0) * c.c3, xb, b.to));
-        b.ti = fma(dr, xb, fma(c.c3, fma(1.0 / 20.0, xb, (-1.0 / 12.0) * sb), b.ti));
-        ao_coeffs_rev(c, q, fma(xb, w, -(sb * h12)), (d0 * to) * yb, (d0 * ti) * ((1.0 / 6.0) * xb), S, zb);
+        const Real w = fma(1.0 / 30.0, to, (1.0 / 20.0) * ti), h12 = (1.0 / 12.0) * ti;
+        const Real B = fma(c.c0, a10, fma(c.cm, a11, c.c2 * a12)), D = fma(c.c0, s0, fma(c.cm, s1, c.c2 * s2));
+        const Real c3w = c.c3 * w;
+        v = fma(1.0 / 12.0, D, SGN > 0 ? fma(h, B, -c3w) : fma(h, B, c3w));
+        sl = fma(-c.c3, h12, fma(h, D, B));
+        const Real xb = SGN > 0 ? -vb : vb;
+        const Real Bb = fma(h, vb, sb), Db = fma(1.0 / 12.0, vb, h * sb);
+        b.a10 = c.c0 * Bb; b.a11 = c.cm * Bb; b.a12 = c.c2 * Bb;
+        b.s0 = fma(c.c0, Db, b.s0); b.s1 = fma(c.cm, Db, b.s1); b.s2 = fma(c.c2, Db, b.s2);
+        b.to = fma((1.0 / 30.0) * c.c3, xb, b.to);
+        b.ti = fma(c.c3, fma(1.0 / 20.0, xb, (-1.0 / 12.0) * sb), b.ti);
+        ao_coeffs_rev(c, q, fma(Bb, a10, Db * s0), fma(Bb, a11, Db * s1), fma(Bb, a12, Db * s2), fma(xb, w, -(sb * h12)), S, zb);
     } else {
+        b.a10 = b.a11 = b.a12 = 0.0;
         zb[0] = zb[1] = zb[2] = zb[3] = 0.0;
     }
     if (lim) ao_limiter_rev(q, c, Real::raw(wb), zb);
-    b.a11 = 0.0;
-    ao_ratios_rev<SGN>(q, c, zb, fb, ff, s0, s1, s2, a11, T, U, 0.0, 0.0, b);
+    ao_ratios_rev<SGN>(q, c, zb, s0, s1, s2, a10, a11, a12, T, U, 0.0, 0.0, b);
 }
 
 // TAPED: the normal reconstructions' ratios are read from the tape the forward sweep wrote

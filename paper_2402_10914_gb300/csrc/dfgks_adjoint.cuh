@@ -589,38 +589,40 @@ DFK_HD void gks_flux_vjp(const GPState& L, const GPState& R, double dt, const Sc
 // ------------------------------------------------------------------------------------------
 // WENO-AO in undivided differences, the reverse of ao_weights and of its evaluations
 //
-// With z_k = r_k^2, c_3 = (1 + z_3)/sum, p_k = (z_k - z_3)/sum (k = 0, 2) and sum = 1 + sum_k d_k z_k; the
-// differences of one reconstruction are fb, ff, the second ones s0, s1, s2 and the third ones to, ti (outer and
+// With z_k = r_k^2 and sum = 1 + sum_k d_k z_k the weights are c_3 = (1 + z_3)/sum, c_0, c_2 = d_0 (z_k - z_3)/sum and
+// c_m = c_3 + d_1 (z_1 - z_3)/sum (ao_sum); the differences of one reconstruction are fb, ff, the second ones s0, s1, s2 and the third ones to, ti (outer and
 // inner: t1, t2 of the forward for SGN +1, t3, t2 for the mirrored stencil), T = to + ti, U = SGN (ti - to).
 // Bound by the FP64 units like the forward.  The sub-stencil polynomials' form (weno_ao_rev above, which stays as
 // the plain statement this one is checked against) and a tape of 29 values a reconstruction instead of 6 took, with
 // the forward: 400 x 400 L-F stage 5.76 -> 3.93 ms, 67 x 83 GKS stage 0.620 -> 0.483, 10-step GKS gradient on
 // 256 x 256 53.1 -> 42.6.
 // ------------------------------------------------------------------------------------------
-struct AODiffBar { Real fb, ff, s0, s1, s2, a11, to, ti; };
+struct AODiffBar { Real fb, ff, s0, s1, s2, a10, a11, a12, to, ti; };
 
-// c_3, p_0, p_2 of a reconstruction (SchemeConsts: d_0 = d_2)
-struct AOCoeffs { Real r[4], c3, p0, p2; };
-DFK_HD AOCoeffs ao_coeffs(const AORatios& q) {
+// the weights of a reconstruction (SchemeConsts: d_0 = d_2)
+struct AOCoeffs { Real r[4], c0, cm, c2, c3; };
+DFK_HD AOCoeffs ao_coeffs(const AORatios& q, const SchemeConsts& S) {
     AOCoeffs c;
 #pragma unroll
     for (int k = 0; k < 4; ++k) c.r[k] = q.tau * q.ie[k];
     const Real z3 = c.r[3] * c.r[3];
     c.c3 = fma(z3, q.iv, q.iv);
-    c.p0 = fma(c.r[0], c.r[0], -z3) * q.iv;
-    c.p2 = fma(c.r[2], c.r[2], -z3) * q.iv;
+    const Real di = S.d[0] * q.iv;
+    c.c0 = fma(c.r[0], c.r[0], -z3) * di;
+    c.c2 = fma(c.r[2], c.r[2], -z3) * di;
+    c.cm = fma(S.d[1] * q.iv, fma(c.r[1], c.r[1], -z3), c.c3);
     return c;
 }
 
-// four times the adjoints of z_k for those of c_3, p_0, p_2 (the factors 2 of z = r^2 and of the squares in the
-// smoothness indicators, once)
-DFK_HD void ao_coeffs_rev(const AOCoeffs& c, const AORatios& q, Real c3b, Real p0b, Real p2b, const SchemeConsts& S, Real zb[4]) {
-    const Real n = fma(c3b, c.c3, fma(p0b, c.p0, p2b * c.p2));          // minus the sum's adjoint times the sum
-    const Real iv = 4.0 * q.iv;
-    zb[0] = iv * fma(-S.d[0], n, p0b);
-    zb[1] = iv * (Real(-S.d[1]) * n);
-    zb[2] = iv * fma(-S.d[0], n, p2b);
-    zb[3] = iv * (fma(-S.d[3], n, c3b) - (p0b + p2b));
+// four times the adjoints of z_k for those of the weights (the factors 2 of z = r^2 and of the squares in the
+// smoothness indicators, once).  As in the forward, each is a difference of terms of its own sub-stencil's size
+DFK_HD void ao_coeffs_rev(const AOCoeffs& c, const AORatios& q, Real c0b, Real cmb, Real c2b, Real c3b, const SchemeConsts& S, Real zb[4]) {
+    const Real n = fma(c0b, c.c0, fma(cmb, c.cm, fma(c2b, c.c2, c3b * c.c3)));     // minus the sum's adjoint times the sum
+    const Real iv = 4.0 * q.iv, di = S.d[0] * iv, em = cmb - n;
+    zb[0] = di * (c0b - n);
+    zb[1] = (S.d[1] * iv) * em;
+    zb[2] = di * (c2b - n);
+    zb[3] = iv * fma(S.d[0], fma(2.0, cmb, -(c0b + c2b)), fma(S.d[3], em, c3b));   // 1 - d_1 = 2 d_0 + d_3
 }
 
 // the limiter weight 2 (1 + z_min) / ((1 + z_max) + (1 + z_min)): adds to (four times) the adjoints of the z it was made of
@@ -643,11 +645,11 @@ DFK_HD void ao_limiter_rev(const AORatios& q, const AOCoeffs& c, Real wb, Real z
     }
 }
 
-// four times the adjoints of the z_k, and those of T, U so far, to the differences (b accumulates; b.a11 holds the
-// evaluation's share of the adjoint of a11 = fb + SGN s1/2)
+// four times the adjoints of the z_k, and those of T, U so far, to the differences (b accumulates; b.a10, b.a11, b.a12
+// hold the evaluation's share of the adjoints of a10 = fb + SGN s0/2, a11 = fb + SGN s1/2, a12 = ff - SGN s2/2)
 template <int SGN>
-DFK_HD void ao_ratios_rev(const AORatios& q, const AOCoeffs& c, const Real zb[4], Real fb, Real ff, Real s0, Real s1, Real s2,
-                          Real a11, Real T, Real U, Real Tb, Real Ub, AODiffBar& b) {
+DFK_HD void ao_ratios_rev(const AORatios& q, const AOCoeffs& c, const Real zb[4], Real s0, Real s1, Real s2, Real a10, Real a11,
+                          Real a12, Real T, Real U, Real Tb, Real Ub, AODiffBar& b) {
     // r_k = tau / e_k; eb: twice the adjoints of e_k
     Real eb[4], g[4];
 #pragma unroll
@@ -663,7 +665,7 @@ DFK_HD void ao_ratios_rev(const AORatios& q, const AOCoeffs& c, const Real zb[4]
     }
     eb[3] = fma(t3, below < 2 ? (below ? Real(1.0) : Real(3.0)) : (below == 2 ? Real(-1.0) : Real(-3.0)), eb[3]);
     const Real h = 0.5 * SGN;
-    const Real a10b = eb[0] * fma(h, s0, fb), a12b = eb[2] * fma(-h, s2, ff);
+    const Real a10b = fma(eb[0], a10, b.a10), a12b = fma(eb[2], a12, b.a12);
     const Real m1b = eb[3] * fma(-1.0 / 12.0, T, a11), m2b = (13.0 / 12.0) * eb[3] * fma(-11.0 / 130.0, U, s1);
     const Real a11b = fma(eb[1], a11, m1b + b.a11);
     Tb = fma((781.0 / 2880.0) * eb[3], T, fma(-1.0 / 12.0, m1b, Tb));

@@ -203,30 +203,19 @@ template <bool VALUES>
 DFK_HD void line_component(const Real f[5], bool acoustic, bool dfL, bool dfR, double alL, double alR, Real idn,
                            const SchemeConsts& S, Real q[4], AOWeights& L, AOWeights& R) {
     const Real s1 = f[1] - f[0], s2 = f[2] - f[1], s3 = f[3] - f[2], s4 = f[4] - f[3];
-    const Real f3 = f[2], hf = 0.5 * f3;
-    // both sides' central quadratics at the face: cell f-1 at xi = +1/2, cell f mirrored
-    const Real baseL = fma(-1.0 / 6.0, s2, hf), baseR = fma(-1.0 / 6.0, s3, -hf);
+    const Real f3 = f[2];
     if (!dfL || !dfR || (!VALUES && S.time_limiter)) {
         const Real eps = acoustic ? Real(4.0 * S.eps) : Real(S.eps);
         const Real t1 = s2 - s1, t2 = s3 - s2, t3 = s4 - s3;
         const Real w1 = second_difference_energy(s1, eps), w2 = second_difference_energy(s2, eps);
         const Real w3 = second_difference_energy(s3, eps), w4 = second_difference_energy(s4, eps);
         L = ao_weights<+1>(f[1], f3, s1, s2, s3, w1, w2, w3, fma(0.5, s2, f[1]), t1 + t2, t2 - t1, eps, S);
+        if (!dfL) ao_diff_at_edge<+1>(L, f[1], f3, s2, t1, t2, idn, S, q);
         R = ao_weights<-1>(f[3], f3, s4, s3, s2, w4, w3, w2, fma(-0.5, s3, f[3]), t2 + t3, t3 - t2, eps, S);
-        const Real h2 = 0.5 * t2, h12 = (1.0 / 12.0) * t2, h20 = (1.0 / 20.0) * t2, d03 = (1.0 / 3.0) * S.d[0];
-        if (!dfL) {
-            const Real iv = ao_inverse_sum(L), p = L.y0 * t1;
-            const Real v = fma(d03, fma(h2, L.y2, p), L.x3 * fma(1.0 / 30.0, t1, h20));
-            q[0] = fma(-iv, v, baseL);
-            q[1] = idn * fma(-iv, fma(S.d[0], p, L.x3 * h12), f3);
-        }
-        if (!dfR) {
-            const Real iv = ao_inverse_sum(R), p = R.y0 * t3;
-            const Real v = fma(d03, fma(h2, R.y2, p), R.x3 * fma(1.0 / 30.0, t3, h20));
-            q[2] = fma(iv, v, baseR);
-            q[3] = idn * fma(-iv, fma(S.d[0], p, R.x3 * h12), f3);
-        }
+        if (!dfR) ao_diff_at_edge<-1>(R, f[3], f3, s3, t3, t2, idn, S, q + 2);
     }
+    // the central quadratics there
+    const Real hf = 0.5 * f3, baseL = fma(-1.0 / 6.0, s2, hf), baseR = fma(-1.0 / 6.0, s3, -hf);
     if (dfL) { q[0] = Real::raw(alL) * baseL; q[1] = idn * (Real::raw(alL) * f3); }
     if (dfR) { q[2] = Real::raw(alR) * baseR; q[3] = idn * (Real::raw(alR) * f3); }
 }

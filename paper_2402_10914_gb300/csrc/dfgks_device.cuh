@@ -325,13 +325,16 @@ DFK_HD AO weno_ao(const double q[5], const SchemeConsts& S) { return weno_ao_t(q
 // the quartic's smoothness indicator completes to squares,
 //   beta_3 = (a1_1 - T/12)^2 + 13/12 (s1 - 11U/130)^2 + 781/2880 T^2 + 1421461/1310400 U^2,
 // and, because the linear weights sum to one, with x_k = 1 + r_k^2 and y_k = x_k - x_3 the weights are
-//   c_3 = x_3 / sum, c_k = d_k y_k / sum,  sum = x_3 + sum_{k<3} d_k y_k,
-// so that A1 = a1_1 - 5/48 c_3 T - (c_0 t1 + c_2 t2)/2 and A2 = s1/2 - c_3 U/16 - (c_0 t1 - c_2 t2)/2: the
-// evaluations need no sub-stencil polynomial any more.  These kernels are bound by the two FP64 units of
-// an SM, so what counts is FP64 instructions: about 70 per reconstruction, against 114 from the
-// coefficients of the four polynomials.  Differences also cancel before they are projected.
-// Per 400 x 400 step the face-line kernel went from 1.36 to 0.91 ms and the tangential one from 1.40
-// to 1.05 ms (1097 -> 737 FP64 instructions per line, 575 -> 429 per face side).
+//   c_3 = x_3 / sum, c_k = d_k y_k / sum,  sum = x_3 + sum_{k<3} d_k y_k.
+// The quartic is the central polynomial and a correction in T and U, so that with c_m = c_1 + c_3 and
+//   B = c_0 a1_0 + c_m a1_1 + c_2 a1_2,  D = c_0 s0 + c_m s1 + c_2 s2
+// A1 = B - 5/48 c_3 T and 2 A2 = D - c_3 U/8, without a coefficient of a quadratic beside its own weight.  (As a
+// departure from the central polynomial, A1 = a1_1 - 5/48 c_3 T - (c_0 t1 + c_2 t2)/2, it is two instructions
+// shorter, but beside a jump the jump then cancels out of terms of weight one: the quiet side takes up
+// rounding noise of the jump's size, 2e-10 of data of order 1 beside a jump of 1e6, instead of 1e-15.)
+// These kernels are bound by the two FP64 units of an SM, so what counts is FP64 instructions: about 75 per
+// reconstruction, against 114 from the coefficients of the four polynomials.  Differences also cancel before they
+// are projected.
 // ------------------------------------------------------------------------------------------
 
 // 1/x for x in [1e-300, 1e300]: the hardware's approximation (2^-20) refined by one third-order
@@ -348,10 +351,12 @@ DFK_HD Real rcp(Real x) {
 #endif
 }
 
-// weights of one reconstruction: c_3 = x3 / sum, c_0 = d0 y0 / sum, c_2 = d0 y2 / sum, and the extreme
-// x_k, all carried scaled by (3 prod)^2, prod = the product of the four beta_k + eps (the scale cancels)
+// weights of one reconstruction: c_3 = x3 / sum, c_0 = d0 y0 / sum, c_2 = d0 y2 / sum, c_m = xm / sum, c_m + c_2 =
+// xr / sum, and the extreme x_k, all carried scaled by (3 prod)^2, prod = the product of the four beta_k + eps (the
+// scale cancels)
 struct AOWeights {
-    Real x3, y0, y2, sum, xmax, xmin;
+    Real x3, y0, y2, xm, xr, sum, xmax, xmin;
+    Real a10, a12, s0, s2;                 // the outer quadratics' coefficients (2 a2_k = s_k)
     Real e[4], tau3, prod, p2;             // beta_k + eps, 3 tau, the scale: for ao_ratios
     bool scaled;
 };
@@ -395,7 +400,10 @@ DFK_HD AOWeights ao_weights(Real fb, Real ff, Real s0, Real s1, Real s2, Real w0
     o.y0 = fma(t0, t0, -z3);
     o.y2 = fma(t2, t2, -z3);
     const Real y1 = fma(t1, t1, -z3);
-    o.sum = fma(S.d[0], o.y0 + o.y2, fma(S.d[1], y1, o.x3));
+    o.xm = fma(S.d[1], y1, o.x3);
+    o.xr = fma(S.d[0], o.y2, o.xm);
+    o.sum = fma(S.d[0], o.y0, o.xr);
+    o.a10 = a10; o.a12 = a12; o.s0 = s0; o.s2 = s2;
     o.xmax = fma(tmax, tmax, p2);                  // the time limiter's; dropped where it is not used
     o.xmin = fma(tmin, tmin, p2);
     o.e[0] = e0; o.e[1] = e1; o.e[2] = e2; o.e[3] = e3;
@@ -442,16 +450,34 @@ DFK_HD AORatios tape_get_ratios(const Tape& tp, int b) {
     return a;
 }
 
-// values minus q0 and d/deta (unscaled) at the two Gauss points eta = -g (m=1), +g (m=2), g = sqrt(3)/6
-DFK_HD void ao_diff_at_gauss(const AOWeights& o, Real a11, Real s1, Real t1, Real t2, Real T, Real U,
+// B and D times the sum of the weights, of coefficients a10, a11, a12 or s0, s1, s2
+DFK_HD Real ao_sum(const AOWeights& o, Real a0, Real am, Real a2, const SchemeConsts& S) {
+    return fma(S.d[0], fma(o.y0, a0, o.y2 * a2), o.xm * am);
+}
+
+// the polynomial's value minus the average (q[0]) and slope (q[1], times idn) at the face, xi = SGN/2 of a cell whose
+// third differences are to (outer) and ti: with D and the slope's H = c_0 (fb + SGN s0) + (c_m + c_2) ff, the central
+// and the inner quadratic having the face's difference ff as their slope there,
+//   value = SGN (H/2 - c_3 (to/30 + ti/20)) - D/6,  slope = H - c_3 ti/12
+template <int SGN>
+DFK_HD void ao_diff_at_edge(const AOWeights& o, Real fb, Real ff, Real s1, Real to, Real ti, Real idn, const SchemeConsts& S, Real q[2]) {
+    const Real iv = ao_inverse_sum(o), D = ao_sum(o, o.s0, s1, o.s2, S);
+    const Real H = fma(S.d[0], Real(o.y0 * (SGN > 0 ? fb + o.s0 : fb - o.s0)), o.xr * ff);
+    const Real w = o.x3 * fma(1.0 / 30.0, to, (1.0 / 20.0) * ti);
+    q[0] = iv * fma(-1.0 / 6.0, D, SGN > 0 ? fma(0.5, H, -w) : fma(-0.5, H, w));
+    q[1] = (idn * iv) * fma(-o.x3, (1.0 / 12.0) * ti, H);
+}
+
+// values minus q0 and d/deta (unscaled) at the two Gauss points eta = -g (m=1), +g (m=2), g = sqrt(3)/6, from a11, s1
+// and the third differences (their sum T and difference U)
+DFK_HD void ao_diff_at_gauss(const AOWeights& o, Real a11, Real s1, Real, Real, Real T, Real U,
                              const SchemeConsts& S, Real val[2], Real slope[2]) {
     const Real g = kGaussEta;
-    const Real iv = ao_inverse_sum(o), di = S.d[0] * iv, c3 = o.x3 * iv;
-    const Real p = (o.y0 * di) * t1, r = (o.y2 * di) * t2;         // c_0 t1, c_2 t2
+    const Real iv = ao_inverse_sum(o), c3 = o.x3 * iv;
+    const Real B = iv * ao_sum(o, o.a10, a11, o.a12, S), D = iv * ao_sum(o, o.s0, s1, o.s2, S);
     const Real c3T = c3 * T, c3U = c3 * U;
-    const Real B = fma(-0.5, p + r, a11);
     const Real O = g * fma(-7.0 / 72.0, c3T, B), Es = fma(-1.0 / 12.0, c3T, B);
-    const Real Os = fma(-1.0 / 9.0, c3U, s1 - (p - r)), E = (-1.0 / 4320.0) * c3U;
+    const Real Os = fma(-1.0 / 9.0, c3U, D), E = (-1.0 / 4320.0) * c3U;
     val[0] = E - O; val[1] = E + O;
     slope[0] = fma(-g, Os, Es); slope[1] = fma(g, Os, Es);
 }
