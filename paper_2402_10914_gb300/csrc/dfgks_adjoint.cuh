@@ -592,8 +592,8 @@ DFK_HD void gks_flux_vjp(const GPState& L, const GPState& R, double dt, const Sc
 // With z_k = r_k^2 and sum = 1 + sum_k d_k z_k the weights are c_3 = (1 + z_3)/sum, c_0, c_2 = d_0 (z_k - z_3)/sum and
 // c_m = c_3 + d_1 (z_1 - z_3)/sum (ao_sum); the differences of one reconstruction are fb, ff, the second ones s0, s1, s2 and the third ones to, ti (outer and
 // inner: t1, t2 of the forward for SGN +1, t3, t2 for the mirrored stencil), T = to + ti, U = SGN (ti - to).
-// Bound by the FP64 units like the forward.  The sub-stencil polynomials' form (weno_ao_rev above, which stays as
-// the plain statement this one is checked against) and a tape of 29 values a reconstruction instead of 6 took, with
+// Bound by the FP64 units like the forward.  The sub-stencil polynomials' form (weno_ao_rev above, which stays with
+// the other plain statements as what these routines are tested against; no kernel calls it) and a tape of 29 values a reconstruction instead of 6 took, with
 // the forward: 400 x 400 L-F stage 5.76 -> 3.93 ms, 67 x 83 GKS stage 0.620 -> 0.483, 10-step GKS gradient on
 // 256 x 256 53.1 -> 42.6.
 // ------------------------------------------------------------------------------------------

@@ -4,13 +4,16 @@
 // dfgks_kernels.cu move data between them.
 //
 // Arithmetic choices (each algebraically identical to the paper's formulas):
-//   * characteristic projection L W and back-projection R Q in factored form (12 + 14 flops
-//     instead of two 4x4 products);
-//   * WENO-AO sub-stencil polynomials kept as cell-centred coefficients a1..a4 (the cell mean
-//     fixes a0), so smoothness indicators (Eq. 38) and every evaluation point share them;
+//   * characteristic projection and back-projection of differences of states, in factored form (DiffBasis: ten
+//     instructions each way);
+//   * WENO-AO in undivided differences (ao_weights): smoothness indicators (Eq. 38), weights and evaluations
+//     without the sub-stencil polynomials' coefficients;
+//   * GKS and L-F fluxes in gradient form: primitive gradients in place of slope coefficients and flux Jacobians;
+//   * every FP64 operand in a vector register (Real), Gaussians and erfc from tables;
 //   * S2O4 flux coefficients (Eq. 27) combined analytically per kinetic term before the moments
-//     are summed, using E(dt) = E(dt/2)^2, which avoids the cancellation of 4(F(dt)-2F(dt/2));
-//   * GKS moments of slope polynomials (Sect. 2.2) as derivatives of the moments themselves.
+//     are summed, using E(dt) = E(dt/2)^2, which avoids the cancellation of 4(F(dt)-2F(dt/2)).
+// The plain statements (project, back_project, weno_ao_t and its evaluations, df_at_*, limiter_alpha) are what the
+// kernels' forms and their reverses are tested against; no kernel calls them.
 #pragma once
 #include <cuda_runtime.h>
 #include <math.h>
@@ -122,10 +125,6 @@ struct SchemeConsts {
 // ------------------------------------------------------------------------------------------
 // Euler state helpers
 // ------------------------------------------------------------------------------------------
-DFK_HD double pressure_of(const double W[4], double gm1) {
-    return gm1 * (W[3] - 0.5 * (W[1] * W[1] + W[2] * W[2]) / W[0]);
-}
-
 // rotate a global-frame state into the local frame of a y-face (theta = pi/2): (rho, rhoV, -rhoU, rhoE)
 template <int DIR>
 DFK_HD void to_local(double W[4]) {
@@ -1084,9 +1083,8 @@ DFK_HD void lf_flux(const GPState& L, const GPState& R, const SchemeConsts& S, d
     lf_flux_sides<false>(L, R, side_state(L.W, S), side_state(R.W, S), S, F, dF);
 }
 
-// DF factor of one Gauss point (Sect. 3.2, Eq. 33) from the Maxwellians of its two local-frame
-// states (maxw_pair, which the GKS flux shares): reciprocal square roots for the sound speeds, one
-// division at the end
+// DF factor (Sect. 3.2, Eq. 33) of a face's two cell averages in its local frame (df_states = 1), from their
+// Maxwellians (maxw_pair): reciprocal square roots for the sound speeds, one division at the end
 DFK_HD double df_alpha_maxw(const Maxw& l, const Maxw& r, const SchemeConsts& S) {
     // 1/c = sqrt(rho / (gamma p)) = sqrt(2/gamma) lambda / sqrt(lambda) on each side
     const double icl = S.r2g * (0.5 * l.tl) * l.isl, icr = S.r2g * (0.5 * r.tl) * r.isl;
