@@ -72,8 +72,8 @@ inline unsigned sweep_blocks(int lx, int ly, int threads = kSweepThreads) { retu
 
 // Which sweep kernels take four threads per item (lines_quad, faces_quad) on a mesh that `beside` meshes of its size
 // are swept at the same time as (itself included, the blocks of a decomposition on their streams): those whose whole
-// items, of all these meshes, are at most two (lines) or three (sides) warps per SM.  A line's 740 FP64 instructions
-// keep an SM's units 6 us per warp, a side's 430 3.5; the quads' 1200 and 620 take 10 and 5, against the 31 and
+// items, of all these meshes, are at most two (lines) or three (sides) warps per SM.  A line's 790 FP64 instructions
+// keep an SM's units 6 us per warp, a side's 440 3.5; the quads' 1250 and 640 take 10 and 5, against the 31 and
 // 19 us that one thread takes however few there are: the quads win below three warps of lines and four of sides.
 // Counting each block of a decomposition by itself costs 14 % in 4 x 4 blocks of 60 x 60 (1374 us a step, 1208 by the
 // warps of eight) and 23 % in 2 x 2 of 50 x 50 (398, 323); blocks of 20 x 20 take the quads either way (433).
@@ -209,10 +209,12 @@ DFK_HD void line_component(const Real f[5], bool acoustic, bool dfL, bool dfR, d
         const Real t1 = s2 - s1, t2 = s3 - s2, t3 = s4 - s3;
         const Real w1 = second_difference_energy(s1, eps), w2 = second_difference_energy(s2, eps);
         const Real w3 = second_difference_energy(s3, eps), w4 = second_difference_energy(s4, eps);
+        // both sides' evaluations without a branch, so that the two chains run side by side (a DF side's is overwritten
+        // below): 20 L-F steps of 40 x 40 2.00 ms, 2.07 with a branch around each
         L = ao_weights<+1>(f[1], f3, s1, s2, s3, w1, w2, w3, fma(0.5, s2, f[1]), t1 + t2, t2 - t1, eps, S);
-        if (!dfL) ao_diff_at_edge<+1>(L, f[1], f3, s2, t1, t2, idn, S, q);
+        ao_diff_at_edge<+1>(L, f[1], f3, s2, t1, t2, idn, S, q);
         R = ao_weights<-1>(f[3], f3, s4, s3, s2, w4, w3, w2, fma(-0.5, s3, f[3]), t2 + t3, t3 - t2, eps, S);
-        if (!dfR) ao_diff_at_edge<-1>(R, f[3], f3, s3, t3, t2, idn, S, q + 2);
+        ao_diff_at_edge<-1>(R, f[3], f3, s3, t3, t2, idn, S, q + 2);
     }
     // the central quadratics there
     const Real hf = 0.5 * f3, baseL = fma(-1.0 / 6.0, s2, hf), baseR = fma(-1.0 / 6.0, s3, -hf);

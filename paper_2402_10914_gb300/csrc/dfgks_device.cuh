@@ -64,7 +64,8 @@ DFK_HD bool in_range(double a, double lo, double hi) { const long long x = dbits
 // these units busy all the time, so their arithmetic runs in this type: x + y is fma(x, 1, y) and x y is
 // fma(x, y, -0), the same bits as the two-operand forms, with 1, -0 and every other constant held as a value
 // the compiler cannot prove uniform.  A product met by a sum fuses, as the compiler fuses plain doubles.
-// Per 400 x 400 step: face lines 0.906 -> 0.807 ms, tangential 1.050 -> 0.934, flux 1.381 -> 1.311.
+// Measured on one state of the kernels, per 400 x 400 step: face lines 0.906 -> 0.807 ms, tangential 1.050 -> 0.934,
+// flux 1.381 -> 1.311.
 #ifdef __CUDACC__
 static __constant__ unsigned kOpaqueZero;      // never written
 #endif
@@ -333,7 +334,9 @@ DFK_HD AO weno_ao(const double q[5], const SchemeConsts& S) { return weno_ao_t(q
 // rounding noise of the jump's size, 2e-10 of data of order 1 beside a jump of 1e6, instead of 1e-15.)
 // These kernels are bound by the two FP64 units of an SM, so what counts is FP64 instructions: about 75 per
 // reconstruction, against 114 from the coefficients of the four polynomials.  Differences also cancel before they
-// are projected.
+// are projected.  790 FP64 instructions per face line and 442 per face side, against 1097 and 575: the face-line
+// kernel takes 0.87 ms per 400 x 400 step, the tangential one 0.94 (1.36 and 1.40 in that form and with two-operand
+// instructions).
 // ------------------------------------------------------------------------------------------
 
 // 1/x for x in [1e-300, 1e300]: the hardware's approximation (2^-20) refined by one third-order
@@ -711,7 +714,7 @@ DFK_HD void finish_moments(const FlowState& s, HalfMom& h) {
 // for the two sides; the reductions below take 11 and 10, and table entries arrive in vector registers.
 // exp(-y): Tang's table-driven method, y = -n ln2/64 - r, a degree-5 polynomial in |r| <= ln2/128 and 2^(n/64)
 // from a table; relative error below 1.2 ulp.  erfcx: see the table.  The tables (0.5 and 12 KB) stay in L1:
-// neighbouring threads read neighbouring rows.  601 -> 514 FP64 instructions per Gauss point; flux kernel
+// neighbouring threads read neighbouring rows.  601 -> 522 FP64 instructions per Gauss point; flux kernel
 // 1.311 -> 1.090 ms per 400 x 400 step.
 #ifdef __CUDACC__
 static __device__ const double kExp2Dev[64] = {
