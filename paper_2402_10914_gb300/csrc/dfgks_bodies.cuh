@@ -72,7 +72,7 @@ inline unsigned sweep_blocks(int lx, int ly, int threads = kSweepThreads) { retu
 
 // Which sweep kernels take four threads per item (lines_quad, faces_quad) on a mesh that `beside` meshes of its size
 // are swept at the same time as (itself included, the blocks of a decomposition on their streams): those whose whole
-// items, of all these meshes, are at most two (lines) or three (sides) warps per SM.  A line's 790 FP64 instructions
+// items, of all these meshes, are at most two (lines) or three (sides) warps per SM.  A line's 785 FP64 instructions
 // keep an SM's units 6 us per warp, a side's 440 3.5; the quads' 1250 and 640 take 10 and 5, against the 31 and
 // 19 us that one thread takes however few there are: the quads win below three warps of lines and four of sides.
 // Counting each block of a decomposition by itself costs 14 % in 4 x 4 blocks of 60 x 60 (1374 us a step, 1208 by the

@@ -334,8 +334,8 @@ DFK_HD AO weno_ao(const double q[5], const SchemeConsts& S) { return weno_ao_t(q
 // rounding noise of the jump's size, 2e-10 of data of order 1 beside a jump of 1e6, instead of 1e-15.)
 // These kernels are bound by the two FP64 units of an SM, so what counts is FP64 instructions: about 75 per
 // reconstruction, against 114 from the coefficients of the four polynomials.  Differences also cancel before they
-// are projected.  790 FP64 instructions per face line and 442 per face side, against 1097 and 575: the face-line
-// kernel takes 0.87 ms per 400 x 400 step, the tangential one 0.94 (1.36 and 1.40 in that form and with two-operand
+// are projected.  785 FP64 instructions per face line and 442 per face side, against 1097 and 575: the face-line
+// kernel takes 0.85 ms per 400 x 400 step, the tangential one 0.94 (1.36 and 1.40 in that form and with two-operand
 // instructions).
 // ------------------------------------------------------------------------------------------
 
